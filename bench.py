@@ -102,7 +102,7 @@ def step_bytes(wl):
     return 3 * Q * e + 2 * rb, 0, 2 * Q * e
 
 
-KERNEL_SOURCES = ("flb_device.cuh", "flb_kernels.cuh", "flb_prec.cuh")
+KERNEL_SOURCES = ("flb_device.cuh", "flb_kernels.cuh", "flb_force.cuh", "flb_prec.cuh")
 
 
 def max_over_ranks(x: float, world: int, device="cuda") -> float:
@@ -165,7 +165,7 @@ def kernel_name(wl):
     if wl["fe"] and wl["fe"].get("model", 0) == 1:
         return "k_step_swift"
     if wl["fe"] and wl["lattice"] == 19:
-        return "k_step_march2" if packed else "k_step_march"
+        return "k_force_collide" if wl["precision"] in ("fp32", "bf16") else "k_step_march"
     return "k_step2" if packed else "k_step"
 
 

@@ -141,8 +141,9 @@ typedef struct {
                             64 KiB guard zones of a fixed byte pattern on both sides,
                             checked by flb_check_guards (a bounds check of the
                             kernels' writes for debugging; default 0) */
-    int z_chunk;         /* D3Q19 non-ideal step (z-marching kernels): planes of z per
-                            thread block.  0 (default): flb_step times candidate
+    int z_chunk;         /* D3Q19 non-ideal step of FP64 storage (z-marching kernel): planes
+                            of z per thread block (FP32 and BF16 storage step in passes
+                            and do not use it).  0 (default): flb_step times candidate
                             lengths on its first steps (three launches each, CUDA
                             events, one host wait on them when done) and keeps
                             the fastest; > 0: that length (at most Z).  The chunk
@@ -255,10 +256,10 @@ int flb_check_guards(flb_ctx* ctx);
  * sums: host, 4*nsteps doubles, written when the call returns (it waits for
  * the context's stream once, at the end; device-addressable page-locked
  * memory is written in place by the reduction, other memory through a copy).  The D3Q19 force-model step with
- * FP32 or BF16 storage and even X forms these sums inside the step kernel
- * (per-block partial sums of the mass deviation and momentum its collision
- * forms from the pulled populations); every other step runs the reduction of
- * flb_conservation before the step.  Errors as flb_step. */
+ * FP32 or BF16 storage forms these sums inside its density pass (per-warp
+ * partial sums of the mass deviation and momentum of the pulled populations,
+ * those of several steps added up by one launch); every other step runs the
+ * reduction of flb_conservation before the step.  Errors as flb_step. */
 int flb_step_sums(flb_ctx* ctx, int nsteps, double* sums);
 
 /* flb_step_sums without the wait: enqueues the nsteps steps and the delivery

@@ -94,6 +94,7 @@ struct flb_ctx {
     void* mu = nullptr;                 // chemical potential (observables)
     void* F = nullptr;                  // force field, 3 components (observables)
     double* partials = nullptr;         // per-block reduction rows
+    unsigned* ticks = nullptr;          // counters of in-kernel reductions
     double* red = nullptr;              // reduced columns (device)
     double2* fft = nullptr;             // FFT work array
     double2* fft_scratch = nullptr;
@@ -176,7 +177,7 @@ int alloc_guarded(flb_ctx* c, void** p, size_t bytes, const char* name)
 void free_all(flb_ctx* c)
 {
     void* ptrs[] = {c->buf[0], c->buf[1], c->drho, c->mu, c->F, c->partials, c->red, c->fft, c->fft_scratch, c->sk_tmp,
-                    c->adj_work, c->adj_rows, c->adj_lam2, c->adj_rb, c->ss_dev, c->h_dev, c->hs_work, c->hs_scratch, c->hs_acc,
+                    c->adj_work, c->adj_rows, c->adj_lam2, c->adj_rb, c->ss_dev, c->ticks, c->h_dev, c->hs_work, c->hs_scratch, c->hs_acc,
                     c->hs_tmp, c->sw_chol, c->sw_work, c->sw_xi};
     for (void* p : ptrs) {
         bool guarded = false;
@@ -238,11 +239,24 @@ const PrecOps* ops_for(int prec)
     }
 }
 
+size_t partial_bytes(const flb_ctx* c)
+{
+    return std::max((size_t)c->ops->partial_rows_max(c->m) * 2 * c->m.Q * sizeof(double), (size_t)1 << 18);
+}
+
 int ensure_partials(flb_ctx* c)
 {
-    int rc = alloc((void**)&c->partials, (size_t)c->ops->partial_rows_max(c->m) * 2 * c->m.Q * sizeof(double));
+    int rc = alloc((void**)&c->partials, partial_bytes(c));
     if (rc) return rc;
     return alloc((void**)&c->red, 64 * sizeof(double));
+}
+
+// Steps whose warp rows (nrow float4 each) and block sums fit the partial-sum
+// buffer together: at least 4 (nrow <= 4 rows_max), at most kSumStepsMax.
+int step_rows_capacity(const flb_ctx* c, int nrow)
+{
+    const size_t per = (size_t)nrow * sizeof(float4) + 4 * flb::kSumBlocksMax * sizeof(double);
+    return (int)std::min<size_t>(flb::kSumStepsMax, std::max<size_t>(1, partial_bytes(c) / per));
 }
 
 // Reduce per-block partial rows into ncol doubles on the host.
@@ -265,7 +279,7 @@ constexpr int kZTuneRounds = 3;
 void ztune_start(flb_ctx* c)
 {
     const HostModel& m = c->m;
-    if (m.zchunk != 0 || m.Q != 19 || !m.nonideal || m.Z <= 16) return;
+    if (m.zchunk != 0 || m.Q != 19 || !m.nonideal || m.Z <= 16 || c->ops->step_in_passes(m)) return;
     std::vector<int> all;
     for (int nc = (m.Z + 39) / 40; nc <= (m.Z + 11) / 12; ++nc) {
         const int len = (m.Z + nc - 1) / nc;
@@ -449,6 +463,22 @@ int flb_create(flb_ctx** out, int lattice, const int dims[3], double omega_shear
         delete c;
         return rc;
     }
+    if (c->ops->step_in_passes(m)) {
+        const size_t nt = flb::kSumStepsMax * sizeof(unsigned);
+        if ((rc = alloc_guarded(c, &c->mu, c->field_bytes(), "chemical potential field")) ||
+            (rc = alloc((void**)&c->ticks, nt))) {
+            free_all(c);
+            delete c;
+            return rc;
+        }
+        const cudaError_t ce = cudaMemsetAsync(c->ticks, 0, nt, c->stream);
+        if (ce != cudaSuccess) {
+            free_all(c);
+            delete c;
+            return fail(FLB_ECUDA, std::string("reduction counters: ") + cudaGetErrorString(ce));
+        }
+        m.mu = c->mu;
+    }
     if (m.nonideal && m.model == 1 && m.kT > 0.0) {
         std::vector<double> chol(3 * (size_t)m.V);
         std::string err;
@@ -521,6 +551,8 @@ int flb_init(flb_ctx* c, const double* rho, const double* u, int thermal_init)
 static int step_impl(flb_ctx* c, int nsteps, double* dev_sums)
 {
     const double m0 = c->m.rho0 * (double)c->m.V;
+    const int nrow = dev_sums ? c->ops->step_row_count(c->m) : 0;
+    const int kmax = nrow > 0 ? step_rows_capacity(c, nrow) : 1;
     for (int t = 0; t < nsteps; ++t) {
         const void* src = c->buf[c->cur];
         void* dst = c->buf[c->cur ^ 1];
@@ -543,17 +575,20 @@ static int step_impl(flb_ctx* c, int nsteps, double* dev_sums)
             FLB_CUDA(cudaEventRecord(c->zt.ev[2 * c->zt.issued], c->stream));
         }
         cudaError_t se;
-        if (dev_sums) {
+        if (dev_sums && nrow > 0) {
+            // the steps' warp rows side by side in the partial-sum buffer, summed
+            // together once it is full
+            float4* rows = (float4*)(c->partials + 4 * (size_t)flb::kSumBlocksMax * kmax);
+            se = c->ops->step_rows(c->m, c->step, src, dst, c->drho, rows + (size_t)(t % kmax) * nrow, c->stream);
+            if (se == cudaSuccess && (t % kmax == kmax - 1 || t == nsteps - 1))
+                se = flb::sum_steps(rows, nrow, t % kmax + 1, c->partials, c->ticks,
+                                    dev_sums + 4 * (size_t)(t - t % kmax), m0, c->stream);
+        } else if (dev_sums) {
+            // this step kernel has no partial sums: reduce the state first
             int nrows = 0;
-            se = c->ops->step_rows(c->m, c->step, src, dst, c->drho, c->partials, &nrows, c->stream);
-            if (se == cudaErrorNotSupported) {
-                // this step kernel has no partial sums: reduce the state first
-                FLB_CUDA(c->ops->cons_partials(c->m, src, c->partials, &nrows, c->stream));
-                FLB_CUDA(flb::sum_columns(c->partials, nrows, 4, dev_sums + 4 * (size_t)t, c->stream, m0));
-                se = c->ops->step(c->m, c->step, src, dst, c->drho, c->stream);
-            } else if (se == cudaSuccess) {
-                se = flb::sum_columns(c->partials, nrows, 4, dev_sums + 4 * (size_t)t, c->stream, m0);
-            }
+            FLB_CUDA(c->ops->cons_partials(c->m, src, c->partials, &nrows, c->stream));
+            FLB_CUDA(flb::sum_columns(c->partials, nrows, 4, dev_sums + 4 * (size_t)t, c->stream, m0));
+            se = c->ops->step(c->m, c->step, src, dst, c->drho, c->stream);
         } else {
             se = c->ops->step(c->m, c->step, src, dst, c->drho, c->stream);
         }

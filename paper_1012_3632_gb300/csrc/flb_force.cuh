@@ -1,0 +1,339 @@
+// flb_force.cuh -- the D3Q19 force-model step with FP32 or BF16 storage, as
+// three launches in packed FP32: density (pull and sum), mu = psi'(rho) -
+// kappa lap rho, then pull + collide with F = -rho grad mu.
+//
+// Every site's density and mu are formed once, and each pass runs at the
+// occupancy that suits it.  One launch that marched columns of sites through z
+// with the densities in shared-memory rings formed them 1.9 and 1.3 times over
+// (tile halos, ring fills), held 12 warps per SM at two barriers a plane and
+// left the chip part empty below 256^3.  Measured, march -> passes, per step:
+// 256^3 FP32 757 -> 698 us (with sums 790 -> 716), BF16 660 -> 597, 128^3 FP32
+// 111 -> 91, 64^3 35 -> 14.6, 129x95x67 84 -> 67.
+//
+// What bounds them at 256^3 FP32: density 196 us, DRAM (80 B/site, 6.8 TB/s);
+// mu 46 us, L1 wavefronts of the row loads; collision 474 us, DRAM (156 B/site,
+// 5.3 TB/s) with issue slots 52 % and the FMA-heavy pipe (integer multiplies of
+// the noise) near as busy; with BF16 storage the issue slots alone.
+//
+// The collision takes the planes in descending order, so that it starts on the
+// lines the density pass read last and leaves the ones the next density pass
+// reads first in L2: 91.0 against 94.8 us at 128^3, 699 against 707 at 256^3.
+#pragma once
+
+#include "flb_kernels.cuh"
+
+namespace flb {
+
+// Blocks of 128 threads over the lattice: rows of 2^lw threads (each N sites
+// along x), 64 >> lw rows in y and two planes in z.  Blocks are numbered along
+// one grid dimension, x fastest (no axis meets a grid limit of 65535).
+struct Tiling {
+    int lw;
+    int ntx, nty, ntz;
+    uint32_t mx, sx, my, sy;  // quotients by ntx and nty: (umulhi(n, m) + n) >> s, n < 2^31
+    unsigned blocks() const { return (unsigned)((long)ntx * nty * ntz); }
+};
+
+inline void fast_div(uint32_t d, uint32_t& m, uint32_t& s)
+{
+    for (s = 0; (1u << s) < d; ++s) {
+    }
+    m = (uint32_t)(((1ull << 32) * ((1ull << s) - d)) / d + 1);
+}
+__device__ __forceinline__ uint32_t fast_quot(uint32_t n, uint32_t m, uint32_t s) { return (__umulhi(n, m) + n) >> s; }
+
+// The row width that covers an X x Y plane with the fewest blocks, the widest
+// of equals (a wide row has the fewest partial sectors).
+inline Tiling make_tiling(int X, int Y, int Z, int N)
+{
+    Tiling t{};
+    long best = 0;
+    for (int lw = 5; lw >= 2; --lw) {
+        const int w = N << lw, h = 64 >> lw, nx = (X + w - 1) / w, ny = (Y + h - 1) / h;
+        if (best && (long)nx * ny >= best) continue;
+        best = (long)nx * ny;
+        t.lw = lw;
+        t.ntx = nx;
+        t.nty = ny;
+    }
+    t.ntz = (Z + 1) / 2;
+    fast_div((uint32_t)t.ntx, t.mx, t.sx);
+    fast_div((uint32_t)t.nty, t.my, t.sy);
+    return t;
+}
+
+// First site (x, y, z) of this thread; REV: the z planes in descending order.
+template <int N, bool REV>
+__device__ __forceinline__ int3 tile_site(const Tiling& t)
+{
+    const uint32_t b = blockIdx.x, r = fast_quot(b, t.mx, t.sx), bx = b - r * t.ntx;
+    const uint32_t rz = fast_quot(r, t.my, t.sy), by = r - rz * t.nty;
+    const int bz = REV ? t.ntz - 1 - (int)rz : (int)rz;
+    const int tx = threadIdx.x & ((1 << t.lw) - 1), row = threadIdx.x >> t.lw, h = 64 >> t.lw;
+    const int ty = row & (h - 1), tz = row >> (6 - t.lw);
+    return make_int3(N * (((int)bx << t.lw) + tx), (int)by * h + ty, 2 * bz + tz);
+}
+
+// A row of a field around the N sites x .. x+N-1: v[0] = f(x-1), v[1..N],
+// v[N+1] = f(x+N) (periodic: xm, xe; x1 the periodic x+1 of unaligned pairs).
+template <int N, bool AL>
+__device__ __forceinline__ void load_row(const float* p, int x, int x1, int xm, int xe, bool ends, float v[N + 2])
+{
+    if constexpr (N == 4) {
+        const float4 m = *reinterpret_cast<const float4*>(p + x);
+        v[1] = m.x;
+        v[2] = m.y;
+        v[3] = m.z;
+        v[4] = m.w;
+    } else if constexpr (AL) {
+        const float2 m = *reinterpret_cast<const float2*>(p + x);
+        v[1] = m.x;
+        v[2] = m.y;
+    } else {
+        v[1] = p[x];
+        v[2] = p[x1];
+    }
+    if (ends) {
+        v[0] = p[xm];
+        v[N + 1] = p[xe];
+    }
+}
+
+// Density: drho(r) = sum_i g*_i(r - c_i).  GX: X % 4 == 0 (4: a quad of sites
+// per thread), X even (2: a pair) or any X (1: a pair by single loads).
+// SUMS: every warp also writes the mass deviation and momentum of its sites
+// (FP32 within the warp).  This pass waits for memory and has the issue slots
+// for it; in the collision the same sums cost 9 % (474 -> 519 us at 256^3).  At
+// least 7 blocks per SM: the sums would take 88 registers and with them the
+// warps that hide the loads (a step with sums 716 us, at 6 blocks 727, 8: 740).
+template <class S, int GX, bool SUMS>
+__global__ void __launch_bounds__(128, 7) k_force_density(const __grid_constant__ Planes<S> P, float* __restrict__ rho,
+                                                       float* __restrict__ rows, int X, int Y, int Z, const Tiling t)
+{
+    using L = D3Q19;
+    using A = Packed<S>;
+    constexpr int N = GX == 4 ? 4 : 2;
+    pdl_begin();
+    const int3 r0 = tile_site<N, false>(t);
+    const int x = r0.x, y = r0.y, z = r0.z, XY = X * Y;
+    const bool in = x < X && y < Y && z < Z;
+    if (!SUMS && !in) return;
+    float v4[4] = {0.f, 0.f, 0.f, 0.f};
+    if (in) {
+        const int zo[3] = {XY * (z == 0 ? Z - 1 : z - 1), XY * z, XY * (z == Z - 1 ? 0 : z + 1)};
+        const int yo[3] = {X * wrap_once(y - 1, Y), X * y, X * wrap_once(y + 1, Y)};
+        const int xm = x == 0 ? X - 1 : x - 1, x1 = x + 1 == X ? 0 : x + 1;
+        const int xl = N == 4 ? x + 3 : x1, xe = xl + 1 == X ? 0 : xl + 1;
+        float* out = rho + (XY * z + X * y + x);
+        if constexpr (GX == 4) {
+            F2 lo[L::Q], hi[L::Q], m[L::Q], n[L::Q];
+#pragma unroll
+            for (int i = 0; i < L::Q; ++i) {
+                const S* r = P.src[i] + (yo[1 - Vel<L>::cy(i)] + zo[1 - Vel<L>::cz(i)]);
+                const float4 v = A::keep4(r + x);
+                const int cx = Vel<L>::cx(i);
+                if (cx == 0) {
+                    lo[i] = F2(v.x, v.y);
+                    hi[i] = F2(v.z, v.w);
+                } else if (cx > 0) {
+                    lo[i] = F2(A::keep1(r + xm), v.x);
+                    hi[i] = F2(v.y, v.z);
+                } else {
+                    lo[i] = F2(v.y, v.z);
+                    hi[i] = F2(v.w, A::keep1(r + xe));
+                }
+            }
+            L::moments(lo, m);
+            L::moments(hi, n);
+            *reinterpret_cast<float4*>(out) = make_float4(m[0].v.x, m[0].v.y, n[0].v.x, n[0].v.y);
+            if constexpr (SUMS) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const F2 c = m[k] + n[k];
+                    v4[k] = c.v.x + c.v.y;
+                }
+            }
+        } else {
+            F2 g[L::Q], m[L::Q];
+#pragma unroll
+            for (int i = 0; i < L::Q; ++i) {
+                const S* r = P.src[i] + (yo[1 - Vel<L>::cy(i)] + zo[1 - Vel<L>::cz(i)]);
+                const int cx = Vel<L>::cx(i);
+                if (cx == 0)
+                    g[i] = GX == 2 ? mk2(A::plain2(r + x)) : F2(A::plain1(r + x), A::plain1(r + x1));
+                else if (cx > 0)
+                    g[i] = F2(A::plain1(r + xm), A::plain1(r + x));
+                else
+                    g[i] = F2(A::plain1(r + x1), A::plain1(r + xe));
+            }
+            L::moments(g, m);
+            const bool two = GX == 2 || x + 1 < X;
+            if constexpr (GX == 2) {
+                *reinterpret_cast<float2*>(out) = m[0].v;
+            } else {
+                out[0] = m[0].v.x;
+                if (two) out[1] = m[0].v.y;
+            }
+            if constexpr (SUMS) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) v4[k] = two ? m[k].v.x + m[k].v.y : m[k].v.x;
+            }
+        }
+    }
+    if constexpr (SUMS) {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        // the sums of four values over a warp in six exchanges: halves keep two, quarters one
+        const bool h16 = lane & 16, h8 = lane & 8;
+        float p = h16 ? v4[2] : v4[0], q = h16 ? v4[3] : v4[1];
+        p += __shfl_xor_sync(0xffffffffu, h16 ? v4[0] : v4[2], 16);
+        q += __shfl_xor_sync(0xffffffffu, h16 ? v4[1] : v4[3], 16);
+        float c = h8 ? q : p;
+        c += __shfl_xor_sync(0xffffffffu, h8 ? p : q, 8);
+        for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+        if ((lane & 7) == 0) rows[4 * (4 * (long)blockIdx.x + warp) + (lane >> 3)] = c;
+    }
+}
+
+// mu = psi'(rho) - kappa lap rho of the sites of two planes z, z + 1: the 12
+// rows of four planes serve both (51 -> 46 us at 256^3 against a plane per
+// thread with its 9 rows).
+template <int GX>
+__global__ void __launch_bounds__(128)
+    k_force_mu(const StepArgs<float> a, const float* __restrict__ rho, float* __restrict__ mu, const Tiling t)
+{
+    using L = D3Q19;
+    constexpr int N = GX == 4 ? 4 : 2;
+    pdl_begin();
+    int3 r0 = tile_site<N, true>(t);
+    const int X = a.X, Y = a.Y, Z = a.Z, XY = X * Y;
+    // the tiling's two planes are rows of threads: here each thread takes a pair of planes
+    const int x = r0.x, y = r0.y, z = 2 * r0.z;
+    if (x >= X || y >= Y || z >= Z) return;
+    const int z1 = z + 1 == Z ? 0 : z + 1, z2 = z1 + 1 == Z ? 0 : z1 + 1;
+    const int zo[4] = {XY * (z == 0 ? Z - 1 : z - 1), XY * z, XY * z1, XY * z2};
+    const int yo[3] = {X * wrap_once(y - 1, Y), X * y, X * wrap_once(y + 1, Y)};
+    const int xm = x == 0 ? X - 1 : x - 1, x1 = x + 1 == X ? 0 : x + 1;
+    const int xl = N == 4 ? x + 3 : x1, xe = xl + 1 == X ? 0 : xl + 1;
+    float r[4][3][N + 2];  // rows (plane, dy)
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int dy = 0; dy < 3; ++dy)
+            load_row<N, GX != 1>(rho + (yo[dy] + zo[k]), x, x1, xm, xe, dy == 1 || k == 1 || k == 2, r[k][dy]);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        float out[N];
+#pragma unroll
+        for (int k = 0; k < N; k += 2) {
+            // sum_i w_i (rho_i - rho) = (1/18) (axis sum) + (1/36) (edge sum) - (2/3) rho
+            // (the Laplacian is 6 times it)
+            F2 sax(0.f), sed(0.f);
+#pragma unroll
+            for (int i = 1; i < L::Q; ++i) {
+                const float* w = r[h + 1 + Vel<L>::cz(i)][1 + Vel<L>::cy(i)] + (k + 1 + Vel<L>::cx(i));
+                if (i < 7)
+                    sax += F2(w[0], w[1]);
+                else
+                    sed += F2(w[0], w[1]);
+            }
+            const F2 rc(r[h + 1][1][k + 1], r[h + 1][1][k + 2]);
+            const F2 lap = (1.0f / 18.0f) * sax + (1.0f / 36.0f) * sed - (2.0f / 3.0f) * rc;
+            const F2 d = rc + a.rho0_minus_rhoc;
+            const F2 m = d * (a.A + a.B * (d * d)) - (6.0f * a.kappa) * lap;
+            out[k] = m.v.x;
+            out[k + 1] = m.v.y;
+        }
+        if (h == 1 && z + 1 == Z) return;
+        float* o = mu + (zo[1 + h] + X * y + x);
+        if constexpr (N == 4) {
+            *reinterpret_cast<float4*>(o) = make_float4(out[0], out[1], out[2], out[3]);
+        } else if constexpr (GX == 2) {
+            *reinterpret_cast<float2*>(o) = make_float2(out[0], out[1]);
+        } else {
+            o[0] = out[0];
+            if (x + 1 < X) o[1] = out[1];
+        }
+    }
+}
+
+// Pull, collide with F = -rho grad mu and store, a site pair per thread.  AL:
+// X even.  TOTAL: psi is the total bulk free energy, F gains cs^2 grad rho
+// (read from the density field).  4 blocks per SM: 128 registers; 5 (96, 72
+// bytes spilled) measured 474 -> 480 us at 256^3.
+template <class S, bool AL, bool TOTAL>
+__global__ void __launch_bounds__(128, 4)
+    k_force_collide(const StepArgs<float> a, const __grid_constant__ Planes<S> P, const float* __restrict__ rho,
+                    const float* __restrict__ mu, const Tiling t)
+{
+    using L = D3Q19;
+    using A = Packed<S>;
+    pdl_begin();
+    const int3 r0 = tile_site<2, true>(t);
+    const int x = r0.x, y = r0.y, z = r0.z, X = a.X, Y = a.Y, Z = a.Z, XY = X * Y;
+    if (x >= X || y >= Y || z >= Z) return;
+    const int xm = x == 0 ? X - 1 : x - 1, x1 = x + 1 == X ? 0 : x + 1, xe = x1 + 1 == X ? 0 : x1 + 1;
+    const int yo[3] = {X * wrap_once(y - 1, Y), X * y, X * wrap_once(y + 1, Y)};
+    const int zo[3] = {XY * (z == 0 ? Z - 1 : z - 1), XY * z, XY * (z == Z - 1 ? 0 : z + 1)};
+    F2 g[L::Q];
+#pragma unroll
+    for (int i = 0; i < L::Q; ++i) {
+        const S* r = P.src[i] + (yo[1 - Vel<L>::cy(i)] + zo[1 - Vel<L>::cz(i)]);
+        const int cx = Vel<L>::cx(i);
+        if (cx == 0)
+            g[i] = AL ? mk2(A::stream2(r + x)) : F2(A::stream1(r + x), A::stream1(r + x1));
+        else if (cx > 0)
+            g[i] = F2(A::stream1(r + xm), A::stream1(r + x));
+        else
+            g[i] = F2(A::stream1(r + x1), A::stream1(r + xe));
+    }
+    // sum_i w_i c_i f_i (a gradient / 3) from the differences f(c) - f(-c) of
+    // the nine velocity pairs (2p-1, 2p): axis pairs weigh 1/18, edge pairs
+    // 1/36; pairs 4..9: (1,1,0) (1,-1,0) (1,0,1) (1,0,-1) (0,1,1) (0,1,-1)
+    auto grad = [&](const float* f, F2& gx, F2& gy, F2& gz) {
+        float r[3][3][4];
+#pragma unroll
+        for (int dz = 0; dz < 3; ++dz)
+#pragma unroll
+            for (int dy = 0; dy < 3; ++dy)
+                load_row<2, AL>(f + (yo[dy] + zo[dz]), x, x1, xm, xe, dy == 1 || dz == 1, r[dz][dy]);
+        F2 dp[10];
+#pragma unroll
+        for (int k = 1; k <= 9; ++k) {
+            const int i = 2 * k - 1;
+            const float* u = r[1 + Vel<L>::cz(i)][1 + Vel<L>::cy(i)] + (1 + Vel<L>::cx(i));
+            const float* w = r[1 - Vel<L>::cz(i)][1 - Vel<L>::cy(i)] + (1 - Vel<L>::cx(i));
+            dp[k] = F2(u[0], u[1]) - F2(w[0], w[1]);
+        }
+        gx = (1.0f / 18.0f) * dp[1] + (1.0f / 36.0f) * ((dp[4] + dp[5]) + (dp[6] + dp[7]));
+        gy = (1.0f / 18.0f) * dp[2] + (1.0f / 36.0f) * ((dp[4] - dp[5]) + (dp[8] + dp[9]));
+        gz = (1.0f / 18.0f) * dp[3] + (1.0f / 36.0f) * ((dp[6] - dp[7]) + (dp[8] - dp[9]));
+    };
+    F2 gx, gy, gz;
+    grad(mu, gx, gy, gz);
+    // the density of the pulled populations, as k_force_density sums it
+    F2 m[L::Q];
+    L::moments(g, m);
+    const F2 pre = -3.0f * (a.c.rho0 + m[0]);
+    F2 fx = pre * gx, fy = pre * gy, fz = pre * gz;
+    if constexpr (TOTAL) {
+        F2 px, py, pz;
+        grad(rho, px, py, pz);
+        fx += px;
+        fy += py;
+        fz += pz;
+    }
+    const int site = x + X * y + XY * z;
+    const bool two = AL || x + 1 < X;
+    L::collide(g, fx, fy, fz, a.c, (uint32_t)site, a.c.step);
+#pragma unroll
+    for (int i = 0; i < L::Q; ++i) {
+        if constexpr (AL) {
+            A::store2(P.dst[i] + site, g[i].v);
+        } else {
+            A::store1(P.dst[i] + site, g[i].v.x);
+            if (two) A::store1(P.dst[i] + site + 1, g[i].v.y);
+        }
+    }
+}
+
+}  // namespace flb

@@ -44,6 +44,7 @@ struct HostModel {
     uint32_t replica;
     int noise_local;
     int zchunk = 0;  // z-marching kernels: planes per block (0: the built-in default)
+    void* mu = nullptr;  // force-model step in passes: the context's chemical potential field
 };
 
 // Kernels whose code depends on the compute/storage type.  Pointers are device
@@ -73,27 +74,55 @@ struct PrecOps {
     cudaError_t (*mode_field)(const HostModel&, const void* src, int mode, void* out, bool fp32, cudaStream_t);
     int (*partial_rows_max)(const HostModel&);
     int (*step_needs_density)(const HostModel&);
+    int (*step_in_passes)(const HostModel&);  // the step uses the density and mu fields itself
     // pre-collision deviations in the storage type, [i][s], to / from a device buffer
     cudaError_t (*pull_state)(const HostModel&, const void* src, void* out, cudaStream_t);
     cudaError_t (*push_state)(const HostModel&, const void* in, void* dst, cudaStream_t);
     // pre-collision populations f_i at n sites (device list), out[i*n + k]
     cudaError_t (*get_sites)(const HostModel&, const void* src, const long long* sites, int n, double* out,
                              cudaStream_t);
-    // the step, also writing *nrows rows of 4 partial sums (mass deviation,
-    // momentum) of the state it steps from; cudaErrorNotSupported (nothing
-    // launched) where the step kernel does not provide them
+    // float4 rows of mass deviation and momentum that step_rows writes (the sums
+    // over warps of the state it steps from); 0: the step does not provide them
+    int (*step_row_count)(const HostModel&);
     cudaError_t (*step_rows)(const HostModel&, uint64_t step, const void* src, void* dst, const void* drho,
-                             double* rows, int* nrows, cudaStream_t);
+                             float4* rows, cudaStream_t);
 };
 
 const PrecOps& ops_fp64();
 const PrecOps& ops_fp32();
 const PrecOps& ops_bf16();
 
+// Launch a kernel that begins with pdl_begin() on a stream: it may start while
+// the kernel before it drains (programmatic dependent launch), which hides the
+// launch latency between the kernels of a step.
+template <class... P, class... A>
+cudaError_t launch_chain(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args)
+{
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kernel, P(args)...);
+}
+
 // Deterministic column sums: out[c] = sum_r partials[r*ncol + c], plus add0
 // on column 0 (flb_fft.cu).
 cudaError_t sum_columns(const double* partials, int nrows, int ncol, double* out, cudaStream_t s,
                         double add0 = 0.0);
+
+// Sums of k steps' warp rows (flb_fft.cu): rows holds k times nrows float4 rows
+// (mass deviation and momentum); out[4 i ..] receives the sums of step i's, the
+// mass with add0.  part: kSumBlocksMax k doubles x 4, ticks: k counters that are
+// zero between launches.
+cudaError_t sum_steps(const float4* rows, int nrows, int k, double* part, unsigned* ticks, double* out, double add0,
+                      cudaStream_t s);
+constexpr int kSumBlocksMax = 64;  // blocks per step
+constexpr int kSumStepsMax = 16;   // steps summed by one launch
 
 // True when an axis of length L is transformed by the in-place mixed-radix FFT
 // (L a product of 2, 3 and 5, at most 4096); other lengths need `scratch`.

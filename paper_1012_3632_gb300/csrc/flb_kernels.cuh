@@ -21,6 +21,16 @@
 
 namespace flb {
 
+// Programmatic dependent launch: a kernel launched with launch_chain may start
+// while the kernel before it on the stream drains.  pdl_begin lets the next
+// one do the same and waits until everything before this kernel is complete
+// and visible; it comes before any access to memory.
+__device__ __forceinline__ void pdl_begin()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // Indices of the 3x3x3 neighbourhood of (x, y, z) on a periodic X*Y*Z lattice:
 // xv[1+dx] + rb[1+dy][1+dz] is the site index of (x+dx, y+dy, z+dz).
 struct Nbhd {
@@ -167,6 +177,7 @@ struct Packed<float> {
     static __device__ __forceinline__ float2 plain2(const float* p) { return *reinterpret_cast<const float2*>(p); }
     static __device__ __forceinline__ float plain1(const float* p) { return *p; }
     static __device__ __forceinline__ void store2(float* p, float2 v) { __stcs(reinterpret_cast<float2*>(p), v); }
+    static __device__ __forceinline__ void store1(float* p, float v) { __stcs(p, v); }
 };
 template <>
 struct Packed<__nv_bfloat16> {
@@ -208,6 +219,7 @@ struct Packed<__nv_bfloat16> {
         const __nv_bfloat162 b = __float22bfloat162_rn(v);
         __stcs(reinterpret_cast<unsigned int*>(p), *reinterpret_cast<const unsigned int*>(&b));
     }
+    static __device__ __forceinline__ void store1(B* p, float v) { store_stream<float, B>(p, v); }
 };
 
 // ---------------------------------------------------------------------------
@@ -631,254 +643,6 @@ __global__ void __launch_bounds__(TX* TY, MINB)
         ra = ra1;
         mb = mb1;
         zc = zc == Z - 1 ? 0 : zc + 1;
-    }
-}
-
-
-// ---------------------------------------------------------------------------
-// Packed-FP32 form of k_step_march (FP32 or BF16 storage S): each thread owns
-// the two sites (x, x+1) of its column pair, and every stage (density gather,
-// mu, F, collision) works on site pairs with FADD2/FMUL2/FFMA2.  X must be
-// even.  Same algorithm and ring layout as k_step_march; the density and mu
-// planes are stored as float2 pairs.  GX = 4 (X % 4 == 0): the density gather
-// works on quads of sites, one 4-element load per direction plus one
-// 1-element load for c_x = +-1, and the density plane starts at x = xb - 4 so
-// that its quads stay aligned; GX = 2: it works on pairs and starts at
-// xb - 2.  Excess free energy only (pgrad = 0): the total-free-energy force
-// runs through k_step_march.
-// ---------------------------------------------------------------------------
-// SUMS: the block also adds up the mass deviation and the momentum of the
-// state it steps from -- sum_i g_i and sum_i c_i g_i of each collided site's
-// pulled populations, the first moments its collision forms -- and writes
-// them as one row of 4 doubles (rows[block * 4 + 0..3]; FP32 within a warp,
-// FP64 above).
-template <class S, int TXT, int TY, int MINB, int GX, bool SUMS = false>
-__global__ void __launch_bounds__(TXT* TY, MINB)
-    k_step_march2(const StepArgs<float> a, const __grid_constant__ Planes<S> P, double* __restrict__ rows)
-{
-    using A = Packed<S>;
-    F2 sum_r(0.f), sum_jx(0.f), sum_jy(0.f), sum_jz(0.f);
-    using L = D3Q19;
-    constexpr bool QUAD = GX == 4;
-    constexpr int NT = TXT * TY;
-    constexpr int OX = QUAD ? 4 : 2;                           // density plane starts at x = xb - OX
-    constexpr int RY = TY + 4;                                 // density rows (tile + 2 halo)
-    constexpr int RX = 2 * TXT + 2 * OX;                       // density floats per row
-    constexpr int RXG = RX / GX, RPG = RXG * RY;               // gather items (pairs or quads) per plane
-    constexpr int MXP = TXT + 1, MY = TY + 2, MPP = MXP * MY;  // mu pairs per plane (tile + 1 halo)
-    constexpr int MX = 2 * MXP;                                // mu floats per row
-    __shared__ __align__(16) float srho[5][RX * RY];
-    __shared__ __align__(16) float smu[3][MPP * 2];
-    const int tid = threadIdx.x + TXT * threadIdx.y;
-    const int X = a.X, Y = a.Y, Z = a.Z;
-    const int XY = X * Y;
-    const int xb = blockIdx.x * 2 * TXT, yb = blockIdx.y * TY, zb = blockIdx.z * a.nzc;
-    const int nz = min(a.nzc, Z - zb);
-    const bool small = X < RX || Y < RY;
-
-    // gather items of this thread (first site gx, a multiple of GX): the sites
-    // gx - 1, gx and gx + GX after periodic wrap, and the rows gy - 1, gy, gy + 1
-    constexpr int NRH = (RPG + NT - 1) / NT;
-    int hx[NRH][3], hy[NRH][3];
-#pragma unroll
-    for (int h = 0; h < NRH; ++h) {
-        const int e = min(tid + h * NT, RPG - 1);
-        const int gx0 = xb - OX + GX * (e % RXG), gy0 = yb - 2 + e / RXG;
-        const int gx = small ? wrap_any(gx0, X) : wrap_once(gx0, X);
-        const int gy = small ? wrap_any(gy0, Y) : wrap_once(gy0, Y);
-        hx[h][0] = gx == 0 ? X - 1 : gx - 1;
-        hx[h][1] = gx;
-        hx[h][2] = gx + GX == X ? 0 : gx + GX;
-        hy[h][0] = X * wrap_once(gy - 1, Y);
-        hy[h][1] = X * gy;
-        hy[h][2] = X * wrap_once(gy + 1, Y);
-    }
-    constexpr int NMU = (MPP + NT - 1) / NT;
-    int mc[NMU];  // float offset of the first site of a mu pair in the density plane
-#pragma unroll
-    for (int j = 0; j < NMU; ++j) {
-        const int e = min(tid + j * NT, MPP - 1);
-        mc[j] = 2 * (e % MXP) + OX - 1 + RX * (e / MXP + 1);
-    }
-
-    const int x = xb + 2 * threadIdx.x, y = yb + threadIdx.y;
-    const int cm = 2 * threadIdx.x + 1 + MX * (threadIdx.y + 1);   // first site in the mu plane
-    const int cr = 2 * threadIdx.x + OX + RX * (threadIdx.y + 2);  // first site in the density plane
-    int ra = 3, mb = 2;
-    int zc = wrap_any(zb - 2, Z);
-#pragma unroll 1
-    for (int k = -4; k < nz; ++k) {
-        const int ra1 = ra == 4 ? 0 : ra + 1, ra2 = ra1 == 4 ? 0 : ra1 + 1;
-        const int mb1 = mb == 2 ? 0 : mb + 1, mb2 = mb1 == 2 ? 0 : mb1 + 1;
-        // (1) density of plane zb+k+2, tile + 2 halo
-        {
-            const int zo[3] = {XY * (zc == 0 ? Z - 1 : zc - 1), XY * zc, XY * (zc == Z - 1 ? 0 : zc + 1)};
-            float* out = srho[ra2];
-#pragma unroll
-            for (int h = 0; h < NRH; ++h) {
-                const int e = tid + h * NT;
-                if (e < RPG) {
-                    if constexpr (QUAD) {
-                        // sites gx .. gx+3: pulls from gx-1 .. gx+4
-                        F2 glo[L::Q], ghi[L::Q], m[L::Q];
-#pragma unroll
-                        for (int i = 0; i < L::Q; ++i) {
-                            const S* p = P.src[i] + hy[h][1 - Vel<L>::cy(i)] + zo[1 - Vel<L>::cz(i)];
-                            const float4 v = A::keep4(p + hx[h][1]);
-                            const int cx = Vel<L>::cx(i);
-                            if (cx == 0) {
-                                glo[i] = F2(v.x, v.y);
-                                ghi[i] = F2(v.z, v.w);
-                            } else if (cx > 0) {
-                                glo[i] = F2(A::keep1(p + hx[h][0]), v.x);
-                                ghi[i] = F2(v.y, v.z);
-                            } else {
-                                glo[i] = F2(v.y, v.z);
-                                ghi[i] = F2(v.w, A::keep1(p + hx[h][2]));
-                            }
-                        }
-                        L::moments(glo, m);
-                        const float2 lo = m[0].v;
-                        L::moments(ghi, m);
-                        *reinterpret_cast<float4*>(out + 4 * e) = make_float4(lo.x, lo.y, m[0].v.x, m[0].v.y);
-                    } else {
-                        // sites gx, gx+1: pulls from gx-1 .. gx+2
-                        F2 g[L::Q], m[L::Q];
-#pragma unroll
-                        for (int i = 0; i < L::Q; ++i) {
-                            const S* p = P.src[i] + hy[h][1 - Vel<L>::cy(i)] + zo[1 - Vel<L>::cz(i)];
-                            const int cx = Vel<L>::cx(i);
-                            if (cx == 0)
-                                g[i] = mk2(A::plain2(p + hx[h][1]));
-                            else if (cx > 0)
-                                g[i] = F2(A::plain1(p + hx[h][0]), A::plain1(p + hx[h][1]));
-                            else
-                                g[i] = F2(A::plain1(p + hx[h][1] + 1), A::plain1(p + hx[h][2]));
-                        }
-                        L::moments(g, m);
-                        *reinterpret_cast<float2*>(out + 2 * e) = m[0].v;
-                    }
-                }
-            }
-        }
-        __syncthreads();
-        // (2) mu pairs of plane zb+k+1, tile + 1 halo
-        if (k >= -2) {
-            const float* rm = srho[ra];
-            const float* r0 = srho[ra1];
-            const float* rp = srho[ra2];
-            float* out = smu[mb2];
-#pragma unroll
-            for (int j = 0; j < NMU; ++j) {
-                const int e = tid + j * NT;
-                if (e < MPP) {
-                    const int c = mc[j];
-                    const F2 rc = F2(r0[c], r0[c + 1]);
-                    // sum_i w_i (rho_i - rho) = (1/18) (axis sum) + (1/36) (edge sum) - (2/3) rho
-                    // (the Laplacian is 6 times it)
-                    F2 sax(0.f), sed(0.f);
-#pragma unroll
-                    for (int i = 1; i < L::Q; ++i) {
-                        const int cz = Vel<L>::cz(i);
-                        const float* pl = cz > 0 ? rp : (cz < 0 ? rm : r0);
-                        // c is odd: pairs at c + cx are aligned only for cx = +-1
-                        const int o = c + Vel<L>::cx(i) + RX * Vel<L>::cy(i);
-                        const F2 v = Vel<L>::cx(i) != 0 ? mk2(*reinterpret_cast<const float2*>(pl + o))
-                                                        : F2(pl[o], pl[o + 1]);
-                        if (i < 7)
-                            sax += v;
-                        else
-                            sed += v;
-                    }
-                    const F2 lap = (1.0f / 18.0f) * sax + (1.0f / 36.0f) * sed - (2.0f / 3.0f) * rc;
-                    const F2 d = rc + a.rho0_minus_rhoc;
-                    const F2 mu = d * (a.A + a.B * (d * d)) - (6.0f * a.kappa) * lap;
-                    out[2 * e] = mu.v.x;
-                    out[2 * e + 1] = mu.v.y;
-                }
-            }
-        }
-        __syncthreads();
-        // (3) collide the pair of plane zb+k with F = -rho grad mu
-        if (k >= 0 && x < X && y < Y) {
-            const int z = zb + k;
-            const float* mlo = smu[mb];
-            const float* mmid = smu[mb1];
-            const float* mhi = smu[mb2];
-            // sum_i w_i c_i mu_i (grad mu / 3; F = -3 rho times it) from the
-            // differences mu(c) - mu(-c) of the nine velocity pairs (2p-1, 2p):
-            // axis pairs weigh 1/18, edge pairs 1/36
-            F2 dp[10];
-#pragma unroll
-            for (int q = 1; q <= 9; ++q) {
-                F2 v2[2];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int i = 2 * q - 1 + h;
-                    const int cz = Vel<L>::cz(i);
-                    const float* pl = cz > 0 ? mhi : (cz < 0 ? mlo : mmid);
-                    const int o = cm + Vel<L>::cx(i) + MX * Vel<L>::cy(i);
-                    v2[h] = Vel<L>::cx(i) != 0 ? mk2(*reinterpret_cast<const float2*>(pl + o)) : F2(pl[o], pl[o + 1]);
-                }
-                dp[q] = v2[0] - v2[1];
-            }
-            // pairs 4..9: (1,1,0) (1,-1,0) (1,0,1) (1,0,-1) (0,1,1) (0,1,-1)
-            const F2 gx = (1.0f / 18.0f) * dp[1] + (1.0f / 36.0f) * ((dp[4] + dp[5]) + (dp[6] + dp[7]));
-            const F2 gy = (1.0f / 18.0f) * dp[2] + (1.0f / 36.0f) * ((dp[4] - dp[5]) + (dp[8] + dp[9]));
-            const F2 gz = (1.0f / 18.0f) * dp[3] + (1.0f / 36.0f) * ((dp[6] - dp[7]) + (dp[8] - dp[9]));
-            const F2 rho = a.c.rho0 + mk2(*reinterpret_cast<const float2*>(srho[ra] + cr));
-            const F2 pre = -3.0f * rho;
-            // pull the pair (its lines were fetched by the gather of this plane;
-            // plain loads: measured faster than the last-use or evict-first hints)
-            const int xm = x == 0 ? X - 1 : x - 1, x2 = x + 2 == X ? 0 : x + 2;
-            const int yv[3] = {wrap_once(y - 1, Y), y, wrap_once(y + 1, Y)};
-            const int zv[3] = {XY * wrap_once(z - 1, Z), XY * z, XY * wrap_once(z + 1, Z)};
-            F2 g[L::Q];
-#pragma unroll
-            for (int i = 0; i < L::Q; ++i) {
-                const S* p = P.src[i] + X * yv[1 - Vel<L>::cy(i)] + zv[1 - Vel<L>::cz(i)];
-                const int cx = Vel<L>::cx(i);
-                if (cx == 0)
-                    g[i] = mk2(A::plain2(p + x));
-                else if (cx > 0)
-                    g[i] = F2(A::plain1(p + xm), A::plain1(p + x));
-                else
-                    g[i] = F2(A::plain1(p + x + 1), A::plain1(p + x2));
-            }
-            const int s = x + X * y + XY * z;
-            if constexpr (SUMS) {
-                // the pre-collision mass deviation and momentum the collision forms
-                F2 first[4];
-                L::collide(g, pre * gx, pre * gy, pre * gz, a.c, (uint32_t)s, a.c.step, first);
-                sum_r += first[0];
-                sum_jx += first[1];
-                sum_jy += first[2];
-                sum_jz += first[3];
-            } else {
-                L::collide(g, pre * gx, pre * gy, pre * gz, a.c, (uint32_t)s, a.c.step);
-            }
-#pragma unroll
-            for (int i = 0; i < L::Q; ++i) A::store2(P.dst[i] + s, g[i].v);
-        }
-        ra = ra1;
-        mb = mb1;
-        zc = zc == Z - 1 ? 0 : zc + 1;
-    }
-    if constexpr (SUMS) {
-        __shared__ double red[NT / 32][4];
-        float v[4] = {sum_r.v.x + sum_r.v.y, sum_jx.v.x + sum_jx.v.y, sum_jy.v.x + sum_jy.v.y,
-                      sum_jz.v.x + sum_jz.v.y};
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-            for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-        if ((tid & 31) == 0)
-            for (int k = 0; k < 4; ++k) red[tid >> 5][k] = (double)v[k];
-        __syncthreads();
-        if (tid < 4) {
-            double acc = 0.0;
-            for (int w = 0; w < NT / 32; ++w) acc += red[w][tid];
-            rows[4 * (blockIdx.x + (long)gridDim.x * (blockIdx.y + (long)gridDim.y * blockIdx.z)) + tid] = acc;
-        }
     }
 }
 

@@ -38,12 +38,8 @@
 #ifndef FLB_STEP2_MINB_BF16
 #define FLB_STEP2_MINB_BF16 4
 #endif
-#ifndef FLB_MARCH2_MINB
-#define FLB_MARCH2_MINB 3
-#endif
-#ifndef FLB_MARCH2_TY
-#define FLB_MARCH2_TY 8
-#endif
+
+#include "flb_force.cuh"
 
 namespace flb {
 
@@ -490,20 +486,68 @@ struct Prec {
             a, make_planes<S>(src, dst, L::Q, m.V), (const R*)drho);
         return cudaGetLastError();
     }
+    // The D3Q19 force-model step of FP32 and BF16 storage (flb_force.cuh).
+    static int step_in_passes(const HostModel& m) { return kPackedStorage && m.Q == 19 && m.nonideal; }
+    static int gather_width(const HostModel& m) { return m.X % 4 == 0 ? 4 : m.X % 2 == 0 ? 2 : 1; }
+    // density: quads of sites per thread, or pairs
+    static Tiling density_tiling(const HostModel& m)
+    {
+        return make_tiling(m.X, m.Y, m.Z, gather_width(m) == 4 ? 4 : 2);
+    }
+    static int step_row_count(const HostModel& m)
+    {
+        return step_in_passes(m) ? 4 * (int)density_tiling(m).blocks() : 0;  // one per warp
+    }
+    static cudaError_t step_force(const HostModel& m, uint64_t step, const void* src, void* dst, float* rho,
+                                  float* rows, cudaStream_t st)
+    {
+        const StepArgs<R> a = make_args<D3Q19, R>(m, step);
+        const Planes<S> pl = make_planes<S>(src, dst, 19, m.V);
+        float* mu = (float*)m.mu;
+        const float* crho = rho;
+        const float* cmu = mu;
+        const int gx = gather_width(m);
+        const Tiling tc = make_tiling(m.X, m.Y, m.Z, 2), td = density_tiling(m);  // collision: site pairs
+        const Tiling tm = make_tiling(m.X, m.Y, (m.Z + 1) / 2, gx == 4 ? 4 : 2);  // mu: two planes per thread
+        auto grid = [](const Tiling& t) { return dim3(t.blocks()); };
+        const dim3 b(128);
+        auto fields = [&](auto G) {
+            constexpr int GX = decltype(G)::value;
+            const cudaError_t e =
+                rows ? launch_chain(k_force_density<S, GX, true>, grid(td), b, st, pl, rho, rows, m.X, m.Y, m.Z, td)
+                     : launch_chain(k_force_density<S, GX, false>, grid(td), b, st, pl, rho, rows, m.X, m.Y, m.Z, td);
+            return e != cudaSuccess ? e : launch_chain(k_force_mu<GX>, grid(tm), b, st, a, crho, mu, tm);
+        };
+        const cudaError_t e = gx == 4   ? fields(std::integral_constant<int, 4>{})
+                              : gx == 2 ? fields(std::integral_constant<int, 2>{})
+                                        : fields(std::integral_constant<int, 1>{});
+        if (e != cudaSuccess) return e;
+        auto collide = [&](auto AL, auto TOTAL) {
+            return launch_chain(k_force_collide<S, decltype(AL)::value, decltype(TOTAL)::value>,
+                                grid(tc), b, st, a, pl, crho, cmu, tc);
+        };
+        const std::true_type yes;
+        const std::false_type no;
+        if (gx == 1) return m.total ? collide(no, yes) : collide(no, no);
+        return m.total ? collide(yes, yes) : collide(yes, no);
+    }
     // The step; with rows (non-NULL) also the mass deviation and momentum of
-    // the state it steps from, as *nrows rows of 4 partial sums, where the
-    // step kernel provides them (cudaErrorNotSupported elsewhere, before any
+    // the state it steps from, as step_row_count rows of 4 partial sums, where
+    // the step kernels provide them (cudaErrorNotSupported elsewhere, before any
     // launch).
     static cudaError_t step(const HostModel& m, uint64_t t, const void* src, void* dst, const void* drho,
                             cudaStream_t st)
     {
-        return step_rows(m, t, src, dst, drho, nullptr, nullptr, st);
+        return step_rows(m, t, src, dst, drho, nullptr, st);
     }
     static cudaError_t step_rows(const HostModel& m, uint64_t t, const void* src, void* dst, const void* drho,
-                                 double* rows, int* nrows, cudaStream_t st)
+                                 float4* rows, cudaStream_t st)
     {
-        if (rows && !(kPackedStorage && m.Q == 19 && m.nonideal && m.X % 2 == 0 && FLB_PACKED && !m.total))
-            return cudaErrorNotSupported;
+        if constexpr (kPackedStorage) {
+            // drho: the context's density field, scratch of this step
+            if (step_in_passes(m)) return step_force(m, t, src, dst, (float*)const_cast<void*>(drho), (float*)rows, st);
+        }
+        if (rows) return cudaErrorNotSupported;
         if (m.Q == 9 && m.nonideal && m.model == 1) {
             const StepArgs<R> a = make_args<D2Q9, R>(m, t);
             const dim3 b(32, 8, 1);
@@ -514,30 +558,6 @@ struct Prec {
         }
         if (m.Q == 19) {
             if (m.nonideal) {
-                if constexpr (kPackedStorage) {
-                    if (m.X % 2 == 0 && FLB_PACKED && !m.total) {
-                        constexpr int TXT = 16, TY = FLB_MARCH2_TY;
-                        const StepArgs<R> a = make_args<D3Q19, R>(m, t);
-                        const dim3 b(TXT, TY, 1);
-                        const dim3 g((m.X + 2 * TXT - 1) / (2 * TXT), (m.Y + TY - 1) / TY,
-                                     (m.Z + a.nzc - 1) / a.nzc);
-                        // density gather by quads of sites when rows hold whole quads
-                        const Planes<S> pl = make_planes<S>(src, dst, 19, m.V);
-                        if (rows) *nrows = (int)(g.x * g.y * g.z);
-                        if (m.X % 4 == 0) {
-                            if (rows)
-                                k_step_march2<S, TXT, TY, FLB_MARCH2_MINB, 4, true><<<g, b, 0, st>>>(a, pl, rows);
-                            else
-                                k_step_march2<S, TXT, TY, FLB_MARCH2_MINB, 4><<<g, b, 0, st>>>(a, pl, nullptr);
-                        } else {
-                            if (rows)
-                                k_step_march2<S, TXT, TY, FLB_MARCH2_MINB, 2, true><<<g, b, 0, st>>>(a, pl, rows);
-                            else
-                                k_step_march2<S, TXT, TY, FLB_MARCH2_MINB, 2><<<g, b, 0, st>>>(a, pl, nullptr);
-                        }
-                        return cudaGetLastError();
-                    }
-                }
                 constexpr int TX = 32, TY = FLB_MARCH_TY;
                 const StepArgs<R> a = make_args<D3Q19, R>(m, t);
                 const dim3 b(TX, TY, 1);
@@ -732,8 +752,8 @@ struct Prec {
     static const PrecOps& ops()
     {
         static const PrecOps o = {(int)sizeof(S), (int)sizeof(R), density, step, init, get_pop, set_pop, moments,
-                                  mu_force, mode_partials, cons_partials, mode_field, rows, needs_density,
-                                  pull_state, push_state, get_sites, step_rows};
+                                  mu_force, mode_partials, cons_partials, mode_field, rows, needs_density, step_in_passes,
+                                  pull_state, push_state, get_sites, step_row_count, step_rows};
         return o;
     }
 };
