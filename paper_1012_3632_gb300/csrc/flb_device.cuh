@@ -152,16 +152,12 @@ __device__ __forceinline__ void box_muller(uint32_t a, uint32_t b, float& z0, fl
     z0 = -r * cos_approx(w);
     z1 = -r * sin_approx(w);
 }
-__device__ __forceinline__ void box_muller(uint32_t a, uint32_t b, double& z0, double& z1)
-{
-    const double u0 = ((double)a + 0.5) * 2.3283064365386963e-10;
-    const double u1 = ((double)b + 0.5) * 2.3283064365386963e-10;
-    const double r = sqrt(-2.0 * log(u0));
-    double s, c;
-    sincospi(2.0 * u1, &s, &c);
-    z0 = r * c;
-    z1 = r * s;
-}
+
+}  // namespace flb
+
+#include "flb_normal64.cuh"  // box_muller of the FP64 paths
+
+namespace flb {
 
 // Four standard normals from the call (site, step, call | tag << 8, replica).
 template <class R>
