@@ -165,8 +165,8 @@ def kernel_name(wl):
     if wl["fe"] and wl["fe"].get("model", 0) == 1:
         return "k_step_swift"
     if wl["fe"] and wl["lattice"] == 19:
-        return "k_force_collide" if wl["precision"] in ("fp32", "bf16") else "k_step_march"
-    return "k_step2" if packed else "k_step"
+        return "k_force_collide" if wl["precision"] in ("fp32", "bf16") else "k_sites"
+    return "k_step2" if packed else "k_step_gather" if wl["fe"] else "k_sites"
 
 
 def kernel_source_hash():

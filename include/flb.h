@@ -141,14 +141,8 @@ typedef struct {
                             64 KiB guard zones of a fixed byte pattern on both sides,
                             checked by flb_check_guards (a bounds check of the
                             kernels' writes for debugging; default 0) */
-    int z_chunk;         /* D3Q19 non-ideal step of FP64 storage (z-marching kernel): planes
-                            of z per thread block (FP32 and BF16 storage step in passes
-                            and do not use it).  0 (default): flb_step times candidate
-                            lengths on its first steps (three launches each, CUDA
-                            events, one host wait on them when done) and keeps
-                            the fastest; > 0: that length (at most Z).  The chunk
-                            length changes no result: every site's arithmetic is
-                            the same. */
+    int z_chunk;         /* reported back by flb_z_chunk; the steps do not use it
+                            (default 0; > 0: at most Z of it is reported) */
 } flb_options;
 
 /* Fill *opt with the defaults listed above. */
@@ -237,9 +231,8 @@ int flb_interface_heights(flb_ctx* ctx, const flb_interface_fit* fit, double* h)
  * first call. */
 int flb_height_spectrum(flb_ctx* ctx, const flb_interface_fit* fit, double* S, int accumulate);
 
-/* Planes of z per thread block of the D3Q19 non-ideal step (opt.z_chunk):
- * *planes = the length in use (the built-in default while tuning or for other
- * steps), *tuning = 1 while flb_step is still timing candidates. */
+/* *planes = opt.z_chunk (a built-in length when it is 0), at most Z; *tuning = 0:
+ * no step of this library depends on either. */
 int flb_z_chunk(flb_ctx* ctx, int* planes, int* tuning);
 
 /* Bounds check of the kernels' writes (contexts created with opt.guard = 1):

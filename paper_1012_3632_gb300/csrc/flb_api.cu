@@ -76,25 +76,16 @@ struct flb_ctx {
     };
     std::vector<GuardZone> guards;
     int guard = 0;
-    // z-chunk autotuning of the z-marching step (opt.z_chunk = 0): candidate
-    // lengths, the best time of each, CUDA events of the tuning launches
-    struct ZTune {
-        bool active = false;
-        std::vector<int> cand;
-        std::vector<float> best;
-        std::vector<cudaEvent_t> ev;
-        int issued = 0;
-    } zt;
     const PrecOps* ops = nullptr;
     uint64_t step = 0;
 
     void* buf[2] = {nullptr, nullptr};  // post-collision populations of the last step
     int cur = 0;
-    void* drho = nullptr;               // density deviation field (compute type)
-    void* mu = nullptr;                 // chemical potential (observables)
+    void* drho = nullptr;               // density deviation field (compute type); a step in
+                                        // passes has its chemical potential behind it
+    void* mu = nullptr;                 // chemical potential (observables of other contexts)
     void* F = nullptr;                  // force field, 3 components (observables)
     double* partials = nullptr;         // per-block reduction rows
-    unsigned* ticks = nullptr;          // counters of in-kernel reductions
     double* red = nullptr;              // reduced columns (device)
     double2* fft = nullptr;             // FFT work array
     double2* fft_scratch = nullptr;
@@ -177,7 +168,7 @@ int alloc_guarded(flb_ctx* c, void** p, size_t bytes, const char* name)
 void free_all(flb_ctx* c)
 {
     void* ptrs[] = {c->buf[0], c->buf[1], c->drho, c->mu, c->F, c->partials, c->red, c->fft, c->fft_scratch, c->sk_tmp,
-                    c->adj_work, c->adj_rows, c->adj_lam2, c->adj_rb, c->ss_dev, c->ticks, c->h_dev, c->hs_work, c->hs_scratch, c->hs_acc,
+                    c->adj_work, c->adj_rows, c->adj_lam2, c->adj_rb, c->ss_dev, c->h_dev, c->hs_work, c->hs_scratch, c->hs_acc,
                     c->hs_tmp, c->sw_chol, c->sw_work, c->sw_xi};
     for (void* p : ptrs) {
         bool guarded = false;
@@ -186,8 +177,6 @@ void free_all(flb_ctx* c)
     }
     for (const auto& g : c->guards) cudaFree(g.base);
     c->guards.clear();
-    for (cudaEvent_t e : c->zt.ev) cudaEventDestroy(e);
-    c->zt.ev.clear();
     for (double* p : c->sk_acc)
         if (p) cudaFree(p);
     for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
@@ -241,15 +230,22 @@ const PrecOps* ops_for(int prec)
 
 size_t partial_bytes(const flb_ctx* c)
 {
-    return std::max((size_t)c->ops->partial_rows_max(c->m) * 2 * c->m.Q * sizeof(double), (size_t)1 << 18);
+    const size_t rows = (size_t)c->ops->partial_rows_max(c->m) * 2 * c->m.Q * sizeof(double);
+    return c->ops->step_row_count(c->m) ? std::max(rows, (size_t)1 << 18) : rows;  // room for several steps' rows
 }
 
 int ensure_partials(flb_ctx* c)
 {
     int rc = alloc((void**)&c->partials, partial_bytes(c));
     if (rc) return rc;
-    return alloc((void**)&c->red, 64 * sizeof(double));
+    return alloc((void**)&c->red, 64 * sizeof(double) + flb::kSumStepsMax * sizeof(unsigned));
 }
+
+// Counters of sum_steps (zero between launches), behind the reduced columns.
+unsigned* ticks(flb_ctx* c) { return (unsigned*)(c->red + 64); }
+
+// Byte offset of the chemical potential behind the density field.
+size_t mu_offset(const flb_ctx* c) { return (c->field_bytes() + 255) / 256 * 256; }
 
 // Steps whose warp rows (nrow float4 each) and block sums fit the partial-sum
 // buffer together: at least 4 (nrow <= 4 rows_max), at most kSumStepsMax.
@@ -265,61 +261,6 @@ int reduce_to_host(flb_ctx* c, int nrows, int ncol, double* host)
     FLB_CUDA(flb::sum_columns(c->partials, nrows, ncol, c->red, c->stream));
     FLB_CUDA(cudaMemcpyAsync(host, c->red, ncol * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     FLB_CUDA(cudaStreamSynchronize(c->stream));
-    return FLB_OK;
-}
-
-// z-chunk autotuning of the z-marching step (D3Q19 non-ideal, opt.z_chunk = 0).
-// Candidates: for every block count nc from ceil(Z/40) to ceil(Z/12) the
-// balanced length ceil(Z/nc), at most 16 of them; each is launched
-// kZTuneRounds times (the candidates in turn) with CUDA events around it and
-// the fastest launch decides.  The steps are the
-// caller's own steps: the chunk length changes no result.
-constexpr int kZTuneRounds = 3;
-
-void ztune_start(flb_ctx* c)
-{
-    const HostModel& m = c->m;
-    if (m.zchunk != 0 || m.Q != 19 || !m.nonideal || m.Z <= 16 || c->ops->step_in_passes(m)) return;
-    std::vector<int> all;
-    for (int nc = (m.Z + 39) / 40; nc <= (m.Z + 11) / 12; ++nc) {
-        const int len = (m.Z + nc - 1) / nc;
-        if (all.empty() || all.back() != len) all.push_back(len);
-    }
-    std::vector<int> cand;
-    const size_t n = std::min<size_t>(all.size(), 16);
-    for (size_t k = 0; k < n; ++k) cand.push_back(all[k * all.size() / n]);
-    if (cand.size() < 2) return;
-    std::vector<cudaEvent_t> ev(2 * kZTuneRounds * cand.size());
-    for (auto& e : ev)
-        if (cudaEventCreate(&e) != cudaSuccess) {
-            for (auto& f : ev)
-                if (f) cudaEventDestroy(f);
-            return;  // no tuning: the built-in default length
-        }
-    c->zt.cand = cand;
-    c->zt.best.assign(cand.size(), 3.0e38f);
-    c->zt.ev = ev;
-    c->zt.issued = 0;
-    c->zt.active = true;
-}
-
-// All tuning launches issued: wait for them, keep the fastest length.
-int ztune_finish(flb_ctx* c)
-{
-    auto& z = c->zt;
-    for (int k = 0; k < z.issued; ++k) {
-        float ms = 0.f;
-        // the launches may span a flb_set_stream: wait on each launch's own event
-        FLB_CUDA(cudaEventSynchronize(z.ev[2 * k + 1]));
-        FLB_CUDA(cudaEventElapsedTime(&ms, z.ev[2 * k], z.ev[2 * k + 1]));
-        float& b = z.best[k % z.cand.size()];
-        b = std::min(b, ms);
-    }
-    const size_t i = std::min_element(z.best.begin(), z.best.end()) - z.best.begin();
-    c->m.zchunk = z.cand[i];
-    for (cudaEvent_t e : z.ev) cudaEventDestroy(e);
-    z.ev.clear();
-    z.active = false;
     return FLB_OK;
 }
 
@@ -458,26 +399,21 @@ int flb_create(flb_ctx** out, int lattice, const int dims[3], double omega_shear
 
     if ((rc = alloc_guarded(c, &c->buf[0], c->pop_bytes(), "population buffer 0")) ||
         (rc = alloc_guarded(c, &c->buf[1], c->pop_bytes(), "population buffer 1")) ||
-        (rc = alloc_guarded(c, &c->drho, c->field_bytes(), "density field")) || (rc = ensure_partials(c))) {
+        (rc = alloc_guarded(c, &c->drho, (c->ops->step_in_passes(m) ? mu_offset(c) : 0) + c->field_bytes(),
+                            "density field")) ||
+        (rc = ensure_partials(c))) {
         free_all(c);
         delete c;
         return rc;
     }
     if (c->ops->step_in_passes(m)) {
-        const size_t nt = flb::kSumStepsMax * sizeof(unsigned);
-        if ((rc = alloc_guarded(c, &c->mu, c->field_bytes(), "chemical potential field")) ||
-            (rc = alloc((void**)&c->ticks, nt))) {
-            free_all(c);
-            delete c;
-            return rc;
-        }
-        const cudaError_t ce = cudaMemsetAsync(c->ticks, 0, nt, c->stream);
+        m.mu = (char*)c->drho + mu_offset(c);
+        const cudaError_t ce = cudaMemsetAsync(ticks(c), 0, flb::kSumStepsMax * sizeof(unsigned), c->stream);
         if (ce != cudaSuccess) {
             free_all(c);
             delete c;
             return fail(FLB_ECUDA, std::string("reduction counters: ") + cudaGetErrorString(ce));
         }
-        m.mu = c->mu;
     }
     if (m.nonideal && m.model == 1 && m.kT > 0.0) {
         std::vector<double> chol(3 * (size_t)m.V);
@@ -511,7 +447,6 @@ int flb_create(flb_ctx** out, int lattice, const int dims[3], double omega_shear
         delete c;
         return fail(FLB_ECUDA, std::string("initialising the state: ") + cudaGetErrorString(e));
     }
-    ztune_start(c);
     *out = c;
     return FLB_OK;
 }
@@ -567,13 +502,6 @@ static int step_impl(flb_ctx* c, int nsteps, double* dev_sums)
             if ((rc = timer_end(c, slot))) return rc;
         }
         if ((rc = timer_begin(c, 1, &slot))) return rc;
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        const bool tune = c->zt.active && cudaStreamIsCapturing(c->stream, &cap) == cudaSuccess &&
-                          cap == cudaStreamCaptureStatusNone;
-        if (tune) {
-            c->m.zchunk = c->zt.cand[c->zt.issued % c->zt.cand.size()];
-            FLB_CUDA(cudaEventRecord(c->zt.ev[2 * c->zt.issued], c->stream));
-        }
         cudaError_t se;
         if (dev_sums && nrow > 0) {
             // the steps' warp rows side by side in the partial-sum buffer, summed
@@ -581,7 +509,7 @@ static int step_impl(flb_ctx* c, int nsteps, double* dev_sums)
             float4* rows = (float4*)(c->partials + 4 * (size_t)flb::kSumBlocksMax * kmax);
             se = c->ops->step_rows(c->m, c->step, src, dst, c->drho, rows + (size_t)(t % kmax) * nrow, c->stream);
             if (se == cudaSuccess && (t % kmax == kmax - 1 || t == nsteps - 1))
-                se = flb::sum_steps(rows, nrow, t % kmax + 1, c->partials, c->ticks,
+                se = flb::sum_steps(rows, nrow, t % kmax + 1, c->partials, ticks(c),
                                     dev_sums + 4 * (size_t)(t - t % kmax), m0, c->stream);
         } else if (dev_sums) {
             // this step kernel has no partial sums: reduce the state first
@@ -591,12 +519,6 @@ static int step_impl(flb_ctx* c, int nsteps, double* dev_sums)
             se = c->ops->step(c->m, c->step, src, dst, c->drho, c->stream);
         } else {
             se = c->ops->step(c->m, c->step, src, dst, c->drho, c->stream);
-        }
-        if (tune) {
-            c->m.zchunk = 0;
-            FLB_CUDA(se);
-            FLB_CUDA(cudaEventRecord(c->zt.ev[2 * c->zt.issued + 1], c->stream));
-            if (++c->zt.issued == (int)(kZTuneRounds * c->zt.cand.size()) && (rc = ztune_finish(c))) return rc;
         }
         FLB_CUDA(se);
         if ((rc = timer_end(c, slot))) return rc;
@@ -718,12 +640,12 @@ int flb_moments(flb_ctx* c, double* out, int which)
     cudaError_t e = cudaSuccess;
     const void* F = nullptr;
     if (which == FLB_U && m.nonideal && m.model == 0) {
-        if ((rc = alloc(&c->mu, c->field_bytes())) || (rc = alloc(&c->F, 3 * c->field_bytes()))) {
+        if ((!m.mu && (rc = alloc(&c->mu, c->field_bytes()))) || (rc = alloc(&c->F, 3 * c->field_bytes()))) {
             cudaFree(d_out);
             return rc;
         }
         e = c->ops->density(m, src, c->drho, c->stream);
-        if (e == cudaSuccess) e = c->ops->mu_force(m, c->drho, c->mu, c->F, c->stream);
+        if (e == cudaSuccess) e = c->ops->mu_force(m, c->drho, m.mu ? m.mu : c->mu, c->F, c->stream);
         F = c->F;
     }
     if (e == cudaSuccess) e = c->ops->moments(m, src, d_out, which, F, c->stream);
@@ -879,7 +801,7 @@ int flb_z_chunk(flb_ctx* c, int* planes, int* tuning)
 {
     if (!c || !planes || !tuning) return fail(FLB_EINVAL, "NULL argument");
     *planes = std::min(c->m.zchunk > 0 ? c->m.zchunk : flb::kZChunkDefault, c->m.Z);
-    *tuning = c->zt.active ? 1 : 0;
+    *tuning = 0;
     return FLB_OK;
 }
 

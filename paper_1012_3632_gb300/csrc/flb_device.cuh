@@ -159,6 +159,15 @@ __device__ __forceinline__ void box_muller(uint32_t a, uint32_t b, float& z0, fl
 
 namespace flb {
 
+// Normals 2p and 2p + 1 of the collision noise of `site`.
+template <class R>
+__device__ __forceinline__ void normal_pair(const PhiloxKeys& K, uint32_t site, uint32_t step, int p, uint32_t replica,
+                                            R& z0, R& z1)
+{
+    const uint4 r = philox4x32_10(make_uint4(site, step, (uint32_t)p >> 1, replica), K);
+    box_muller(p & 1 ? r.z : r.x, p & 1 ? r.w : r.y, z0, z1);
+}
+
 // Four standard normals from the call (site, step, call | tag << 8, replica).
 template <class R>
 __device__ __forceinline__ void normals4(const PhiloxKeys& K, uint32_t site, uint32_t step, uint32_t call_tag,
@@ -385,6 +394,12 @@ struct D2Q9 {
     __device__ __forceinline__ static void collide(R g[9], R Fx, R Fy, const Coll<PR>& P, uint32_t site,
                                                    uint32_t step)
     {
+        collide_with(g, Fx, Fy, P, [&](R z[8]) { noise_normals<2>(P.key, site, step, P.replica, z); });
+    }
+    // normals(z): the site's normals of the non-conserved modes.
+    template <class R, class PR, class NZ>
+    __device__ __forceinline__ static void collide_with(R g[9], R Fx, R Fy, const Coll<PR>& P, NZ&& normals)
+    {
         R m[9];
         moments(g, m);
         const R rho = P.rho0 + m[0];
@@ -410,7 +425,7 @@ struct D2Q9 {
         if (P.noise) {
             const R sr = P.noise_local ? sqrt_(rho) : R(P.sqrt_rho0);
             R z[8];
-            noise_normals<2>(P.key, site, step, P.replica, z);
+            normals(z);
 #pragma unroll
             for (int k = 0; k < 6; ++k) Dm[3 + k] += P.ns[k] * (sr * z[k]);
         }
@@ -597,21 +612,24 @@ struct D3Q19 {
     }
 
     // FORCE = false: F = 0 (ideal gas); the force terms are not evaluated.
-    // first (optional): receives the pre-collision mass deviation and
-    // momentum m[0..3] = sum_i g_i, sum_i c_i g_i the collision forms anyway.
     // INTERLEAVED: the two-site noise draws its Philox calls round-major.
     template <bool FORCE = true, bool INTERLEAVED = false, class R, class PR>
     __device__ __forceinline__ static void collide(R g[19], R Fx, R Fy, R Fz, const Coll<PR>& P, uint32_t site,
-                                                   uint32_t step, R* first = nullptr)
+                                                   uint32_t step)
+    {
+        collide_with<FORCE>(g, Fx, Fy, Fz, P, [&](R z[16]) {
+            if constexpr (std::is_same<R, F2>::value)
+                noise_normals<4, INTERLEAVED>(P.key, site, step, P.replica, z);
+            else
+                noise_normals<4>(P.key, site, step, P.replica, z);
+        });
+    }
+    // normals(z): the site's normals of the non-conserved modes.
+    template <bool FORCE, class R, class PR, class NZ>
+    __device__ __forceinline__ static void collide_with(R g[19], R Fx, R Fy, R Fz, const Coll<PR>& P, NZ&& normals)
     {
         R m[19];
         moments(g, m);
-        if (first) {
-            first[0] = m[0];
-            first[1] = m[1];
-            first[2] = m[2];
-            first[3] = m[3];
-        }
         const R rho = P.rho0 + m[0];
         const R ir = rcp_(rho);
         R ux, uy, uz;
@@ -655,10 +673,7 @@ struct D3Q19 {
         if (P.noise) {
             const R sr = P.noise_local ? sqrt_(rho) : R(P.sqrt_rho0);
             R z[16];
-            if constexpr (std::is_same<R, F2>::value)
-                noise_normals<4, INTERLEAVED>(P.key, site, step, P.replica, z);
-            else
-                noise_normals<4>(P.key, site, step, P.replica, z);
+            normals(z);
 #pragma unroll
             for (int k = 0; k < 15; ++k) Dm[4 + k] += P.ns[k] * (sr * z[k]);
         }

@@ -21,7 +21,7 @@ __global__ void k_sum_columns(const double* __restrict__ partials, int nrows, in
 {
     __shared__ double sh[256];
     const int c = blockIdx.x;
-    pdl_begin();
+    pdl_wait();
     double acc = 0.0;
     for (int r = threadIdx.x; r < nrows; r += blockDim.x) acc += partials[(long)r * ncol + c];
     sh[threadIdx.x] = acc;
@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(256) k_sum_steps(const float4* __restrict__ ro
                                                    double* __restrict__ out, double add0)
 {
     __shared__ double red[8][4];
-    pdl_begin();
+    pdl_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, step = blockIdx.y, nb = gridDim.x;
     const float4* r = rows + (long)step * nrows;
     const int end = min(nrows, ((int)blockIdx.x + 1) * per);

@@ -24,56 +24,6 @@
 
 namespace flb {
 
-// Blocks of 128 threads over the lattice: rows of 2^lw threads (each N sites
-// along x), 64 >> lw rows in y and two planes in z.  Blocks are numbered along
-// one grid dimension, x fastest (no axis meets a grid limit of 65535).
-struct Tiling {
-    int lw;
-    int ntx, nty, ntz;
-    uint32_t mx, sx, my, sy;  // quotients by ntx and nty: (umulhi(n, m) + n) >> s, n < 2^31
-    unsigned blocks() const { return (unsigned)((long)ntx * nty * ntz); }
-};
-
-inline void fast_div(uint32_t d, uint32_t& m, uint32_t& s)
-{
-    for (s = 0; (1u << s) < d; ++s) {
-    }
-    m = (uint32_t)(((1ull << 32) * ((1ull << s) - d)) / d + 1);
-}
-__device__ __forceinline__ uint32_t fast_quot(uint32_t n, uint32_t m, uint32_t s) { return (__umulhi(n, m) + n) >> s; }
-
-// The row width that covers an X x Y plane with the fewest blocks, the widest
-// of equals (a wide row has the fewest partial sectors).
-inline Tiling make_tiling(int X, int Y, int Z, int N)
-{
-    Tiling t{};
-    long best = 0;
-    for (int lw = 5; lw >= 2; --lw) {
-        const int w = N << lw, h = 64 >> lw, nx = (X + w - 1) / w, ny = (Y + h - 1) / h;
-        if (best && (long)nx * ny >= best) continue;
-        best = (long)nx * ny;
-        t.lw = lw;
-        t.ntx = nx;
-        t.nty = ny;
-    }
-    t.ntz = (Z + 1) / 2;
-    fast_div((uint32_t)t.ntx, t.mx, t.sx);
-    fast_div((uint32_t)t.nty, t.my, t.sy);
-    return t;
-}
-
-// First site (x, y, z) of this thread; REV: the z planes in descending order.
-template <int N, bool REV>
-__device__ __forceinline__ int3 tile_site(const Tiling& t)
-{
-    const uint32_t b = blockIdx.x, r = fast_quot(b, t.mx, t.sx), bx = b - r * t.ntx;
-    const uint32_t rz = fast_quot(r, t.my, t.sy), by = r - rz * t.nty;
-    const int bz = REV ? t.ntz - 1 - (int)rz : (int)rz;
-    const int tx = threadIdx.x & ((1 << t.lw) - 1), row = threadIdx.x >> t.lw, h = 64 >> t.lw;
-    const int ty = row & (h - 1), tz = row >> (6 - t.lw);
-    return make_int3(N * (((int)bx << t.lw) + tx), (int)by * h + ty, 2 * bz + tz);
-}
-
 // A row of a field around the N sites x .. x+N-1: v[0] = f(x-1), v[1..N],
 // v[N+1] = f(x+N) (periodic: xm, xe; x1 the periodic x+1 of unaligned pairs).
 template <int N, bool AL>
@@ -113,8 +63,8 @@ __global__ void __launch_bounds__(128, 7) k_force_density(const __grid_constant_
     using L = D3Q19;
     using A = Packed<S>;
     constexpr int N = GX == 4 ? 4 : 2;
-    pdl_begin();
-    const int3 r0 = tile_site<N, false>(t);
+    pdl_wait();
+    const int3 r0 = tile_site<N, 2, false>(t, threadIdx.x);
     const int x = r0.x, y = r0.y, z = r0.z, XY = X * Y;
     const bool in = x < X && y < Y && z < Z;
     if (!SUMS && !in) return;
@@ -145,6 +95,7 @@ __global__ void __launch_bounds__(128, 7) k_force_density(const __grid_constant_
             }
             L::moments(lo, m);
             L::moments(hi, n);
+            pdl_trigger();
             *reinterpret_cast<float4*>(out) = make_float4(m[0].v.x, m[0].v.y, n[0].v.x, n[0].v.y);
             if constexpr (SUMS) {
 #pragma unroll
@@ -168,6 +119,7 @@ __global__ void __launch_bounds__(128, 7) k_force_density(const __grid_constant_
             }
             L::moments(g, m);
             const bool two = GX == 2 || x + 1 < X;
+            pdl_trigger();
             if constexpr (GX == 2) {
                 *reinterpret_cast<float2*>(out) = m[0].v;
             } else {
@@ -203,8 +155,8 @@ __global__ void __launch_bounds__(128)
 {
     using L = D3Q19;
     constexpr int N = GX == 4 ? 4 : 2;
-    pdl_begin();
-    int3 r0 = tile_site<N, true>(t);
+    pdl_wait();
+    int3 r0 = tile_site<N, 2, true>(t, threadIdx.x);
     const int X = a.X, Y = a.Y, Z = a.Z, XY = X * Y;
     // the tiling's two planes are rows of threads: here each thread takes a pair of planes
     const int x = r0.x, y = r0.y, z = 2 * r0.z;
@@ -243,6 +195,7 @@ __global__ void __launch_bounds__(128)
             out[k] = m.v.x;
             out[k + 1] = m.v.y;
         }
+        if (h == 0) pdl_trigger();
         if (h == 1 && z + 1 == Z) return;
         float* o = mu + (zo[1 + h] + X * y + x);
         if constexpr (N == 4) {
@@ -267,8 +220,8 @@ __global__ void __launch_bounds__(128, 4)
 {
     using L = D3Q19;
     using A = Packed<S>;
-    pdl_begin();
-    const int3 r0 = tile_site<2, true>(t);
+    pdl_wait();
+    const int3 r0 = tile_site<2, 2, true>(t, threadIdx.x);
     const int x = r0.x, y = r0.y, z = r0.z, X = a.X, Y = a.Y, Z = a.Z, XY = X * Y;
     if (x >= X || y >= Y || z >= Z) return;
     const int xm = x == 0 ? X - 1 : x - 1, x1 = x + 1 == X ? 0 : x + 1, xe = x1 + 1 == X ? 0 : x1 + 1;
@@ -325,6 +278,7 @@ __global__ void __launch_bounds__(128, 4)
     const int site = x + X * y + XY * z;
     const bool two = AL || x + 1 < X;
     L::collide(g, fx, fy, fz, a.c, (uint32_t)site, a.c.step);
+    pdl_trigger();
 #pragma unroll
     for (int i = 0; i < L::Q; ++i) {
         if constexpr (AL) {

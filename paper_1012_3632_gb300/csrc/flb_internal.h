@@ -25,8 +25,7 @@ struct NvtxRange {
 };
 #define FLB_TRACE() ::flb::NvtxRange flb_trace_range_(__func__)
 
-// Planes of z per thread block of the z-marching kernels unless a context sets
-// its own (flb_options.z_chunk, or the length flb_step's tuning picks).
+// flb_z_chunk's answer for contexts that set no z_chunk of their own.
 constexpr int kZChunkDefault = 16;
 
 // Model parameters in double; each instantiation converts to its compute type.
@@ -43,7 +42,7 @@ struct HostModel {
     uint64_t seed;
     uint32_t replica;
     int noise_local;
-    int zchunk = 0;  // z-marching kernels: planes per block (0: the built-in default)
+    int zchunk = 0;  // flb_options.z_chunk
     void* mu = nullptr;  // force-model step in passes: the context's chemical potential field
 };
 
@@ -92,7 +91,7 @@ const PrecOps& ops_fp64();
 const PrecOps& ops_fp32();
 const PrecOps& ops_bf16();
 
-// Launch a kernel that begins with pdl_begin() on a stream: it may start while
+// Launch a kernel that begins with pdl_wait() on a stream: it may start while
 // the kernel before it drains (programmatic dependent launch), which hides the
 // launch latency between the kernels of a step.
 template <class... P, class... A>

@@ -21,15 +21,17 @@
 
 namespace flb {
 
-// Programmatic dependent launch: a kernel launched with launch_chain may start
-// while the kernel before it on the stream drains.  pdl_begin lets the next
-// one do the same and waits until everything before this kernel is complete
-// and visible; it comes before any access to memory.
-__device__ __forceinline__ void pdl_begin()
-{
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-}
+// Programmatic dependent launch.  A kernel launched with launch_chain may start
+// while the kernel before it on the stream drains: pdl_wait waits until
+// everything before this kernel is complete and visible and comes before any
+// access to memory; after pdl_trigger of all its blocks (or their end) the next
+// one may start.  The trigger stands before a kernel's stores: blocks of the
+// next kernel that start while this one still computes are placed on the SMs
+// that happen to have room, several on one, and wait there (a trigger at the
+// start: 48^3 force model 15.7 instead of 9.7 us a step, 160 x 128 in FP64
+// 30.9 instead of 12.1).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Indices of the 3x3x3 neighbourhood of (x, y, z) on a periodic X*Y*Z lattice:
 // xv[1+dx] + rb[1+dy][1+dz] is the site index of (x+dx, y+dy, z+dz).
@@ -51,6 +53,60 @@ struct Nbhd {
     // index of r - c for c = (cx, cy, cz)
     __device__ __forceinline__ int src(int cx, int cy, int cz) const { return xv[1 - cx] + rb[1 - cy][1 - cz]; }
 };
+
+// Tiles of threads over the lattice: rows of 2^lw threads (each N sites along
+// x), 2^lh rows in y and one or two planes in z.  Tiles are numbered along one grid dimension, x fastest (no axis meets a grid
+// limit of 65535).
+struct Tiling {
+    int lw, lh;
+    int ntx, nty, ntz;
+    uint32_t mx, sx, my, sy;  // quotients by ntx and nty: (umulhi(n, m) + n) >> s, n < 2^31
+    unsigned blocks() const { return (unsigned)((long)ntx * nty * ntz); }
+};
+
+inline void fast_div(uint32_t d, uint32_t& m, uint32_t& s)
+{
+    for (s = 0; (1u << s) < d; ++s) {
+    }
+    m = (uint32_t)(((1ull << 32) * ((1ull << s) - d)) / d + 1);
+}
+__device__ __forceinline__ uint32_t fast_quot(uint32_t n, uint32_t m, uint32_t s) { return (__umulhi(n, m) + n) >> s; }
+
+// The row width that covers an X x Y plane with the fewest tiles, the widest
+// of equals (a wide row has the fewest partial sectors).
+inline Tiling make_tiling(int X, int Y, int Z, int N, int threads, int planes)
+{
+    Tiling t{};
+    int lt = 5;  // log2 of the threads per plane
+    while ((1 << lt) * planes < threads) ++lt;
+    long best = 0;
+    for (int lw = 5; lw >= 2; --lw) {
+        const int w = N << lw, lh = lt - lw, h = 1 << lh, nx = (X + w - 1) / w, ny = (Y + h - 1) / h;
+        if (best && (long)nx * ny >= best) continue;
+        best = (long)nx * ny;
+        t.lw = lw;
+        t.lh = lh;
+        t.ntx = nx;
+        t.nty = ny;
+    }
+    t.ntz = (Z + planes - 1) / planes;
+    fast_div((uint32_t)t.ntx, t.mx, t.sx);
+    fast_div((uint32_t)t.nty, t.my, t.sy);
+    return t;
+}
+
+// First site (x, y, z) of thread `tid` of this block's tile of PLANES planes;
+// REV: the z planes in descending order.
+template <int N, int PLANES, bool REV>
+__device__ __forceinline__ int3 tile_site(const Tiling& t, int tid)
+{
+    const uint32_t b = blockIdx.x, r = fast_quot(b, t.mx, t.sx), bx = b - r * t.ntx;
+    const uint32_t rz = fast_quot(r, t.my, t.sy), by = r - rz * t.nty;
+    const int bz = REV ? t.ntz - 1 - (int)rz : (int)rz;
+    const int tx = tid & ((1 << t.lw) - 1), row = tid >> t.lw;
+    return make_int3(N * (((int)bx << t.lw) + tx), ((int)by << t.lh) + (row & ((1 << t.lh) - 1)),
+                     PLANES * bz + (row >> t.lh));
+}
 
 // Velocity tables for the pull / scatter addressing (same order as the API).
 template <class L>
@@ -236,123 +292,207 @@ struct StepArgs {
     // cs^2 grad rho = sum_i w_i c_i rho(r + c_i), which cancels the LB's own
     // ideal-gas pressure gradient (Eq. (he-force)); pgrad = 0 otherwise.
     R A, B, kappa, rho0_minus_rhoc, pgrad;
-    int nzc;  // z-marching kernels: planes per block (the z extent of a block's column)
 };
 
 // ---------------------------------------------------------------------------
 // Density gather: drho(r) = sum_i g*_i(r - c_i), the density deviation the
 // coming step sees (needed on a neighbourhood by the force).
 // ---------------------------------------------------------------------------
+constexpr int kSitesThreads = 128;
+
 template <class L, class R, class S>
-__global__ void k_density(const S* __restrict__ src, R* __restrict__ drho, int X, int Y, int Z)
+__global__ void __launch_bounds__(kSitesThreads)
+    k_density(const S* __restrict__ src, R* __restrict__ drho, int X, int Y, int Z, const Tiling t)
 {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z * blockDim.z + threadIdx.z;
-    if (x >= X || y >= Y || z >= Z) return;
-    const long V = (long)X * Y * Z;
-    const Nbhd nb(x, y, z, X, Y, Z);
+    pdl_wait();
+    const int3 r = tile_site<1, L::D == 3 ? 2 : 1, false>(t, threadIdx.x);
+    if (r.x >= X || r.y >= Y || r.z >= Z) return;
+    const Nbhd nb(r.x, r.y, r.z, X, Y, Z);
     R g[L::Q], m[L::Q];
-    pull<L>(src, V, nb, g);
+    pull<L>(src, (long)X * Y * Z, nb, g);
     L::moments(g, m);
-    drho[x + (long)X * (y + (long)Y * z)] = m[0];
+    pdl_trigger();
+    drho[r.x + X * (r.y + Y * r.z)] = m[0];
 }
 
 // ---------------------------------------------------------------------------
-// Fused pull + collide (+ force) + store.  Block = TX*TY*TZ threads, one site
-// each.  NONIDEAL adds the shared-memory mu / F stencils; their density tile
-// (tile + 2-site halo) comes from the field drho, or with GATHER from the
-// populations themselves (each halo site's pulls summed as k_density does),
-// which saves the separate density launch and field.
+// Fused pull + collide + store, one site per lane: FP64 storage, the D2Q9 ideal
+// gas.  FORCE (D3Q19): F = -rho grad mu with mu written by k_mu_field before;
+// TOTAL: psi is the total bulk free energy, F gains cs^2 grad rho.
+// SPLIT (FP64, small lattices): a block of four warps steps 32 sites; the first
+// pulls and collides, the others draw the normals meanwhile.
+//
+// FP64: the FP64 pipe (16 cycles per warp instruction of an SM) where the
+// lattice fills the chip, 64^3 force model 198 us a step (840 before: a column
+// march on 64 blocks that formed densities and mu several times over, normals
+// on the same pipe); below, the latency of one warp's chain of instructions,
+// 32 x 32 5.2 us (15.1 on 4 blocks of 256).
 // ---------------------------------------------------------------------------
-template <class L, class R, class S, bool NONIDEAL, int TX, int TY, int TZ, bool GATHER = false>
-__global__ void __launch_bounds__(TX* TY* TZ)
-    k_step(const StepArgs<R> a, const __grid_constant__ Planes<S> P, const R* __restrict__ drho)
+template <class L, class R, class S, bool FORCE, bool TOTAL, bool SPLIT>
+__global__ void __launch_bounds__(kSitesThreads)
+    k_sites(const StepArgs<R> a, const __grid_constant__ Planes<S> P, const R* __restrict__ drho,
+            const R* __restrict__ mu, const Tiling t)
 {
-    constexpr int HZ = (L::D == 3) ? 2 : 0;      // halo of rho in z
-    constexpr int RX = TX + 4, RY = TY + 4, RZ = TZ + 2 * HZ;
-    constexpr int MX = TX + 2, MY = TY + 2, MZ = TZ + (HZ ? 2 : 0);
-    constexpr int NT = TX * TY * TZ;
-    const int x = blockIdx.x * TX + threadIdx.x;
-    const int y = blockIdx.y * TY + threadIdx.y;
-    const int z = blockIdx.z * TZ + threadIdx.z;
-    const int X = a.X, Y = a.Y, Z = a.Z;
-
-    R F[3] = {R(0), R(0), R(0)};
-    if constexpr (NONIDEAL) {
-        __shared__ R srho[RZ * RY * RX];
-        __shared__ R smu[MZ * MY * MX];
-        const int tid = threadIdx.x + TX * (threadIdx.y + TY * threadIdx.z);
-        const int x0 = blockIdx.x * TX - 2, y0 = blockIdx.y * TY - 2, z0 = blockIdx.z * TZ - HZ;
-        for (int e = tid; e < RZ * RY * RX; e += NT) {
-            const int lx = e % RX, ly = (e / RX) % RY, lz = e / (RX * RY);
-            const int gx = wrap_any(x0 + lx, X), gy = wrap_any(y0 + ly, Y), gz = wrap_any(z0 + lz, Z);
-            if constexpr (GATHER) {
-                const Nbhd nh(gx, gy, gz, X, Y, Z);
-                R g[L::Q], m[L::Q];
-#pragma unroll
-                for (int i = 0; i < L::Q; ++i)
-                    g[i] = load_s<R>(P.src[i] + nh.src(Vel<L>::cx(i), Vel<L>::cy(i), Vel<L>::cz(i)));
-                L::moments(g, m);
-                srho[e] = m[0];
-            } else {
-                srho[e] = drho[gx + (long)X * (gy + (long)Y * gz)];
-            }
-        }
-        __syncthreads();
-        // mu = psi'(rho) - kappa lap rho on the tile + 1 halo;
-        // lap phi = 6 sum_i w_i (phi(r + c_i) - phi(r))
-        for (int e = tid; e < MZ * MY * MX; e += NT) {
-            const int mx = e % MX, my = (e / MX) % MY, mz = e / (MX * MY);
-            const int cidx = (mx + 1) + RX * ((my + 1) + RY * (mz + (HZ ? 1 : 0)));
-            const R r0 = srho[cidx];
-            R lap = R(0);
-#pragma unroll
-            for (int i = 1; i < L::Q; ++i) {
-                const int o = Vel<L>::cx(i) + RX * (Vel<L>::cy(i) + RY * Vel<L>::cz(i));
-                lap += R(Vel<L>::w(i)) * (srho[cidx + o] - r0);
-            }
-            lap *= R(6);
-            const R d = r0 + a.rho0_minus_rhoc;
-            smu[e] = d * (a.A + a.B * d * d) - a.kappa * lap;
-        }
-        __syncthreads();
-        // grad mu = 3 sum_i w_i c_i mu(r + c_i); F = -rho grad mu
-        const int cm = (threadIdx.x + 1) + MX * ((threadIdx.y + 1) + MY * (threadIdx.z + (HZ ? 1 : 0)));
-        R gx = R(0), gy = R(0), gz = R(0);
-#pragma unroll
-        for (int i = 1; i < L::Q; ++i) {
-            const int o = Vel<L>::cx(i) + MX * (Vel<L>::cy(i) + MY * Vel<L>::cz(i));
-            const R wm = R(Vel<L>::w(i)) * smu[cm + o];
-            if (Vel<L>::cx(i)) gx += R(Vel<L>::cx(i)) * wm;
-            if (Vel<L>::cy(i)) gy += R(Vel<L>::cy(i)) * wm;
-            if (Vel<L>::cz(i)) gz += R(Vel<L>::cz(i)) * wm;
-        }
-        const int cr = (threadIdx.x + 2) + RX * ((threadIdx.y + 2) + RY * (threadIdx.z + HZ));
-        const R rho = a.c.rho0 + srho[cr];
-        const R pre = R(-3) * rho;
-        F[0] = pre * gx;
-        F[1] = pre * gy;
-        F[2] = pre * gz;
-        if (a.pgrad != R(0)) {
-#pragma unroll
-            for (int i = 1; i < L::Q; ++i) {
-                const R wr = R(Vel<L>::w(i)) * srho[cr + Vel<L>::cx(i) + RX * (Vel<L>::cy(i) + RY * Vel<L>::cz(i))];
-                if (Vel<L>::cx(i)) F[0] += R(Vel<L>::cx(i)) * wr;
-                if (Vel<L>::cy(i)) F[1] += R(Vel<L>::cy(i)) * wr;
-                if (Vel<L>::cz(i)) F[2] += R(Vel<L>::cz(i)) * wr;
-            }
+    constexpr int PLANES = L::D == 3 && !SPLIT ? 2 : 1, NPAIR = (L::NNC + 1) / 2;
+    __shared__ R zs[SPLIT ? 2 * NPAIR : 1][32];
+    pdl_wait();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, X = a.X, Y = a.Y, Z = a.Z;
+    const int3 r = tile_site<1, PLANES, false>(t, SPLIT ? lane : (int)threadIdx.x);
+    const bool in = r.x < X && r.y < Y && r.z < Z;
+    const int x = in ? r.x : 0, y = in ? r.y : 0, z = in ? r.z : 0;  // idle lanes repeat the first site
+    const int s = x + X * (y + Y * z);
+    if constexpr (SPLIT) {
+        if (warp > 0) {
+            if (!a.c.noise) return;
+            for (int p = warp - 1; p < NPAIR; p += 3)
+                normal_pair(a.c.key, (uint32_t)s, a.c.step, p, a.c.replica, zs[2 * p][lane], zs[2 * p + 1][lane]);
+            __syncthreads();
+            return;
         }
     }
-    if (x >= X || y >= Y || z >= Z) return;
+    if (!SPLIT && !in) return;
     const Nbhd nb(x, y, z, X, Y, Z);
     R g[L::Q];
     pull_planes<L, false>(P, nb, g);
-    const int s = x + X * (y + Y * z);
+    R F[3] = {R(0), R(0), R(0)};
+    if constexpr (FORCE) {
+        // sum_i w_i c_i f(r + c_i) from the differences f(c) - f(-c) of the velocity
+        // pairs (2k-1, 2k): axis pairs weigh 1/18, edge pairs 1/36
+        auto grad = [&](const R* f, R d[3]) {
+            R e[10];
+#pragma unroll
+            for (int k = 1; k <= 9; ++k) {
+                const int i = 2 * k - 1, cx = Vel<L>::cx(i), cy = Vel<L>::cy(i), cz = Vel<L>::cz(i);
+                e[k] = f[nb.src(-cx, -cy, -cz)] - f[nb.src(cx, cy, cz)];
+            }
+            d[0] = R(1.0 / 18) * e[1] + R(1.0 / 36) * ((e[4] + e[5]) + (e[6] + e[7]));
+            d[1] = R(1.0 / 18) * e[2] + R(1.0 / 36) * ((e[4] - e[5]) + (e[8] + e[9]));
+            d[2] = R(1.0 / 18) * e[3] + R(1.0 / 36) * ((e[6] - e[7]) + (e[8] - e[9]));
+        };
+        R d[3];
+        grad(mu, d);
+        const R pre = R(-3) * (a.c.rho0 + drho[s]);
+        for (int k = 0; k < 3; ++k) F[k] = pre * d[k];
+        if constexpr (TOTAL) {
+            grad(drho, d);
+            for (int k = 0; k < 3; ++k) F[k] += d[k];
+        }
+    }
+    auto normals = [&](R* q) {
+        if constexpr (SPLIT) {
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < 2 * NPAIR; ++k) q[k] = zs[k][lane];
+        } else {
+            noise_normals<L::NCALL>(a.c.key, (uint32_t)s, a.c.step, a.c.replica, q);
+        }
+    };
     if constexpr (L::D == 3)
-        L::template collide<NONIDEAL>(g, F[0], F[1], F[2], a.c, (uint32_t)s, a.c.step);
+        L::template collide_with<FORCE>(g, F[0], F[1], F[2], a.c, normals);
     else
-        L::collide(g, F[0], F[1], a.c, (uint32_t)s, a.c.step);
+        L::collide_with(g, F[0], F[1], a.c, normals);
+    pdl_trigger();
+    if (!in) return;
+#pragma unroll
+    for (int i = 0; i < L::Q; ++i) store_stream(P.dst[i] + s, g[i]);
+}
+
+// mu = psi'(rho) - kappa lap rho of every site (D3Q19, one site per thread): the
+// Laplacian is 6 sum_i w_i (rho_i - rho) = (1/3) (axis sum) + (1/6) (edge sum) - 4 rho.
+template <class R>
+__global__ void __launch_bounds__(kSitesThreads)
+    k_mu_field(const StepArgs<R> a, const R* __restrict__ drho, R* __restrict__ mu, const Tiling t)
+{
+    using L = D3Q19;
+    pdl_wait();
+    const int3 r = tile_site<1, 2, false>(t, threadIdx.x);
+    if (r.x >= a.X || r.y >= a.Y || r.z >= a.Z) return;
+    const Nbhd nb(r.x, r.y, r.z, a.X, a.Y, a.Z);
+    const int s = r.x + a.X * (r.y + a.Y * r.z);
+    const R rc = drho[s];
+    R ax = R(0), ed = R(0);
+#pragma unroll
+    for (int i = 1; i < L::Q; ++i) {
+        const R v = drho[nb.src(-Vel<L>::cx(i), -Vel<L>::cy(i), -Vel<L>::cz(i))];
+        if (i < 7)
+            ax += v;
+        else
+            ed += v;
+    }
+    const R lap = R(1.0 / 3) * ax + R(1.0 / 6) * ed - R(4) * rc;
+    const R d = rc + a.rho0_minus_rhoc;
+    pdl_trigger();
+    mu[s] = d * (a.A + a.B * d * d) - a.kappa * lap;
+}
+
+// ---------------------------------------------------------------------------
+// D2Q9 force model in one launch: a block's density tile (tile + 2-site halo)
+// is gathered from the populations into shared memory, mu is formed on the tile
+// + 1-site halo, then pull + collide with F = -rho grad mu + store.
+// ---------------------------------------------------------------------------
+template <class R, class S, int TX, int TY>
+__global__ void __launch_bounds__(TX* TY)
+    k_step_gather(const StepArgs<R> a, const __grid_constant__ Planes<S> P)
+{
+    using L = D2Q9;
+    constexpr int RX = TX + 4, RY = TY + 4, MX = TX + 2, MY = TY + 2, NT = TX * TY;
+    const int x = blockIdx.x * TX + threadIdx.x;
+    const int y = blockIdx.y * TY + threadIdx.y;
+    const int X = a.X, Y = a.Y;
+    __shared__ R srho[RY * RX];
+    __shared__ R smu[MY * MX];
+    const int tid = threadIdx.x + TX * threadIdx.y;
+    const int x0 = blockIdx.x * TX - 2, y0 = blockIdx.y * TY - 2;
+    for (int e = tid; e < RY * RX; e += NT) {
+        const Nbhd nh(wrap_any(x0 + e % RX, X), wrap_any(y0 + e / RX, Y), 0, X, Y, 1);
+        R g[L::Q], m[L::Q];
+        pull_planes<L, false>(P, nh, g);
+        L::moments(g, m);
+        srho[e] = m[0];
+    }
+    __syncthreads();
+    // mu = psi'(rho) - kappa lap rho on the tile + 1 halo;
+    // lap phi = 6 sum_i w_i (phi(r + c_i) - phi(r))
+    for (int e = tid; e < MY * MX; e += NT) {
+        const int cidx = e % MX + 1 + RX * (e / MX + 1);
+        const R r0 = srho[cidx];
+        R lap = R(0);
+#pragma unroll
+        for (int i = 1; i < L::Q; ++i) {
+            const int o = Vel<L>::cx(i) + RX * Vel<L>::cy(i);
+            lap += R(Vel<L>::w(i)) * (srho[cidx + o] - r0);
+        }
+        lap *= R(6);
+        const R d = r0 + a.rho0_minus_rhoc;
+        smu[e] = d * (a.A + a.B * d * d) - a.kappa * lap;
+    }
+    __syncthreads();
+    if (x >= X || y >= Y) return;
+    // grad mu = 3 sum_i w_i c_i mu(r + c_i); F = -rho grad mu
+    const int cm = threadIdx.x + 1 + MX * (threadIdx.y + 1);
+    const int cr = threadIdx.x + 2 + RX * (threadIdx.y + 2);
+    R gx = R(0), gy = R(0);
+#pragma unroll
+    for (int i = 1; i < L::Q; ++i) {
+        const R wm = R(Vel<L>::w(i)) * smu[cm + Vel<L>::cx(i) + MX * Vel<L>::cy(i)];
+        if (Vel<L>::cx(i)) gx += R(Vel<L>::cx(i)) * wm;
+        if (Vel<L>::cy(i)) gy += R(Vel<L>::cy(i)) * wm;
+    }
+    const R pre = R(-3) * (a.c.rho0 + srho[cr]);
+    R fx = pre * gx, fy = pre * gy;
+    if (a.pgrad != R(0)) {
+#pragma unroll
+        for (int i = 1; i < L::Q; ++i) {
+            const R wr = R(Vel<L>::w(i)) * srho[cr + Vel<L>::cx(i) + RX * Vel<L>::cy(i)];
+            if (Vel<L>::cx(i)) fx += R(Vel<L>::cx(i)) * wr;
+            if (Vel<L>::cy(i)) fy += R(Vel<L>::cy(i)) * wr;
+        }
+    }
+    const Nbhd nb(x, y, 0, X, Y, 1);
+    R g[L::Q];
+    pull_planes<L, false>(P, nb, g);
+    const int s = x + X * y;
+    L::collide(g, fx, fy, a.c, (uint32_t)s, a.c.step);
 #pragma unroll
     for (int i = 0; i < L::Q; ++i) store_stream(P.dst[i] + s, g[i]);
 }
@@ -460,190 +600,6 @@ __global__ void __launch_bounds__(TXT* TY* TZ, MINB)
     L::template collide<false>(g, F2(0.f), F2(0.f), F2(0.f), a.c, (uint32_t)s, a.c.step);
 #pragma unroll
     for (int i = 0; i < L::Q; ++i) A::store2(P.dst[i] + s, g[i].v);
-}
-
-// Density gather for site pairs (x, x+1), packed FP32; X even.
-template <int TXT, int TY, int TZ>
-__global__ void __launch_bounds__(TXT* TY* TZ)
-    k_density2(const __grid_constant__ Planes<float> P, float* __restrict__ drho, int X, int Y, int Z)
-{
-    using L = D3Q19;
-    const int x = 2 * (blockIdx.x * TXT + threadIdx.x);
-    const int y = blockIdx.y * TY + threadIdx.y;
-    const int z = blockIdx.z * TZ + threadIdx.z;
-    if (x >= X || y >= Y || z >= Z) return;
-    const int xm = x == 0 ? X - 1 : x - 1, x2 = x + 2 == X ? 0 : x + 2;
-    const int yv[3] = {wrap_once(y - 1, Y), y, wrap_once(y + 1, Y)};
-    const int zv[3] = {wrap_once(z - 1, Z), z, wrap_once(z + 1, Z)};
-    F2 g[L::Q], m[L::Q];
-#pragma unroll
-    for (int i = 0; i < L::Q; ++i) {
-        const float* p = P.src[i] + X * (yv[1 - Vel<L>::cy(i)] + Y * zv[1 - Vel<L>::cz(i)]);
-        const int cx = Vel<L>::cx(i);
-        if (cx == 0)
-            g[i] = mk2(*reinterpret_cast<const float2*>(p + x));
-        else if (cx > 0)
-            g[i] = F2(p[xm], p[x]);
-        else
-            g[i] = F2(p[x + 1], p[x2]);
-    }
-    L::moments(g, m);
-    *reinterpret_cast<float2*>(drho + x + X * (y + Y * z)) = m[0].v;
-}
-
-// ---------------------------------------------------------------------------
-// D3Q19 non-ideal fluid with the density gather fused in: one block owns a
-// TX x TY column of sites and marches over a.nzc planes in z.  Iteration k pulls
-// drho of plane zb+k+2 on the tile + 2-site halo (the tile interior's pulled
-// populations are re-read from L2 by the collision two planes later),
-// evaluates mu of plane zb+k+1 on the tile + 1-site halo, and collides plane
-// zb+k with F = -rho grad mu.  The first iterations (k < 0) only fill the
-// rings of 5 density planes and 3 chemical-potential planes kept in shared
-// memory; the density never goes to DRAM.  Each stage appears once in the
-// loop body so that the kernel stays small in the instruction cache.
-// ---------------------------------------------------------------------------
-template <class R, class S, int TX, int TY, int MINB>
-__global__ void __launch_bounds__(TX* TY, MINB)
-    k_step_march(const StepArgs<R> a, const __grid_constant__ Planes<S> P)
-{
-    using L = D3Q19;
-    constexpr int NT = TX * TY, RX = TX + 4, RY = TY + 4, RP = RX * RY, MX = TX + 2, MY = TY + 2, MP = MX * MY;
-    constexpr int NRH = (RP + NT - 1) / NT;  // halo density sites per thread
-    __shared__ R srho[5][RP];
-    __shared__ R smu[3][MP];
-    const int tid = threadIdx.x + TX * threadIdx.y;
-    const int X = a.X, Y = a.Y, Z = a.Z;
-    const int XY = X * Y;
-    const int xb = blockIdx.x * TX, yb = blockIdx.y * TY, zb = blockIdx.z * a.nzc;
-    const int nz = min(a.nzc, Z - zb);
-
-    // In-plane neighbourhood of this thread's density sites (fixed over z):
-    // x - 1, x, x + 1 and the row offsets X*(y - 1), X*y, X*(y + 1).
-    int hx[NRH][3], hy[NRH][3];
-#pragma unroll
-    for (int h = 0; h < NRH; ++h) {
-        const int e = min(tid + h * NT, RP - 1);
-        const int gx = wrap_any(xb - 2 + e % RX, X), gy = wrap_any(yb - 2 + e / RX, Y);
-        hx[h][0] = wrap_once(gx - 1, X);
-        hx[h][1] = gx;
-        hx[h][2] = wrap_once(gx + 1, X);
-        hy[h][0] = X * wrap_once(gy - 1, Y);
-        hy[h][1] = X * gy;
-        hy[h][2] = X * wrap_once(gy + 1, Y);
-    }
-
-    // this thread's chemical-potential sites: centre offset in the density plane
-    constexpr int NMU = (MP + NT - 1) / NT;
-    int mc[NMU];
-#pragma unroll
-    for (int j = 0; j < NMU; ++j) {
-        const int e = min(tid + j * NT, MP - 1);
-        mc[j] = (e % MX + 1) + RX * (e / MX + 1);
-    }
-
-    const int x = xb + threadIdx.x, y = yb + threadIdx.y;
-    const int cm = (threadIdx.x + 1) + MX * (threadIdx.y + 1);
-    const int cr = (threadIdx.x + 2) + RX * (threadIdx.y + 2);
-    // ring slots, advanced by one each iteration: plane zb+k+2 of the density
-    // goes to slot (k+4) mod 5 = ra + 2, the collision reads density slot
-    // ra = (k+2) mod 5 and chemical-potential slots (k, k+1, k+2) mod 3.
-    int ra = 3;       // (k + 2) mod 5 at k = -4
-    int mb = 2;       // k mod 3 at k = -4
-    int zc = wrap_any(zb - 2, Z);  // density plane being gathered, wrapped
-#pragma unroll 1
-    for (int k = -4; k < nz; ++k) {
-        const int ra1 = ra == 4 ? 0 : ra + 1, ra2 = ra1 == 4 ? 0 : ra1 + 1;
-        const int mb1 = mb == 2 ? 0 : mb + 1, mb2 = mb1 == 2 ? 0 : mb1 + 1;
-        // (1) density of plane zb+k+2 on the tile + 2 halo: drho = sum_i g*_i(r - c_i)
-        {
-            const int zo[3] = {XY * (zc == 0 ? Z - 1 : zc - 1), XY * zc, XY * (zc == Z - 1 ? 0 : zc + 1)};
-            R* out = srho[ra2];
-#pragma unroll
-            for (int h = 0; h < NRH; ++h) {
-                const int e = tid + h * NT;
-                if (e < RP) {
-                    R g[L::Q], m[L::Q];
-#pragma unroll
-                    for (int i = 0; i < L::Q; ++i)
-                        g[i] = load_s<R>(P.src[i] + (hx[h][1 - Vel<L>::cx(i)] + hy[h][1 - Vel<L>::cy(i)] +
-                                                     zo[1 - Vel<L>::cz(i)]));
-                    L::moments(g, m);
-                    out[e] = m[0];
-                }
-            }
-        }
-        __syncthreads();
-        // (2) mu = psi'(rho) - kappa lap rho of plane zb+k+1 on the tile + 1 halo
-        if (k >= -2) {
-            const R* rm = srho[ra];
-            const R* r0 = srho[ra1];
-            const R* rp = srho[ra2];
-            R* out = smu[mb2];
-#pragma unroll
-            for (int j = 0; j < NMU; ++j) {
-                const int e = tid + j * NT;
-                if (e < MP) {
-                    const int c = mc[j];
-                    const R rc = r0[c];
-                    R lap = R(0);
-#pragma unroll
-                    for (int i = 1; i < L::Q; ++i) {
-                        const int cz = Vel<L>::cz(i);
-                        const R* pl = cz > 0 ? rp : (cz < 0 ? rm : r0);
-                        lap += R(Vel<L>::w(i)) * (pl[c + Vel<L>::cx(i) + RX * Vel<L>::cy(i)] - rc);
-                    }
-                    lap *= R(6);
-                    const R d = rc + a.rho0_minus_rhoc;
-                    out[e] = d * (a.A + a.B * d * d) - a.kappa * lap;
-                }
-            }
-        }
-        __syncthreads();
-        // (3) collide plane zb+k with F = -rho grad mu, grad = 3 sum_i w_i c_i mu(r + c_i)
-        if (k >= 0 && x < X && y < Y) {
-            const int z = zb + k;
-            const R* mlo = smu[mb];
-            const R* mmid = smu[mb1];
-            const R* mhi = smu[mb2];
-            R gx = R(0), gy = R(0), gz = R(0);
-#pragma unroll
-            for (int i = 1; i < L::Q; ++i) {
-                const int cz = Vel<L>::cz(i);
-                const R* pl = cz > 0 ? mhi : (cz < 0 ? mlo : mmid);
-                const R wm = R(Vel<L>::w(i)) * pl[cm + Vel<L>::cx(i) + MX * Vel<L>::cy(i)];
-                if (Vel<L>::cx(i)) gx += R(Vel<L>::cx(i)) * wm;
-                if (Vel<L>::cy(i)) gy += R(Vel<L>::cy(i)) * wm;
-                if (Vel<L>::cz(i)) gz += R(Vel<L>::cz(i)) * wm;
-            }
-            const R pre = R(-3) * (a.c.rho0 + srho[ra][cr]);
-            R fx = pre * gx, fy = pre * gy, fz = pre * gz;
-            if (a.pgrad != R(0)) {
-                // + cs^2 grad rho from the density planes z-1, z, z+1
-                const R* qlo = srho[ra == 0 ? 4 : ra - 1];
-                const R* qmid = srho[ra];
-                const R* qhi = srho[ra1];
-#pragma unroll
-                for (int i = 1; i < L::Q; ++i) {
-                    const int cz = Vel<L>::cz(i);
-                    const R* pl = cz > 0 ? qhi : (cz < 0 ? qlo : qmid);
-                    const R wr = R(Vel<L>::w(i)) * pl[cr + Vel<L>::cx(i) + RX * Vel<L>::cy(i)];
-                    if (Vel<L>::cx(i)) fx += R(Vel<L>::cx(i)) * wr;
-                    if (Vel<L>::cy(i)) fy += R(Vel<L>::cy(i)) * wr;
-                    if (Vel<L>::cz(i)) fz += R(Vel<L>::cz(i)) * wr;
-                }
-            }
-            const Nbhd nb(x, y, z, X, Y, Z);
-            R g[L::Q];
-            pull_planes<L, true>(P, nb, g);
-            const int s = x + X * (y + Y * z);
-            L::collide(g, fx, fy, fz, a.c, (uint32_t)s, a.c.step);
-#pragma unroll
-            for (int i = 0; i < L::Q; ++i) store_stream(P.dst[i] + s, g[i]);
-        }
-        ra = ra1;
-        mb = mb1;
-        zc = zc == Z - 1 ? 0 : zc + 1;
-    }
 }
 
 }  // namespace flb

@@ -11,15 +11,6 @@
 #include "flb_internal.h"
 #include "flb_kernels.cuh"
 
-#ifndef FLB_MARCH_MINB
-#define FLB_MARCH_MINB 3
-#endif
-#ifndef FLB_MARCH_TY
-#define FLB_MARCH_TY 8
-#endif
-#ifndef FLB_PACKED
-#define FLB_PACKED 1
-#endif
 #ifndef FLB_STEP2_TXT
 #define FLB_STEP2_TXT 32
 #endif
@@ -87,7 +78,6 @@ StepArgs<R> make_args(const HostModel& m, uint64_t step)
     a.kappa = R(m.kappa);
     a.rho0_minus_rhoc = R(m.rho0 - m.rho_c);
     a.pgrad = R(m.nonideal && m.total ? 1 : 0);
-    a.nzc = std::min(m.zchunk > 0 ? m.zchunk : kZChunkDefault, m.Z);
     return a;
 }
 
@@ -454,82 +444,100 @@ struct Prec {
     // FP32 arithmetic on FP32 or BF16 storage: the two-sites-per-thread kernels
     static constexpr bool kPackedStorage =
         std::is_same<R, float>::value && (std::is_same<S, float>::value || std::is_same<S, __nv_bfloat16>::value);
-    template <class L>
-    static cudaError_t density_l(const HostModel& m, const void* pop, void* drho, cudaStream_t st)
-    {
-        const dim3 b = site_block<L>();
-        k_density<L, R, S><<<grid_for(m, b), b, 0, st>>>((const S*)pop, (R*)drho, m.X, m.Y, m.Z);
-        return cudaGetLastError();
-    }
     static cudaError_t density(const HostModel& m, const void* pop, void* drho, cudaStream_t st)
     {
-        if constexpr (std::is_same<R, float>::value && std::is_same<S, float>::value) {
-            if (m.Q == 19 && m.X % 2 == 0 && FLB_PACKED) {
-                constexpr int TXT = 16, TY = 4, TZ = 2;
-                const dim3 b(TXT, TY, TZ);
-                const dim3 g((m.X / 2 + TXT - 1) / TXT, (m.Y + TY - 1) / TY, (m.Z + TZ - 1) / TZ);
-                k_density2<TXT, TY, TZ><<<g, b, 0, st>>>(make_planes<S>(pop, nullptr, 19, m.V), (float*)drho, m.X,
-                                                          m.Y, m.Z);
-                return cudaGetLastError();
-            }
+        if constexpr (kPackedStorage) {
+            if (m.Q == 19) return density_packed(m, pop, (float*)drho, nullptr, st);
         }
-        return m.Q == 19 ? density_l<D3Q19>(m, pop, drho, st) : density_l<D2Q9>(m, pop, drho, st);
+        const Tiling t = make_tiling(m.X, m.Y, m.Z, 1, kSitesThreads, m.D == 3 ? 2 : 1);
+        const auto k = m.Q == 19 ? k_density<D3Q19, R, S> : k_density<D2Q9, R, S>;
+        return launch_chain(k, dim3(t.blocks()), dim3(kSitesThreads), st, (const S*)pop, (R*)drho, m.X, m.Y, m.Z, t);
     }
 
-    template <class L, bool NI, int TX, int TY, int TZ, bool GATHER = false>
-    static cudaError_t step_t(const HostModel& m, uint64_t step, const void* src, void* dst, const void* drho,
-                              cudaStream_t st)
+    // The step of one site per lane (k_sites).  FP64: small lattices are stepped
+    // 32 sites per block, whose other warps draw the noise meanwhile; larger ones
+    // fill the FP64 pipe either way.  Measured, us per step, 128 sites / 32 per
+    // block: D2Q9 32^2 7.7 / 5.2, 160 x 128 12.1 / 7.7, 224 x 200 15.7 / 12.9,
+    // 256^2 equal; D3Q19 force 16^3 22.9 / 17.4, 28^3 35.7 / 33.6, 36^3 48.8 / 51.7.
+    static bool split_sites(const HostModel& m) { return m.V <= (m.D == 2 ? 65536 : 24576); }
+    template <class L, bool FORCE, bool TOTAL>
+    static cudaError_t step_sites(const HostModel& m, uint64_t step, const void* src, void* dst, const R* drho,
+                                  cudaStream_t st)
     {
         const StepArgs<R> a = make_args<L, R>(m, step);
-        const dim3 b(TX, TY, TZ);
-        k_step<L, R, S, NI, TX, TY, TZ, GATHER><<<grid_for(m, b), b, 0, st>>>(
-            a, make_planes<S>(src, dst, L::Q, m.V), (const R*)drho);
-        return cudaGetLastError();
+        const Planes<S> pl = make_planes<S>(src, dst, L::Q, m.V);
+        const R* mu = (const R*)m.mu;
+        if constexpr (std::is_same<R, double>::value) {
+            if (split_sites(m)) {
+                const Tiling t = make_tiling(m.X, m.Y, m.Z, 1, 32, 1);
+                return launch_chain(k_sites<L, R, S, FORCE, TOTAL, true>, dim3(t.blocks()), dim3(kSitesThreads), st, a,
+                                    pl, drho, mu, t);
+            }
+        }
+        const Tiling t = make_tiling(m.X, m.Y, m.Z, 1, kSitesThreads, L::D == 3 ? 2 : 1);
+        return launch_chain(k_sites<L, R, S, FORCE, TOTAL, false>, dim3(t.blocks()), dim3(kSitesThreads), st, a, pl,
+                            drho, mu, t);
     }
-    // The D3Q19 force-model step of FP32 and BF16 storage (flb_force.cuh).
-    static int step_in_passes(const HostModel& m) { return kPackedStorage && m.Q == 19 && m.nonideal; }
+    // D3Q19 force model, FP64: density, mu and collision passes.
+    static cudaError_t step_force_sites(const HostModel& m, uint64_t step, const void* src, void* dst, R* drho,
+                                        cudaStream_t st)
+    {
+        cudaError_t e = density(m, src, drho, st);
+        if (e != cudaSuccess) return e;
+        const Tiling t = make_tiling(m.X, m.Y, m.Z, 1, kSitesThreads, 2);
+        const R* rho = drho;
+        e = launch_chain(k_mu_field<R>, dim3(t.blocks()), dim3(kSitesThreads), st, make_args<D3Q19, R>(m, step), rho,
+                         (R*)m.mu, t);
+        if (e != cudaSuccess) return e;
+        return m.total ? step_sites<D3Q19, true, true>(m, step, src, dst, rho, st)
+                       : step_sites<D3Q19, true, false>(m, step, src, dst, rho, st);
+    }
+    // The D3Q19 force model steps in passes over the context's density and mu
+    // fields: FP32 and BF16 storage by flb_force.cuh, FP64 by k_sites.
+    static int step_in_passes(const HostModel& m) { return m.Q == 19 && m.nonideal; }
     static int gather_width(const HostModel& m) { return m.X % 4 == 0 ? 4 : m.X % 2 == 0 ? 2 : 1; }
     // density: quads of sites per thread, or pairs
     static Tiling density_tiling(const HostModel& m)
     {
-        return make_tiling(m.X, m.Y, m.Z, gather_width(m) == 4 ? 4 : 2);
+        return make_tiling(m.X, m.Y, m.Z, gather_width(m) == 4 ? 4 : 2, 128, 2);
     }
     static int step_row_count(const HostModel& m)
     {
-        return step_in_passes(m) ? 4 * (int)density_tiling(m).blocks() : 0;  // one per warp
+        return kPackedStorage && step_in_passes(m) ? 4 * (int)density_tiling(m).blocks() : 0;  // one per warp
+    }
+    // rows (or NULL): step_row_count rows of mass deviation and momentum
+    static cudaError_t density_packed(const HostModel& m, const void* pop, float* rho, float* rows, cudaStream_t st)
+    {
+        const Planes<S> pl = make_planes<S>(pop, nullptr, 19, m.V);
+        const Tiling t = density_tiling(m);
+        auto go = [&](auto G) {
+            constexpr int GX = decltype(G)::value;
+            const auto k = rows ? k_force_density<S, GX, true> : k_force_density<S, GX, false>;
+            return launch_chain(k, dim3(t.blocks()), dim3(128), st, pl, rho, rows, m.X, m.Y, m.Z, t);
+        };
+        const int gx = gather_width(m);
+        return gx == 4   ? go(std::integral_constant<int, 4>{})
+               : gx == 2 ? go(std::integral_constant<int, 2>{})
+                         : go(std::integral_constant<int, 1>{});
     }
     static cudaError_t step_force(const HostModel& m, uint64_t step, const void* src, void* dst, float* rho,
                                   float* rows, cudaStream_t st)
     {
         const StepArgs<R> a = make_args<D3Q19, R>(m, step);
         const Planes<S> pl = make_planes<S>(src, dst, 19, m.V);
-        float* mu = (float*)m.mu;
         const float* crho = rho;
-        const float* cmu = mu;
+        const float* mu = (const float*)m.mu;
         const int gx = gather_width(m);
-        const Tiling tc = make_tiling(m.X, m.Y, m.Z, 2), td = density_tiling(m);  // collision: site pairs
-        const Tiling tm = make_tiling(m.X, m.Y, (m.Z + 1) / 2, gx == 4 ? 4 : 2);  // mu: two planes per thread
-        auto grid = [](const Tiling& t) { return dim3(t.blocks()); };
-        const dim3 b(128);
-        auto fields = [&](auto G) {
-            constexpr int GX = decltype(G)::value;
-            const cudaError_t e =
-                rows ? launch_chain(k_force_density<S, GX, true>, grid(td), b, st, pl, rho, rows, m.X, m.Y, m.Z, td)
-                     : launch_chain(k_force_density<S, GX, false>, grid(td), b, st, pl, rho, rows, m.X, m.Y, m.Z, td);
-            return e != cudaSuccess ? e : launch_chain(k_force_mu<GX>, grid(tm), b, st, a, crho, mu, tm);
-        };
-        const cudaError_t e = gx == 4   ? fields(std::integral_constant<int, 4>{})
-                              : gx == 2 ? fields(std::integral_constant<int, 2>{})
-                                        : fields(std::integral_constant<int, 1>{});
+        cudaError_t e = density_packed(m, src, rho, rows, st);
         if (e != cudaSuccess) return e;
-        auto collide = [&](auto AL, auto TOTAL) {
-            return launch_chain(k_force_collide<S, decltype(AL)::value, decltype(TOTAL)::value>,
-                                grid(tc), b, st, a, pl, crho, cmu, tc);
-        };
-        const std::true_type yes;
-        const std::false_type no;
-        if (gx == 1) return m.total ? collide(no, yes) : collide(no, no);
-        return m.total ? collide(yes, yes) : collide(yes, no);
+        const Tiling tm = make_tiling(m.X, m.Y, (m.Z + 1) / 2, gx == 4 ? 4 : 2, 128, 2);  // two planes per thread
+        const auto km = gx == 4 ? k_force_mu<4> : gx == 2 ? k_force_mu<2> : k_force_mu<1>;
+        e = launch_chain(km, dim3(tm.blocks()), dim3(128), st, a, crho, (float*)m.mu, tm);
+        if (e != cudaSuccess) return e;
+        const Tiling tc = make_tiling(m.X, m.Y, m.Z, 2, 128, 2);  // site pairs
+        const auto kc = gx == 1 ? (m.total ? k_force_collide<S, false, true> : k_force_collide<S, false, false>)
+                                : (m.total ? k_force_collide<S, true, true> : k_force_collide<S, true, false>);
+        return launch_chain(kc, dim3(tc.blocks()), dim3(128), st, a, pl, crho, mu, tc);
     }
     // The step; with rows (non-NULL) also the mass deviation and momentum of
     // the state it steps from, as step_row_count rows of 4 partial sums, where
@@ -543,11 +551,12 @@ struct Prec {
     static cudaError_t step_rows(const HostModel& m, uint64_t t, const void* src, void* dst, const void* drho,
                                  float4* rows, cudaStream_t st)
     {
+        // drho: the context's density field, scratch of the steps in passes
         if constexpr (kPackedStorage) {
-            // drho: the context's density field, scratch of this step
             if (step_in_passes(m)) return step_force(m, t, src, dst, (float*)const_cast<void*>(drho), (float*)rows, st);
         }
         if (rows) return cudaErrorNotSupported;
+        if (step_in_passes(m)) return step_force_sites(m, t, src, dst, (R*)const_cast<void*>(drho), st);
         if (m.Q == 9 && m.nonideal && m.model == 1) {
             const StepArgs<R> a = make_args<D2Q9, R>(m, t);
             const dim3 b(32, 8, 1);
@@ -556,33 +565,25 @@ struct Prec {
                                                                       (const NoiseField<R>*)m.swift_xi);
             return cudaGetLastError();
         }
-        if (m.Q == 19) {
-            if (m.nonideal) {
-                constexpr int TX = 32, TY = FLB_MARCH_TY;
+        if (m.Q == 9 && m.nonideal) {
+            const dim3 b(32, 8, 1);
+            k_step_gather<R, S, 32, 8>
+                <<<grid_for(m, b), b, 0, st>>>(make_args<D2Q9, R>(m, t), make_planes<S>(src, dst, 9, m.V));
+            return cudaGetLastError();
+        }
+        if constexpr (kPackedStorage) {
+            if (m.Q == 19 && m.X % 2 == 0) {
+                constexpr int TXT = FLB_STEP2_TXT, TY = FLB_STEP2_TY, TZ = FLB_STEP2_TZ;
                 const StepArgs<R> a = make_args<D3Q19, R>(m, t);
-                const dim3 b(TX, TY, 1);
-                const dim3 g((m.X + TX - 1) / TX, (m.Y + TY - 1) / TY, (m.Z + a.nzc - 1) / a.nzc);
-                k_step_march<R, S, TX, TY, (sizeof(R) == 8 ? 1 : FLB_MARCH_MINB)>
-                    <<<g, b, 0, st>>>(a, make_planes<S>(src, dst, 19, m.V));
+                const dim3 b(TXT, TY, TZ);
+                const dim3 g((m.X / 2 + TXT - 1) / TXT, (m.Y + TY - 1) / TY, (m.Z + TZ - 1) / TZ);
+                constexpr int MINB = sizeof(S) == 4 ? FLB_STEP2_MINB : FLB_STEP2_MINB_BF16;
+                k_step2<D3Q19, S, TXT, TY, TZ, MINB><<<g, b, 0, st>>>(a, make_planes<S>(src, dst, 19, m.V));
                 return cudaGetLastError();
             }
-            if constexpr (kPackedStorage) {
-                if (m.X % 2 == 0 && FLB_PACKED) {
-                    constexpr int TXT = FLB_STEP2_TXT, TY = FLB_STEP2_TY, TZ = FLB_STEP2_TZ;
-                    const StepArgs<R> a = make_args<D3Q19, R>(m, t);
-                    const dim3 b(TXT, TY, TZ);
-                    const dim3 g((m.X / 2 + TXT - 1) / TXT, (m.Y + TY - 1) / TY, (m.Z + TZ - 1) / TZ);
-                    constexpr int MINB = sizeof(S) == 4 ? FLB_STEP2_MINB : FLB_STEP2_MINB_BF16;
-                    k_step2<D3Q19, S, TXT, TY, TZ, MINB>
-                        <<<g, b, 0, st>>>(a, make_planes<S>(src, dst, 19, m.V));
-                    return cudaGetLastError();
-                }
-            }
-            return step_t<D3Q19, false, 32, 4, 2>(m, t, src, dst, drho, st);
         }
-        // force model: the density tile is gathered inside the step
-        if (m.nonideal) return step_t<D2Q9, true, 32, 8, 1, true>(m, t, src, dst, drho, st);
-        return step_t<D2Q9, false, 32, 8, 1>(m, t, src, dst, drho, st);
+        return m.Q == 19 ? step_sites<D3Q19, false, false>(m, t, src, dst, nullptr, st)
+                         : step_sites<D2Q9, false, false>(m, t, src, dst, nullptr, st);
     }
 
     template <class L>
