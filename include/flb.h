@@ -249,7 +249,7 @@ int flb_check_guards(flb_ctx* ctx);
  * sums: host, 4*nsteps doubles, written when the call returns (it waits for
  * the context's stream once, at the end; device-addressable page-locked
  * memory is written in place by the reduction, other memory through a copy).  The D3Q19 force-model step with
- * FP32 or BF16 storage forms these sums inside its density pass (per-warp
+ * FP32 or BF16 storage, even X and the excess free energy forms these sums inside its density pass (per-warp
  * partial sums of the mass deviation and momentum of the pulled populations,
  * those of several steps added up by one launch); every other step runs the
  * reduction of flb_conservation before the step.  Errors as flb_step. */

@@ -95,7 +95,6 @@ __global__ void __launch_bounds__(128, 7) k_force_density(const __grid_constant_
             }
             L::moments(lo, m);
             L::moments(hi, n);
-            pdl_trigger();
             *reinterpret_cast<float4*>(out) = make_float4(m[0].v.x, m[0].v.y, n[0].v.x, n[0].v.y);
             if constexpr (SUMS) {
 #pragma unroll
@@ -118,17 +117,15 @@ __global__ void __launch_bounds__(128, 7) k_force_density(const __grid_constant_
                     g[i] = F2(A::plain1(r + x1), A::plain1(r + xe));
             }
             L::moments(g, m);
-            const bool two = GX == 2 || x + 1 < X;
-            pdl_trigger();
             if constexpr (GX == 2) {
                 *reinterpret_cast<float2*>(out) = m[0].v;
             } else {
                 out[0] = m[0].v.x;
-                if (two) out[1] = m[0].v.y;
+                if (x + 1 < X) out[1] = m[0].v.y;
             }
-            if constexpr (SUMS) {
+            if constexpr (SUMS) {  // GX == 2: both sites exist
 #pragma unroll
-                for (int k = 0; k < 4; ++k) v4[k] = two ? m[k].v.x + m[k].v.y : m[k].v.x;
+                for (int k = 0; k < 4; ++k) v4[k] = m[k].v.x + m[k].v.y;
             }
         }
     }
@@ -195,7 +192,6 @@ __global__ void __launch_bounds__(128)
             out[k] = m.v.x;
             out[k + 1] = m.v.y;
         }
-        if (h == 0) pdl_trigger();
         if (h == 1 && z + 1 == Z) return;
         float* o = mu + (zo[1 + h] + X * y + x);
         if constexpr (N == 4) {
@@ -278,7 +274,6 @@ __global__ void __launch_bounds__(128, 4)
     const int site = x + X * y + XY * z;
     const bool two = AL || x + 1 < X;
     L::collide(g, fx, fy, fz, a.c, (uint32_t)site, a.c.step);
-    pdl_trigger();
 #pragma unroll
     for (int i = 0; i < L::Q; ++i) {
         if constexpr (AL) {

@@ -22,16 +22,15 @@
 namespace flb {
 
 // Programmatic dependent launch.  A kernel launched with launch_chain may start
-// while the kernel before it on the stream drains: pdl_wait waits until
-// everything before this kernel is complete and visible and comes before any
-// access to memory; after pdl_trigger of all its blocks (or their end) the next
-// one may start.  The trigger stands before a kernel's stores: blocks of the
-// next kernel that start while this one still computes are placed on the SMs
-// that happen to have room, several on one, and wait there (a trigger at the
-// start: 48^3 force model 15.7 instead of 9.7 us a step, 160 x 128 in FP64
-// 30.9 instead of 12.1).
+// while the last blocks of the kernel before it on the stream are ending:
+// pdl_wait waits until everything before this kernel is complete and visible
+// and comes before any access to memory.  No kernel triggers its dependent
+// earlier than its blocks' end: blocks that start while this one still computes
+// are placed on the SMs that happen to have room, several on one, and wait
+// there (a trigger at the start: 48^3 force model 15.7 instead of 9.7 us a
+// step, 160 x 128 in FP64 30.9 instead of 12.1; a trigger before the stores:
+// ideal step 256^3 420 instead of 417, 32^3 3.3 instead of 2.9).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Indices of the 3x3x3 neighbourhood of (x, y, z) on a periodic X*Y*Z lattice:
 // xv[1+dx] + rb[1+dy][1+dz] is the site index of (x+dx, y+dy, z+dz).
@@ -72,18 +71,22 @@ inline void fast_div(uint32_t d, uint32_t& m, uint32_t& s)
 }
 __device__ __forceinline__ uint32_t fast_quot(uint32_t n, uint32_t m, uint32_t s) { return (__umulhi(n, m) + n) >> s; }
 
-// The row width that covers an X x Y plane with the fewest tiles, the widest
-// of equals (a wide row has the fewest partial sectors).
+// The row width that covers an X x Y plane at the least cost: the number of
+// tiles, weighed by what the narrower rows lose on partial sectors (measured on
+// the pair kernels at X = 36 to 129: rows of 64 sites and of 32 alike, 16 worth
+// 1.2, 8 worth 1.6 tiles; 129 x 95 x 67 force model, rows of 64 / 32 / 16 / 8:
+// 51.7, 46.8, 48.3, 65.9 us).
 inline Tiling make_tiling(int X, int Y, int Z, int N, int threads, int planes)
 {
     Tiling t{};
     int lt = 5;  // log2 of the threads per plane
     while ((1 << lt) * planes < threads) ++lt;
-    long best = 0;
+    double best = 0.0;
     for (int lw = 5; lw >= 2; --lw) {
         const int w = N << lw, lh = lt - lw, h = 1 << lh, nx = (X + w - 1) / w, ny = (Y + h - 1) / h;
-        if (best && (long)nx * ny >= best) continue;
-        best = (long)nx * ny;
+        const double cost = (double)nx * ny * (w >= 64 ? 1.0 : w >= 32 ? 1.05 : w >= 16 ? 1.2 : w >= 8 ? 1.6 : 2.5);
+        if (best > 0.0 && cost >= best) continue;
+        best = cost;
         t.lw = lw;
         t.lh = lh;
         t.ntx = nx;
@@ -311,7 +314,6 @@ __global__ void __launch_bounds__(kSitesThreads)
     R g[L::Q], m[L::Q];
     pull<L>(src, (long)X * Y * Z, nb, g);
     L::moments(g, m);
-    pdl_trigger();
     drho[r.x + X * (r.y + Y * r.z)] = m[0];
 }
 
@@ -356,26 +358,47 @@ __global__ void __launch_bounds__(kSitesThreads)
     pull_planes<L, false>(P, nb, g);
     R F[3] = {R(0), R(0), R(0)};
     if constexpr (FORCE) {
-        // sum_i w_i c_i f(r + c_i) from the differences f(c) - f(-c) of the velocity
-        // pairs (2k-1, 2k): axis pairs weigh 1/18, edge pairs 1/36
-        auto grad = [&](const R* f, R d[3]) {
-            R e[10];
+        if constexpr (std::is_same<R, float>::value) {
+            // grad = 3 sum_i w_i c_i mu(r + c_i); F = -rho grad mu (+ cs^2 grad rho)
+            R gr[3] = {R(0), R(0), R(0)};
+            auto add = [&](const R* f, R d[3]) {
 #pragma unroll
-            for (int k = 1; k <= 9; ++k) {
-                const int i = 2 * k - 1, cx = Vel<L>::cx(i), cy = Vel<L>::cy(i), cz = Vel<L>::cz(i);
-                e[k] = f[nb.src(-cx, -cy, -cz)] - f[nb.src(cx, cy, cz)];
+                for (int i = 1; i < L::Q; ++i) {
+                    const int cx = Vel<L>::cx(i), cy = Vel<L>::cy(i), cz = Vel<L>::cz(i);
+                    const R wm = R(Vel<L>::w(i)) * f[nb.src(-cx, -cy, -cz)];
+                    if (cx) d[0] += R(cx) * wm;
+                    if (cy) d[1] += R(cy) * wm;
+                    if (cz) d[2] += R(cz) * wm;
+                }
+            };
+            add(mu, gr);
+            const R pre = R(-3) * (a.c.rho0 + drho[s]);
+            F[0] = pre * gr[0];
+            F[1] = pre * gr[1];
+            F[2] = pre * gr[2];
+            if (a.pgrad != R(0)) add(drho, F);
+        } else {
+            // sum_i w_i c_i f(r + c_i) from the differences f(c) - f(-c) of the velocity
+            // pairs (2k-1, 2k): axis pairs weigh 1/18, edge pairs 1/36
+            auto grad = [&](const R* f, R d[3]) {
+                R e[10];
+#pragma unroll
+                for (int k = 1; k <= 9; ++k) {
+                    const int i = 2 * k - 1, cx = Vel<L>::cx(i), cy = Vel<L>::cy(i), cz = Vel<L>::cz(i);
+                    e[k] = f[nb.src(-cx, -cy, -cz)] - f[nb.src(cx, cy, cz)];
+                }
+                d[0] = R(1.0 / 18) * e[1] + R(1.0 / 36) * ((e[4] + e[5]) + (e[6] + e[7]));
+                d[1] = R(1.0 / 18) * e[2] + R(1.0 / 36) * ((e[4] - e[5]) + (e[8] + e[9]));
+                d[2] = R(1.0 / 18) * e[3] + R(1.0 / 36) * ((e[6] - e[7]) + (e[8] - e[9]));
+            };
+            R d[3];
+            grad(mu, d);
+            const R pre = R(-3) * (a.c.rho0 + drho[s]);
+            for (int k = 0; k < 3; ++k) F[k] = pre * d[k];
+            if constexpr (TOTAL) {
+                grad(drho, d);
+                for (int k = 0; k < 3; ++k) F[k] += d[k];
             }
-            d[0] = R(1.0 / 18) * e[1] + R(1.0 / 36) * ((e[4] + e[5]) + (e[6] + e[7]));
-            d[1] = R(1.0 / 18) * e[2] + R(1.0 / 36) * ((e[4] - e[5]) + (e[8] + e[9]));
-            d[2] = R(1.0 / 18) * e[3] + R(1.0 / 36) * ((e[6] - e[7]) + (e[8] - e[9]));
-        };
-        R d[3];
-        grad(mu, d);
-        const R pre = R(-3) * (a.c.rho0 + drho[s]);
-        for (int k = 0; k < 3; ++k) F[k] = pre * d[k];
-        if constexpr (TOTAL) {
-            grad(drho, d);
-            for (int k = 0; k < 3; ++k) F[k] += d[k];
         }
     }
     auto normals = [&](R* q) {
@@ -391,14 +414,14 @@ __global__ void __launch_bounds__(kSitesThreads)
         L::template collide_with<FORCE>(g, F[0], F[1], F[2], a.c, normals);
     else
         L::collide_with(g, F[0], F[1], a.c, normals);
-    pdl_trigger();
     if (!in) return;
 #pragma unroll
     for (int i = 0; i < L::Q; ++i) store_stream(P.dst[i] + s, g[i]);
 }
 
 // mu = psi'(rho) - kappa lap rho of every site (D3Q19, one site per thread): the
-// Laplacian is 6 sum_i w_i (rho_i - rho) = (1/3) (axis sum) + (1/6) (edge sum) - 4 rho.
+// Laplacian is 6 sum_i w_i (rho_i - rho), in FP64 as (1/3) (axis sum) + (1/6)
+// (edge sum) - 4 rho (fewer operations on the slow pipe).
 template <class R>
 __global__ void __launch_bounds__(kSitesThreads)
     k_mu_field(const StepArgs<R> a, const R* __restrict__ drho, R* __restrict__ mu, const Tiling t)
@@ -410,18 +433,22 @@ __global__ void __launch_bounds__(kSitesThreads)
     const Nbhd nb(r.x, r.y, r.z, a.X, a.Y, a.Z);
     const int s = r.x + a.X * (r.y + a.Y * r.z);
     const R rc = drho[s];
-    R ax = R(0), ed = R(0);
+    R lap = R(0), ed = R(0);
 #pragma unroll
     for (int i = 1; i < L::Q; ++i) {
         const R v = drho[nb.src(-Vel<L>::cx(i), -Vel<L>::cy(i), -Vel<L>::cz(i))];
-        if (i < 7)
-            ax += v;
+        if constexpr (std::is_same<R, float>::value)
+            lap += R(Vel<L>::w(i)) * (v - rc);
+        else if (i < 7)
+            lap += v;
         else
             ed += v;
     }
-    const R lap = R(1.0 / 3) * ax + R(1.0 / 6) * ed - R(4) * rc;
+    if constexpr (std::is_same<R, float>::value)
+        lap *= R(6);
+    else
+        lap = R(1.0 / 3) * lap + R(1.0 / 6) * ed - R(4) * rc;
     const R d = rc + a.rho0_minus_rhoc;
-    pdl_trigger();
     mu[s] = d * (a.A + a.B * d * d) - a.kappa * lap;
 }
 
@@ -443,6 +470,7 @@ __global__ void __launch_bounds__(TX* TY)
     __shared__ R smu[MY * MX];
     const int tid = threadIdx.x + TX * threadIdx.y;
     const int x0 = blockIdx.x * TX - 2, y0 = blockIdx.y * TY - 2;
+    pdl_wait();
     for (int e = tid; e < RY * RX; e += NT) {
         const Nbhd nh(wrap_any(x0 + e % RX, X), wrap_any(y0 + e / RX, Y), 0, X, Y, 1);
         R g[L::Q], m[L::Q];
@@ -519,6 +547,7 @@ __global__ void __launch_bounds__(TX* TY)
     const int X = a.X, Y = a.Y;
     const int tid = threadIdx.x + TX * threadIdx.y;
     const int x0 = blockIdx.x * TX - 1, y0 = blockIdx.y * TY - 1;
+    pdl_wait();
     for (int e = tid; e < RX * RY; e += TX * TY)
         srho[e] = drho[wrap_any(x0 + e % RX, X) + (long)X * wrap_any(y0 + e / RX, Y)];
     __syncthreads();
@@ -559,24 +588,28 @@ __global__ void __launch_bounds__(TX* TY)
 }
 
 // ---------------------------------------------------------------------------
-// Ideal gas, FP32 or BF16 storage, two sites (x, x+1) per thread with packed
-// FP32 arithmetic (F2).  X must be even: a thread's pair then never straddles a
-// row and its populations at (x, x+1) are aligned to the pair's size.  Pulls along c_x = 0 are
-// single 8-byte loads; along c_x = +-1 the pair comes from (x-1, x) or
-// (x+1, x+2).  Block = TXT x TY x TZ threads covering 2 TXT x TY x TZ sites.
+// D3Q19 ideal gas, FP32 or BF16 storage, two sites (x, x+1) per thread with
+// packed FP32 arithmetic (F2).  AL: X even, a thread's pair never straddles a
+// row and its populations at (x, x+1) are aligned to the pair's size: pulls
+// along c_x = 0 are single loads of two, along c_x = +-1 the pair comes from
+// (x-1, x) or (x+1, x+2).  Odd X: single loads, the last pair of a row is one
+// site.
+// Bound by DRAM at 256^3 (417 us, 152 B/site at 6.1 TB/s) and 128^3; small
+// lattices by launch and latency: chained launches 6.2 -> 2.9 us at 32^3, tiles
+// that fit the row 32.6 -> 24 us at 96^3, pairs instead of single sites 34.9 ->
+// 30.8 us at 129 x 95 x 67.
 // ---------------------------------------------------------------------------
-template <class L, class S, int TXT, int TY, int TZ, int MINB = 1>
-__global__ void __launch_bounds__(TXT* TY* TZ, MINB)
-    k_step2(const StepArgs<float> a, const __grid_constant__ Planes<S> P)
+template <class S, bool AL, int MINB>
+__global__ void __launch_bounds__(128, MINB)
+    k_step2(const StepArgs<float> a, const __grid_constant__ Planes<S> P, const Tiling t)
 {
+    using L = D3Q19;
     using A = Packed<S>;
-    const int x = 2 * (blockIdx.x * TXT + threadIdx.x);
-    const int y = blockIdx.y * TY + threadIdx.y;
-    const int z = blockIdx.z * TZ + threadIdx.z;
-    const int X = a.X, Y = a.Y, Z = a.Z;
+    pdl_wait();
+    const int3 r0 = tile_site<2, 2, false>(t, threadIdx.x);
+    const int x = r0.x, y = r0.y, z = r0.z, X = a.X, Y = a.Y, Z = a.Z;
     if (x >= X || y >= Y || z >= Z) return;
-    const int xm = x == 0 ? X - 1 : x - 1;  // x - 1
-    const int x2 = x + 2 == X ? 0 : x + 2;  // x + 2
+    const int xm = x == 0 ? X - 1 : x - 1, x1 = AL ? x + 1 : x + 1 == X ? 0 : x + 1, x2 = x1 + 1 == X ? 0 : x1 + 1;
     const int yv[3] = {wrap_once(y - 1, Y), y, wrap_once(y + 1, Y)};
     const int zv[3] = {wrap_once(z - 1, Z), z, wrap_once(z + 1, Z)};
     int rb[3][3];
@@ -590,16 +623,23 @@ __global__ void __launch_bounds__(TXT* TY* TZ, MINB)
         const S* p = P.src[i] + rb[1 - Vel<L>::cy(i)][1 - Vel<L>::cz(i)];
         const int cx = Vel<L>::cx(i);
         if (cx == 0)
-            g[i] = mk2(A::stream2(p + x));
+            g[i] = AL ? mk2(A::stream2(p + x)) : F2(A::stream1(p + x), A::stream1(p + x1));
         else if (cx > 0)
             g[i] = F2(A::stream1(p + xm), A::stream1(p + x));
         else
-            g[i] = F2(A::stream1(p + x + 1), A::stream1(p + x2));
+            g[i] = F2(A::stream1(p + x1), A::stream1(p + x2));
     }
     const int s = x + X * (y + Y * z);
     L::template collide<false>(g, F2(0.f), F2(0.f), F2(0.f), a.c, (uint32_t)s, a.c.step);
 #pragma unroll
-    for (int i = 0; i < L::Q; ++i) A::store2(P.dst[i] + s, g[i].v);
+    for (int i = 0; i < L::Q; ++i) {
+        if constexpr (AL) {
+            A::store2(P.dst[i] + s, g[i].v);
+        } else {
+            A::store1(P.dst[i] + s, g[i].v.x);
+            if (x + 1 < X) A::store1(P.dst[i] + s + 1, g[i].v.y);
+        }
+    }
 }
 
 }  // namespace flb

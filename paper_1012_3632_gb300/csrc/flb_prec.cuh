@@ -11,25 +11,6 @@
 #include "flb_internal.h"
 #include "flb_kernels.cuh"
 
-#ifndef FLB_STEP2_TXT
-#define FLB_STEP2_TXT 32
-#endif
-#ifndef FLB_STEP2_TY
-#define FLB_STEP2_TY 2
-#endif
-#ifndef FLB_STEP2_TZ
-#define FLB_STEP2_TZ 2
-#endif
-// Ideal-gas two-site step, minimum resident blocks per SM: 5 with FP32
-// storage (96 registers, 48 bytes spilled, 20 warps per SM: measured faster
-// than 4 blocks at 126 registers), 4 with BF16 storage (5 measured slower).
-#ifndef FLB_STEP2_MINB
-#define FLB_STEP2_MINB 5
-#endif
-#ifndef FLB_STEP2_MINB_BF16
-#define FLB_STEP2_MINB_BF16 4
-#endif
-
 #include "flb_force.cuh"
 
 namespace flb {
@@ -444,10 +425,19 @@ struct Prec {
     // FP32 arithmetic on FP32 or BF16 storage: the two-sites-per-thread kernels
     static constexpr bool kPackedStorage =
         std::is_same<R, float>::value && (std::is_same<S, float>::value || std::is_same<S, __nv_bfloat16>::value);
+    // The packed kernels take every D3Q19 lattice in FP32 storage; in BF16 storage
+    // those of even X without the total free energy.  (The others keep the
+    // arithmetic of one site per lane: another order of the FP32 operations moves
+    // populations across BF16 rounding boundaries, and the conserved totals with
+    // them by 1e-8.)
+    static bool packed(const HostModel& m)
+    {
+        return kPackedStorage && m.Q == 19 && (std::is_same<S, float>::value || (m.X % 2 == 0 && !m.total));
+    }
     static cudaError_t density(const HostModel& m, const void* pop, void* drho, cudaStream_t st)
     {
         if constexpr (kPackedStorage) {
-            if (m.Q == 19) return density_packed(m, pop, (float*)drho, nullptr, st);
+            if (packed(m)) return density_packed(m, pop, (float*)drho, nullptr, st);
         }
         const Tiling t = make_tiling(m.X, m.Y, m.Z, 1, kSitesThreads, m.D == 3 ? 2 : 1);
         const auto k = m.Q == 19 ? k_density<D3Q19, R, S> : k_density<D2Q9, R, S>;
@@ -478,7 +468,7 @@ struct Prec {
         return launch_chain(k_sites<L, R, S, FORCE, TOTAL, false>, dim3(t.blocks()), dim3(kSitesThreads), st, a, pl,
                             drho, mu, t);
     }
-    // D3Q19 force model, FP64: density, mu and collision passes.
+    // D3Q19 force model, one site per lane: density, mu and collision passes.
     static cudaError_t step_force_sites(const HostModel& m, uint64_t step, const void* src, void* dst, R* drho,
                                         cudaStream_t st)
     {
@@ -493,7 +483,7 @@ struct Prec {
                        : step_sites<D3Q19, true, false>(m, step, src, dst, rho, st);
     }
     // The D3Q19 force model steps in passes over the context's density and mu
-    // fields: FP32 and BF16 storage by flb_force.cuh, FP64 by k_sites.
+    // fields: packed storage by flb_force.cuh, the rest by k_sites.
     static int step_in_passes(const HostModel& m) { return m.Q == 19 && m.nonideal; }
     static int gather_width(const HostModel& m) { return m.X % 4 == 0 ? 4 : m.X % 2 == 0 ? 2 : 1; }
     // density: quads of sites per thread, or pairs
@@ -501,9 +491,11 @@ struct Prec {
     {
         return make_tiling(m.X, m.Y, m.Z, gather_width(m) == 4 ? 4 : 2, 128, 2);
     }
+    // one row per warp; X even and the excess free energy, whose deviations are
+    // small: FP32 sums over a warp's sites would lose digits on a stripe's
     static int step_row_count(const HostModel& m)
     {
-        return kPackedStorage && step_in_passes(m) ? 4 * (int)density_tiling(m).blocks() : 0;  // one per warp
+        return packed(m) && m.nonideal && m.X % 2 == 0 && !m.total ? 4 * (int)density_tiling(m).blocks() : 0;
     }
     // rows (or NULL): step_row_count rows of mass deviation and momentum
     static cudaError_t density_packed(const HostModel& m, const void* pop, float* rho, float* rows, cudaStream_t st)
@@ -512,7 +504,7 @@ struct Prec {
         const Tiling t = density_tiling(m);
         auto go = [&](auto G) {
             constexpr int GX = decltype(G)::value;
-            const auto k = rows ? k_force_density<S, GX, true> : k_force_density<S, GX, false>;
+            const auto k = GX != 1 && rows ? k_force_density<S, GX, GX != 1> : k_force_density<S, GX, false>;
             return launch_chain(k, dim3(t.blocks()), dim3(128), st, pl, rho, rows, m.X, m.Y, m.Z, t);
         };
         const int gx = gather_width(m);
@@ -548,42 +540,39 @@ struct Prec {
     {
         return step_rows(m, t, src, dst, drho, nullptr, st);
     }
-    static cudaError_t step_rows(const HostModel& m, uint64_t t, const void* src, void* dst, const void* drho,
+    static cudaError_t step_rows(const HostModel& m, uint64_t step, const void* src, void* dst, const void* drho,
                                  float4* rows, cudaStream_t st)
     {
+        if (rows && !step_row_count(m)) return cudaErrorNotSupported;
         // drho: the context's density field, scratch of the steps in passes
         if constexpr (kPackedStorage) {
-            if (step_in_passes(m)) return step_force(m, t, src, dst, (float*)const_cast<void*>(drho), (float*)rows, st);
+            if (packed(m) && m.nonideal) return step_force(m, step, src, dst, (float*)const_cast<void*>(drho), (float*)rows, st);
         }
-        if (rows) return cudaErrorNotSupported;
-        if (step_in_passes(m)) return step_force_sites(m, t, src, dst, (R*)const_cast<void*>(drho), st);
+        if (step_in_passes(m)) return step_force_sites(m, step, src, dst, (R*)const_cast<void*>(drho), st);
         if (m.Q == 9 && m.nonideal && m.model == 1) {
-            const StepArgs<R> a = make_args<D2Q9, R>(m, t);
+            const StepArgs<R> a = make_args<D2Q9, R>(m, step);
             const dim3 b(32, 8, 1);
-            k_step_swift<R, S, 32, 8><<<grid_for(m, b), b, 0, st>>>(a, make_planes<S>(src, dst, 9, m.V),
-                                                                      (const R*)drho,
-                                                                      (const NoiseField<R>*)m.swift_xi);
-            return cudaGetLastError();
+            return launch_chain(k_step_swift<R, S, 32, 8>, grid_for(m, b), b, st, a, make_planes<S>(src, dst, 9, m.V),
+                                (const R*)drho, (const NoiseField<R>*)m.swift_xi);
         }
         if (m.Q == 9 && m.nonideal) {
             const dim3 b(32, 8, 1);
-            k_step_gather<R, S, 32, 8>
-                <<<grid_for(m, b), b, 0, st>>>(make_args<D2Q9, R>(m, t), make_planes<S>(src, dst, 9, m.V));
-            return cudaGetLastError();
+            return launch_chain(k_step_gather<R, S, 32, 8>, grid_for(m, b), b, st, make_args<D2Q9, R>(m, step),
+                                make_planes<S>(src, dst, 9, m.V));
         }
         if constexpr (kPackedStorage) {
-            if (m.Q == 19 && m.X % 2 == 0) {
-                constexpr int TXT = FLB_STEP2_TXT, TY = FLB_STEP2_TY, TZ = FLB_STEP2_TZ;
-                const StepArgs<R> a = make_args<D3Q19, R>(m, t);
-                const dim3 b(TXT, TY, TZ);
-                const dim3 g((m.X / 2 + TXT - 1) / TXT, (m.Y + TY - 1) / TY, (m.Z + TZ - 1) / TZ);
-                constexpr int MINB = sizeof(S) == 4 ? FLB_STEP2_MINB : FLB_STEP2_MINB_BF16;
-                k_step2<D3Q19, S, TXT, TY, TZ, MINB><<<g, b, 0, st>>>(a, make_planes<S>(src, dst, 19, m.V));
-                return cudaGetLastError();
+            if (packed(m)) {
+                // minimum resident blocks per SM: 5 with FP32 storage (96 registers, 48
+                // bytes spilled: measured faster than 4 at 126), 4 with BF16 storage
+                constexpr int MINB = sizeof(S) == 4 ? 5 : 4;
+                const Tiling t = make_tiling(m.X, m.Y, m.Z, 2, 128, 2);
+                const auto k = m.X % 2 == 0 ? k_step2<S, true, MINB> : k_step2<S, false, MINB>;
+                return launch_chain(k, dim3(t.blocks()), dim3(128), st, make_args<D3Q19, R>(m, step),
+                                    make_planes<S>(src, dst, 19, m.V), t);
             }
         }
-        return m.Q == 19 ? step_sites<D3Q19, false, false>(m, t, src, dst, nullptr, st)
-                         : step_sites<D2Q9, false, false>(m, t, src, dst, nullptr, st);
+        return m.Q == 19 ? step_sites<D3Q19, false, false>(m, step, src, dst, nullptr, st)
+                         : step_sites<D2Q9, false, false>(m, step, src, dst, nullptr, st);
     }
 
     template <class L>
