@@ -619,11 +619,18 @@ int flb_moments(flb_ctx* c, double* out, int which)
     if (which == FLB_MODE_VAR) {
         int rc = ensure_partials(c);
         if (rc) return rc;
-        int nrows = 0;
-        FLB_CUDA(c->ops->mode_partials(m, src, c->partials, &nrows, c->stream));
+        flb::ModeSums a;
+        a.n = 0;
+        a.rows = c->partials;
+        a.lat[0].first = 0;
+        // one warp per block while that leaves SMs without a block
+        const int warps = ((long)((m.X + 31) / 32) * m.Y * m.Z) < 8 * 152 ? 1 : 8;
+        flb::mode_blocks(a, src, m.X, m.Y, m.Z, warps);
+        FLB_CUDA(c->ops->mode_sums(a, m.Q, warps, c->stream));
+        FLB_CUDA(flb::sum_lattices(a, 2 * m.Q, c->red, c->stream));
         std::vector<double> h(2 * m.Q);
-        rc = reduce_to_host(c, nrows, 2 * m.Q, h.data());
-        if (rc) return rc;
+        FLB_CUDA(cudaMemcpyAsync(h.data(), c->red, h.size() * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+        FLB_CUDA(cudaStreamSynchronize(c->stream));
         c->mv_count += 1;
         for (int a = 0; a < m.Q; ++a) {
             const double mean = h[a] / (double)m.V;

@@ -495,20 +495,19 @@ int flb_batch_mode_variance(flb_batch* b, double* out)
     if (!b || !out) return bfail(FLB_EINVAL, "NULL argument");
     Dev guard(b->device);
     const flb::PrecOps& ops = flb::ops_fp32();
+    // one launch over every replica's sites, one over their rows, one copy, one wait
+    flb::ModeSums a;
+    a.n = 0;
+    a.lat[0].first = 0;
+    for (int r = 0; r < b->n; ++r) flb::mode_blocks(a, rep_src(b, r), b->m[r].X, b->m[r].Y, b->m[r].Z, 8);
     if (!b->partials) {
-        int rows = 0;
-        for (int r = 0; r < b->n; ++r) rows = std::max(rows, ops.partial_rows_max(b->m[r]));
-        BCUDA(cudaMalloc(&b->partials, (size_t)rows * 38 * sizeof(double)));
+        BCUDA(cudaMalloc(&b->partials, (size_t)a.lat[a.n].first * 38 * sizeof(double)));
         BCUDA(cudaMalloc(&b->red, (size_t)b->n * 38 * sizeof(double)));
     }
+    a.rows = b->partials;
     b->mv_count += 1;
-    // every replica's 38 column sums into its own row of red (the partial-sum
-    // rows are reused in stream order), then one copy and one wait
-    for (int r = 0; r < b->n; ++r) {
-        int nrows = 0;
-        BCUDA(ops.mode_partials(b->m[r], rep_src(b, r), b->partials, &nrows, b->stream));
-        BCUDA(flb::sum_columns(b->partials, nrows, 38, b->red + 38 * (size_t)r, b->stream));
-    }
+    BCUDA(ops.mode_sums(a, 19, 8, b->stream));
+    BCUDA(flb::sum_lattices(a, 38, b->red, b->stream));
     std::vector<double> h((size_t)b->n * 38);
     BCUDA(cudaMemcpyAsync(h.data(), b->red, h.size() * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
     BCUDA(cudaStreamSynchronize(b->stream));

@@ -38,6 +38,25 @@ cudaError_t sum_columns(const double* partials, int nrows, int ncol, double* out
     return launch_chain(k_sum_columns, dim3(ncol), dim3(256), s, partials, nrows, ncol, out, add0);
 }
 
+__global__ void __launch_bounds__(128) k_sum_lattices(const __grid_constant__ ModeSums a, int ncol,
+                                                      double* __restrict__ out)
+{
+    __shared__ double sh[4];
+    pdl_wait();
+    const int c = blockIdx.x, r = blockIdx.y, end = a.lat[r + 1].first;
+    double acc = 0.0;
+    for (int k = a.lat[r].first + threadIdx.x; k < end; k += 128) acc += a.rows[(long)k * ncol + c];
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) out[r * ncol + c] = (sh[0] + sh[1]) + (sh[2] + sh[3]);
+}
+
+cudaError_t sum_lattices(const ModeSums& a, int ncol, double* out, cudaStream_t s)
+{
+    return launch_chain(k_sum_lattices, dim3(ncol, a.n), dim3(128), s, a, ncol, out);
+}
+
 // Step blockIdx.y: its rows are split over gridDim.x blocks; the block that
 // comes last adds their partial sums in block order (deterministic).
 __global__ void __launch_bounds__(256) k_sum_steps(const float4* __restrict__ rows, int nrows, int per,

@@ -46,6 +46,37 @@ struct HostModel {
     void* mu = nullptr;  // force-model step in passes: the context's chemical potential field
 };
 
+// Lattices whose mode sums one launch forms; lattice r owns the blocks and rows
+// lat[r].first .. lat[r + 1].first of 2 Q doubles.
+struct ModeLattice {
+    const void* src;
+    int X, Y, Z, first;
+};
+struct ModeSums {
+    int n;
+    double* rows;
+    ModeLattice lat[FLB_BATCH_MAX + 1];
+};
+constexpr int kModeRowsMin = 512;  // rows that a partial-sum buffer holds at least
+// Append a lattice; returns its blocks.  Sixteen groups of 32 sites per warp and
+// at most six blocks per SM: long enough that the block's own sums do not count.
+inline int mode_blocks(ModeSums& a, const void* src, int X, int Y, int Z, int warps)
+{
+    const long groups = (long)((X + 31) / 32) * Y * Z, most = 6 * 152;
+    long nb = (groups + 16 * warps - 1) / (16 * warps);
+    if (nb < 152) nb = (groups + warps - 1) / warps < 152 ? (groups + warps - 1) / warps : 152;
+    if (nb > most) nb = most;
+    ModeLattice& q = a.lat[a.n];
+    q.src = src;
+    q.X = X;
+    q.Y = Y;
+    q.Z = Z;
+    a.lat[++a.n].first = q.first + (int)nb;
+    return (int)nb;
+}
+// Column sums of each lattice's rows: out[r * ncol + c] (flb_fft.cu).
+cudaError_t sum_lattices(const ModeSums& a, int ncol, double* out, cudaStream_t s);
+
 // Kernels whose code depends on the compute/storage type.  Pointers are device
 // pointers; `pop` buffers hold Q*V elements of the storage type, `field`
 // buffers V (or 3V) elements of the compute type.
@@ -63,9 +94,9 @@ struct PrecOps {
     cudaError_t (*moments)(const HostModel&, const void* src, double* out, int which, const void* F,
                            cudaStream_t);
     cudaError_t (*mu_force)(const HostModel&, const void* drho, void* mu, void* F, cudaStream_t);
+    // per-block sums of m_a and m_a^2, warps per block as mode_blocks returns
+    cudaError_t (*mode_sums)(const ModeSums&, int Q, int warps, cudaStream_t);
     // per-block partial sums; returns the number of partial rows written
-    cudaError_t (*mode_partials)(const HostModel&, const void* src, double* partials, int* nrows,
-                                 cudaStream_t);
     cudaError_t (*cons_partials)(const HostModel&, const void* src, double* partials, int* nrows,
                                  cudaStream_t);
     // mode a of the pre-collision state as a complex field: double2, or float2

@@ -305,28 +305,95 @@ __device__ __forceinline__ long block_linear()
     return blockIdx.x + (long)gridDim.x * (blockIdx.y + (long)gridDim.y * blockIdx.z);
 }
 
-// Per block: sum m_a and sum m_a^2 of the pre-collision moments (m_0 = drho).
-template <class L, class R, class S>
-__global__ void k_mode_partials(const S* __restrict__ src, double* __restrict__ partials, int X, int Y, int Z)
+// Sums of m_a and m_a^2 of the pre-collision moments (m_0 = drho) over one or
+// many lattices.  A warp takes groups of 32 sites along x and adds the 2 Q
+// values of its lanes in the compute type by exchanging halves: at distance 16,
+// 8, .. 1 a lane keeps half of its columns and adds what the other lane holds
+// of them (39 exchanges for 38 columns; a shuffle tree per column takes 190).
+// Two columns are left per lane, and only these go to FP64, once per group.
+// Bound by DRAM (76 B/site): 128^3 FP32 148 -> 28 us; the trees and a
+// conversion of every column per warp and block kept the FP64 pipe busy.
+template <int N, int O, class R>
+__device__ __forceinline__ void halve_columns(R* v)
 {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z * blockDim.z + threadIdx.z;
-    R v[2 * L::Q];
-    for (int q = 0; q < 2 * L::Q; ++q) v[q] = R(0);
-    if (x < X && y < Y && z < Z) {
-        const long V = (long)X * Y * Z;
-        const Nbhd nb(x, y, z, X, Y, Z);
-        R g[L::Q], m[L::Q];
-        pull<L>(src, V, nb, g);
-        L::moments(g, m);
+    constexpr int H = (N + 1) / 2;
+    const bool up = threadIdx.x & O;
 #pragma unroll
-        for (int q = 0; q < L::Q; ++q) {
-            v[q] = m[q];
-            v[L::Q + q] = m[q] * m[q];
-        }
+    for (int k = 0; k < H; ++k) {
+        const R hi = k + H < N ? v[k + H] : R(0);
+        const R keep = up ? hi : v[k], send = up ? v[k] : hi;
+        v[k] = keep + __shfl_xor_sync(0xffffffffu, send, O);
     }
-    block_sum_row<2 * L::Q>(v, partials + block_linear() * (2 * L::Q));
+    if constexpr (O > 1) halve_columns<H, O / 2>(v);
+}
+// Column of value k after halve_columns<N, 16>, or -1 for padding.
+template <int N, int O>
+__device__ __forceinline__ int halved_column(int k)
+{
+    constexpr int H = (N + 1) / 2;
+    if constexpr (O > 1) k = halved_column<H, O / 2>(k);
+    if (k < 0 || k >= H) return -1;
+    k += (threadIdx.x & O) ? H : 0;
+    return k < N ? k : -1;
+}
+
+constexpr int kModeWarps = 8;
+
+template <class L, class R, class S>
+__global__ void __launch_bounds__(32 * kModeWarps) k_mode_sums(const __grid_constant__ ModeSums a)
+{
+    constexpr int NC = 2 * L::Q, NK = 2;  // columns, columns left per lane
+    static_assert(NC <= 64, "two columns per lane");
+    __shared__ double red[kModeWarps][NC];
+    pdl_wait();
+    int lo = 0, hi = a.n;  // the lattice of this block
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) / 2;
+        if ((int)blockIdx.x >= a.lat[mid].first)
+            lo = mid;
+        else
+            hi = mid;
+    }
+    const ModeLattice& q = a.lat[lo];
+    const int X = q.X, Y = q.Y, Z = q.Z, nx = (X + 31) / 32;
+    const long V = (long)X * Y * Z;
+    const S* src = (const S*)q.src;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
+    const int nb = a.lat[lo + 1].first - q.first;
+    const long groups = (long)nx * Y * Z, stride = (long)nb * wpb;
+    double acc[NK] = {0.0, 0.0};
+    for (long g = ((int)blockIdx.x - q.first) * wpb + warp; g < groups; g += stride) {
+        const long row = g / nx;
+        const int x = (int)(g - row * nx) * 32 + lane, y = (int)(row % Y), z = (int)(row / Y);
+        R v[NC + 1];
+#pragma unroll
+        for (int k = 0; k < NC + 1; ++k) v[k] = R(0);
+        if (x < X) {
+            const Nbhd nb3(x, y, z, X, Y, Z);
+            R f[L::Q], m[L::Q];
+            pull<L>(src, V, nb3, f);
+            L::moments(f, m);
+#pragma unroll
+            for (int k = 0; k < L::Q; ++k) {
+                v[k] = m[k];
+                v[L::Q + k] = m[k] * m[k];
+            }
+        }
+        halve_columns<NC, 16>(v);
+#pragma unroll
+        for (int k = 0; k < NK; ++k) acc[k] += (double)v[k];
+    }
+#pragma unroll
+    for (int k = 0; k < NK; ++k) {
+        const int c = halved_column<NC, 16>(k);
+        if (c >= 0) red[warp][c] = acc[k];
+    }
+    __syncthreads();
+    for (int c = threadIdx.x; c < NC; c += blockDim.x) {
+        double t = 0.0;
+        for (int w = 0; w < wpb; ++w) t += red[w][c];
+        a.rows[(long)blockIdx.x * NC + c] = t;
+    }
 }
 
 // Per block: sum of g and of g c over the stored buffer (a permutation of the
@@ -646,30 +713,25 @@ struct Prec {
     // a density field written before the step: only the modified-equilibrium
     // step reads one (the force-model steps gather their density themselves)
     static int needs_density(const HostModel& m) { return m.nonideal && m.Q == 9 && m.model == 1 ? 1 : 0; }
-    static int rows(const HostModel& m)
+    static int site_blocks(const HostModel& m)
     {
         const dim3 b = m.Q == 19 ? site_block<D3Q19>() : site_block<D2Q9>();
         const dim3 g = grid_for(m, b);
         return (int)(g.x * g.y * g.z);
     }
-    static cudaError_t mode_partials(const HostModel& m, const void* src, double* partials, int* nrows,
-                                     cudaStream_t st)
+    static int rows(const HostModel& m) { return std::max(site_blocks(m), kModeRowsMin); }
+    // one launch over a.n lattices whose `first` and `rows` are set (mode_blocks)
+    static cudaError_t mode_sums(const ModeSums& a, int Q, int warps, cudaStream_t st)
     {
-        *nrows = rows(m);
-        if (m.Q == 19) {
-            const dim3 b = site_block<D3Q19>();
-            k_mode_partials<D3Q19, R, S><<<grid_for(m, b), b, 0, st>>>((const S*)src, partials, m.X, m.Y, m.Z);
-        } else {
-            const dim3 b = site_block<D2Q9>();
-            k_mode_partials<D2Q9, R, S><<<grid_for(m, b), b, 0, st>>>((const S*)src, partials, m.X, m.Y, m.Z);
-        }
-        return cudaGetLastError();
+        const dim3 g(a.lat[a.n].first), b(32 * warps);
+        return Q == 19 ? launch_chain(k_mode_sums<D3Q19, R, S>, g, b, st, a)
+                       : launch_chain(k_mode_sums<D2Q9, R, S>, g, b, st, a);
     }
     static cudaError_t cons_partials(const HostModel& m, const void* src, double* partials, int* nrows,
                                      cudaStream_t st)
     {
         if constexpr (std::is_same<R, float>::value) {
-            // at most rows(m): cons_blocks(V) <= ceil(V / 256) <= the site grid
+            // at most site_blocks(m): cons_blocks(V) <= ceil(V / 256) <= the site grid
             *nrows = cons_blocks(m.V);
             if (m.Q == 19)
                 k_cons_partials_sp<D3Q19, S><<<*nrows, kConsThreads, 0, st>>>((const S*)src, partials, m.V);
@@ -677,7 +739,7 @@ struct Prec {
                 k_cons_partials_sp<D2Q9, S><<<*nrows, kConsThreads, 0, st>>>((const S*)src, partials, m.V);
             return cudaGetLastError();
         }
-        *nrows = rows(m);
+        *nrows = site_blocks(m);
         if (m.Q == 19) {
             const dim3 b = site_block<D3Q19>();
             k_cons_partials<D3Q19, R, S><<<grid_for(m, b), b, 0, st>>>((const S*)src, partials, m.X, m.Y, m.Z);
@@ -742,7 +804,7 @@ struct Prec {
     static const PrecOps& ops()
     {
         static const PrecOps o = {(int)sizeof(S), (int)sizeof(R), density, step, init, get_pop, set_pop, moments,
-                                  mu_force, mode_partials, cons_partials, mode_field, rows, needs_density, step_in_passes,
+                                  mu_force, mode_sums, cons_partials, mode_field, rows, needs_density, step_in_passes,
                                   pull_state, push_state, get_sites, step_row_count, step_rows};
         return o;
     }
