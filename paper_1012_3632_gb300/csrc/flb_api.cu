@@ -96,7 +96,7 @@ struct flb_ctx {
     int mv_count = 0;
 
     // modified-equilibrium model: Cholesky table and the two noise fields
-    double* sw_chol = nullptr;
+    void* sw_chol = nullptr;  // in the compute type
     double2* sw_work = nullptr;
     double2* sw_xi = nullptr;
 
@@ -423,14 +423,18 @@ int flb_create(flb_ctx** out, int lattice, const int dims[3], double omega_shear
             delete c;
             return fail(FLB_EINVAL, err);
         }
-        if ((rc = alloc((void**)&c->sw_chol, chol.size() * sizeof(double))) ||
+        std::vector<float> chol_sp;
+        if (c->prec != FLB_FP64) chol_sp.assign(chol.begin(), chol.end());
+        const void* table = c->prec != FLB_FP64 ? (const void*)chol_sp.data() : chol.data();
+        const size_t table_bytes = chol.size() * (c->prec != FLB_FP64 ? sizeof(float) : sizeof(double));
+        if ((rc = alloc(&c->sw_chol, table_bytes)) ||
             (rc = alloc((void**)&c->sw_work, m.V * sizeof(double2))) ||
             (rc = alloc((void**)&c->sw_xi, m.V * sizeof(double2)))) {
             free_all(c);
             delete c;
             return rc;
         }
-        const cudaError_t ce = cudaMemcpy(c->sw_chol, chol.data(), chol.size() * sizeof(double), cudaMemcpyHostToDevice);
+        const cudaError_t ce = cudaMemcpy(c->sw_chol, table, table_bytes, cudaMemcpyHostToDevice);
         if (ce != cudaSuccess) {
             free_all(c);
             delete c;
@@ -671,37 +675,32 @@ int flb_structure_factor(flb_ctx* c, double* S, int mode, int accumulate)
     if (mode < 0 || mode >= m.Q) return fail(FLB_EINVAL, "mode out of range");
     DeviceGuard guard(c->device);
     int rc;
-    if ((rc = alloc((void**)&c->fft, m.V * sizeof(double2))) || (rc = alloc((void**)&c->fft_scratch, m.V * sizeof(double2))))
+    if ((rc = alloc((void**)&c->fft, (m.V + 1) * sizeof(double2))) || (rc = alloc((void**)&c->fft_scratch, m.V * sizeof(double2))))
         return rc;
     double* target = nullptr;
     if (accumulate) {
         if ((rc = alloc((void**)&c->sk_acc[mode], m.V * sizeof(double)))) return rc;
         if (c->sk_count[mode] == 0) FLB_CUDA(cudaMemsetAsync(c->sk_acc[mode], 0, m.V * sizeof(double), c->stream));
         target = c->sk_acc[mode];
-    } else {
-        if ((rc = alloc((void**)&c->sk_tmp, m.V * sizeof(double)))) return rc;
     }
+    if ((S || !accumulate) && (rc = alloc((void**)&c->sk_tmp, m.V * sizeof(double)))) return rc;
+    double* out = S || !accumulate ? c->sk_tmp : nullptr;
+    const double scale = accumulate ? 1.0 / (c->sk_count[mode] + 1) : 1.0;  // out: the mean over the snapshots
     // single-precision states are transformed in single precision (GB300's
     // FP64 rate is a small fraction of its FP32 rate); |F|^2 accumulates in FP64
-    const bool fp32 = c->prec != FLB_FP64;
-    FLB_CUDA(c->ops->mode_field(m, c->buf[c->cur], mode, c->fft, fp32, c->stream));
-    if (fp32) {
-        FLB_CUDA(flb::fft3d((float2*)c->fft, m.X, m.Y, m.Z, (float2*)c->fft_scratch, c->stream));
-        FLB_CUDA(flb::power_spectrum((const float2*)c->fft, m.V, target, c->sk_tmp, c->stream));
+    if (c->prec != FLB_FP64) {
+        float* real = (float*)(c->fft + m.V / 2 + 1);  // behind the V complex numbers of the transform
+        FLB_CUDA(c->ops->mode_field(m, c->buf[c->cur], mode, real, c->stream));
+        FLB_CUDA(flb::spectrum((float2*)c->fft, real, m.X, m.Y, m.Z, (float2*)c->fft_scratch, target, out, scale,
+                               c->stream));
     } else {
+        FLB_CUDA(c->ops->mode_field(m, c->buf[c->cur], mode, c->fft, c->stream));
         FLB_CUDA(flb::fft3d(c->fft, m.X, m.Y, m.Z, c->fft_scratch, c->stream));
-        FLB_CUDA(flb::power_spectrum(c->fft, m.V, target, c->sk_tmp, c->stream));
+        FLB_CUDA(flb::power_spectrum(c->fft, m.V, target, out, c->stream, scale));
     }
     if (accumulate) c->sk_count[mode] += 1;
     if (S) {
-        const double* src = c->sk_tmp;
-        if (accumulate) {
-            // the mean over the snapshots, formed on the device
-            if ((rc = alloc((void**)&c->sk_tmp, m.V * sizeof(double)))) return rc;
-            FLB_CUDA(flb::scale_copy(c->sk_acc[mode], 1.0 / c->sk_count[mode], m.V, c->sk_tmp, c->stream));
-            src = c->sk_tmp;
-        }
-        FLB_CUDA(cudaMemcpyAsync(S, src, m.V * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+        FLB_CUDA(cudaMemcpyAsync(S, out, m.V * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
         FLB_CUDA(cudaStreamSynchronize(c->stream));
     }
     return FLB_OK;

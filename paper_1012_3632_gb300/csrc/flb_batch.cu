@@ -533,7 +533,7 @@ int flb_batch_structure_factor(flb_batch* b, int replica, double* S, int mode, i
     if (!b->fft) {
         long vmax = 0;
         for (auto& mm : b->m) vmax = std::max(vmax, mm.V);
-        BCUDA(cudaMalloc(&b->fft, vmax * sizeof(double2)));
+        BCUDA(cudaMalloc(&b->fft, (vmax + 1) * sizeof(double2)));
         BCUDA(cudaMalloc(&b->fft_scratch, vmax * sizeof(double2)));
         BCUDA(cudaMalloc(&b->sk_tmp, vmax * sizeof(double)));
     }
@@ -546,13 +546,13 @@ int flb_batch_structure_factor(flb_batch* b, int replica, double* S, int mode, i
         slot.second += 1;
     }
     // FP32 states: FP32 transform, |F|^2 summed in FP64 (as flb_structure_factor)
-    BCUDA(ops.mode_field(m, rep_src(b, replica), mode, b->fft, true, b->stream));
-    BCUDA(flb::fft3d((float2*)b->fft, m.X, m.Y, m.Z, (float2*)b->fft_scratch, b->stream));
-    BCUDA(flb::power_spectrum((const float2*)b->fft, m.V, target, b->sk_tmp, b->stream));
+    float* real = (float*)(b->fft + m.V / 2 + 1);  // behind the V complex numbers of the transform
+    double* out = S || !accumulate ? b->sk_tmp : nullptr;
+    const double scale = accumulate ? 1.0 / b->sk_acc[{replica, mode}].second : 1.0;
+    BCUDA(ops.mode_field(m, rep_src(b, replica), mode, real, b->stream));
+    BCUDA(flb::spectrum((float2*)b->fft, real, m.X, m.Y, m.Z, (float2*)b->fft_scratch, target, out, scale, b->stream));
     if (S) {
-        if (accumulate)
-            BCUDA(flb::scale_copy(target, 1.0 / b->sk_acc[{replica, mode}].second, m.V, b->sk_tmp, b->stream));
-        BCUDA(cudaMemcpyAsync(S, b->sk_tmp, m.V * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
+        BCUDA(cudaMemcpyAsync(S, out, m.V * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
         BCUDA(cudaStreamSynchronize(b->stream));
     }
     return FLB_OK;

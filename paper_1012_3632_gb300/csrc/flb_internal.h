@@ -99,9 +99,9 @@ struct PrecOps {
     // per-block partial sums; returns the number of partial rows written
     cudaError_t (*cons_partials)(const HostModel&, const void* src, double* partials, int* nrows,
                                  cudaStream_t);
-    // mode a of the pre-collision state as a complex field: double2, or float2
-    // when fp32 (the transform of single-precision states)
-    cudaError_t (*mode_field)(const HostModel&, const void* src, int mode, void* out, bool fp32, cudaStream_t);
+    // mode a of the pre-collision state: double2 of an FP64 state, float (real)
+    // of the others
+    cudaError_t (*mode_field)(const HostModel&, const void* src, int mode, void* out, cudaStream_t);
     int (*partial_rows_max)(const HostModel&);
     int (*step_needs_density)(const HostModel&);
     int (*step_in_passes)(const HostModel&);  // the step uses the density and mu fields itself
@@ -126,11 +126,12 @@ const PrecOps& ops_bf16();
 // the kernel before it drains (programmatic dependent launch), which hides the
 // launch latency between the kernels of a step.
 template <class... P, class... A>
-cudaError_t launch_chain(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args)
+cudaError_t launch_chain_smem(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args)
 {
     cudaLaunchConfig_t c{};
     c.gridDim = grid;
     c.blockDim = block;
+    c.dynamicSmemBytes = smem;
     c.stream = st;
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -138,6 +139,11 @@ cudaError_t launch_chain(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream
     c.attrs = &at;
     c.numAttrs = 1;
     return cudaLaunchKernelEx(&c, kernel, P(args)...);
+}
+template <class... P, class... A>
+cudaError_t launch_chain(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args)
+{
+    return launch_chain_smem(kernel, grid, block, 0, st, args...);
 }
 
 // Deterministic column sums: out[c] = sum_r partials[r*ncol + c], plus add0
@@ -172,12 +178,13 @@ cudaError_t fft_rows(double2* data, int X, int n, double2* scratch, cudaStream_t
 // (c11, c21, c22) per wavevector, the lower Cholesky factor of the lattice
 // covariance of the e and eps noise; false (with a message) where it is not
 // positive definite.  swift_noise draws the white e/eps normals of `step`,
-// transforms them to Fourier space, colours them with chol and leaves in
+// transforms them to Fourier space, colours them with chol (float when fp32,
+// else double) and leaves in
 // `out` a field whose real part times 1/V is xi_e and minus imaginary part
 // times 1/V is xi_eps; `work` is scratch (both V complex numbers, float2 when
 // fp32, else double2).
 bool swift_table(const HostModel& m, double* chol, std::string& err);
-cudaError_t swift_noise(const HostModel& m, uint64_t step, const double* chol, void* work, void* out, bool fp32,
+cudaError_t swift_noise(const HostModel& m, uint64_t step, const void* chol, void* work, void* out, bool fp32,
                         cudaStream_t s);
 
 // Interface heights of a stripe (flb_capillary.cu): drho is the density
@@ -203,10 +210,12 @@ cudaError_t adjoint_step(const HostModel& m, int prec, uint64_t step, const void
 cudaError_t adjoint_add_rb(const HostModel& m, int prec, void* lam, const void* rb, cudaStream_t st);
 int adjoint_rows(const HostModel& m);
 
-// p = |data|^2 / V with p(0) = 0; accumulate: acc += p, else out = p.
-cudaError_t power_spectrum(const double2* data, long V, double* acc, double* out, cudaStream_t s);
-cudaError_t power_spectrum(const float2* data, long V, double* acc, double* out, cudaStream_t s);
-// out[s] = a * in[s], s < V
-cudaError_t scale_copy(const double* in, double a, long V, double* out, cudaStream_t s);
+// p = |data|^2 / V with p(0) = 0: acc += p and out = scale * acc (out may be
+// NULL), or without acc out = p.
+cudaError_t power_spectrum(const double2* data, long V, double* acc, double* out, cudaStream_t s, double scale = 1.0);
+// The same of an FP32 field of real numbers: transform (data: work, V complex
+// numbers, scratch as many) and power spectrum.
+cudaError_t spectrum(float2* data, const float* real, int X, int Y, int Z, float2* scratch, double* acc, double* out,
+                     double scale, cudaStream_t s);
 
 }  // namespace flb

@@ -295,6 +295,7 @@ struct StepArgs {
     // cs^2 grad rho = sum_i w_i c_i rho(r + c_i), which cancels the LB's own
     // ideal-gas pressure gradient (Eq. (he-force)); pgrad = 0 otherwise.
     R A, B, kappa, rho0_minus_rhoc, pgrad;
+    R inv_v, inv_v_lo;  // 1 / V and what its rounding left
 };
 
 // ---------------------------------------------------------------------------
@@ -575,9 +576,14 @@ __global__ void __launch_bounds__(TX* TY)
     R xe = R(0), xp = R(0);
     if (a.c.noise) {
         const NoiseField<R> v = xi[s];
-        const double iv = 1.0 / (double)a.V;
-        xe = R(v.x * iv);
-        xp = R(-v.y * iv);
+        if constexpr (std::is_same<R, float>::value) {
+            // v / V with 1 / V in two floats: rounded once, and off the FP64 pipe
+            xe = fmaf(v.x, a.inv_v, v.x * a.inv_v_lo);
+            xp = -fmaf(v.y, a.inv_v, v.y * a.inv_v_lo);
+        } else {
+            xe = v.x * a.inv_v;
+            xp = -v.y * a.inv_v;
+        }
     }
     const Nbhd nb(x, y, 0, X, Y, 1);
     R g[L::Q];

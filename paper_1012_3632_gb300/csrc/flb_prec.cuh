@@ -59,6 +59,8 @@ StepArgs<R> make_args(const HostModel& m, uint64_t step)
     a.kappa = R(m.kappa);
     a.rho0_minus_rhoc = R(m.rho0 - m.rho_c);
     a.pgrad = R(m.nonideal && m.total ? 1 : 0);
+    a.inv_v = R(1.0 / (double)m.V);
+    a.inv_v_lo = R(1.0 / (double)m.V - (double)a.inv_v);
     return a;
 }
 
@@ -465,23 +467,24 @@ inline int cons_blocks(long V)
 }
 
 template <class L, class R, class S, class T>
-__global__ void k_mode_field(const S* __restrict__ src, int mode, T* __restrict__ out, int X, int Y, int Z)
+__global__ void __launch_bounds__(kSitesThreads)
+    k_mode_field(const S* __restrict__ src, int mode, T* __restrict__ out, int X, int Y, int Z, const Tiling t)
 {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z * blockDim.z + threadIdx.z;
-    if (x >= X || y >= Y || z >= Z) return;
-    const long V = (long)X * Y * Z;
-    const Nbhd nb(x, y, z, X, Y, Z);
+    pdl_wait();
+    const int3 r = tile_site<1, L::D == 3 ? 2 : 1, false>(t, threadIdx.x);
+    if (r.x >= X || r.y >= Y || r.z >= Z) return;
+    const Nbhd nb(r.x, r.y, r.z, X, Y, Z);
     R g[L::Q], m[L::Q];
-    pull<L>(src, V, nb, g);
+    pull<L>(src, (long)X * Y * Z, nb, g);
     L::moments(g, m);
     R v = m[0];
 #pragma unroll
     for (int q = 1; q < L::Q; ++q)
         if (q == mode) v = m[q];
-    using E = decltype(T::x);
-    out[x + X * (y + Y * z)] = T{E(v), E(0)};
+    if constexpr (std::is_same<T, double2>::value)
+        out[r.x + X * (r.y + Y * r.z)] = make_double2(v, 0.0);
+    else
+        out[r.x + X * (r.y + Y * r.z)] = v;
 }
 
 // ---------------------------------------------------------------------------
@@ -749,21 +752,17 @@ struct Prec {
         }
         return cudaGetLastError();
     }
-    template <class T>
-    static cudaError_t mode_field_t(const HostModel& m, const void* src, int mode, T* out, cudaStream_t st)
+    static cudaError_t mode_field(const HostModel& m, const void* src, int mode, void* out, cudaStream_t st)
     {
-        if (m.Q == 19) {
-            const dim3 b = site_block<D3Q19>();
-            k_mode_field<D3Q19, R, S, T><<<grid_for(m, b), b, 0, st>>>((const S*)src, mode, out, m.X, m.Y, m.Z);
-        } else {
-            const dim3 b = site_block<D2Q9>();
-            k_mode_field<D2Q9, R, S, T><<<grid_for(m, b), b, 0, st>>>((const S*)src, mode, out, m.X, m.Y, m.Z);
+        if constexpr (kPackedStorage) {
+            if (mode == 0 && packed(m) && ((uintptr_t)out & 15) == 0)
+                return density_packed(m, src, (float*)out, nullptr, st);  // the same sums, a quad per thread
         }
-        return cudaGetLastError();
-    }
-    static cudaError_t mode_field(const HostModel& m, const void* src, int mode, void* out, bool fp32, cudaStream_t st)
-    {
-        return fp32 ? mode_field_t(m, src, mode, (float2*)out, st) : mode_field_t(m, src, mode, (double2*)out, st);
+        using T = typename std::conditional<std::is_same<R, double>::value, double2, float>::type;
+        const Tiling t = make_tiling(m.X, m.Y, m.Z, 1, kSitesThreads, m.D == 3 ? 2 : 1);
+        const auto k = m.Q == 19 ? k_mode_field<D3Q19, R, S, T> : k_mode_field<D2Q9, R, S, T>;
+        return launch_chain(k, dim3(t.blocks()), dim3(kSitesThreads), st, (const S*)src, mode, (T*)out, m.X, m.Y, m.Z,
+                            t);
     }
 
     static cudaError_t pull_state(const HostModel& m, const void* src, void* out, cudaStream_t st)

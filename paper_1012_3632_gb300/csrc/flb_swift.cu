@@ -24,37 +24,32 @@
 // transforms (a random field that needs no more precision).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <string>
 
 #include "../../include/flb.h"
-#include "flb_device.cuh"
+#include "flb_kernels.cuh"
 #include "flb_internal.h"
+#include "flb_swift.cuh"
 
 namespace flb {
 namespace {
 
-// Z(r) = z_e(r) + i z_eps(r): normals 0 and 5 of the D2Q9 collision draw
-// (calls 0 and 1 of tag 0), stored as T: Box-Muller in FP64 for double2 and in
-// FP32 for float2, as the collision kernels of those precisions draw them.
+// Z(r) = z_e(r) + i z_eps(r)
 template <class T>
 __global__ void k_swift_white(PhiloxKeys key, uint32_t step, uint32_t replica, long V, T* __restrict__ Z)
 {
-    using E = decltype(T::x);
-    for (long s = blockIdx.x * (long)blockDim.x + threadIdx.x; s < V; s += (long)gridDim.x * blockDim.x) {
-        E a[4], b[4];
-        normals4<E>(key, (uint32_t)s, step, 0u, replica, a);
-        normals4<E>(key, (uint32_t)s, step, 1u, replica, b);
-        Z[s] = T{a[0], b[1]};
-    }
+    pdl_wait();
+    for (long s = blockIdx.x * (long)blockDim.x + threadIdx.x; s < V; s += (long)gridDim.x * blockDim.x)
+        Z[s] = swift_white<T>(key, (uint32_t)s, step, replica);
 }
 
 // out(k) = conj(Ze'(k) + i Zp'(k)) with (Ze', Zp') = chol(k) (E, P).
-template <class T>
-__global__ void k_swift_colour(const T* __restrict__ Z, const double* __restrict__ chol, int X, int Y,
-                               T* __restrict__ out)
+template <class T, class E = decltype(T::x)>
+__global__ void k_swift_colour(const T* __restrict__ Z, const E* __restrict__ chol, int X, int Y, T* __restrict__ out)
 {
-    using E = decltype(T::x);
+    pdl_wait();
     const long V = (long)X * Y;
     for (long s = blockIdx.x * (long)blockDim.x + threadIdx.x; s < V; s += (long)gridDim.x * blockDim.x) {
         const int nx = (int)(s % X), ny = (int)(s / X);
@@ -63,7 +58,7 @@ __global__ void k_swift_colour(const T* __restrict__ Z, const double* __restrict
         // E = (Z(k) + conj Z(-k)) / 2, P = (Z(k) - conj Z(-k)) / (2i)
         const E er = E(0.5) * (zk.x + zm.x), ei = E(0.5) * (zk.y - zm.y);
         const E pr = E(0.5) * (zk.y + zm.y), pi = E(-0.5) * (zk.x - zm.x);
-        const E c11 = E(chol[3 * s]), c21 = E(chol[3 * s + 1]), c22 = E(chol[3 * s + 2]);
+        const E c11 = chol[3 * s], c21 = chol[3 * s + 1], c22 = chol[3 * s + 2];
         const E Er = c11 * er, Ei = c11 * ei;
         const E Pr = c21 * er + c22 * pr, Pi = c21 * ei + c22 * pi;
         // E' + i P' = (Er - Pi) + i (Ei + Pr); conjugate
@@ -71,17 +66,15 @@ __global__ void k_swift_colour(const T* __restrict__ Z, const double* __restrict
     }
 }
 
-template <class T>
-cudaError_t swift_noise_t(const HostModel& m, uint64_t step, const double* chol, T* work, T* out, cudaStream_t s)
+template <class T, class E = decltype(T::x)>
+cudaError_t swift_noise_t(const HostModel& m, uint64_t step, const E* chol, T* work, T* out, cudaStream_t s)
 {
     const long V = m.V;
-    const unsigned nb = (unsigned)std::min<long>((V + 255) / 256, 152 * 16);
-    k_swift_white<T><<<nb, 256, 0, s>>>(philox_keys(m.seed), (uint32_t)step, m.replica, V, work);
-    cudaError_t e = cudaGetLastError();
+    const dim3 nb((unsigned)std::min<long>((V + 255) / 256, 152 * 16)), b(256);
+    cudaError_t e = launch_chain(k_swift_white<T>, nb, b, s, philox_keys(m.seed), (uint32_t)step, m.replica, V, work);
     if (e != cudaSuccess) return e;
     if ((e = fft3d(work, m.X, m.Y, 1, out, s)) != cudaSuccess) return e;
-    k_swift_colour<T><<<nb, 256, 0, s>>>(work, chol, m.X, m.Y, out);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_chain(k_swift_colour<T>, nb, b, s, (const T*)work, chol, m.X, m.Y, out)) != cudaSuccess) return e;
     return fft3d(out, m.X, m.Y, 1, work, s);
 }
 
@@ -123,11 +116,14 @@ bool swift_table(const HostModel& m, double* chol, std::string& err)
     return true;
 }
 
-cudaError_t swift_noise(const HostModel& m, uint64_t step, const double* chol, void* work, void* out, bool fp32,
+cudaError_t swift_noise(const HostModel& m, uint64_t step, const void* chol, void* work, void* out, bool fp32,
                         cudaStream_t s)
 {
-    if (fp32) return swift_noise_t(m, step, chol, (float2*)work, (float2*)out, s);
-    return swift_noise_t(m, step, chol, (double2*)work, (double2*)out, s);
+    if (!fp32) return swift_noise_t(m, step, (const double*)chol, (double2*)work, (double2*)out, s);
+    if (swift_noise_lengths(m.X, m.Y))
+        return swift_noise_fp32(philox_keys(m.seed), (uint32_t)step, m.replica, m.X, m.Y, (const float*)chol,
+                                (float2*)work, (float2*)out, s);
+    return swift_noise_t(m, step, (const float*)chol, (float2*)work, (float2*)out, s);
 }
 
 }  // namespace flb
