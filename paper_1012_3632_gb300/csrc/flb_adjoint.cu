@@ -10,17 +10,25 @@
 // the step computes lam^n = dJ/dg^n and adds dJ/dtheta for
 // theta = (omega_shear, omega_bulk, omega_ghost, kappa, A, B).
 //
-// Kernels (per step, all hand-written VJPs):
-//   k_adj_collide  pull lam^{n+1}(r + c_i) (adjoint of streaming), replay the
-//                  forward collision at r and propagate through it: the local
-//                  part of lam^n, the force adjoint Fbar(r) and the relaxation
-//                  parameter gradients;
+// Kernels (all hand-written VJPs):
+//   k_adj_density, k_force_mu / k_mu_field
+//                  rho and mu of the states of up to kAdjBatch steps, a launch each;
+//   k_adj_collide  per step: pull lam^{n+1}(r + c_i) (adjoint of streaming), replay
+//                  the forward collision at r and propagate through it: the local
+//                  part of lam^n, the force adjoint Fbar(r), the direct term
+//                  -Fbar . grad mu of rho and the relaxation parameter gradients;
 //   k_adj_mu       mubar(y) = -3 sum_i w_i c_i . rho(y - c_i) Fbar(y - c_i)
-//                  (adjoint of F = -rho grad mu) and the direct rho term
-//                  Fbar . F / rho;
+//                  (adjoint of F = -rho grad mu);
 //   k_adj_rho      rhobar = psi''(rho) mubar - kappa lap(mubar) + direct term,
 //                  added to every population (rho = sum_i g_i), and the
-//                  kappa, A, B gradients.
+//                  kappa, A, B gradients;
+//   k_sum_grads, k_add_grads
+//                  the gradients' block sums of those steps into grad.
+// At 64^3 a launch takes little more than its latency, so that fields which the
+// states of several steps give at once are not a launch per step, neighbours are
+// read once (30 values for mubar, not 90) and the launches are chained: a segment
+// of 20 steps, recomputed and swept back, takes 1.07 ms; with density, mu, force
+// and gradient launches per step and its states pulled apart it took 1.9 ms.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -39,122 +47,162 @@ namespace {
 
 using L = D3Q19;
 
-template <class R>
-__device__ __forceinline__ R d_sqrt(R x)
-{
-    return sqrt(x);
-}
-
 // Adjoint parameters per launch.
 template <class R>
 struct AdjArgs {
     Coll<R> c;
     int X, Y, Z;
     long V;
-    int nonideal;
-    R A, B, kappa, rho0_minus_rhoc, pgrad;
-    // d(rel)/d omega = -1/N_a, d(frc)/d omega = -1/(2 N_a), d(ns)/d omega per mode
-    R drel[16], dfrc[6], dns[16];
-    int cls[16];  // 0 bulk, 1 shear, 2 ghost of non-conserved mode k
+    R A, B, kappa, rho0_minus_rhoc;
+    // per class of modes (0 bulk: mode 0 of the non-conserved ones, 1 shear: 1-5,
+    // 2 ghost: 6-14): 1 / omega, d ln(ns) / d omega
+    R inv_om[3], dln_ns[3];
 };
 
-// Per-site VJP of the collision.  gn: pre-collision deviations at r; F: force
-// at r; lb: adjoint of the post-collision populations at r (pulled from step
-// n+1).  Out: lg (adjoint of gn, local part), Fb (force adjoint), gp[3]
-// (gradients of omega_bulk, omega_shear, omega_ghost).
-template <class R>
-__device__ __forceinline__ void collide_vjp(const R gn[19], const R F[3], const R lb[19], const AdjArgs<R>& a,
-                                            uint32_t site, uint32_t step, R lg[19], R Fb[3], R gp[3])
+__device__ __forceinline__ double mad(double a, double b, double c) { return a * b + c; }
+__device__ __forceinline__ float mad(float a, float b, float c) { return a * b + c; }
+__device__ __forceinline__ F2 mad(F2 a, F2 b, F2 c) { return mk2(__ffma2_rn(a.v, b.v, c.v)); }
+__device__ __forceinline__ F2 mad(float a, F2 b, F2 c) { return mk2(__ffma2_rn(make_float2(a, a), b.v, c.v)); }
+
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+
+// sites per thread
+template <class T>
+constexpr int kSites = std::is_same<T, F2>::value ? 2 : 1;
+__device__ __forceinline__ double value_sum(double v, bool) { return v; }
+__device__ __forceinline__ float value_sum(float v, bool) { return v; }
+__device__ __forceinline__ float value_sum(F2 v, bool two) { return two ? v.v.x + v.v.y : v.v.x; }
+
+// lb_i += sum_a T_ai b_a, the transpose of L::moments
+template <class T>
+__device__ __forceinline__ void add_transposed(const T b[19], T lb[19])
 {
-    const Coll<R>& P = a.c;
-    R m[19];
-    L::moments(gn, m);
-    const R rho = P.rho0 + m[0];
-    const R ir = R(1) / rho;
-    const R ux = (m[1] + R(0.5) * F[0]) * ir, uy = (m[2] + R(0.5) * F[1]) * ir, uz = (m[3] + R(0.5) * F[2]) * ir;
-    const R Fx = F[0], Fy = F[1], Fz = F[2];
-    const R uxx = ux * ux, uyy = uy * uy, uzz = uz * uz, uu = uxx + uyy + uzz;
-    const R uF = ux * Fx + uy * Fy + uz * Fz;
-    R z[16];
-    R sr = R(0), dsr = R(0);  // noise amplitude factor and its rho derivative
-    if (P.noise) {
-        noise_normals<4>(P.key, site, step, P.replica, z);
-        if (P.noise_local) {
-            sr = d_sqrt(rho);
-            dsr = R(0.5) / sr;
-        } else {
-            sr = P.sqrt_rho0;
-        }
-    } else {
-        for (int k = 0; k < 16; ++k) z[k] = R(0);
+    const T a10 = T(1.0 / 3) * b[10], a11 = T(1.0 / 3) * b[11], a12 = T(1.0 / 3) * b[12];
+    const T t16 = T(1.0 / 3) * b[16], h17 = T(0.5) * b[17], h18 = T(0.5) * b[18];
+    lb[0] += b[0] - b[4] + t16;
+    const T Ea = mad(T(-2), t16, b[0]), Ee = b[0] + b[4] + t16;
+    const T s56 = b[5] + b[6], d56 = b[6] - b[5];
+    const T E1 = Ea + mad(T(2), b[5], T(-1) * b[17]), O1 = mad(T(-2), a10, b[1]);
+    const T E2 = Ea + d56 + (h17 - h18), O2 = mad(T(-2), a11, b[2]);
+    const T E3 = Ea - s56 + (h17 + h18), O3 = mad(T(-2), a12, b[3]);
+    const T Exy = Ee + s56 + (h17 + h18), Exz = Ee - d56 + (h17 - h18), Eyz = Ee - mad(T(2), b[5], b[17]);
+    const T jx = b[1] + a10, jy = b[2] + a11, jz = b[3] + a12;
+    const T E[10] = {Ea, E1, E2, E3, Exy + b[7], Exy - b[7], Exz + b[9], Exz - b[9], Eyz + b[8], Eyz - b[8]};
+    const T O[10] = {Ea, O1, O2, O3, jx + jy + (b[13] - b[14]), jx - jy + (b[13] + b[14]), jx + jz - (b[13] - b[15]),
+                     jx - jz - (b[13] + b[15]), jy + jz + (b[14] - b[15]), jy - jz + (b[14] + b[15])};
+#pragma unroll
+    for (int k = 1; k < 10; ++k) {
+        lb[2 * k - 1] += E[k] + O[k];
+        lb[2 * k] += E[k] - O[k];
     }
-    // adjoint of the increments: Db_a = sum_i w_i T_ai lb_i
-    R wl[19], Db[19];
-#pragma unroll
-    for (int i = 0; i < 19; ++i) wl[i] = R(Vel<L>::w(i)) * lb[i];
-    L::moments(wl, Db);
-
-    // forward pieces needed for the parameter gradients
-    const R neq[6] = {m[4] - rho * uu, m[5] - rho * (R(3) * uxx - uu), m[6] - rho * (uyy - uzz),
-                      m[7] - rho * ux * uy, m[8] - rho * uy * uz, m[9] - rho * uz * ux};
-    const R mF[6] = {R(2) * uF, R(2) * (R(3) * ux * Fx - uF), R(2) * (uy * Fy - uz * Fz),
-                     ux * Fy + uy * Fx, uy * Fz + uz * Fy, uz * Fx + ux * Fz};
-
-    R mb[19];  // adjoint of the moments
-    R rb = R(0), ubx = R(0), uby = R(0), ubz = R(0);
-    R fbx = R(3) * Db[1], fby = R(3) * Db[2], fbz = R(3) * Db[3];
-    gp[0] = gp[1] = gp[2] = R(0);
-#pragma unroll
-    for (int k = 0; k < 15; ++k) {
-        const int aidx = 4 + k;
-        const R d = Db[aidx];
-        mb[aidx] = P.rel[k] * d;
-        // parameter gradient of this mode
-        R g = a.drel[k] * (k < 6 ? neq[k] : m[aidx]) + a.dns[k] * sr * z[k];
-        if (k < 6) g += a.dfrc[k] * mF[k];
-        gp[a.cls[k]] += d * g;
-        // noise amplitude through rho
-        rb += d * P.ns[k] * z[k] * dsr;
-    }
-    const R* rl = P.rel;
-    const R* fr = P.frc;
-    const R d4 = Db[4], d5 = Db[5], d6 = Db[6], d7 = Db[7], d8 = Db[8], d9 = Db[9];
-    // d/drho at fixed u of the equilibrium parts
-    rb += -rl[0] * uu * d4 - rl[1] * (R(3) * uxx - uu) * d5 - rl[2] * (uyy - uzz) * d6 - rl[3] * ux * uy * d7 -
-          rl[4] * uy * uz * d8 - rl[5] * uz * ux * d9;
-    // d/du
-    ubx += d4 * (R(-2) * rl[0] * rho * ux + R(2) * fr[0] * Fx) + d5 * (R(-4) * rl[1] * rho * ux + R(4) * fr[1] * Fx) +
-           d7 * (-rl[3] * rho * uy + fr[3] * Fy) + d9 * (-rl[5] * rho * uz + fr[5] * Fz);
-    uby += d4 * (R(-2) * rl[0] * rho * uy + R(2) * fr[0] * Fy) + d5 * (R(2) * rl[1] * rho * uy - R(2) * fr[1] * Fy) +
-           d6 * (R(-2) * rl[2] * rho * uy + R(2) * fr[2] * Fy) + d7 * (-rl[3] * rho * ux + fr[3] * Fx) +
-           d8 * (-rl[4] * rho * uz + fr[4] * Fz);
-    ubz += d4 * (R(-2) * rl[0] * rho * uz + R(2) * fr[0] * Fz) + d5 * (R(2) * rl[1] * rho * uz - R(2) * fr[1] * Fz) +
-           d6 * (R(2) * rl[2] * rho * uz - R(2) * fr[2] * Fz) + d8 * (-rl[4] * rho * uy + fr[4] * Fy) +
-           d9 * (-rl[5] * rho * ux + fr[5] * Fx);
-    // d/dF at fixed u
-    fbx += d4 * R(2) * fr[0] * ux + d5 * R(4) * fr[1] * ux + d7 * fr[3] * uy + d9 * fr[5] * uz;
-    fby += d4 * R(2) * fr[0] * uy - d5 * R(2) * fr[1] * uy + d6 * R(2) * fr[2] * uy + d7 * fr[3] * ux + d8 * fr[4] * uz;
-    fbz += d4 * R(2) * fr[0] * uz - d5 * R(2) * fr[1] * uz - d6 * R(2) * fr[2] * uz + d8 * fr[4] * uy + d9 * fr[5] * ux;
-    // u = (j + F/2) / rho
-    mb[1] = ubx * ir;
-    mb[2] = uby * ir;
-    mb[3] = ubz * ir;
-    fbx += R(0.5) * ubx * ir;
-    fby += R(0.5) * uby * ir;
-    fbz += R(0.5) * ubz * ir;
-    rb -= (ubx * ux + uby * uy + ubz * uz) * ir;
-    mb[0] = rb;
-    // lg = lb + T^T mb  (T^T mb = from_moments(mb) / w)
-    R t[19];
-    L::from_moments(mb, t);
-#pragma unroll
-    for (int i = 0; i < 19; ++i) lg[i] = lb[i] + t[i] * R(1.0 / Vel<L>::w(i));
-    Fb[0] = fbx;
-    Fb[1] = fby;
-    Fb[2] = fbz;
 }
 
-__device__ __forceinline__ long blin() { return blockIdx.x + (long)gridDim.x * (blockIdx.y + (long)gridDim.y * blockIdx.z); }
+// VJP of the collision of one site (two with T = F2).  m: moments of the
+// pre-collision deviations; F: force; l: adjoint of the post-collision
+// populations (pulled from step n+1), turned into the local part of the adjoint
+// of the deviations.  Out: fb (force adjoint), gp[3] (gradients of omega_bulk,
+// omega_shear, omega_ghost).
+// The collision is D_k = rel_k (m_k - rho u.Q_k u) + frc_k 2 u.Q_k F + ns_k s z_k
+// with 15 modes k, of which 0-5 have a quadratic form Q_k: all derivatives of
+// those six in u, F and rho go through the two symmetric matrices
+//   E = 2 sum_k e_k Q_k,  M = 2 sum_k f_k Q_k,  e_k = rel_k d_k, f_k = frc_k d_k,
+// d = L::moments(w lb).
+template <bool FORCE, class T, class R>
+__device__ __forceinline__ void collide_vjp(const T m[19], const T F[3], T l[19], const AdjArgs<R>& a, uint32_t site,
+                                            T fb[3], T gp[3])
+{
+    const Coll<R>& P = a.c;
+    const T rho = P.rho0 + m[0];
+    T ir;
+    if constexpr (std::is_same<T, F2>::value)
+        ir = F2(1.0f / rho.v.x, 1.0f / rho.v.y);
+    else
+        ir = T(1) / rho;
+    T u[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) u[k] = (FORCE ? mad(T(0.5), F[k], m[1 + k]) : m[1 + k]) * ir;
+    T d[19], b[19];
+    {
+        T wl[19];
+#pragma unroll
+        for (int i = 0; i < 19; ++i) wl[i] = T(Vel<L>::w(i)) * l[i];
+        L::moments(wl, d);
+    }
+    // noise: A_c = sum_k ns_k z_k d_k over the modes of class c
+    T rb(0);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) gp[c] = T(0);
+    if (P.noise) {
+        T z[16], A[3] = {T(0), T(0), T(0)};
+        noise_normals<4>(P.key, site, P.step, P.replica, z);
+#pragma unroll
+        for (int k = 0; k < 15; ++k) {
+            const int c = k == 0 ? 0 : k < 6 ? 1 : 2;
+            A[c] = mad(P.ns[k] * d[4 + k], z[k], A[c]);
+        }
+        T sr;
+        if constexpr (std::is_same<T, F2>::value)
+            sr = P.noise_local ? F2(sqrtf(rho.v.x), sqrtf(rho.v.y)) : F2(P.sqrt_rho0);
+        else
+            sr = P.noise_local ? T(sqrt(rho)) : T(P.sqrt_rho0);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) gp[c] = sr * (a.dln_ns[c] * A[c]);
+        if (P.noise_local) rb = T(0.5) * (A[0] + A[1] + A[2]) * (sr * ir);  // d sqrt(rho) = sqrt(rho) / (2 rho)
+    }
+#pragma unroll
+    for (int k = 0; k < 15; ++k) b[4 + k] = P.rel[k] * d[4 + k];
+    auto symmetric = [](const T* e, const T v[3], T out[3]) {  // 2 sum_k e_k Q_k v
+        const T e0 = T(2) * e[0], e1 = T(2) * e[1], e2 = T(2) * e[2];
+        const T xx = mad(T(2), e1, e0), yy = e0 - e1 + e2, zz = e0 - e1 - e2;
+        out[0] = mad(xx, v[0], mad(e[3], v[1], e[5] * v[2]));
+        out[1] = mad(e[3], v[0], mad(yy, v[1], e[4] * v[2]));
+        out[2] = mad(e[5], v[0], mad(e[4], v[1], zz * v[2]));
+    };
+    T Eu[3];
+    symmetric(b + 4, u, Eu);
+    const T uu = mad(u[0], u[0], mad(u[1], u[1], u[2] * u[2]));
+    const T huEu = T(0.5) * mad(u[0], Eu[0], mad(u[1], Eu[1], u[2] * Eu[2]));  // sum_k e_k u.Q_k u
+    // omega gradients: d rel = rel / omega, d frc = rel / (2 omega)
+    T g0 = m[4] - rho * uu, g1 = b[4] * uu - huEu, gm(0), g2(0);
+#pragma unroll
+    for (int k = 1; k < 6; ++k) gm = mad(b[4 + k], m[4 + k], gm);
+    g1 = mad(rho, g1, gm);
+#pragma unroll
+    for (int k = 6; k < 15; ++k) g2 = mad(b[4 + k], m[4 + k], g2);
+    rb = rb - huEu;
+    T ub[3];
+    if constexpr (FORCE) {
+        const T uF = mad(u[0], F[0], mad(u[1], F[1], u[2] * F[2]));
+        const T uEF = mad(F[0], Eu[0], mad(F[1], Eu[1], F[2] * Eu[2]));  // 2 sum_k e_k u.Q_k F
+        g0 += uF;
+        g1 += mad(T(0.5), uEF, T(-1) * (b[4] * uF));
+        T f[6], Mu[3], MF[3];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) f[k] = P.frc[k] * d[4 + k];
+        symmetric(f, u, Mu);
+        symmetric(f, F, MF);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            ub[k] = (MF[k] - rho * Eu[k]) * ir;
+            fb[k] = mad(T(0.5), ub[k], mad(T(3), d[1 + k], Mu[k]));
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) ub[k] = T(-1) * Eu[k];
+    }
+    gp[0] = mad(a.inv_om[0], b[4] * g0, gp[0]);
+    gp[1] = mad(a.inv_om[1], g1, gp[1]);
+    gp[2] = mad(a.inv_om[2], g2, gp[2]);
+    // u = (j + F/2) / rho
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        b[1 + k] = ub[k];
+        rb = rb - ub[k] * u[k];
+    }
+    b[0] = rb;
+    add_transposed(b, l);
+}
 
 // Block sums of NV per-thread values: warp sums in the compute type (32
 // terms; FP64 arithmetic per thread would run on GB300's slow FP64 pipe),
@@ -178,10 +226,13 @@ __device__ __forceinline__ void block_rows(R v[NV], double* __restrict__ row)
     }
 }
 
-// densities and forces of the state g^n (pre-collision deviations)
+// densities of the states g^n (pre-collision deviations) blockIdx.y = 0, 1, ..
 template <class R>
-__global__ void k_adj_rho(const R* __restrict__ gn, R* __restrict__ drho, long V)
+__global__ void __launch_bounds__(128) k_adj_density(const R* __restrict__ gn, R* __restrict__ drho, long V)
 {
+    pdl_wait();
+    gn += (long)blockIdx.y * 19 * V;
+    drho += (long)blockIdx.y * V;
     for (long s = blockIdx.x * (long)blockDim.x + threadIdx.x; s < V; s += (long)gridDim.x * blockDim.x) {
         R g[19], m[19];
 #pragma unroll
@@ -191,101 +242,181 @@ __global__ void k_adj_rho(const R* __restrict__ gn, R* __restrict__ drho, long V
     }
 }
 
-// rb_next (or NULL): the density part of lam_next kept apart by the previous
-// adjoint step of a segment; lam_next + rb_next is the full adjoint state.
-template <class R>
-__global__ void k_adj_collide(const AdjArgs<R> a, uint32_t step, const R* __restrict__ gn, const R* __restrict__ F,
-                              const R* __restrict__ lam_next, const R* __restrict__ rb_next, R* __restrict__ lam,
-                              R* __restrict__ Fbar, double* __restrict__ rows)
-{
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z * blockDim.z + threadIdx.z;
-    R gp[3] = {R(0), R(0), R(0)};
-    if (x < a.X && y < a.Y && z < a.Z) {
-        const long V = a.V;
-        const int s = x + a.X * (y + a.Y * z);
-        const Nbhd nb(x, y, z, a.X, a.Y, a.Z);
-        R g[19], lb[19], lg[19], Fs[3] = {R(0), R(0), R(0)}, Fb[3];
-#pragma unroll
-        for (int i = 0; i < 19; ++i) {
-            g[i] = gn[(long)i * V + s];
-            // streaming moved the post-collision population i from r to r + c_i
-            const int q = nb.src(-Vel<L>::cx(i), -Vel<L>::cy(i), -Vel<L>::cz(i));
-            lb[i] = rb_next ? lam_next[(long)i * V + q] + rb_next[q] : lam_next[(long)i * V + q];
-        }
-        if (a.nonideal)
-            for (int d = 0; d < 3; ++d) Fs[d] = F[d * V + s];
-        collide_vjp(g, Fs, lb, a, (uint32_t)s, step, lg, Fb, gp);
-#pragma unroll
-        for (int i = 0; i < 19; ++i) lam[(long)i * V + s] = lg[i];
-        if (a.nonideal)
-            for (int d = 0; d < 3; ++d) Fbar[d * V + s] = Fb[d];
+// Loads of the kSites<T> values of a row from x on, one site or two: two at x
+// by one load with AL (X even, rows aligned), single ones elsewhere.
+template <class T, class R>
+struct Row {
+    int x, x1, xm, xe;  // the sites, their neighbours -1 and +1
+    template <bool AL>
+    __device__ __forceinline__ T at(const R* p, int c) const
+    {
+        if constexpr (kSites<T> == 1)
+            return p[c == 0 ? x : c < 0 ? xm : xe];
+        else if (c == 0)
+            return AL ? mk2(*reinterpret_cast<const float2*>(p + x)) : F2(p[x], p[x1]);
+        else
+            return c < 0 ? F2(p[xm], p[x]) : F2(p[x1], p[xe]);
     }
-    block_rows<3>(gp, rows + blin() * 6);
+};
+template <class T, bool AL, class R>
+__device__ __forceinline__ void put(R* p, T v, bool two)
+{
+    if constexpr (kSites<T> == 1) {
+        *p = v;
+    } else if constexpr (AL) {
+        *reinterpret_cast<float2*>(p) = v.v;
+    } else {
+        p[0] = v.v.x;
+        if (two) p[1] = v.v.y;
+    }
 }
 
-// F(r) = -rho(r) grad mu(r) + pgrad sum_i w_i c_i rho(r + c_i).  Adjoint:
-// mubar(y) = -3 sum_i w_i c_i . rho(y - c_i) Fbar(y - c_i);
-// rb1(y) = Fbar(y) . (-grad mu(y)) + pgrad sum_i w_i c_i . Fbar(y - c_i),
-// with -grad mu(y) = (F(y) - pgrad sum_i w_i c_i rho(y + c_i)) / rho(y).
-template <class R>
-__global__ void k_adj_mu(const AdjArgs<R> a, const R* __restrict__ drho, const R* __restrict__ F,
-                         const R* __restrict__ Fbar, R* __restrict__ mubar, R* __restrict__ rb1)
+// The VJP of the collision.  T = F2: two sites per thread (FP32), which halves
+// the instructions: 64^3 23.0 -> 18.9 us, the 60 MB of states and adjoints in
+// L2 and DRAM take 9.  3 blocks per SM: 168 registers; 4 (spilled) and 2 make a
+// step back 1.5 and 2.7 us longer.  AL: X even and every pointer aligned to two values.
+// rb_next (or NULL): the density part of lam_next kept apart by the previous
+// adjoint step of a segment; lam_next + rb_next is the full adjoint state.
+// W: rho Fbar (TOTAL: Fbar), three fields; rb1: -Fbar . grad mu.
+template <class T, class R, bool AL, bool FORCE, bool TOTAL>
+__global__ void __launch_bounds__(128, kSites<T> == 2 ? 3 : 2)
+    k_adj_collide(const AdjArgs<R> a, const R* __restrict__ gn, const R* __restrict__ drho, const R* __restrict__ mu,
+                  const R* __restrict__ lam_next, const R* __restrict__ rb_next, R* __restrict__ lam,
+                  R* __restrict__ W, R* __restrict__ rb1, double* __restrict__ rows, const Tiling t)
 {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z * blockDim.z + threadIdx.z;
-    if (x >= a.X || y >= a.Y || z >= a.Z) return;
+    pdl_wait();
+    const int3 r = tile_site<kSites<T>, 2, false>(t, threadIdx.x);
+    const int x = r.x, y = r.y, z = r.z, X = a.X, Y = a.Y, Z = a.Z, XY = X * Y;
+    R gs[3] = {R(0), R(0), R(0)};
+    if (x < X && y < Y && z < Z) {
+        const long V = a.V;
+        const int x1 = x + 1 == X ? 0 : x + 1;
+        const Row<T, R> row{x, x1, x == 0 ? X - 1 : x - 1, kSites<T> == 1 ? x1 : x1 + 1 == X ? 0 : x1 + 1};
+        const int yo[3] = {X * wrap_once(y - 1, Y), X * y, X * wrap_once(y + 1, Y)};
+        const int zo[3] = {XY * (z == 0 ? Z - 1 : z - 1), XY * z, XY * (z == Z - 1 ? 0 : z + 1)};
+        const bool two = AL || x + 1 < X;
+        T l[19], m[19], F[3], fb[3], gp[3], d[3];
+        {
+            T g[19];
+#pragma unroll
+            for (int i = 0; i < 19; ++i) g[i] = row.template at<AL>(gn + (i * V + yo[1] + zo[1]), 0);
+            L::moments(g, m);
+        }
+#pragma unroll
+        for (int i = 0; i < 19; ++i) {
+            // streaming moved the post-collision population i from r to r + c_i
+            const int o = yo[1 + Vel<L>::cy(i)] + zo[1 + Vel<L>::cz(i)];
+            l[i] = row.template at<AL>(lam_next + (i * V + o), Vel<L>::cx(i));
+            if (rb_next) l[i] += row.template at<AL>(rb_next + o, Vel<L>::cx(i));
+        }
+        // sum_i w_i c_i f(r + c_i) (a gradient / 3) from the differences f(c) - f(-c)
+        // of the velocity pairs (2k-1, 2k): axis pairs weigh 1/18, edge pairs 1/36
+        auto gradient = [&](const R* f, T out[3]) {
+            T e[10];
+#pragma unroll
+            for (int k = 1; k <= 9; ++k) {
+                const int cx = Vel<L>::cx(2 * k - 1), cy = Vel<L>::cy(2 * k - 1), cz = Vel<L>::cz(2 * k - 1);
+                e[k] = row.template at<AL>(f + (yo[1 + cy] + zo[1 + cz]), cx) -
+                       row.template at<AL>(f + (yo[1 - cy] + zo[1 - cz]), -cx);
+            }
+            out[0] = T(1.0 / 18) * e[1] + T(1.0 / 36) * ((e[4] + e[5]) + (e[6] + e[7]));
+            out[1] = T(1.0 / 18) * e[2] + T(1.0 / 36) * ((e[4] - e[5]) + (e[8] + e[9]));
+            out[2] = T(1.0 / 18) * e[3] + T(1.0 / 36) * ((e[6] - e[7]) + (e[8] - e[9]));
+        };
+        const T rho = a.c.rho0 + m[0];
+        if constexpr (FORCE) {
+            gradient(mu, d);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) F[k] = T(-3) * rho * d[k];
+            if constexpr (TOTAL) {
+                T p[3];
+                gradient(drho, p);
+#pragma unroll
+                for (int k = 0; k < 3; ++k) F[k] += p[k];
+            }
+        }
+        const int s = x + yo[1] + zo[1];
+        collide_vjp<FORCE>(m, F, l, a, (uint32_t)s, fb, gp);
+#pragma unroll
+        for (int i = 0; i < 19; ++i) put<T, AL>(lam + (i * V + s), l[i], two);
+        if constexpr (FORCE) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) put<T, AL>(W + (k * V + s), TOTAL ? fb[k] : rho * fb[k], two);
+            put<T, AL>(rb1 + s, T(-3) * (d[0] * fb[0] + d[1] * fb[1] + d[2] * fb[2]), two);
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) gs[c] = value_sum(gp[c], two);
+    }
+    block_rows<3>(gs, rows + 3 * (long)blockIdx.x);
+}
+
+// mubar(y) = -3 sum_i w_i c_i . rho(y - c_i) Fbar(y - c_i); TOTAL (F gains
+// cs^2 grad rho): rb1 += sum_i w_i c_i . Fbar(y - c_i) as well.
+template <class R, bool TOTAL>
+__global__ void __launch_bounds__(128)
+    k_adj_mu(const AdjArgs<R> a, const R* __restrict__ drho, const R* __restrict__ W, R* __restrict__ mubar,
+             R* __restrict__ rb1, const Tiling t)
+{
+    pdl_wait();
+    const int3 r = tile_site<1, 2, false>(t, threadIdx.x);
+    if (r.x >= a.X || r.y >= a.Y || r.z >= a.Z) return;
     const long V = a.V;
-    const int s = x + a.X * (y + a.Y * z);
-    const Nbhd nb(x, y, z, a.X, a.Y, a.Z);
-    R acc = R(0), accp = R(0), pr[3] = {R(0), R(0), R(0)};
+    const int s = r.x + a.X * (r.y + a.Y * r.z);
+    const Nbhd nb(r.x, r.y, r.z, a.X, a.Y, a.Z);
+    R ax = R(0), ed = R(0), axp = R(0), edp = R(0);  // axis and edge velocities, weights 1/18 and 1/36
 #pragma unroll
     for (int i = 1; i < 19; ++i) {
-        const int q = nb.src(Vel<L>::cx(i), Vel<L>::cy(i), Vel<L>::cz(i));  // y - c_i
-        const R rq = a.c.rho0 + drho[q];
-        const R cf = Vel<L>::cx(i) * Fbar[q] + Vel<L>::cy(i) * Fbar[V + q] + Vel<L>::cz(i) * Fbar[2 * V + q];
-        acc += R(Vel<L>::w(i)) * rq * cf;
-        accp += R(Vel<L>::w(i)) * cf;
-        const R wr = R(Vel<L>::w(i)) * drho[nb.src(-Vel<L>::cx(i), -Vel<L>::cy(i), -Vel<L>::cz(i))];  // y + c_i
-        pr[0] += R(Vel<L>::cx(i)) * wr;
-        pr[1] += R(Vel<L>::cy(i)) * wr;
-        pr[2] += R(Vel<L>::cz(i)) * wr;
+        const int cx = Vel<L>::cx(i), cy = Vel<L>::cy(i), cz = Vel<L>::cz(i);
+        const int q = nb.src(cx, cy, cz);  // y - c_i
+        R cf = R(0);
+        if (cx) cf += R(cx) * W[q];
+        if (cy) cf += R(cy) * W[V + q];
+        if (cz) cf += R(cz) * W[2 * V + q];
+        R rf = cf;
+        if constexpr (TOTAL) {
+            rf = mul_rn(a.c.rho0 + drho[q], cf);  // rounded: c and -c cancel where nothing varies
+            if (i < 7)
+                axp += cf;
+            else
+                edp += cf;
+        }
+        if (i < 7)
+            ax += rf;
+        else
+            ed += rf;
     }
-    mubar[s] = R(-3) * acc;
-    const R rho = a.c.rho0 + drho[s];
-    R fg = R(0);
-    for (int d = 0; d < 3; ++d) fg += Fbar[d * V + s] * (F[d * V + s] - a.pgrad * pr[d]);
-    rb1[s] = fg / rho + a.pgrad * accp;
+    mubar[s] = R(-3.0 / 18) * ax + R(-3.0 / 36) * ed;
+    if constexpr (TOTAL) rb1[s] += R(1.0 / 18) * axp + R(1.0 / 36) * edp;
 }
 
 // rhobar = rb1 + psi''(rho) mubar - kappa lap(mubar), added to every population
 // (or, with rb_out, stored for the next adjoint step of a segment to add);
-// kappa, A, B gradients
+// kappa, A, B gradients.  The kappa gradient -sum mubar lap(rho) is formed as
+// -sum rho lap(mubar): the lattice Laplacian is symmetric.
 template <class R>
-__global__ void k_adj_rho(const AdjArgs<R> a, const R* __restrict__ drho, const R* __restrict__ mubar,
-                          const R* __restrict__ rb1, R* __restrict__ lam, R* __restrict__ rb_out,
-                          double* __restrict__ rows)
+__global__ void __launch_bounds__(128)
+    k_adj_rho(const AdjArgs<R> a, const R* __restrict__ drho, const R* __restrict__ mubar,
+              const R* __restrict__ rb1, R* __restrict__ lam, R* __restrict__ rb_out, double* __restrict__ rows,
+              const Tiling t)
 {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z * blockDim.z + threadIdx.z;
+    pdl_wait();
+    const int3 r = tile_site<1, 2, false>(t, threadIdx.x);
     R gp[3] = {R(0), R(0), R(0)};
-    if (x < a.X && y < a.Y && z < a.Z) {
+    if (r.x < a.X && r.y < a.Y && r.z < a.Z) {
         const long V = a.V;
-        const int s = x + a.X * (y + a.Y * z);
-        const Nbhd nb(x, y, z, a.X, a.Y, a.Z);
+        const int s = r.x + a.X * (r.y + a.Y * r.z);
+        const Nbhd nb(r.x, r.y, r.z, a.X, a.Y, a.Z);
         const R mb = mubar[s], r0 = drho[s];
-        R lapm = R(0), lapr = R(0);
+        R ax = R(0), ed = R(0);
 #pragma unroll
         for (int i = 1; i < 19; ++i) {
-            const int q = nb.src(-Vel<L>::cx(i), -Vel<L>::cy(i), -Vel<L>::cz(i));  // y + c_i
-            lapm += R(Vel<L>::w(i)) * (mubar[q] - mb);
-            lapr += R(Vel<L>::w(i)) * (drho[q] - r0);
+            const R v = mubar[nb.src(-Vel<L>::cx(i), -Vel<L>::cy(i), -Vel<L>::cz(i))] - mb;
+            if (i < 7)
+                ax += v;
+            else
+                ed += v;
         }
-        lapm *= R(6);
-        lapr *= R(6);
+        const R lapm = R(1.0 / 3) * ax + R(1.0 / 6) * ed;  // 6 sum_i w_i (..)
         const R d = r0 + a.rho0_minus_rhoc;
         const R psi2 = a.A + R(3) * a.B * d * d;
         const R rb = rb1[s] + psi2 * mb - a.kappa * lapm;
@@ -294,17 +425,18 @@ __global__ void k_adj_rho(const AdjArgs<R> a, const R* __restrict__ drho, const 
         else
 #pragma unroll
             for (int i = 0; i < 19; ++i) lam[(long)i * V + s] += rb;
-        gp[0] = -mb * lapr;   // kappa
-        gp[1] = mb * d;       // A
+        gp[0] = -r0 * lapm;      // kappa
+        gp[1] = mb * d;          // A
         gp[2] = mb * d * d * d;  // B
     }
-    block_rows<3>(gp, rows + blin() * 6 + 3);
+    block_rows<3>(gp, rows + 3 * (long)blockIdx.x);
 }
 
 // lam += rb on every population: the deferred density part of the last step
 template <class R>
 __global__ void k_add_rb(R* __restrict__ lam, const R* __restrict__ rb, long V)
 {
+    pdl_wait();
     for (long s = blockIdx.x * (long)blockDim.x + threadIdx.x; s < V; s += (long)gridDim.x * blockDim.x) {
         const R r = rb[s];
 #pragma unroll
@@ -312,24 +444,38 @@ __global__ void k_add_rb(R* __restrict__ lam, const R* __restrict__ rb, long V)
     }
 }
 
-// Column c of the per-block rows summed (in the order of k_sum_columns) and
-// added to its parameter: columns (bulk, shear, ghost, kappa, A, B) go to
-// grad (omega_shear, omega_bulk, omega_ghost, kappa, A, B).  One block per
-// column; the free-energy columns only for the non-ideal fluid.
-__global__ void k_add_grads(const double* __restrict__ rows, int nrows, double* __restrict__ grad, int nonideal)
+// Column blockIdx.x of the block rows of step blockIdx.y (nc rows of the
+// collision's three columns, then nr of k_adj_rho's) summed into
+// part[step * 6 + column].
+__global__ void __launch_bounds__(256) k_sum_grads(const double* __restrict__ rows, int nc, int nr,
+                                                   double* __restrict__ part)
 {
     __shared__ double sh[256];
-    const int c = blockIdx.x;
-    if (c >= 3 && !nonideal) return;
+    pdl_wait();
+    const int c = blockIdx.x, n = c < 3 ? nc : nr;
+    const double* p = rows + 3 * ((long)blockIdx.y * (nc + nr) + (c < 3 ? 0 : nc)) + c % 3;
     double acc = 0.0;
-    for (int r = threadIdx.x; r < nrows; r += blockDim.x) acc += rows[(long)r * 6 + c];
+    for (int r = threadIdx.x; r < n; r += blockDim.x) acc += p[(long)r * 3];
     sh[threadIdx.x] = acc;
     __syncthreads();
     for (int o = blockDim.x / 2; o > 0; o >>= 1) {
         if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
         __syncthreads();
     }
-    if (threadIdx.x == 0) grad[c == 0 ? 1 : c == 1 ? 0 : c] += sh[0];
+    if (threadIdx.x == 0) part[blockIdx.y * 6 + c] = sh[0];
+}
+
+// The steps' sums added to their parameters, the last step first: columns
+// (bulk, shear, ghost, kappa, A, B) go to grad (omega_shear, omega_bulk,
+// omega_ghost, kappa, A, B), the free-energy columns only for the non-ideal fluid.
+__global__ void k_add_grads(const double* __restrict__ part, int n, double* __restrict__ grad, int nonideal)
+{
+    pdl_wait();
+    const int c = threadIdx.x;
+    if (c >= 6 || (c >= 3 && !nonideal)) return;
+    double acc = grad[c == 0 ? 1 : c == 1 ? 0 : c];
+    for (int k = n - 1; k >= 0; --k) acc += part[k * 6 + c];
+    grad[c == 0 ? 1 : c == 1 ? 0 : c] = acc;
 }
 
 template <class R>
@@ -341,100 +487,137 @@ AdjArgs<R> make_adj(const HostModel& m, const Coll<R>& c)
     a.Y = m.Y;
     a.Z = m.Z;
     a.V = m.V;
-    a.nonideal = m.nonideal;
     a.A = R(m.A);
     a.B = R(m.B);
     a.kappa = R(m.kappa);
     a.rho0_minus_rhoc = R(m.rho0 - m.rho_c);
-    a.pgrad = R(m.nonideal && m.total ? 1 : 0);
-    for (int k = 0; k < 15; ++k) {
-        const int aidx = 4 + k;
-        const double om = k == 0 ? m.om_b : k < 6 ? m.om_s : m.om_g;
-        const double Na = L::N(aidx);
-        a.cls[k] = k == 0 ? 0 : k < 6 ? 1 : 2;
-        a.drel[k] = R(-1.0 / Na);
-        if (k < 6) a.dfrc[k] = R(-0.5 / Na);
-        const double ns = std::sqrt(m.kT * (2.0 - om) * om * Na * 3.0) / Na;
-        a.dns[k] = R(ns * (1.0 - om) / (om * (2.0 - om)));
+    const double om[3] = {m.om_b, m.om_s, m.om_g};
+    for (int c = 0; c < 3; ++c) {
+        a.inv_om[c] = R(1.0 / om[c]);
+        a.dln_ns[c] = R((1.0 - om[c]) / (om[c] * (2.0 - om[c])));
     }
     return a;
 }
 
+// rho and mu of `n` states, V values each, the states one after another.
 template <class R>
-cudaError_t adjoint_step_t(const HostModel& m, const Coll<R>& c, uint64_t step, const R* gn, const R* lam_next,
-                           const R* rb_next, R* lam, R* rb_out, R* work, double* rows, double* grad,
+cudaError_t adjoint_fields_t(const HostModel& m, const Coll<R>& c, const R* states, int n, R* rho, R* mu,
+                             cudaStream_t st)
+{
+    const unsigned nb = (unsigned)std::min<long>((m.V + 127) / 128, 152 * 16);
+    cudaError_t e = launch_chain(k_adj_density<R>, dim3(nb, n), dim3(128), st, states, rho, m.V);
+    if (e != cudaSuccess) return e;
+    const AdjArgs<R> a = make_adj<R>(m, c);
+    StepArgs<R> sa{};
+    sa.c = c;
+    sa.X = m.X;
+    sa.Y = m.Y;
+    sa.Z = m.Z;
+    sa.V = m.V;
+    sa.A = a.A;
+    sa.B = a.B;
+    sa.kappa = a.kappa;
+    sa.rho0_minus_rhoc = a.rho0_minus_rhoc;
+    sa.pgrad = R(m.total ? 1 : 0);
+    const R* crho = rho;
+    if constexpr (std::is_same<R, float>::value) {
+        const int gx = m.X % 4 == 0 && m.V % 4 == 0 ? 4 : m.X % 2 == 0 ? 2 : 1;
+        const Tiling t = make_tiling(m.X, m.Y, (m.Z + 1) / 2, gx == 4 ? 4 : 2, 128, 2);
+        const auto k = gx == 4 ? k_force_mu<4> : gx == 2 ? k_force_mu<2> : k_force_mu<1>;
+        return launch_chain(k, dim3(t.blocks(), n), dim3(128), st, sa, crho, mu, t);
+    } else {
+        const Tiling t = make_tiling(m.X, m.Y, m.Z, 1, kSitesThreads, 2);
+        return launch_chain(k_mu_field<R>, dim3(t.blocks(), n), dim3(kSitesThreads), st, sa, crho, mu, t);
+    }
+}
+
+// the collision (two sites per thread in FP32) and k_adj_mu, k_adj_rho
+Tiling collide_tiling(const HostModel& m, int prec)
+{
+    return make_tiling(m.X, m.Y, m.Z, prec == FLB_FP64 ? 1 : 2, 128, 2);
+}
+Tiling adjoint_tiling(const HostModel& m) { return make_tiling(m.X, m.Y, m.Z, 1, 128, 2); }
+
+template <class T, class R, bool AL>
+auto collide_kernel(const HostModel& m)
+{
+    return !m.nonideal ? k_adj_collide<T, R, AL, false, false>
+           : m.total   ? k_adj_collide<T, R, AL, true, true>
+                       : k_adj_collide<T, R, AL, true, false>;
+}
+
+template <class R>
+cudaError_t adjoint_step_t(const HostModel& m, const Coll<R>& c, const R* gn, const R* rho, const R* mu,
+                           const R* lam_next, const R* rb_next, R* lam, R* rb_out, R* work, double* rows,
                            cudaStream_t st)
 {
+    constexpr bool f32 = std::is_same<R, float>::value;
+    using T = std::conditional_t<f32, F2, R>;
     const long V = m.V;
-    R* drho = work;
-    R* mu = work + V;
-    R* F = work + 2 * V;
-    R* Fbar = work + 5 * V;
-    R* mubar = work + 8 * V;
-    R* rb1 = work + 9 * V;
+    R* W = work;
+    R* mubar = work + 3 * V;
+    R* rb1 = work + 4 * V;
     const AdjArgs<R> a = make_adj<R>(m, c);
-    const dim3 b(32, 4, 2);
-    const dim3 g((m.X + 31) / 32, (m.Y + 3) / 4, (m.Z + 1) / 2);
-    const int nrows = (int)(g.x * g.y * g.z);
-    cudaError_t e = cudaSuccess;
-    // every block writes columns 0-2 (collision) and, for the non-ideal fluid,
-    // 3-5 (free-energy parameters); the ideal gas leaves 3-5 at zero
-    if (!m.nonideal && (e = cudaMemsetAsync(rows, 0, (size_t)nrows * 6 * sizeof(double), st)) != cudaSuccess)
-        return e;
-    if (m.nonideal) {
-        k_adj_rho<R><<<(unsigned)std::min<long>((V + 255) / 256, 152 * 16), 256, 0, st>>>(gn, drho, V);
-        StepArgs<R> sa{};
-        sa.c = c;
-        sa.X = m.X;
-        sa.Y = m.Y;
-        sa.Z = m.Z;
-        sa.V = V;
-        sa.A = a.A;
-        sa.B = a.B;
-        sa.kappa = a.kappa;
-        sa.rho0_minus_rhoc = a.rho0_minus_rhoc;
-        sa.pgrad = a.pgrad;
-        k_mu<L, R><<<g, b, 0, st>>>(sa, drho, mu);
-        k_force<L, R><<<g, b, 0, st>>>(sa, drho, mu, F);
-    }
-    k_adj_collide<R><<<g, b, 0, st>>>(a, (uint32_t)step, gn, F, lam_next, rb_next, lam, Fbar, rows);
-    if (m.nonideal) {
-        k_adj_mu<R><<<g, b, 0, st>>>(a, drho, F, Fbar, mubar, rb1);
-        k_adj_rho<R><<<g, b, 0, st>>>(a, drho, mubar, rb1, lam, rb_out, rows);
-    }
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_add_grads<<<6, 256, 0, st>>>(rows, nrows, grad, m.nonideal);
-    return cudaGetLastError();
+    const Tiling tc = collide_tiling(m, f32 ? FLB_FP32 : FLB_FP64), t = adjoint_tiling(m);
+    const dim3 b(128);
+    // the caller's arrays may begin at any value
+    const bool al = f32 && m.X % 2 == 0 && (((uintptr_t)gn | (uintptr_t)lam_next | (uintptr_t)lam) & 7) == 0;
+    const auto k = al ? collide_kernel<T, R, f32>(m) : collide_kernel<T, R, false>(m);
+    cudaError_t e = launch_chain(k, dim3(tc.blocks()), b, st, a, gn, rho, mu, lam_next, rb_next, lam, W, rb1, rows, tc);
+    if (e != cudaSuccess || !m.nonideal) return e;
+    const R* cW = W;
+    const R* cmubar = mubar;
+    const R* crb1 = rb1;
+    const dim3 g(t.blocks());
+    e = launch_chain(m.total ? k_adj_mu<R, true> : k_adj_mu<R, false>, g, b, st, a, rho, cW, mubar, rb1, t);
+    if (e != cudaSuccess) return e;
+    return launch_chain(k_adj_rho<R>, g, b, st, a, rho, cmubar, crb1, lam, rb_out, rows + 3 * (size_t)tc.blocks(), t);
 }
 
 }  // namespace
 
-cudaError_t adjoint_step(const HostModel& m, int prec, uint64_t step, const void* gn, const void* lam_next,
-                         const void* rb_next, void* lam, void* rb_out, void* work, double* rows, double* grad,
+cudaError_t adjoint_fields(const HostModel& m, int prec, const void* states, int n, void* rho, void* mu,
+                           cudaStream_t st)
+{
+    if (!m.nonideal) return cudaSuccess;
+    if (prec == FLB_FP64)
+        return adjoint_fields_t<double>(m, coll_fp64(m, 0), (const double*)states, n, (double*)rho, (double*)mu, st);
+    return adjoint_fields_t<float>(m, coll_fp32(m, 0), (const float*)states, n, (float*)rho, (float*)mu, st);
+}
+
+cudaError_t adjoint_step(const HostModel& m, int prec, uint64_t step, const void* gn, const void* rho, const void* mu,
+                         const void* lam_next, const void* rb_next, void* lam, void* rb_out, void* work, double* rows,
                          cudaStream_t st)
 {
     if (prec == FLB_FP64)
-        return adjoint_step_t<double>(m, coll_fp64(m, step), step, (const double*)gn, (const double*)lam_next,
-                                      (const double*)rb_next, (double*)lam, (double*)rb_out, (double*)work, rows,
-                                      grad, st);
-    return adjoint_step_t<float>(m, coll_fp32(m, step), step, (const float*)gn, (const float*)lam_next,
-                                 (const float*)rb_next, (float*)lam, (float*)rb_out, (float*)work, rows, grad,
-                                 st);
+        return adjoint_step_t<double>(m, coll_fp64(m, step), (const double*)gn, (const double*)rho,
+                                      (const double*)mu, (const double*)lam_next, (const double*)rb_next, (double*)lam,
+                                      (double*)rb_out, (double*)work, rows, st);
+    return adjoint_step_t<float>(m, coll_fp32(m, step), (const float*)gn, (const float*)rho, (const float*)mu,
+                                 (const float*)lam_next, (const float*)rb_next, (float*)lam, (float*)rb_out,
+                                 (float*)work, rows, st);
+}
+
+cudaError_t adjoint_grads(const HostModel& m, int prec, const double* rows, int n, double* part, double* grad,
+                          cudaStream_t st)
+{
+    const int nc = (int)collide_tiling(m, prec).blocks();
+    cudaError_t e = launch_chain(k_sum_grads, dim3(m.nonideal ? 6 : 3, n), dim3(256), st, rows, nc,
+                                 adjoint_rows(m, prec) - nc, part);
+    if (e != cudaSuccess) return e;
+    return launch_chain(k_add_grads, dim3(1), dim3(32), st, (const double*)part, n, grad, m.nonideal);
 }
 
 cudaError_t adjoint_add_rb(const HostModel& m, int prec, void* lam, const void* rb, cudaStream_t st)
 {
-    const unsigned nb = (unsigned)std::min<long>((m.V + 255) / 256, 152 * 16);
-    if (prec == FLB_FP64)
-        k_add_rb<double><<<nb, 256, 0, st>>>((double*)lam, (const double*)rb, m.V);
-    else
-        k_add_rb<float><<<nb, 256, 0, st>>>((float*)lam, (const float*)rb, m.V);
-    return cudaGetLastError();
+    const dim3 nb((unsigned)std::min<long>((m.V + 255) / 256, 152 * 16)), b(256);
+    if (prec == FLB_FP64) return launch_chain(k_add_rb<double>, nb, b, st, (double*)lam, (const double*)rb, m.V);
+    return launch_chain(k_add_rb<float>, nb, b, st, (float*)lam, (const float*)rb, m.V);
 }
 
-int adjoint_rows(const HostModel& m)
+int adjoint_rows(const HostModel& m, int prec)
 {
-    return ((m.X + 31) / 32) * ((m.Y + 3) / 4) * ((m.Z + 1) / 2);
+    return (int)(collide_tiling(m, prec).blocks() + adjoint_tiling(m).blocks());
 }
 
 }  // namespace flb

@@ -109,10 +109,11 @@ struct flb_ctx {
     int hs_count = 0;
 
     // adjoint scratch
-    void* adj_work = nullptr;
-    double* adj_rows = nullptr;
-    void* adj_lam2 = nullptr;  // flb_adjoint_segment: second adjoint state (ping-pong)
-    void* adj_rb = nullptr;    // flb_adjoint_segment: deferred density parts (2 fields)
+    void* adj_work = nullptr;  // kAdjFields fields, rho and mu of one state
+    double* adj_rows = nullptr;  // block sums of kAdjBatch steps, then the steps' sums
+    void* adj_seg = nullptr;  // flb_adjoint_segment: second adjoint state (ping-pong), two
+                              // deferred density parts, then rho and mu of adj_batch states
+    int adj_batch = 0;
     double* ss_dev = nullptr;  // flb_step_sums: 4 sums per step (device)
     size_t ss_cap = 0;
 
@@ -168,7 +169,7 @@ int alloc_guarded(flb_ctx* c, void** p, size_t bytes, const char* name)
 void free_all(flb_ctx* c)
 {
     void* ptrs[] = {c->buf[0], c->buf[1], c->drho, c->mu, c->F, c->partials, c->red, c->fft, c->fft_scratch, c->sk_tmp,
-                    c->adj_work, c->adj_rows, c->adj_lam2, c->adj_rb, c->ss_dev, c->h_dev, c->hs_work, c->hs_scratch, c->hs_acc,
+                    c->adj_work, c->adj_rows, c->adj_seg, c->ss_dev, c->h_dev, c->hs_work, c->hs_scratch, c->hs_acc,
                     c->hs_tmp, c->sw_chol, c->sw_work, c->sw_xi};
     for (void* p : ptrs) {
         bool guarded = false;
@@ -486,8 +487,9 @@ int flb_init(flb_ctx* c, const double* rho, const double* u, int thermal_init)
 // The time steps of flb_step; with dev_sums (device, 4 doubles per step) also
 // the sums of the state each step starts from: the step kernel's own partial
 // sums where it provides them, else the conservation reduction before the step
-// (dev_sums[4 t] is the total mass: rho0 V is added to the summed deviations).
-static int step_impl(flb_ctx* c, int nsteps, double* dev_sums)
+// (dev_sums[4 t] is the total mass: rho0 V is added to the summed deviations);
+// with states (device, pop_bytes per step) each state a step starts from.
+static int step_impl(flb_ctx* c, int nsteps, double* dev_sums, char* states = nullptr)
 {
     const double m0 = c->m.rho0 * (double)c->m.V;
     const int nrow = dev_sums ? c->ops->step_row_count(c->m) : 0;
@@ -521,6 +523,8 @@ static int step_impl(flb_ctx* c, int nsteps, double* dev_sums)
             FLB_CUDA(c->ops->cons_partials(c->m, src, c->partials, &nrows, c->stream));
             FLB_CUDA(flb::sum_columns(c->partials, nrows, 4, dev_sums + 4 * (size_t)t, c->stream, m0));
             se = c->ops->step(c->m, c->step, src, dst, c->drho, c->stream);
+        } else if (states) {
+            se = c->ops->step_state(c->m, c->step, src, dst, c->drho, states + (size_t)t * c->pop_bytes(), c->stream);
         } else {
             se = c->ops->step(c->m, c->step, src, dst, c->drho, c->stream);
         }
@@ -906,6 +910,40 @@ int flb_set_populations(flb_ctx* c, const double* f)
     return FLB_OK;
 }
 
+namespace {
+
+int adjoint_scratch(flb_ctx* c)
+{
+    const size_t rows = ((size_t)flb::adjoint_rows(c->m, c->prec) * 3 + 6) * flb::kAdjBatch;
+    int rc;
+    if ((rc = alloc(&c->adj_work, (flb::kAdjFields + 2) * c->field_bytes())) ||
+        (rc = alloc((void**)&c->adj_rows, rows * sizeof(double))))
+        return rc;
+    return FLB_OK;
+}
+
+// A segment's scratch with room for rho and mu of kAdjBatch states, of half as
+// many and so on where the memory is short (of one state: its place in
+// adj_work).  Made once: a captured segment may still use it.
+int adjoint_segment_scratch(flb_ctx* c)
+{
+    if (c->adj_seg) return FLB_OK;
+    const size_t fixed = c->pop_bytes() + 2 * c->field_bytes();
+    int n = flb::kAdjBatch;
+    if (c->m.nonideal)
+        for (; n > 1; n /= 2) {
+            if (cudaMalloc(&c->adj_seg, fixed + 2 * (size_t)n * c->field_bytes()) == cudaSuccess) break;
+            c->adj_seg = nullptr;
+            cudaGetLastError();
+        }
+    c->adj_batch = n;
+    return alloc(&c->adj_seg, fixed);
+}
+
+double* adjoint_part(flb_ctx* c) { return c->adj_rows + (size_t)flb::adjoint_rows(c->m, c->prec) * flb::kAdjBatch * 3; }
+
+}  // namespace
+
 int flb_get_state_device(flb_ctx* c, void* g)
 {
     FLB_TRACE();
@@ -933,11 +971,13 @@ int flb_adjoint_step(flb_ctx* c, const void* g_n, uint64_t step, const void* lam
     if (lam == lam_next) return fail(FLB_EINVAL, "lam and lam_next must not alias");
     DeviceGuard guard(c->device);
     int rc;
-    if ((rc = alloc(&c->adj_work, 10 * c->field_bytes())) ||
-        (rc = alloc((void**)&c->adj_rows, (size_t)flb::adjoint_rows(c->m) * 6 * sizeof(double))))
-        return rc;
-    FLB_CUDA(flb::adjoint_step(c->m, c->prec, step, g_n, lam_next, nullptr, lam, nullptr, c->adj_work, c->adj_rows,
-                               grad, c->stream));
+    if ((rc = adjoint_scratch(c))) return rc;
+    char* rho = (char*)c->adj_work + flb::kAdjFields * c->field_bytes();
+    char* mu = rho + c->field_bytes();
+    FLB_CUDA(flb::adjoint_fields(c->m, c->prec, g_n, 1, rho, mu, c->stream));
+    FLB_CUDA(flb::adjoint_step(c->m, c->prec, step, g_n, rho, mu, lam_next, nullptr, lam, nullptr, c->adj_work,
+                               c->adj_rows, c->stream));
+    FLB_CUDA(flb::adjoint_grads(c->m, c->prec, c->adj_rows, 1, adjoint_part(c), grad, c->stream));
     return FLB_OK;
 }
 
@@ -951,38 +991,44 @@ int flb_adjoint_segment(flb_ctx* c, const void* g_start, uint64_t step0, int n, 
     if (c->prec == FLB_BF16) return fail(FLB_EINVAL, "the adjoint step needs FLB_FP64 or FLB_FP32 storage");
     DeviceGuard guard(c->device);
     int rc;
-    if ((rc = alloc(&c->adj_work, 10 * c->field_bytes())) ||
-        (rc = alloc((void**)&c->adj_rows, (size_t)flb::adjoint_rows(c->m) * 6 * sizeof(double))) ||
-        (rc = alloc(&c->adj_lam2, c->pop_bytes())) ||
-        (rc = alloc(&c->adj_rb, 2 * c->field_bytes())))
-        return rc;
+    if ((rc = adjoint_scratch(c)) || (rc = adjoint_segment_scratch(c))) return rc;
     const size_t pb = c->pop_bytes();
     char* S = (char*)states;
     // forward: the states at step0 .. step0+n-1 (pre-collision deviations)
-    FLB_CUDA(cudaMemcpyAsync(S, g_start, pb, cudaMemcpyDeviceToDevice, c->stream));
     FLB_CUDA(c->ops->push_state(c->m, g_start, c->buf[c->cur], c->stream));
     c->step = step0;
-    for (int k = 1; k < n; ++k) {
-        if ((rc = flb_step(c, 1))) return rc;
-        FLB_CUDA(c->ops->pull_state(c->m, c->buf[c->cur], S + (size_t)k * pb, c->stream));
-    }
+    if ((rc = step_impl(c, n - 1, nullptr, S))) return rc;
+    FLB_CUDA(c->ops->pull_state(c->m, c->buf[c->cur], S + (size_t)(n - 1) * pb, c->stream));
     // reverse: lam(step0 + n) -> lam(step0), alternating between lam and
-    // adj_lam2; for the non-ideal fluid each step passes its density part on to
+    // adj_seg; for the non-ideal fluid each step passes its density part on to
     // the next (two scalars per site instead of a pass over all 19 planes) and
     // the last one is added at the end, the same additions in the same order
     // as flb_adjoint_step one step at a time
     void* nxt = lam;
-    void* cur = c->adj_lam2;
-    char* rb = (char*)c->adj_rb;
+    void* cur = c->adj_seg;
     const size_t fb = c->field_bytes();
+    char* rb = (char*)c->adj_seg + pb;
     const bool defer = c->m.nonideal != 0;
     const void* rb_in = nullptr;
-    for (int k = n - 1; k >= 0; --k) {
-        void* rb_out = defer ? rb + (size_t)(k & 1) * fb : nullptr;
-        FLB_CUDA(flb::adjoint_step(c->m, c->prec, step0 + (uint64_t)k, S + (size_t)k * pb, nxt, rb_in, cur, rb_out,
-                                   c->adj_work, c->adj_rows, grad, c->stream));
-        rb_in = rb_out;
-        std::swap(nxt, cur);
+    char* rho = c->adj_batch > 1 ? rb + 2 * fb : (char*)c->adj_work + flb::kAdjFields * fb;
+    char* mu = rho + (size_t)c->adj_batch * fb;
+    const size_t nrow = (size_t)flb::adjoint_rows(c->m, c->prec) * 3;
+    for (int last = n; last > 0;) {
+        // densities and chemical potentials of a batch of states, their steps back
+        // from the last, the batch's gradients
+        const int first = std::max(0, last - c->adj_batch), cnt = last - first;
+        FLB_CUDA(flb::adjoint_fields(c->m, c->prec, S + (size_t)first * pb, cnt, rho, mu, c->stream));
+        for (int k = last - 1; k >= first; --k) {
+            void* rb_out = defer ? rb + (size_t)(k & 1) * fb : nullptr;
+            const size_t j = (size_t)(k - first);
+            FLB_CUDA(flb::adjoint_step(c->m, c->prec, step0 + (uint64_t)k, S + (size_t)k * pb, rho + j * fb,
+                                       mu + j * fb, nxt, rb_in, cur, rb_out, c->adj_work, c->adj_rows + j * nrow,
+                                       c->stream));
+            rb_in = rb_out;
+            std::swap(nxt, cur);
+        }
+        FLB_CUDA(flb::adjoint_grads(c->m, c->prec, c->adj_rows, cnt, adjoint_part(c), grad, c->stream));
+        last = first;
     }
     if (rb_in) FLB_CUDA(flb::adjoint_add_rb(c->m, c->prec, nxt, rb_in, c->stream));
     if (nxt != lam) FLB_CUDA(cudaMemcpyAsync(lam, nxt, pb, cudaMemcpyDeviceToDevice, c->stream));

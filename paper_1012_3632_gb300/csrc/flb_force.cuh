@@ -56,7 +56,9 @@ __device__ __forceinline__ void load_row(const float* p, int x, int x1, int xm, 
 // for it; in the collision the same sums cost 9 % (474 -> 519 us at 256^3).  At
 // least 7 blocks per SM: the sums would take 88 registers and with them the
 // warps that hide the loads (a step with sums 716 us, at 6 blocks 727, 8: 740).
-template <class S, int GX, bool SUMS>
+// STATE: the pulled deviations go to P.dst as well, the states that the adjoint
+// keeps (FP32; 64^3 14.7 us, without them 8.3 and a pull of their own 9.5).
+template <class S, int GX, bool SUMS, bool STATE = false>
 __global__ void __launch_bounds__(128, 7) k_force_density(const __grid_constant__ Planes<S> P, float* __restrict__ rho,
                                                        float* __restrict__ rows, int X, int Y, int Z, const Tiling t)
 {
@@ -92,6 +94,9 @@ __global__ void __launch_bounds__(128, 7) k_force_density(const __grid_constant_
                     lo[i] = F2(v.y, v.z);
                     hi[i] = F2(v.w, A::keep1(r + xe));
                 }
+                if constexpr (STATE)
+                    *reinterpret_cast<float4*>(P.dst[i] + (XY * z + X * y + x)) =
+                        make_float4(lo[i].v.x, lo[i].v.y, hi[i].v.x, hi[i].v.y);
             }
             L::moments(lo, m);
             L::moments(hi, n);
@@ -115,6 +120,15 @@ __global__ void __launch_bounds__(128, 7) k_force_density(const __grid_constant_
                     g[i] = F2(A::plain1(r + xm), A::plain1(r + x));
                 else
                     g[i] = F2(A::plain1(r + x1), A::plain1(r + xe));
+                if constexpr (STATE) {
+                    S* o = P.dst[i] + (XY * z + X * y + x);
+                    if constexpr (GX == 2) {
+                        *reinterpret_cast<float2*>(o) = g[i].v;
+                    } else {
+                        o[0] = g[i].v.x;
+                        if (x + 1 < X) o[1] = g[i].v.y;
+                    }
+                }
             }
             L::moments(g, m);
             if constexpr (GX == 2) {
@@ -155,6 +169,8 @@ __global__ void __launch_bounds__(128)
     pdl_wait();
     int3 r0 = tile_site<N, 2, true>(t, threadIdx.x);
     const int X = a.X, Y = a.Y, Z = a.Z, XY = X * Y;
+    rho += (long)blockIdx.y * a.V;  // several fields in one launch (the adjoint's states)
+    mu += (long)blockIdx.y * a.V;
     // the tiling's two planes are rows of threads: here each thread takes a pair of planes
     const int x = r0.x, y = r0.y, z = 2 * r0.z;
     if (x >= X || y >= Y || z >= Z) return;

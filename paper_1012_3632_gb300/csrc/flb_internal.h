@@ -116,6 +116,9 @@ struct PrecOps {
     int (*step_row_count)(const HostModel&);
     cudaError_t (*step_rows)(const HostModel&, uint64_t step, const void* src, void* dst, const void* drho,
                              float4* rows, cudaStream_t);
+    // the step from src, whose pre-collision deviations go to state as well
+    cudaError_t (*step_state)(const HostModel&, uint64_t step, const void* src, void* dst, const void* drho,
+                              void* state, cudaStream_t);
 };
 
 const PrecOps& ops_fp64();
@@ -196,19 +199,27 @@ cudaError_t interface_heights(const void* drho, int real_size, double rho0, int 
 cudaError_t height_power(const double* h, int X, double2* work, double2* scratch, double* acc, double* out,
                          cudaStream_t s);
 
-// Adjoint of one D3Q19 step (flb_adjoint.cu): gn, lam_next, lam are [19][V]
-// pre-collision deviations / adjoints in the storage type (FP64 or FP32);
-// work holds 10 V compute-type scalars, rows adjoint_rows(m) * 6 doubles;
-// grad (6 doubles, device) is incremented.  Within a segment the
-// density part of the adjoint (one scalar per site, added to every
-// population) may be passed on instead of added: rb_out (V scalars or NULL)
-// receives it and the next step takes it as rb_next (NULL: lam_next is
-// complete); adjoint_add_rb adds the last one.
-cudaError_t adjoint_step(const HostModel& m, int prec, uint64_t step, const void* gn, const void* lam_next,
-                         const void* rb_next, void* lam, void* rb_out, void* work, double* rows, double* grad,
+// Adjoint of D3Q19 steps (flb_adjoint.cu).  States and adjoints are [19][V]
+// deviations in the storage type (FP64 or FP32).
+// adjoint_fields: rho and mu (V values each, state after state) of n <= kAdjBatch
+// consecutive states; nothing for the ideal gas.
+// adjoint_step: the adjoint of one step at state gn with its rho and mu; work
+// holds kAdjFields V values, rows adjoint_rows(m, prec) * 3 doubles of block sums of
+// the parameter gradients.  Within a segment the density part of the adjoint
+// (one scalar per site, added to every population) may be passed on instead of
+// added: rb_out (V scalars or NULL) receives it and the next step takes it as
+// rb_next (NULL: lam_next is complete); adjoint_add_rb adds the last one.
+// adjoint_grads: the block sums of n steps (rows step after step, part: n * 6
+// doubles) added to grad (6 doubles, device), the last step first.
+constexpr int kAdjBatch = 8, kAdjFields = 5;
+cudaError_t adjoint_fields(const HostModel& m, int prec, const void* states, int n, void* rho, void* mu,
+                           cudaStream_t st);
+cudaError_t adjoint_step(const HostModel& m, int prec, uint64_t step, const void* gn, const void* rho, const void* mu,
+                         const void* lam_next, const void* rb_next, void* lam, void* rb_out, void* work, double* rows,
                          cudaStream_t st);
+cudaError_t adjoint_grads(const HostModel& m, int prec, const double* rows, int n, double* part, double* grad, cudaStream_t st);
 cudaError_t adjoint_add_rb(const HostModel& m, int prec, void* lam, const void* rb, cudaStream_t st);
-int adjoint_rows(const HostModel& m);
+int adjoint_rows(const HostModel& m, int prec);
 
 // p = |data|^2 / V with p(0) = 0: acc += p and out = scale * acc (out may be
 // NULL), or without acc out = p.

@@ -431,6 +431,8 @@ __global__ void __launch_bounds__(kSitesThreads)
     pdl_wait();
     const int3 r = tile_site<1, 2, false>(t, threadIdx.x);
     if (r.x >= a.X || r.y >= a.Y || r.z >= a.Z) return;
+    drho += (long)blockIdx.y * a.V;  // several fields in one launch (the adjoint's states)
+    mu += (long)blockIdx.y * a.V;
     const Nbhd nb(r.x, r.y, r.z, a.X, a.Y, a.Z);
     const int s = r.x + a.X * (r.y + a.Y * r.z);
     const R rc = drho[s];

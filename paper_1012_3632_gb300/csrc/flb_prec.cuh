@@ -177,6 +177,7 @@ __global__ void k_set_pop(const double* __restrict__ in, S* __restrict__ dst, do
 template <class L, class S>
 __global__ void k_pull_state(const S* __restrict__ src, S* __restrict__ out, int X, int Y, int Z)
 {
+    pdl_wait();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z * blockDim.z + threadIdx.z;
@@ -191,6 +192,7 @@ __global__ void k_pull_state(const S* __restrict__ src, S* __restrict__ out, int
 template <class L, class S>
 __global__ void k_push_state(const S* __restrict__ in, S* __restrict__ dst, int X, int Y, int Z)
 {
+    pdl_wait();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z * blockDim.z + threadIdx.z;
@@ -507,7 +509,7 @@ struct Prec {
     static cudaError_t density(const HostModel& m, const void* pop, void* drho, cudaStream_t st)
     {
         if constexpr (kPackedStorage) {
-            if (packed(m)) return density_packed(m, pop, (float*)drho, nullptr, st);
+            if (packed(m)) return density_packed(m, pop, (float*)drho, nullptr, nullptr, st);
         }
         const Tiling t = make_tiling(m.X, m.Y, m.Z, 1, kSitesThreads, m.D == 3 ? 2 : 1);
         const auto k = m.Q == 19 ? k_density<D3Q19, R, S> : k_density<D2Q9, R, S>;
@@ -567,14 +569,19 @@ struct Prec {
     {
         return packed(m) && m.nonideal && m.X % 2 == 0 && !m.total ? 4 * (int)density_tiling(m).blocks() : 0;
     }
-    // rows (or NULL): step_row_count rows of mass deviation and momentum
-    static cudaError_t density_packed(const HostModel& m, const void* pop, float* rho, float* rows, cudaStream_t st)
+    // rows (or NULL): step_row_count rows of mass deviation and momentum; state
+    // (or NULL, FP32 without rows, 16-byte aligned): the pulled deviations
+    static cudaError_t density_packed(const HostModel& m, const void* pop, float* rho, float* rows, void* state,
+                                      cudaStream_t st)
     {
-        const Planes<S> pl = make_planes<S>(pop, nullptr, 19, m.V);
+        const Planes<S> pl = make_planes<S>(pop, state, 19, m.V);
         const Tiling t = density_tiling(m);
         auto go = [&](auto G) {
             constexpr int GX = decltype(G)::value;
-            const auto k = GX != 1 && rows ? k_force_density<S, GX, GX != 1> : k_force_density<S, GX, false>;
+            auto k = GX != 1 && rows ? k_force_density<S, GX, GX != 1> : k_force_density<S, GX, false>;
+            if constexpr (std::is_same<S, float>::value) {
+                if (state) k = k_force_density<S, GX, false, true>;
+            }
             return launch_chain(k, dim3(t.blocks()), dim3(128), st, pl, rho, rows, m.X, m.Y, m.Z, t);
         };
         const int gx = gather_width(m);
@@ -583,14 +590,14 @@ struct Prec {
                          : go(std::integral_constant<int, 1>{});
     }
     static cudaError_t step_force(const HostModel& m, uint64_t step, const void* src, void* dst, float* rho,
-                                  float* rows, cudaStream_t st)
+                                  float* rows, void* state, cudaStream_t st)
     {
         const StepArgs<R> a = make_args<D3Q19, R>(m, step);
         const Planes<S> pl = make_planes<S>(src, dst, 19, m.V);
         const float* crho = rho;
         const float* mu = (const float*)m.mu;
         const int gx = gather_width(m);
-        cudaError_t e = density_packed(m, src, rho, rows, st);
+        cudaError_t e = density_packed(m, src, rho, rows, state, st);
         if (e != cudaSuccess) return e;
         const Tiling tm = make_tiling(m.X, m.Y, (m.Z + 1) / 2, gx == 4 ? 4 : 2, 128, 2);  // two planes per thread
         const auto km = gx == 4 ? k_force_mu<4> : gx == 2 ? k_force_mu<2> : k_force_mu<1>;
@@ -600,6 +607,18 @@ struct Prec {
         const auto kc = gx == 1 ? (m.total ? k_force_collide<S, false, true> : k_force_collide<S, false, false>)
                                 : (m.total ? k_force_collide<S, true, true> : k_force_collide<S, true, false>);
         return launch_chain(kc, dim3(tc.blocks()), dim3(128), st, a, pl, crho, mu, tc);
+    }
+    // pull_state of src, then the step: one pass over src does both where the
+    // step pulls the state for its density (FP32 force model).
+    static cudaError_t step_state(const HostModel& m, uint64_t t, const void* src, void* dst, const void* drho,
+                                  void* state, cudaStream_t st)
+    {
+        if constexpr (std::is_same<S, float>::value) {
+            if (packed(m) && m.nonideal && ((uintptr_t)state & 15) == 0)
+                return step_force(m, t, src, dst, (float*)const_cast<void*>(drho), nullptr, state, st);
+        }
+        const cudaError_t e = pull_state(m, src, state, st);
+        return e != cudaSuccess ? e : step(m, t, src, dst, drho, st);
     }
     // The step; with rows (non-NULL) also the mass deviation and momentum of
     // the state it steps from, as step_row_count rows of 4 partial sums, where
@@ -616,7 +635,8 @@ struct Prec {
         if (rows && !step_row_count(m)) return cudaErrorNotSupported;
         // drho: the context's density field, scratch of the steps in passes
         if constexpr (kPackedStorage) {
-            if (packed(m) && m.nonideal) return step_force(m, step, src, dst, (float*)const_cast<void*>(drho), (float*)rows, st);
+            if (packed(m) && m.nonideal) return step_force(m, step, src, dst, (float*)const_cast<void*>(drho), (float*)rows,
+                                                              nullptr, st);
         }
         if (step_in_passes(m)) return step_force_sites(m, step, src, dst, (R*)const_cast<void*>(drho), st);
         if (m.Q == 9 && m.nonideal && m.model == 1) {
@@ -756,7 +776,7 @@ struct Prec {
     {
         if constexpr (kPackedStorage) {
             if (mode == 0 && packed(m) && ((uintptr_t)out & 15) == 0)
-                return density_packed(m, src, (float*)out, nullptr, st);  // the same sums, a quad per thread
+                return density_packed(m, src, (float*)out, nullptr, nullptr, st);  // the same sums, a quad per thread
         }
         using T = typename std::conditional<std::is_same<R, double>::value, double2, float>::type;
         const Tiling t = make_tiling(m.X, m.Y, m.Z, 1, kSitesThreads, m.D == 3 ? 2 : 1);
@@ -767,25 +787,17 @@ struct Prec {
 
     static cudaError_t pull_state(const HostModel& m, const void* src, void* out, cudaStream_t st)
     {
-        if (m.Q == 19) {
-            const dim3 b = site_block<D3Q19>();
-            k_pull_state<D3Q19, S><<<grid_for(m, b), b, 0, st>>>((const S*)src, (S*)out, m.X, m.Y, m.Z);
-        } else {
-            const dim3 b = site_block<D2Q9>();
-            k_pull_state<D2Q9, S><<<grid_for(m, b), b, 0, st>>>((const S*)src, (S*)out, m.X, m.Y, m.Z);
-        }
-        return cudaGetLastError();
+        const dim3 b = m.Q == 19 ? site_block<D3Q19>() : site_block<D2Q9>();
+        if (m.Q == 19)
+            return launch_chain(k_pull_state<D3Q19, S>, grid_for(m, b), b, st, (const S*)src, (S*)out, m.X, m.Y, m.Z);
+        return launch_chain(k_pull_state<D2Q9, S>, grid_for(m, b), b, st, (const S*)src, (S*)out, m.X, m.Y, m.Z);
     }
     static cudaError_t push_state(const HostModel& m, const void* in, void* dst, cudaStream_t st)
     {
-        if (m.Q == 19) {
-            const dim3 b = site_block<D3Q19>();
-            k_push_state<D3Q19, S><<<grid_for(m, b), b, 0, st>>>((const S*)in, (S*)dst, m.X, m.Y, m.Z);
-        } else {
-            const dim3 b = site_block<D2Q9>();
-            k_push_state<D2Q9, S><<<grid_for(m, b), b, 0, st>>>((const S*)in, (S*)dst, m.X, m.Y, m.Z);
-        }
-        return cudaGetLastError();
+        const dim3 b = m.Q == 19 ? site_block<D3Q19>() : site_block<D2Q9>();
+        if (m.Q == 19)
+            return launch_chain(k_push_state<D3Q19, S>, grid_for(m, b), b, st, (const S*)in, (S*)dst, m.X, m.Y, m.Z);
+        return launch_chain(k_push_state<D2Q9, S>, grid_for(m, b), b, st, (const S*)in, (S*)dst, m.X, m.Y, m.Z);
     }
 
     static cudaError_t get_sites(const HostModel& m, const void* src, const long long* sites, int n, double* out,
@@ -804,7 +816,7 @@ struct Prec {
     {
         static const PrecOps o = {(int)sizeof(S), (int)sizeof(R), density, step, init, get_pop, set_pop, moments,
                                   mu_force, mode_sums, cons_partials, mode_field, rows, needs_density, step_in_passes,
-                                  pull_state, push_state, get_sites, step_row_count, step_rows};
+                                  pull_state, push_state, get_sites, step_row_count, step_rows, step_state};
         return o;
     }
 };
