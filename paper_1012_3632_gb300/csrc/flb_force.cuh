@@ -1,5 +1,5 @@
-// flb_force.cuh -- the D3Q19 force-model step with FP32 or BF16 storage, as
-// three launches in packed FP32: density (pull and sum), mu = psi'(rho) -
+// flb_force.cuh -- the force-model steps with FP32 or BF16 storage: D2Q9 in one
+// launch (k_step_gather2, at the end), D3Q19 as three launches in packed FP32: density (pull and sum), mu = psi'(rho) -
 // kappa lap rho, then pull + collide with F = -rho grad mu.
 //
 // Every site's density and mu are formed once, and each pass runs at the
@@ -297,6 +297,128 @@ __global__ void __launch_bounds__(128, 4)
         } else {
             A::store1(P.dst[i] + site, g[i].v.x);
             if (two) A::store1(P.dst[i] + site + 1, g[i].v.y);
+        }
+    }
+}
+
+// D2Q9 force model in one launch, a site pair per thread: a block pulls the
+// pairs of its tile, which stay in registers, and those of a 2-site halo, whose
+// densities go to shared memory with the tile's; mu is formed on the tile + 1
+// (pairs of the same grid, so that 2 columns more are formed than used), then
+// the pair collides with F = -rho grad mu.  AL: X even, the pairs of every row
+// begin at even x.
+// 1024 x 400 FP32 lies in L2 and is bound by the latency of its three phases and
+// by issue slots: 14.4 -> 9.6 us a step (9.6 -> 5.1 million warp instructions)
+// against one site per thread with the tile pulled twice; 129 x 97 6.2 -> 3.1.
+// Tiles of 32 x 8: 32 x 16 10.2, 64 x 8 9.9, 64 x 16 14.7, 16 x 16 11.8 us.
+template <class S, bool AL, bool TOTAL, int TX, int TY>
+__global__ void __launch_bounds__(TX* TY / 2)
+    k_step_gather2(const StepArgs<float> a, const __grid_constant__ Planes<S> P, const Tiling t)
+{
+    using L = D2Q9;
+    using A = Packed<S>;
+    constexpr int HX = TX / 2, RX = TX + 4, RP = RX / 2, RY = TY + 4, NT = HX * TY;
+    constexpr int NHALO = RP * RY - NT;  // halo pairs: two rows below and above, then a column on each side
+    __shared__ float2 rho_pad[RY * RP + 2], smu[RY * RP];  // a corner pair of mu reads one site past the field
+    float2* const srho = rho_pad + 1;
+    pdl_wait();
+    const int X = a.X, Y = a.Y, tid = threadIdx.x;
+    const uint32_t ry = fast_quot(blockIdx.x, t.mx, t.sx);
+    const int bx = TX * (int)(blockIdx.x - ry * t.ntx), by = TY * (int)ry;
+    auto pull = [&](int x, int y, F2 g[L::Q]) {  // x, y within a few tiles of the lattice
+        const int xa = wrap_any(x, X), y0 = wrap_any(y, Y);
+        const int xm = xa == 0 ? X - 1 : xa - 1, x1 = xa + 1 == X ? 0 : xa + 1, xe = x1 + 1 == X ? 0 : x1 + 1;
+        const int yo[3] = {X * wrap_once(y0 - 1, Y), X * y0, X * wrap_once(y0 + 1, Y)};
+#pragma unroll
+        for (int i = 0; i < L::Q; ++i) {
+            const S* r = P.src[i] + yo[1 - Vel<L>::cy(i)];
+            const int cx = Vel<L>::cx(i);
+            if (cx == 0)
+                g[i] = AL ? mk2(A::plain2(r + xa)) : F2(A::plain1(r + xa), A::plain1(r + x1));
+            else if (cx > 0)
+                g[i] = F2(A::plain1(r + xm), A::plain1(r + xa));
+            else
+                g[i] = F2(A::plain1(r + x1), A::plain1(r + xe));
+        }
+    };
+    const int px = tid % HX, py = tid / HX, x = bx + 2 * px, y = by + py;
+    const int own = px + 1 + RP * (py + 2);
+    F2 g[L::Q], m[L::Q];
+    pull(x, y, g);
+    L::moments(g, m);
+    srho[own] = m[0].v;
+    for (int e = tid; e < NHALO; e += NT) {
+        int hx, hy;
+        if (e < 4 * RP) {
+            hx = e % RP;
+            hy = e / RP;
+            if (hy >= 2) hy += TY;
+        } else {
+            hx = (e & 1) * (RP - 1);
+            hy = 2 + ((e - 4 * RP) >> 1);
+        }
+        F2 h[L::Q], n[L::Q];
+        pull(bx - 2 + 2 * hx, by - 2 + hy, h);
+        L::moments(h, n);
+        srho[hx + RP * hy] = n[0].v;
+    }
+    __syncthreads();
+    // the differences f(c) - f(-c) of the pair at index e of a shared field
+    struct Rows {
+        float v[3][4];
+        __device__ __forceinline__ Rows(const float2* f, int e)
+        {
+            const float* p = reinterpret_cast<const float*>(f);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const int o = e + RP * (k - 1);
+                v[k][0] = p[2 * o - 1];
+                v[k][1] = f[o].x;
+                v[k][2] = f[o].y;
+                v[k][3] = p[2 * o + 2];
+            }
+        }
+        __device__ __forceinline__ F2 at(int cx, int cy) const { return F2(v[1 + cy][1 + cx], v[1 + cy][2 + cx]); }
+    };
+    // mu = psi'(rho) - kappa lap rho; lap phi = 6 sum_i w_i (phi(r + c_i) - phi(r))
+    for (int e = RP + tid; e < RP * (RY - 1); e += NT) {
+        const Rows r(srho, e);
+        const F2 rc = r.at(0, 0);
+        F2 ax(0.f), ed(0.f);
+#pragma unroll
+        for (int i = 1; i < L::Q; ++i) (i < 5 ? ax : ed) += r.at(Vel<L>::cx(i), Vel<L>::cy(i)) - rc;
+        const F2 lap = (6.0f / 9.0f) * ax + (6.0f / 36.0f) * ed;
+        const F2 d = rc + a.rho0_minus_rhoc;
+        smu[e] = (d * (a.A + a.B * (d * d)) - a.kappa * lap).v;
+    }
+    __syncthreads();
+    if (x >= X || y >= Y) return;
+    // sum_i w_i c_i f(r + c_i) (a gradient / 3)
+    auto gradient = [&](const float2* f, F2& gx, F2& gy) {
+        const Rows r(f, own);
+        const F2 d1 = r.at(1, 0) - r.at(-1, 0), d2 = r.at(0, 1) - r.at(0, -1);
+        const F2 d5 = r.at(1, 1) - r.at(-1, -1), d8 = r.at(1, -1) - r.at(-1, 1);
+        gx = (1.0f / 9.0f) * d1 + (1.0f / 36.0f) * (d5 + d8);
+        gy = (1.0f / 9.0f) * d2 + (1.0f / 36.0f) * (d5 - d8);
+    };
+    F2 gx, gy;
+    gradient(smu, gx, gy);
+    const F2 pre = -3.0f * (a.c.rho0 + m[0]);
+    F2 fx = pre * gx, fy = pre * gy;
+    if constexpr (TOTAL) {
+        gradient(srho, gx, gy);
+        fx += gx;
+        fy += gy;
+    }
+    const int site = x + X * y;
+    L::collide(g, fx, fy, a.c, (uint32_t)site, a.c.step);
+#pragma unroll
+    for (int i = 0; i < L::Q; ++i) {
+        if constexpr (AL) {
+            A::store2(P.dst[i] + site, g[i].v);
+        } else {
+            A::store1(P.dst[i] + site, g[i].v.x);
+            if (x + 1 < X) A::store1(P.dst[i] + site + 1, g[i].v.y);
         }
     }
 }

@@ -456,7 +456,7 @@ __global__ void __launch_bounds__(kSitesThreads)
 }
 
 // ---------------------------------------------------------------------------
-// D2Q9 force model in one launch: a block's density tile (tile + 2-site halo)
+// D2Q9 force model with FP64 storage in one launch: a block's density tile (tile + 2-site halo)
 // is gathered from the populations into shared memory, mu is formed on the tile
 // + 1-site halo, then pull + collide with F = -rho grad mu + store.
 // ---------------------------------------------------------------------------

@@ -646,9 +646,24 @@ struct Prec {
                                 (const R*)drho, (const NoiseField<R>*)m.swift_xi);
         }
         if (m.Q == 9 && m.nonideal) {
-            const dim3 b(32, 8, 1);
-            return launch_chain(k_step_gather<R, S, 32, 8>, grid_for(m, b), b, st, make_args<D2Q9, R>(m, step),
-                                make_planes<S>(src, dst, 9, m.V));
+            if constexpr (kPackedStorage) {
+                constexpr int TX = 32, TY = 8;
+                Tiling t{};
+                t.ntx = (m.X + TX - 1) / TX;
+                t.nty = (m.Y + TY - 1) / TY;
+                t.ntz = 1;
+                fast_div((uint32_t)t.ntx, t.mx, t.sx);
+                const auto k = m.X % 2 == 0 ? (m.total ? k_step_gather2<S, true, true, TX, TY>
+                                                       : k_step_gather2<S, true, false, TX, TY>)
+                                            : (m.total ? k_step_gather2<S, false, true, TX, TY>
+                                                       : k_step_gather2<S, false, false, TX, TY>);
+                return launch_chain(k, dim3(t.blocks()), dim3(TX * TY / 2), st, make_args<D2Q9, R>(m, step),
+                                    make_planes<S>(src, dst, 9, m.V), t);
+            } else {
+                const dim3 b(32, 8, 1);
+                return launch_chain(k_step_gather<R, S, 32, 8>, grid_for(m, b), b, st, make_args<D2Q9, R>(m, step),
+                                    make_planes<S>(src, dst, 9, m.V));
+            }
         }
         if constexpr (kPackedStorage) {
             if (packed(m)) {
