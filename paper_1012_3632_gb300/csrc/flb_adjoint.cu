@@ -524,7 +524,7 @@ cudaError_t adjoint_fields_t(const HostModel& m, const Coll<R>& c, const R* stat
         const int gx = m.X % 4 == 0 && m.V % 4 == 0 ? 4 : m.X % 2 == 0 ? 2 : 1;
         const Tiling t = make_tiling(m.X, m.Y, (m.Z + 1) / 2, gx == 4 ? 4 : 2, 128, 2);
         const auto k = gx == 4 ? k_force_mu<4> : gx == 2 ? k_force_mu<2> : k_force_mu<1>;
-        return launch_chain(k, dim3(t.blocks(), n), dim3(128), st, sa, crho, mu, t);
+        return launch_chain(k, dim3(t.blocks(), n), dim3(128), st, sa, crho, mu, t, false);
     } else {
         const Tiling t = make_tiling(m.X, m.Y, m.Z, 1, kSitesThreads, 2);
         return launch_chain(k_mu_field<R>, dim3(t.blocks(), n), dim3(kSitesThreads), st, sa, crho, mu, t);

@@ -162,11 +162,13 @@ __global__ void __launch_bounds__(128, 7) k_force_density(const __grid_constant_
 // thread with its 9 rows).
 template <int GX>
 __global__ void __launch_bounds__(128)
-    k_force_mu(const StepArgs<float> a, const float* __restrict__ rho, float* __restrict__ mu, const Tiling t)
+    k_force_mu(const StepArgs<float> a, const float* __restrict__ rho, float* __restrict__ mu, const Tiling t,
+               bool trigger)
 {
     using L = D3Q19;
     constexpr int N = GX == 4 ? 4 : 2;
     pdl_wait();
+    if (trigger) pdl_trigger();  // the collision draws its noise meanwhile
     int3 r0 = tile_site<N, 2, true>(t, threadIdx.x);
     const int X = a.X, Y = a.Y, Z = a.Z, XY = X * Y;
     rho += (long)blockIdx.y * a.V;  // several fields in one launch (the adjoint's states)
@@ -223,18 +225,24 @@ __global__ void __launch_bounds__(128)
 
 // Pull, collide with F = -rho grad mu and store, a site pair per thread.  AL:
 // X even.  TOTAL: psi is the total bulk free energy, F gains cs^2 grad rho
-// (read from the density field).  4 blocks per SM: 128 registers; 5 (96, 72
-// bytes spilled) measured 474 -> 480 us at 256^3.
-template <class S, bool AL, bool TOTAL>
-__global__ void __launch_bounds__(128, 4)
+// (read from the density field).  EARLY: the noise is drawn before the wait for
+// mu (k_force_mu's trigger).  4 blocks per SM: 128 registers; 5 (96, 72 bytes
+// spilled) measured 474 -> 480 us at 256^3.
+template <class S, bool AL, bool TOTAL, bool EARLY>
+__global__ void __launch_bounds__(128, EARLY ? 3 : 4)
     k_force_collide(const StepArgs<float> a, const __grid_constant__ Planes<S> P, const float* __restrict__ rho,
                     const float* __restrict__ mu, const Tiling t)
 {
     using L = D3Q19;
     using A = Packed<S>;
-    pdl_wait();
+    if constexpr (!EARLY) pdl_wait();
     const int3 r0 = tile_site<2, 2, true>(t, threadIdx.x);
     const int x = r0.x, y = r0.y, z = r0.z, X = a.X, Y = a.Y, Z = a.Z, XY = X * Y;
+    F2 zn[EARLY ? 16 : 1];
+    if constexpr (EARLY) {
+        if (a.c.noise) noise_normals<4>(a.c.key, (uint32_t)(x + X * y + XY * z), a.c.step, a.c.replica, zn);
+        pdl_wait();
+    }
     if (x >= X || y >= Y || z >= Z) return;
     const int xm = x == 0 ? X - 1 : x - 1, x1 = x + 1 == X ? 0 : x + 1, xe = x1 + 1 == X ? 0 : x1 + 1;
     const int yo[3] = {X * wrap_once(y - 1, Y), X * y, X * wrap_once(y + 1, Y)};
@@ -289,7 +297,13 @@ __global__ void __launch_bounds__(128, 4)
     }
     const int site = x + X * y + XY * z;
     const bool two = AL || x + 1 < X;
-    L::collide(g, fx, fy, fz, a.c, (uint32_t)site, a.c.step);
+    if constexpr (EARLY)
+        L::template collide_with<true>(g, fx, fy, fz, a.c, [&](F2* q) {
+#pragma unroll
+            for (int k = 0; k < 16; ++k) q[k] = zn[k];
+        });
+    else
+        L::collide(g, fx, fy, fz, a.c, (uint32_t)site, a.c.step);
 #pragma unroll
     for (int i = 0; i < L::Q; ++i) {
         if constexpr (AL) {

@@ -24,13 +24,16 @@ namespace flb {
 // Programmatic dependent launch.  A kernel launched with launch_chain may start
 // while the last blocks of the kernel before it on the stream are ending:
 // pdl_wait waits until everything before this kernel is complete and visible
-// and comes before any access to memory.  No kernel triggers its dependent
-// earlier than its blocks' end: blocks that start while this one still computes
-// are placed on the SMs that happen to have room, several on one, and wait
-// there (a trigger at the start: 48^3 force model 15.7 instead of 9.7 us a
-// step, 160 x 128 in FP64 30.9 instead of 12.1; a trigger before the stores:
-// ideal step 256^3 420 instead of 417, 32^3 3.3 instead of 2.9).
+// and comes before any access to memory.  A kernel triggers its dependent
+// before its blocks' end only where that one has work that needs no memory, the
+// noise, and both fit the chip (EARLY), and only after its own wait, so that no
+// more than two kernels are under way.  Elsewhere blocks that start while this
+// kernel still computes are placed on the SMs that happen to have room, several
+// on one, and wait there (a trigger at the start: 48^3 force model 15.7 instead
+// of 9.7 us a step, 160 x 128 in FP64 30.9 instead of 12.1; a trigger before the
+// stores: ideal step 256^3 420 instead of 417).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Indices of the 3x3x3 neighbourhood of (x, y, z) on a periodic X*Y*Z lattice:
 // xv[1+dx] + rb[1+dy][1+dz] is the site index of (x+dx, y+dy, z+dz).
@@ -602,20 +605,30 @@ __global__ void __launch_bounds__(TX* TY)
 // along c_x = 0 are single loads of two, along c_x = +-1 the pair comes from
 // (x-1, x) or (x+1, x+2).  Odd X: single loads, the last pair of a row is one
 // site.
-// Bound by DRAM at 256^3 (417 us, 152 B/site at 6.1 TB/s) and 128^3; small
-// lattices by launch and latency: chained launches 6.2 -> 2.9 us at 32^3, tiles
+// EARLY: the normals are drawn before the wait for the step before (2.9 -> 2.3
+// us at 32^3), in 32 registers more.
+// Bound by DRAM at 256^3 (417 us, 152 B/site at 6.1 TB/s; 378 without the
+// collision) and 128^3; small lattices by latency: chained launches 6.2 -> 2.9 us
+// at 32^3, tiles
 // that fit the row 32.6 -> 24 us at 96^3, pairs instead of single sites 34.9 ->
 // 30.8 us at 129 x 95 x 67.
 // ---------------------------------------------------------------------------
-template <class S, bool AL, int MINB>
+template <class S, bool AL, int MINB, bool EARLY>
 __global__ void __launch_bounds__(128, MINB)
     k_step2(const StepArgs<float> a, const __grid_constant__ Planes<S> P, const Tiling t)
 {
     using L = D3Q19;
     using A = Packed<S>;
-    pdl_wait();
+    if constexpr (!EARLY) pdl_wait();
     const int3 r0 = tile_site<2, 2, false>(t, threadIdx.x);
     const int x = r0.x, y = r0.y, z = r0.z, X = a.X, Y = a.Y, Z = a.Z;
+    const int s = x + X * (y + Y * z);
+    F2 zn[EARLY ? 16 : 1];
+    if constexpr (EARLY) {
+        if (a.c.noise) noise_normals<4>(a.c.key, (uint32_t)s, a.c.step, a.c.replica, zn);
+        pdl_wait();
+        pdl_trigger();
+    }
     if (x >= X || y >= Y || z >= Z) return;
     const int xm = x == 0 ? X - 1 : x - 1, x1 = AL ? x + 1 : x + 1 == X ? 0 : x + 1, x2 = x1 + 1 == X ? 0 : x1 + 1;
     const int yv[3] = {wrap_once(y - 1, Y), y, wrap_once(y + 1, Y)};
@@ -637,8 +650,13 @@ __global__ void __launch_bounds__(128, MINB)
         else
             g[i] = F2(A::stream1(p + x1), A::stream1(p + x2));
     }
-    const int s = x + X * (y + Y * z);
-    L::template collide<false>(g, F2(0.f), F2(0.f), F2(0.f), a.c, (uint32_t)s, a.c.step);
+    if constexpr (EARLY)
+        L::template collide_with<false>(g, F2(0.f), F2(0.f), F2(0.f), a.c, [&](F2* q) {
+#pragma unroll
+            for (int k = 0; k < 16; ++k) q[k] = zn[k];
+        });
+    else
+        L::template collide<false>(g, F2(0.f), F2(0.f), F2(0.f), a.c, (uint32_t)s, a.c.step);
 #pragma unroll
     for (int i = 0; i < L::Q; ++i) {
         if constexpr (AL) {

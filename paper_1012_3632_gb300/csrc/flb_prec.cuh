@@ -516,6 +516,14 @@ struct Prec {
         return launch_chain(k, dim3(t.blocks()), dim3(kSitesThreads), st, (const S*)pop, (R*)drho, m.X, m.Y, m.Z, t);
     }
 
+    // Blocks up to which a step's kernel draws its noise before it waits for the
+    // kernel before it (EARLY), which then lets it start as soon as it has its own
+    // input: two steps share the chip.  Measured, us per step, without / with:
+    // ideal FP32 32^3 2.92 / 2.3, 48^3 (432 blocks) 4.80 / 4.01, 64^3 (1024) 7.85 /
+    // 7.39, 96^3 (3456) 24.7 / 26.4, BF16 48^3 4.32 / 2.97; force model FP32 32^3
+    // 7.1 / 6.6, 48^3 9.9 / 9.0, 56^3 (784) 12.6 / 12.0, 64^3 (1024) 13.8 / 14.1.
+    static constexpr unsigned kEarlyIdealBlocks = 8 * 152, kEarlyForceBlocks = 6 * 152;
+
     // The step of one site per lane (k_sites).  FP64: small lattices are stepped
     // 32 sites per block, whose other warps draw the noise meanwhile; larger ones
     // fill the FP64 pipe either way.  Measured, us per step, 128 sites / 32 per
@@ -601,11 +609,16 @@ struct Prec {
         if (e != cudaSuccess) return e;
         const Tiling tm = make_tiling(m.X, m.Y, (m.Z + 1) / 2, gx == 4 ? 4 : 2, 128, 2);  // two planes per thread
         const auto km = gx == 4 ? k_force_mu<4> : gx == 2 ? k_force_mu<2> : k_force_mu<1>;
-        e = launch_chain(km, dim3(tm.blocks()), dim3(128), st, a, crho, (float*)m.mu, tm);
-        if (e != cudaSuccess) return e;
         const Tiling tc = make_tiling(m.X, m.Y, m.Z, 2, 128, 2);  // site pairs
-        const auto kc = gx == 1 ? (m.total ? k_force_collide<S, false, true> : k_force_collide<S, false, false>)
-                                : (m.total ? k_force_collide<S, true, true> : k_force_collide<S, true, false>);
+        const bool early = tc.blocks() <= kEarlyForceBlocks;
+        e = launch_chain(km, dim3(tm.blocks()), dim3(128), st, a, crho, (float*)m.mu, tm, early);
+        if (e != cudaSuccess) return e;
+        auto pick = [&](auto E) {
+            constexpr bool EARLY = decltype(E)::value;
+            return gx == 1 ? (m.total ? k_force_collide<S, false, true, EARLY> : k_force_collide<S, false, false, EARLY>)
+                           : (m.total ? k_force_collide<S, true, true, EARLY> : k_force_collide<S, true, false, EARLY>);
+        };
+        const auto kc = early ? pick(std::true_type{}) : pick(std::false_type{});
         return launch_chain(kc, dim3(tc.blocks()), dim3(128), st, a, pl, crho, mu, tc);
     }
     // pull_state of src, then the step: one pass over src does both where the
@@ -671,7 +684,10 @@ struct Prec {
                 // bytes spilled: measured faster than 4 at 126), 4 with BF16 storage
                 constexpr int MINB = sizeof(S) == 4 ? 5 : 4;
                 const Tiling t = make_tiling(m.X, m.Y, m.Z, 2, 128, 2);
-                const auto k = m.X % 2 == 0 ? k_step2<S, true, MINB> : k_step2<S, false, MINB>;
+                const bool al = m.X % 2 == 0;
+                const bool early = t.blocks() <= kEarlyIdealBlocks;
+                const auto k = early ? (al ? k_step2<S, true, 3, true> : k_step2<S, false, 3, true>)
+                                     : (al ? k_step2<S, true, MINB, false> : k_step2<S, false, MINB, false>);
                 return launch_chain(k, dim3(t.blocks()), dim3(128), st, make_args<D3Q19, R>(m, step),
                                     make_planes<S>(src, dst, 19, m.V), t);
             }
