@@ -60,7 +60,6 @@ struct AdjArgs {
 };
 
 __device__ __forceinline__ double mad(double a, double b, double c) { return a * b + c; }
-__device__ __forceinline__ float mad(float a, float b, float c) { return a * b + c; }
 __device__ __forceinline__ F2 mad(F2 a, F2 b, F2 c) { return mk2(__ffma2_rn(a.v, b.v, c.v)); }
 __device__ __forceinline__ F2 mad(float a, F2 b, F2 c) { return mk2(__ffma2_rn(make_float2(a, a), b.v, c.v)); }
 
@@ -71,7 +70,6 @@ __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, 
 template <class T>
 constexpr int kSites = std::is_same<T, F2>::value ? 2 : 1;
 __device__ __forceinline__ double value_sum(double v, bool) { return v; }
-__device__ __forceinline__ float value_sum(float v, bool) { return v; }
 __device__ __forceinline__ float value_sum(F2 v, bool two) { return two ? v.v.x + v.v.y : v.v.x; }
 
 // lb_i += sum_a T_ai b_a, the transpose of L::moments

@@ -269,10 +269,9 @@ int conservation(flb_ctx* c, double out[4])
 {
     int rc = ensure_partials(c);
     if (rc) return rc;
-    int nrows = 0;
-    FLB_CUDA(c->ops->cons_partials(c->m, c->buf[c->cur], c->partials, &nrows, c->stream));
+    FLB_CUDA(c->ops->cons_partials(c->m, c->buf[c->cur], c->partials, c->stream));
     double h[4];
-    rc = reduce_to_host(c, nrows, 4, h);
+    rc = reduce_to_host(c, flb::cons_rows(c->m.V), 4, h);
     if (rc) return rc;
     out[0] = c->m.rho0 * (double)c->m.V + h[0];
     out[1] = h[1];
@@ -493,7 +492,9 @@ static int step_impl(flb_ctx* c, int nsteps, double* dev_sums, char* states = nu
 {
     const double m0 = c->m.rho0 * (double)c->m.V;
     const int nrow = dev_sums ? c->ops->step_row_count(c->m) : 0;
-    const int kmax = nrow > 0 ? step_rows_capacity(c, nrow) : 1;
+    const int kmax = nrow > 0   ? step_rows_capacity(c, nrow)
+                     : dev_sums ? (int)std::min<size_t>(16, partial_bytes(c) / (32 * (size_t)flb::cons_rows(c->m.V)))
+                                : 1;
     for (int t = 0; t < nsteps; ++t) {
         const void* src = c->buf[c->cur];
         void* dst = c->buf[c->cur ^ 1];
@@ -518,10 +519,12 @@ static int step_impl(flb_ctx* c, int nsteps, double* dev_sums, char* states = nu
                 se = flb::sum_steps(rows, nrow, t % kmax + 1, c->partials, ticks(c),
                                     dev_sums + 4 * (size_t)(t - t % kmax), m0, c->stream);
         } else if (dev_sums) {
-            // this step kernel has no partial sums: reduce the state first
-            int nrows = 0;
-            FLB_CUDA(c->ops->cons_partials(c->m, src, c->partials, &nrows, c->stream));
-            FLB_CUDA(flb::sum_columns(c->partials, nrows, 4, dev_sums + 4 * (size_t)t, c->stream, m0));
+            // this step kernel has no partial sums: reduce the state first, the
+            // rows of kmax states (4 of the buffer's 2 Q columns each) together
+            const int rows = flb::cons_rows(c->m.V), k = t % kmax;
+            FLB_CUDA(c->ops->cons_partials(c->m, src, c->partials + 4 * (size_t)rows * k, c->stream));
+            if (k == kmax - 1 || t == nsteps - 1)
+                FLB_CUDA(flb::sum_columns(c->partials, rows, 4, dev_sums + 4 * (size_t)(t - k), c->stream, m0, k + 1));
             se = c->ops->step(c->m, c->step, src, dst, c->drho, c->stream);
         } else if (states) {
             se = c->ops->step_state(c->m, c->step, src, dst, c->drho, states + (size_t)t * c->pop_bytes(), c->stream);

@@ -23,6 +23,8 @@ __global__ void k_sum_columns(const double* __restrict__ partials, int nrows, in
 {
     __shared__ double sh[256];
     const int c = blockIdx.x;
+    partials += (long)blockIdx.y * nrows * ncol;
+    out += (long)blockIdx.y * ncol;
     pdl_wait();
     double acc = 0.0;
     for (int r = threadIdx.x; r < nrows; r += blockDim.x) acc += partials[(long)r * ncol + c];
@@ -35,9 +37,9 @@ __global__ void k_sum_columns(const double* __restrict__ partials, int nrows, in
     if (threadIdx.x == 0) out[c] = c == 0 ? sh[0] + add0 : sh[0];
 }
 
-cudaError_t sum_columns(const double* partials, int nrows, int ncol, double* out, cudaStream_t s, double add0)
+cudaError_t sum_columns(const double* partials, int nrows, int ncol, double* out, cudaStream_t s, double add0, int k)
 {
-    return launch_chain(k_sum_columns, dim3(ncol), dim3(256), s, partials, nrows, ncol, out, add0);
+    return launch_chain(k_sum_columns, dim3(ncol, k), dim3(256), s, partials, nrows, ncol, out, add0);
 }
 
 __global__ void __launch_bounds__(128) k_sum_lattices(const __grid_constant__ ModeSums a, int ncol,

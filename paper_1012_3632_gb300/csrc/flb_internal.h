@@ -96,9 +96,8 @@ struct PrecOps {
     cudaError_t (*mu_force)(const HostModel&, const void* drho, void* mu, void* F, cudaStream_t);
     // per-block sums of m_a and m_a^2, warps per block as mode_blocks returns
     cudaError_t (*mode_sums)(const ModeSums&, int Q, int warps, cudaStream_t);
-    // per-block partial sums; returns the number of partial rows written
-    cudaError_t (*cons_partials)(const HostModel&, const void* src, double* partials, int* nrows,
-                                 cudaStream_t);
+    // cons_rows(V) rows of partial sums of mass deviation and momentum
+    cudaError_t (*cons_partials)(const HostModel&, const void* src, double* partials, cudaStream_t);
     // mode a of the pre-collision state: double2 of an FP64 state, float (real)
     // of the others
     cudaError_t (*mode_field)(const HostModel&, const void* src, int mode, void* out, cudaStream_t);
@@ -149,10 +148,20 @@ cudaError_t launch_chain(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream
     return launch_chain_smem(kernel, grid, block, 0, st, args...);
 }
 
-// Deterministic column sums: out[c] = sum_r partials[r*ncol + c], plus add0
-// on column 0 (flb_fft.cu).
+// Deterministic column sums of k arrays of nrows rows, one after another:
+// out[i*ncol + c] = sum_r partials[(i*nrows + r)*ncol + c], plus add0 on the
+// columns 0 (flb_fft.cu).
 cudaError_t sum_columns(const double* partials, int nrows, int ncol, double* out, cudaStream_t s,
-                        double add0 = 0.0);
+                        double add0 = 0.0, int k = 1);
+
+// Rows of cons_partials, a block of kConsThreads each: at most the blocks of one
+// site per thread, for which the buffer of partial sums has 2 Q columns.
+constexpr int kConsThreads = 256, kConsBlocksMax = 152 * 3;
+inline int cons_rows(long V)
+{
+    const long b = (V + kConsThreads - 1) / kConsThreads;
+    return (int)(b < kConsBlocksMax ? b : kConsBlocksMax);
+}
 
 // Sums of k steps' warp rows (flb_fft.cu): rows holds k times nrows float4 rows
 // (mass deviation and momentum); out[4 i ..] receives the sums of step i's, the

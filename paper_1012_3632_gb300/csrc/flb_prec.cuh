@@ -304,11 +304,6 @@ __device__ __forceinline__ void block_sum_row(V v[NV], double* __restrict__ row)
     }
 }
 
-__device__ __forceinline__ long block_linear()
-{
-    return blockIdx.x + (long)gridDim.x * (blockIdx.y + (long)gridDim.y * blockIdx.z);
-}
-
 // Sums of m_a and m_a^2 of the pre-collision moments (m_0 = drho) over one or
 // many lattices.  A warp takes groups of 32 sites along x and adds the 2 Q
 // values of its lanes in the compute type by exchanging halves: at distance 16,
@@ -401,37 +396,19 @@ __global__ void __launch_bounds__(32 * kModeWarps) k_mode_sums(const __grid_cons
 }
 
 // Per block: sum of g and of g c over the stored buffer (a permutation of the
-// pre-collision populations, so the totals are those of the state).
-template <class L, class R, class S>
-__global__ void k_cons_partials(const S* __restrict__ src, double* __restrict__ partials, int X, int Y, int Z)
-{
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z * blockDim.z + threadIdx.z;
-    double v[4] = {0.0, 0.0, 0.0, 0.0};
-    if (x < X && y < Y && z < Z) {
-        const long V = (long)X * Y * Z;
-        const int s = x + X * (y + Y * z);
-#pragma unroll
-        for (int i = 0; i < L::Q; ++i) {
-            const double gi = (double)load_s<R>(src + (long)i * V + s);
-            v[0] += gi;
-            v[1] += Vel<L>::cx(i) * gi;
-            v[2] += Vel<L>::cy(i) * gi;
-            v[3] += Vel<L>::cz(i) * gi;
-        }
-    }
-    block_sum_row<4>(v, partials + block_linear() * 4);
-}
-
-// Single-precision state: the same sums without FP64 arithmetic per population
-// (the FP64 rate of the part is a small fraction of its FP32 rate).  Each
-// thread walks the sites with a fixed stride and adds every population into
-// (hi, lo) single-precision pairs by Knuth's TwoSum, so the rounding error of
-// each addition is kept in lo; the pairs become doubles only for the block sum.
-// The grid depends on V alone, so the result is deterministic.
-constexpr int kConsThreads = 256, kConsBlocksMax = 152 * 8;
-
+// pre-collision populations, so the totals are those of the state).  The grid
+// depends on V alone, so the result is deterministic.
+// Every thread walks the sites with a fixed stride; per velocity pair (c, -c) it
+// keeps the sum of the two populations and that of their difference (which stays
+// small, so that the momentum keeps its digits) and combines the pairs at the
+// end.  FP64 storage: in FP64.  Single precision: in (hi, lo) pairs by Knuth's
+// TwoSum, so the rounding error of each addition is kept in lo (the FP64 rate of
+// the part is a small fraction of its FP32 rate).
+// A sum per component instead, 49 additions per site of D3Q19 in four dependent
+// chains, took longer than the loads.  What a step with sums takes longer than one
+// without: ideal 256^3 FP32 246 -> 220 us (the loads alone 188), 128^3 54 -> 38,
+// 32^3 10.2 -> 5.0; FP64 96^3 170 -> 78 us.  3 blocks of 256 per SM: 6 are 11 us
+// slower at 64^3 and 128^3 (the ends of more threads), 2 with 20 % more registers 23.
 __device__ __forceinline__ void two_sum_add(float& hi, float& lo, float b)
 {
     const float s = hi + b;
@@ -440,32 +417,77 @@ __device__ __forceinline__ void two_sum_add(float& hi, float& lo, float b)
     hi = s;
 }
 
-template <class L, class S>
-__global__ void __launch_bounds__(kConsThreads) k_cons_partials_sp(const S* __restrict__ src,
-                                                                   double* __restrict__ partials, long V)
+// A sum in R: a double, or two floats.
+template <class R>
+struct Sum {
+    double v = 0.0;
+    __device__ __forceinline__ void add(double b) { v += b; }
+    __device__ __forceinline__ void add_difference(double a, double b) { v += a - b; }
+    __device__ __forceinline__ void add(const Sum& b, int sign) { v += sign * b.v; }
+    __device__ __forceinline__ double value() const { return v; }
+};
+template <>
+struct Sum<float> {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float b) { two_sum_add(hi, lo, b); }
+    __device__ __forceinline__ void add_difference(float a, float b)
+    {
+        two_sum_add(a, lo, -b);
+        two_sum_add(hi, lo, a);
+    }
+    __device__ __forceinline__ void add(const Sum& b, int sign)
+    {
+        two_sum_add(hi, lo, sign * b.hi);
+        lo += sign * b.lo;
+    }
+    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
+
+// First velocity of pair k, and the opposite of a velocity (D2Q9: (1,3) (2,4)
+// (5,7) (6,8); D3Q19: (2k + 1, 2k + 2)).
+template <class L>
+__host__ __device__ constexpr int pair_of(int k)
 {
-    float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
+    return L::Q == 19 ? 2 * k + 1 : k < 2 ? k + 1 : k + 3;
+}
+template <class L>
+__host__ __device__ constexpr int opposite(int i)
+{
+    return L::Q == 19 ? i + 1 : i + 2;
+}
+
+template <class L, class R, class S>
+__global__ void __launch_bounds__(kConsThreads, sizeof(R) == 8 ? 2 : 3)
+    k_cons_partials(const S* __restrict__ src, double* __restrict__ partials, long V)
+{
+    pdl_wait();
+    constexpr int NP = (L::Q - 1) / 2;
+    Sum<R> m[NP], d[NP], t[4];
     for (long s = blockIdx.x * (long)kConsThreads + threadIdx.x; s < V; s += (long)gridDim.x * kConsThreads) {
-        float g[L::Q];
+        R g[L::Q];
 #pragma unroll
-        for (int i = 0; i < L::Q; ++i) g[i] = load_s<float>(src + (long)i * V + s);
+        for (int i = 0; i < L::Q; ++i) g[i] = load_s<R>(src + (long)i * V + s);
+        t[0].add(g[0]);
 #pragma unroll
-        for (int i = 0; i < L::Q; ++i) {
-            two_sum_add(hi[0], lo[0], g[i]);
-            if (Vel<L>::cx(i) != 0) two_sum_add(hi[1], lo[1], Vel<L>::cx(i) > 0 ? g[i] : -g[i]);
-            if (Vel<L>::cy(i) != 0) two_sum_add(hi[2], lo[2], Vel<L>::cy(i) > 0 ? g[i] : -g[i]);
-            if (Vel<L>::cz(i) != 0) two_sum_add(hi[3], lo[3], Vel<L>::cz(i) > 0 ? g[i] : -g[i]);
+        for (int k = 0; k < NP; ++k) {
+            const R a = g[pair_of<L>(k)], b = g[opposite<L>(pair_of<L>(k))];
+            m[k].add(a);
+            m[k].add(b);
+            d[k].add_difference(a, b);
         }
+    }
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {
+        const int i = pair_of<L>(k);
+        t[0].add(m[k], 1);
+        if (Vel<L>::cx(i) != 0) t[1].add(d[k], Vel<L>::cx(i));
+        if (Vel<L>::cy(i) != 0) t[2].add(d[k], Vel<L>::cy(i));
+        if (Vel<L>::cz(i) != 0) t[3].add(d[k], Vel<L>::cz(i));
     }
     double v[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] = (double)hi[k] + (double)lo[k];
+    for (int k = 0; k < 4; ++k) v[k] = t[k].value();
     block_sum_row<4>(v, partials + (long)blockIdx.x * 4);
-}
-
-inline int cons_blocks(long V)
-{
-    return (int)std::min<long>((V + kConsThreads - 1) / kConsThreads, kConsBlocksMax);
 }
 
 template <class L, class R, class S, class T>
@@ -781,27 +803,10 @@ struct Prec {
         return Q == 19 ? launch_chain(k_mode_sums<D3Q19, R, S>, g, b, st, a)
                        : launch_chain(k_mode_sums<D2Q9, R, S>, g, b, st, a);
     }
-    static cudaError_t cons_partials(const HostModel& m, const void* src, double* partials, int* nrows,
-                                     cudaStream_t st)
+    static cudaError_t cons_partials(const HostModel& m, const void* src, double* partials, cudaStream_t st)
     {
-        if constexpr (std::is_same<R, float>::value) {
-            // at most site_blocks(m): cons_blocks(V) <= ceil(V / 256) <= the site grid
-            *nrows = cons_blocks(m.V);
-            if (m.Q == 19)
-                k_cons_partials_sp<D3Q19, S><<<*nrows, kConsThreads, 0, st>>>((const S*)src, partials, m.V);
-            else
-                k_cons_partials_sp<D2Q9, S><<<*nrows, kConsThreads, 0, st>>>((const S*)src, partials, m.V);
-            return cudaGetLastError();
-        }
-        *nrows = site_blocks(m);
-        if (m.Q == 19) {
-            const dim3 b = site_block<D3Q19>();
-            k_cons_partials<D3Q19, R, S><<<grid_for(m, b), b, 0, st>>>((const S*)src, partials, m.X, m.Y, m.Z);
-        } else {
-            const dim3 b = site_block<D2Q9>();
-            k_cons_partials<D2Q9, R, S><<<grid_for(m, b), b, 0, st>>>((const S*)src, partials, m.X, m.Y, m.Z);
-        }
-        return cudaGetLastError();
+        const auto k = m.Q == 19 ? k_cons_partials<D3Q19, R, S> : k_cons_partials<D2Q9, R, S>;
+        return launch_chain(k, dim3(cons_rows(m.V)), dim3(kConsThreads), st, (const S*)src, partials, m.V);
     }
     static cudaError_t mode_field(const HostModel& m, const void* src, int mode, void* out, cudaStream_t st)
     {
