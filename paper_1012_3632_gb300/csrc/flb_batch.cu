@@ -341,7 +341,9 @@ int flb_batch_create(flb_batch** out, int lattice, int n, const int* dims, const
         m.replica = o.replica + (uint32_t)r;
         m.noise_local = o.noise_rho_local ? 1 : 0;
         b->off[r] = b->total;
-        b->total += 19LL * m.V;
+        // every replica begins at a multiple of 256 bytes: its pairs of sites are
+        // loaded together, also behind a replica of an odd number of values
+        b->total += (19LL * m.V + 63) / 64 * 64;
         b->sites += m.V;
         if (19LL * m.V >= (1LL << 31)) b->off32 = false;
         b->shape[r] = (m.X % 32 == 0) ? 1 : 4;  // (32,4,2) or (16,8,2) until tuned
