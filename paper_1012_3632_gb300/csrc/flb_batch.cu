@@ -1,6 +1,6 @@
 // flb_batch.cu -- many independent fluctuating ideal-gas D3Q19 lattices of
 // uneven sizes advanced together (ensemble averages for the FDT statistics of
-// Sec. VI).  One persistent kernel per time step walks a flattened work list
+// Sec. VI).  One kernel per time step walks a flattened work list
 // of (replica, tile) items; per-replica sizes, relaxation rates, noise scales
 // and Philox keys live in the kernel's parameter bank; the time step index
 // lives in device memory so that a CUDA graph of two steps can be replayed.
@@ -58,13 +58,24 @@ struct Tile {
 // single-lattice kernel k_step2), otherwise one site per thread in two passes.
 // OFF32: every replica has 19 V < 2^31, so a population's element offset from
 // its replica's base fits in 32 bits (one address operation per access).
+// The step index is read from one counter and the next one written to another,
+// which the next step reads.
+// Bound by DRAM and the latency of its tiles: 64 replicas of 32^3 to 128^3, 1.35
+// ms at 5.9 TB/s.  5 blocks per SM (96 registers), each walking every 16th wave's
+// tile: 1392 -> 1346 us a step (4 blocks 1383; one wave of blocks that walks all
+// tiles 1397, 4 waves 1372, a block per tile 1405, where the replica's parameters
+// are read anew for each; Philox calls round by round 1355).
 template <bool OFF32>
-__global__ void __launch_bounds__(128) k_step_batch(const __grid_constant__ BatchArgs A, const int4* __restrict__ tiles,
-                                                    int ntiles, const unsigned long long* __restrict__ d_step)
+__global__ void __launch_bounds__(128, 5)
+    k_step_batch(const __grid_constant__ BatchArgs A, const int4* __restrict__ tiles, int ntiles,
+                 const unsigned long long* __restrict__ d_step, unsigned long long* __restrict__ d_next)
 {
     using Off = typename std::conditional<OFF32, int, long>::type;
     using L = D3Q19;
-    const uint32_t step = (uint32_t)__ldg(d_step);
+    pdl_wait();
+    const unsigned long long step64 = *d_step;
+    const uint32_t step = (uint32_t)step64;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *d_next = step64 + 1;
     // the next work item is fetched one iteration ahead, off the path of the pulls
     int4 w_next = (int)blockIdx.x < ntiles ? __ldg(tiles + blockIdx.x) : make_int4(0, 0, 0, 0);
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
@@ -97,7 +108,7 @@ __global__ void __launch_bounds__(128) k_step_batch(const __grid_constant__ Batc
                     g[i] = F2(ld_stream1(p + x + 1), ld_stream1(p + x2));
             }
             const int s = x + X * (y + Y * z);
-            L::template collide<false, true>(g, F2(0.f), F2(0.f), F2(0.f), B.c, (uint32_t)s, step);
+            L::template collide<false>(g, F2(0.f), F2(0.f), F2(0.f), B.c, (uint32_t)s, step);
 #pragma unroll
             for (int i = 0; i < L::Q; ++i) __stcs(reinterpret_cast<float2*>(dst + ((Off)i * V + s)), g[i].v);
         } else {
@@ -120,8 +131,6 @@ __global__ void __launch_bounds__(128) k_step_batch(const __grid_constant__ Batc
         }
     }
 }
-
-__global__ void k_advance(unsigned long long* d_step) { *d_step += 1ull; }
 
 int ilog2(int v)
 {
@@ -149,7 +158,7 @@ struct flb_batch {
     long long sites = 0;
     float* buf[2] = {nullptr, nullptr};
     int cur = 0;
-    unsigned long long* d_step = nullptr;
+    unsigned long long* d_step = nullptr;  // step index of the state in buf[0] and in buf[1], that of cur valid
     uint64_t step = 0;
     int4* tiles = nullptr;
     int ntiles = 0;
@@ -245,16 +254,15 @@ int build_tiles(flb_batch* b)
     return FLB_OK;
 }
 
-int launch_step(flb_batch* b, cudaStream_t st)
+// The step from buffer b->cur over a work list.
+int launch_tiles(flb_batch* b, const int4* tiles, int ntiles, cudaStream_t st)
 {
-    if (b->off32)
-        flb::k_step_batch<true><<<b->grid, 128, 0, st>>>(b->args[b->cur], b->tiles, b->ntiles, b->d_step);
-    else
-        flb::k_step_batch<false><<<b->grid, 128, 0, st>>>(b->args[b->cur], b->tiles, b->ntiles, b->d_step);
-    flb::k_advance<<<1, 1, 0, st>>>(b->d_step);
-    BCUDA(cudaGetLastError());
+    const auto k = b->off32 ? flb::k_step_batch<true> : flb::k_step_batch<false>;
+    BCUDA(flb::launch_chain(k, dim3(std::min(b->grid, ntiles)), dim3(128), st, b->args[b->cur], tiles, ntiles,
+                            (const unsigned long long*)(b->d_step + b->cur), b->d_step + (b->cur ^ 1)));
     return FLB_OK;
 }
+int launch_step(flb_batch* b, cudaStream_t st) { return launch_tiles(b, b->tiles, b->ntiles, st); }
 
 // Graph of two steps starting from buffer parity p (ends at parity p).
 int make_graph(flb_batch* b, int p)
@@ -356,10 +364,10 @@ int flb_batch_create(flb_batch** out, int lattice, int n, const int* dims, const
     };
     cudaError_t e = cudaMalloc(&b->buf[0], b->total * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc(&b->buf[1], b->total * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_step, sizeof(unsigned long long));
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_step, 2 * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMemset(b->buf[0], 0, b->total * sizeof(float));
     if (e == cudaSuccess) e = cudaMemset(b->buf[1], 0, b->total * sizeof(float));
-    if (e == cudaSuccess) e = cudaMemset(b->d_step, 0, sizeof(unsigned long long));
+    if (e == cudaSuccess) e = cudaMemset(b->d_step, 0, 2 * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
     if (e != cudaSuccess)
         return cleanup(bfail(e == cudaErrorMemoryAllocation ? FLB_ENOMEM : FLB_ECUDA,
@@ -371,7 +379,7 @@ int flb_batch_create(flb_batch** out, int lattice, int n, const int* dims, const
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, flb::k_step_batch<true>, 128, 0);
     else
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, flb::k_step_batch<false>, 128, 0);
-    b->grid = std::max(1, nsm * std::max(1, per_sm));
+    b->grid = 16 * nsm * std::max(1, per_sm);
     if ((rc = build_tiles(b))) return cleanup(rc);
     *out = b;
     return FLB_OK;
@@ -385,7 +393,7 @@ int flb_batch_init(flb_batch* b, int thermal_init)
     const flb::PrecOps& ops = flb::ops_fp32();
     for (int r = 0; r < b->n; ++r)
         BCUDA(ops.init(b->m[r], b->buf[0] + b->off[r], nullptr, nullptr, thermal_init ? 1 : 0, b->stream));
-    BCUDA(cudaMemsetAsync(b->d_step, 0, sizeof(unsigned long long), b->stream));
+    BCUDA(cudaMemsetAsync(b->d_step, 0, 2 * sizeof(unsigned long long), b->stream));
     BCUDA(cudaStreamSynchronize(b->stream));
     b->cur = 0;
     b->step = 0;
@@ -454,14 +462,7 @@ int flb_batch_autotune(flb_batch* b, int* shapes_out)
             float ms = 0.f;
             for (int rep = 0; rep < 4 && e == cudaSuccess; ++rep) {  // first launch warms up
                 cudaEventRecord(e0, b->stream);
-                for (int it = 0; it < 5; ++it) {
-                    if (b->off32)
-                        flb::k_step_batch<true>
-                            <<<b->grid, 128, 0, b->stream>>>(b->args[b->cur], d_t, (int)t.size(), b->d_step);
-                    else
-                        flb::k_step_batch<false>
-                            <<<b->grid, 128, 0, b->stream>>>(b->args[b->cur], d_t, (int)t.size(), b->d_step);
-                }
+                for (int it = 0; it < 5 && !rc; ++it) rc = launch_tiles(b, d_t, (int)t.size(), b->stream);
                 cudaEventRecord(e1, b->stream);
                 e = cudaEventSynchronize(e1);
                 float m1 = 0.f;
@@ -469,7 +470,7 @@ int flb_batch_autotune(flb_batch* b, int* shapes_out)
                 if (rep > 0) ms += m1;
             }
             if (d_t) cudaFree(d_t);
-            if (e != cudaSuccess) rc = bfail(FLB_ECUDA, std::string("autotune: ") + cudaGetErrorString(e));
+            if (e != cudaSuccess && !rc) rc = bfail(FLB_ECUDA, std::string("autotune: ") + cudaGetErrorString(e));
             else if (ms < best) {
                 best = ms;
                 best_s = sidx;
