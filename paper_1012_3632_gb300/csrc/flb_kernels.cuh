@@ -101,17 +101,23 @@ inline Tiling make_tiling(int X, int Y, int Z, int N, int threads, int planes)
     return t;
 }
 
-// First site (x, y, z) of thread `tid` of this block's tile of PLANES planes;
+// First site (x, y, z) of thread `tid` of tile b (this block's) of PLANES planes;
 // REV: the z planes in descending order.
 template <int N, int PLANES, bool REV>
-__device__ __forceinline__ int3 tile_site(const Tiling& t, int tid)
+__device__ __forceinline__ int3 tile_site(const Tiling& t, int tid, uint32_t b)
 {
-    const uint32_t b = blockIdx.x, r = fast_quot(b, t.mx, t.sx), bx = b - r * t.ntx;
+    const uint32_t r = fast_quot(b, t.mx, t.sx), bx = b - r * t.ntx;
     const uint32_t rz = fast_quot(r, t.my, t.sy), by = r - rz * t.nty;
     const int bz = REV ? t.ntz - 1 - (int)rz : (int)rz;
     const int tx = tid & ((1 << t.lw) - 1), row = tid >> t.lw;
     return make_int3(N * (((int)bx << t.lw) + tx), ((int)by << t.lh) + (row & ((1 << t.lh) - 1)),
                      PLANES * bz + (row >> t.lh));
+}
+
+template <int N, int PLANES, bool REV>
+__device__ __forceinline__ int3 tile_site(const Tiling& t, int tid)
+{
+    return tile_site<N, PLANES, REV>(t, tid, blockIdx.x);
 }
 
 // Velocity tables for the pull / scatter addressing (same order as the API).
@@ -607,12 +613,35 @@ __global__ void __launch_bounds__(TX* TY)
 // site.
 // EARLY: the normals are drawn before the wait for the step before (2.9 -> 2.3
 // us at 32^3), in 32 registers more.
-// Bound by DRAM at 256^3 (417 us, 152 B/site at 6.1 TB/s; 378 without the
+// Bound by DRAM at 256^3 (408 us, 152 B/site at 6.2 TB/s; 378 without the
 // collision) and 128^3; small lattices by latency: chained launches 6.2 -> 2.9 us
 // at 32^3, tiles
 // that fit the row 32.6 -> 24 us at 96^3, pairs instead of single sites 34.9 ->
 // 30.8 us at 129 x 95 x 67.
 // ---------------------------------------------------------------------------
+// FP32 storage, large lattices of whole lines (X % 32 == 0): each warp asks for the lines of its rows in the
+// tile kPrefetchTiles further on, about a wave, so that DRAM has reads to serve
+// while the warps compute: 417 -> 408 us at 256^3, 54.9 -> 53.5 at 128^3 (152
+// tiles 418, 304 413, 1520 416; bulk prefetches of whole rows 430).  Rows that
+// share their lines with the next are better left alone (72^3 12.0 -> 13.3 us), and
+// BF16 storage, whose step is bound by its instructions (374 -> 386).
+constexpr uint32_t kPrefetchTiles = 4 * 152;
+template <class S>
+__device__ __forceinline__ void prefetch_rows(const S* src, const StepArgs<float>& a, const Tiling& t)
+{
+    const uint32_t b = blockIdx.x + kPrefetchTiles;
+    const int lane = threadIdx.x & 31;
+    if (a.X % 32 != 0 || b >= gridDim.x || lane >= D3Q19::Q) return;
+    const int rows = 32 >> t.lw;  // of a warp
+    for (int k = 0, row = (threadIdx.x >> 5) * rows; k < rows; ++k, ++row) {
+        const int3 r = tile_site<2, 2, false>(t, row << t.lw, b);
+        if (r.x >= a.X || r.y >= a.Y || r.z >= a.Z) continue;
+        const char* p = reinterpret_cast<const char*>(src + lane * a.V + (r.x + a.X * (r.y + a.Y * r.z)));
+        const int bytes = min(2 << t.lw, a.X - r.x) * (int)sizeof(S);
+        for (int o = 0; o < bytes; o += 128) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + o));
+    }
+}
+
 template <class S, bool AL, int MINB, bool EARLY>
 __global__ void __launch_bounds__(128, MINB)
     k_step2(const StepArgs<float> a, const __grid_constant__ Planes<S> P, const Tiling t)
@@ -650,6 +679,7 @@ __global__ void __launch_bounds__(128, MINB)
         else
             g[i] = F2(A::stream1(p + x1), A::stream1(p + x2));
     }
+    if constexpr (!EARLY && sizeof(S) == 4) prefetch_rows(P.src[0], a, t);
     if constexpr (EARLY)
         L::template collide_with<false>(g, F2(0.f), F2(0.f), F2(0.f), a.c, [&](F2* q) {
 #pragma unroll
