@@ -28,7 +28,7 @@
 // states of several steps give at once are not a launch per step, neighbours are
 // read once (30 values for mubar, not 90) and the launches are chained: a segment
 // of 20 steps, recomputed and swept back, takes 1.07 ms; with density, mu, force
-// and gradient launches per step and its states pulled apart it took 1.9 ms.
+// and gradient launches per step and its states pulled apart it took 1.8 ms.
 #include <cuda_runtime.h>
 
 #include <cmath>

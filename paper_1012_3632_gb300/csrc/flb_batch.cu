@@ -61,10 +61,10 @@ struct Tile {
 // The step index is read from one counter and the next one written to another,
 // which the next step reads.
 // Bound by DRAM and the latency of its tiles: 64 replicas of 32^3 to 128^3, 1.35
-// ms at 5.9 TB/s.  5 blocks per SM (96 registers), each walking every 16th wave's
-// tile: 1392 -> 1346 us a step (4 blocks 1383; one wave of blocks that walks all
-// tiles 1397, 4 waves 1372, a block per tile 1405, where the replica's parameters
-// are read anew for each; Philox calls round by round 1355).
+// ms at 5.9 TB/s.  5 blocks per SM (96 registers) and 16 waves of blocks, each
+// block walking a few tiles: 1392 -> 1346 us a step (4 blocks per SM 1383; one
+// wave 1397, 4 waves 1372, a block per tile 1405, where the replica's parameters
+// are read anew for each; the thread's eight Philox calls in lock-step 1355).
 template <bool OFF32>
 __global__ void __launch_bounds__(128, 5)
     k_step_batch(const __grid_constant__ BatchArgs A, const int4* __restrict__ tiles, int ntiles,

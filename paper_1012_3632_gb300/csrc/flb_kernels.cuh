@@ -57,8 +57,8 @@ struct Nbhd {
 };
 
 // Tiles of threads over the lattice: rows of 2^lw threads (each N sites along
-// x), 2^lh rows in y and one or two planes in z.  Tiles are numbered along one grid dimension, x fastest (no axis meets a grid
-// limit of 65535).
+// x), 2^lh rows in y and one or two planes in z.  Tiles are numbered along one
+// grid dimension, x fastest (no axis meets a grid limit of 65535).
 struct Tiling {
     int lw, lh;
     int ntx, nty, ntz;
@@ -615,16 +615,16 @@ __global__ void __launch_bounds__(TX* TY)
 // us at 32^3), in 32 registers more.
 // Bound by DRAM at 256^3 (408 us, 152 B/site at 6.2 TB/s; 378 without the
 // collision) and 128^3; small lattices by latency: chained launches 6.2 -> 2.9 us
-// at 32^3, tiles
-// that fit the row 32.6 -> 24 us at 96^3, pairs instead of single sites 34.9 ->
-// 30.8 us at 129 x 95 x 67.
+// at 32^3, tiles that fit the row 32.6 -> 24 us at 96^3, pairs instead of single
+// sites 34.9 -> 30.8 us at 129 x 95 x 67.
 // ---------------------------------------------------------------------------
-// FP32 storage, large lattices of whole lines (X % 32 == 0): each warp asks for the lines of its rows in the
-// tile kPrefetchTiles further on, about a wave, so that DRAM has reads to serve
-// while the warps compute: 417 -> 408 us at 256^3, 54.9 -> 53.5 at 128^3 (152
-// tiles 418, 304 413, 1520 416; bulk prefetches of whole rows 430).  Rows that
-// share their lines with the next are better left alone (72^3 12.0 -> 13.3 us), and
-// BF16 storage, whose step is bound by its instructions (374 -> 386).
+// FP32 storage, large lattices of whole lines (X % 32 == 0): each warp asks for
+// the lines of its rows in the tile kPrefetchTiles further on, about a wave, so
+// that DRAM has reads to serve while the warps compute: 417 -> 408 us at 256^3,
+// 54.9 -> 53.5 at 128^3 (152 tiles 418, 304 413, 1520 416; bulk prefetches of
+// whole rows 430).  Rows that share their lines with the next are better left
+// alone (72^3 12.0 -> 13.3 us), and BF16 storage, whose step is bound by its
+// instructions (374 -> 386).
 constexpr uint32_t kPrefetchTiles = 4 * 152;
 template <class S>
 __device__ __forceinline__ void prefetch_rows(const S* src, const StepArgs<float>& a, const Tiling& t)

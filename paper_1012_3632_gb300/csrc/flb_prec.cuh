@@ -670,15 +670,22 @@ struct Prec {
         if (rows && !step_row_count(m)) return cudaErrorNotSupported;
         // drho: the context's density field, scratch of the steps in passes
         if constexpr (kPackedStorage) {
-            if (packed(m) && m.nonideal) return step_force(m, step, src, dst, (float*)const_cast<void*>(drho), (float*)rows,
-                                                              nullptr, st);
+            if (packed(m) && m.nonideal)
+                return step_force(m, step, src, dst, (float*)const_cast<void*>(drho), (float*)rows, nullptr, st);
         }
         if (step_in_passes(m)) return step_force_sites(m, step, src, dst, (R*)const_cast<void*>(drho), st);
         if (m.Q == 9 && m.nonideal && m.model == 1) {
             const StepArgs<R> a = make_args<D2Q9, R>(m, step);
-            const dim3 b(32, 8, 1);
-            return launch_chain(k_step_swift<R, S, 32, 8>, grid_for(m, b), b, st, a, make_planes<S>(src, dst, 9, m.V),
-                                (const R*)drho, (const NoiseField<R>*)m.swift_xi);
+            const Planes<S> pl = make_planes<S>(src, dst, 9, m.V);
+            const auto* xi = (const NoiseField<R>*)m.swift_xi;
+            if constexpr (kPackedStorage) {
+                const Tiling t = make_tiling(m.X, m.Y, 1, 2, 128, 1);
+                const auto k = m.X % 2 == 0 ? k_step_swift2<S, true> : k_step_swift2<S, false>;
+                return launch_chain(k, dim3(t.blocks()), dim3(128), st, a, pl, (const R*)drho, xi, t);
+            } else {
+                const dim3 b(32, 8, 1);
+                return launch_chain(k_step_swift<R, S, 32, 8>, grid_for(m, b), b, st, a, pl, (const R*)drho, xi);
+            }
         }
         if (m.Q == 9 && m.nonideal) {
             if constexpr (kPackedStorage) {
