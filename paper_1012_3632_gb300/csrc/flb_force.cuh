@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(128, EARLY ? 3 : 4)
     using L = D3Q19;
     using A = Packed<S>;
     if constexpr (!EARLY) pdl_wait();
-    const int3 r0 = tile_site<2, 2, true>(t, threadIdx.x);
+    const int3 r0 = grid_tile<2, 2, true>(t, threadIdx.x);
     const int x = r0.x, y = r0.y, z = r0.z, X = a.X, Y = a.Y, Z = a.Z, XY = X * Y;
     F2 zn[EARLY ? 16 : 1];
     if constexpr (EARLY) {

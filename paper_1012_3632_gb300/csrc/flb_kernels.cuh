@@ -64,6 +64,9 @@ struct Tiling {
     int ntx, nty, ntz;
     uint32_t mx, sx, my, sy;  // quotients by ntx and nty: (umulhi(n, m) + n) >> s, n < 2^31
     unsigned blocks() const { return (unsigned)((long)ntx * nty * ntz); }
+    // a grid of three dimensions where its limits allow, for kernels that find their
+    // tile by grid_tile
+    dim3 grid() const { return nty > 65535 || ntz > 65535 ? dim3(blocks()) : dim3(ntx, nty, ntz); }
 };
 
 inline void fast_div(uint32_t d, uint32_t& m, uint32_t& s)
@@ -118,6 +121,19 @@ template <int N, int PLANES, bool REV>
 __device__ __forceinline__ int3 tile_site(const Tiling& t, int tid)
 {
     return tile_site<N, PLANES, REV>(t, tid, blockIdx.x);
+}
+
+// The same for a grid of Tiling::grid(): ten instructions fewer where no quotient
+// is needed, which the issue-bound steps notice (BF16 256^3 ideal 374.7 -> 372.1
+// us, with the pulls' row offsets as sums of two 370.9).
+template <int N, int PLANES, bool REV>
+__device__ __forceinline__ int3 grid_tile(const Tiling& t, int tid)
+{
+    if (gridDim.y * gridDim.z == 1) return tile_site<N, PLANES, REV>(t, tid, blockIdx.x);
+    const int bz = REV ? t.ntz - 1 - (int)blockIdx.z : (int)blockIdx.z;
+    const int tx = tid & ((1 << t.lw) - 1), row = tid >> t.lw;
+    return make_int3(N * (((int)blockIdx.x << t.lw) + tx), ((int)blockIdx.y << t.lh) + (row & ((1 << t.lh) - 1)),
+                     PLANES * bz + (row >> t.lh));
 }
 
 // Velocity tables for the pull / scatter addressing (same order as the API).
@@ -613,7 +629,7 @@ __global__ void __launch_bounds__(TX* TY)
 // site.
 // EARLY: the normals are drawn before the wait for the step before (2.9 -> 2.3
 // us at 32^3), in 32 registers more.
-// Bound by DRAM at 256^3 (408 us, 152 B/site at 6.2 TB/s; 378 without the
+// Bound by DRAM at 256^3 (406 us, 152 B/site at 6.3 TB/s; 378 without the
 // collision) and 128^3; small lattices by latency: chained launches 6.2 -> 2.9 us
 // at 32^3, tiles that fit the row 32.6 -> 24 us at 96^3, pairs instead of single
 // sites 34.9 -> 30.8 us at 129 x 95 x 67.
@@ -629,9 +645,10 @@ constexpr uint32_t kPrefetchTiles = 4 * 152;
 template <class S>
 __device__ __forceinline__ void prefetch_rows(const S* src, const StepArgs<float>& a, const Tiling& t)
 {
-    const uint32_t b = blockIdx.x + kPrefetchTiles;
     const int lane = threadIdx.x & 31;
-    if (a.X % 32 != 0 || b >= gridDim.x || lane >= D3Q19::Q) return;
+    if (a.X % 32 != 0 || lane >= D3Q19::Q) return;
+    const uint32_t b = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z) + kPrefetchTiles;
+    if (b >= gridDim.x * gridDim.y * gridDim.z) return;
     const int rows = 32 >> t.lw;  // of a warp
     for (int k = 0, row = (threadIdx.x >> 5) * rows; k < rows; ++k, ++row) {
         const int3 r = tile_site<2, 2, false>(t, row << t.lw, b);
@@ -649,7 +666,7 @@ __global__ void __launch_bounds__(128, MINB)
     using L = D3Q19;
     using A = Packed<S>;
     if constexpr (!EARLY) pdl_wait();
-    const int3 r0 = tile_site<2, 2, false>(t, threadIdx.x);
+    const int3 r0 = grid_tile<2, 2, false>(t, threadIdx.x);
     const int x = r0.x, y = r0.y, z = r0.z, X = a.X, Y = a.Y, Z = a.Z;
     const int s = x + X * (y + Y * z);
     F2 zn[EARLY ? 16 : 1];
@@ -660,17 +677,12 @@ __global__ void __launch_bounds__(128, MINB)
     }
     if (x >= X || y >= Y || z >= Z) return;
     const int xm = x == 0 ? X - 1 : x - 1, x1 = AL ? x + 1 : x + 1 == X ? 0 : x + 1, x2 = x1 + 1 == X ? 0 : x1 + 1;
-    const int yv[3] = {wrap_once(y - 1, Y), y, wrap_once(y + 1, Y)};
-    const int zv[3] = {wrap_once(z - 1, Z), z, wrap_once(z + 1, Z)};
-    int rb[3][3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) rb[i][j] = X * (yv[i] + Y * zv[j]);
+    const int XY = X * Y, yo[3] = {X * (y == 0 ? Y - 1 : y - 1), X * y, X * (y == Y - 1 ? 0 : y + 1)};
+    const int zo[3] = {XY * (z == 0 ? Z - 1 : z - 1), XY * z, XY * (z == Z - 1 ? 0 : z + 1)};
     F2 g[L::Q];
 #pragma unroll
     for (int i = 0; i < L::Q; ++i) {
-        const S* p = P.src[i] + rb[1 - Vel<L>::cy(i)][1 - Vel<L>::cz(i)];
+        const S* p = P.src[i] + (yo[1 - Vel<L>::cy(i)] + zo[1 - Vel<L>::cz(i)]);
         const int cx = Vel<L>::cx(i);
         if (cx == 0)
             g[i] = AL ? mk2(A::stream2(p + x)) : F2(A::stream1(p + x), A::stream1(p + x1));

@@ -641,7 +641,7 @@ struct Prec {
                            : (m.total ? k_force_collide<S, true, true, EARLY> : k_force_collide<S, true, false, EARLY>);
         };
         const auto kc = early ? pick(std::true_type{}) : pick(std::false_type{});
-        return launch_chain(kc, dim3(tc.blocks()), dim3(128), st, a, pl, crho, mu, tc);
+        return launch_chain(kc, tc.grid(), dim3(128), st, a, pl, crho, mu, tc);
     }
     // pull_state of src, then the step: one pass over src does both where the
     // step pulls the state for its density (FP32 force model).
@@ -717,7 +717,7 @@ struct Prec {
                 const bool early = t.blocks() <= kEarlyIdealBlocks;
                 const auto k = early ? (al ? k_step2<S, true, 3, true> : k_step2<S, false, 3, true>)
                                      : (al ? k_step2<S, true, MINB, false> : k_step2<S, false, MINB, false>);
-                return launch_chain(k, dim3(t.blocks()), dim3(128), st, make_args<D3Q19, R>(m, step),
+                return launch_chain(k, t.grid(), dim3(128), st, make_args<D3Q19, R>(m, step),
                                     make_planes<S>(src, dst, 19, m.V), t);
             }
         }
