@@ -161,12 +161,13 @@ def initial_density(wl, dims):
 
 def kernel_name(wl):
     """The step kernel the library launches for this workload."""
-    packed = wl["precision"] in ("fp32", "bf16") and wl["dims"][0] % 2 == 0 and wl["lattice"] == 19
-    if wl["fe"] and wl["fe"].get("model", 0) == 1:
-        return "k_step_swift"
-    if wl["fe"] and wl["lattice"] == 19:
-        return "k_force_collide" if wl["precision"] in ("fp32", "bf16") else "k_sites"
-    return "k_step2" if packed else "k_step_gather" if wl["fe"] else "k_sites"
+    packed = wl["precision"] in ("fp32", "bf16")
+    if wl["lattice"] == 19:
+        return ("k_force_collide" if wl["fe"] else "k_step2") if packed else "k_sites"
+    if not wl["fe"]:
+        return "k_sites"
+    name = "k_step_swift" if wl["fe"].get("model", 0) == 1 else "k_step_gather"
+    return name + "2" if packed else name
 
 
 def kernel_source_hash():
@@ -295,7 +296,7 @@ def cpu_baseline(wl, budget_s=12.0):
 def batched_vs_plain(n=64, steps=2000, every=20, seed=4):
     """The batched ensemble workload: 64 D3Q19 ideal-gas replicas, cubic sizes
     drawn from {32,48,64,96,128}, omega_shear ~ U(0.8,1.6), kT = 1e-5, FP32, one
-    persistent launch per step replayed from a CUDA graph, 2000 steps with the
+    launch per step replayed from a CUDA graph, 2000 steps with the
     ensemble observables accumulated in FP64 every 20 steps (every replica's
     mode variances and its density S(k) on the device).  Times the whole run,
     the steps alone, and the plain single-lattice step on the same replicas."""
@@ -351,7 +352,7 @@ def batched_vs_plain(n=64, steps=2000, every=20, seed=4):
             t_plain += cnt * ev0.elapsed_time(ev1) / 50
     shape_of = {int(l): [int(v) for v in shapes[int(np.where(L == l)[0][0])]] for l in set(int(v) for v in L)}
     return {"workload": f"{n} D3Q19 ideal-gas replicas, cubic sizes from {{32,48,64,96,128}} (seed {seed}), "
-                        "omega_shear U(0.8,1.6), kT=1e-5, FP32, graph-replayed persistent launch",
+                        "omega_shear U(0.8,1.6), kT=1e-5, FP32, graph-replayed launch",
             "sites": sites, "batched_mlups": sites / (t_batch * 1e-3) / 1e6,
             "batched_gbs": 152 * sites / (t_batch * 1e-3) / 1e9,
             "plain_mlups": sites / (t_plain * 1e-3) / 1e6, "batched_over_plain": t_plain / t_batch,
@@ -394,7 +395,7 @@ def adjoint_vs_plain(dims=(64, 64, 64), nsteps=200, every=20, precision="fp32"):
         c.get_state_device(g0.data_ptr())
     cfg = dict(dims=dims, kT=1e-6, seed=5, precision=precision, nsteps=nsteps, every=every, nonideal=True, rho_c=1.0)
     # warm-up of the loss (cuFFT loads and plans on its first use) and of the
-    # path, long enough for the step's column-length tuning
+    # path
     density_spectrum_loss(g0, dims).item()
     warm = dict(cfg, nsteps=40, every=20)
     th0 = torch.tensor([1.0, 1.0, 1.0, 0.02, -0.01, 0.1], dtype=torch.float64, requires_grad=True)
@@ -541,13 +542,6 @@ def main():
     ctx.init(rho=rho, u=u, thermal=not wl["fe"])
 
     # ---- device-resident timing ------------------------------------------
-    # setup: the z-marching step times its candidate column lengths on its
-    # first launches; finish that before the warm-up steps so that the timed
-    # steps all run with the chosen length
-    n_tune = 0
-    while ctx.z_chunk()[1] and n_tune < 256:
-        ctx.step(1)
-        n_tune += 1
     ctx.step(args.warmup)
     ctx.synchronize()
     ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -580,7 +574,6 @@ def main():
     kms, kn = ctx.kernel_times()
     ctx.kernel_timing(False)
     n_kt = args.steps
-    z_planes, z_tuning = ctx.z_chunk()
     ms_max = max_over_ranks(ms, world)
     value = whole_job_mlups(world, V, args.steps, ms_max * 1e-3)
 
@@ -639,11 +632,14 @@ def main():
     t_fused = kms[1] / max(n_fused, 1) * 1e-3
     achieved = fused_b * V / t_fused / 1e9
     traffic = ncu_traffic(args.workload)
-    # kernels per step: the timed kinds (gather, step, checks), plus, for the
-    # modified-equilibrium noise, its white draw, colouring and two 2-D FFTs
+    # kernels per step: the timed kinds (gather, step, checks); the D3Q19 force
+    # model's step is three kernels (density, mu, collision), the modified
+    # equilibrium's coloured noise three more (rows, columns and back, rows)
     per_step = (kn[0] + kn[1] + kn[2]) / max(n_kt, 1)
-    if wl["fe"] and wl["fe"].get("model", 0) == 1 and wl["kT"] > 0:
-        per_step += 6
+    if wl["fe"] and wl["fe"].get("model", 0) == 1:
+        per_step += 3 if wl["kT"] > 0 else 0
+    elif wl["fe"] and wl["lattice"] == 19:
+        per_step += 2
     n_launch = int(round(per_step * args.steps))
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
@@ -666,9 +662,7 @@ def main():
                                        "achieved_gbs": gather_b * V / (kms[0] / max(kn[0], 1) * 1e-3) / 1e9
                                        if kn[0] else None},
                     "fused_step": {"launches": n_fused, "avg_ms": kms[1] / max(n_fused, 1)},
-                    "timed_with_events_over_steps": n_kt,
-                    "z_planes_per_block": z_planes, "z_chunk_tuning_steps_before_warmup": n_tune,
-                    "z_chunk_tuned_before_timing": not z_tuning},
+                    "timed_with_events_over_steps": n_kt},
         "whole_step_gbs": (fused_b + gather_b) * V / (ms_max / args.steps * 1e-3) / 1e9,
         "clocks": clk.summary(), "e2e": e2e, "gpu_launches": n_launch,
     }
