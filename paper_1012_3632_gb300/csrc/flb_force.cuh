@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(128)
 // (read from the density field).  EARLY: the noise is drawn before the wait for
 // mu (k_force_mu's trigger).  4 blocks per SM: 128 registers; 5 (96, 72 bytes
 // spilled) measured 474 -> 480 us at 256^3.
-template <class S, bool AL, bool TOTAL, bool EARLY>
+template <class S, bool AL, bool TOTAL, bool EARLY, bool LINE>
 __global__ void __launch_bounds__(128, EARLY ? 3 : 4)
     k_force_collide(const StepArgs<float> a, const __grid_constant__ Planes<S> P, const float* __restrict__ rho,
                     const float* __restrict__ mu, const Tiling t)
@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(128, EARLY ? 3 : 4)
     using L = D3Q19;
     using A = Packed<S>;
     if constexpr (!EARLY) pdl_wait();
-    const int3 r0 = grid_tile<2, 2, true>(t, threadIdx.x);
+    const int3 r0 = grid_tile<2, 2, true, LINE>(t, threadIdx.x);
     const int x = r0.x, y = r0.y, z = r0.z, X = a.X, Y = a.Y, Z = a.Z, XY = X * Y;
     F2 zn[EARLY ? 16 : 1];
     if constexpr (EARLY) {

@@ -122,15 +122,15 @@ inline Tiling make_tiling(int X, int Y, int Z, int N, int threads, int planes)
 }
 
 // First site (x, y, z) of thread `tid` of tile b (this block's) of PLANES planes;
-// REV: the z planes in descending order.
-template <int N, int PLANES, bool REV>
+// REV: the z planes in descending order.  LINE: t may have its threads in line.
+template <int N, int PLANES, bool REV, bool LINE = true>
 __device__ __forceinline__ int3 tile_site(const Tiling& t, int tid, uint32_t b)
 {
-    if (t.threads) b = b * t.threads + tid;
+    if (LINE && t.threads) b = b * t.threads + tid;
     const uint32_t r = fast_quot(b, t.mx, t.sx), bx = b - r * t.ntx;
     const uint32_t rz = fast_quot(r, t.my, t.sy), by = r - rz * t.nty;
     const int bz = REV ? t.ntz - 1 - (int)rz : (int)rz;
-    if (t.threads) return make_int3(N * (int)bx, (int)by, (int)rz < t.ntz ? bz : t.ntz);  // past the last row: outside
+    if (LINE && t.threads) return make_int3(N * (int)bx, (int)by, (int)rz < t.ntz ? bz : t.ntz);  // past the last row: outside
     const int tx = tid & ((1 << t.lw) - 1), row = tid >> t.lw;
     return make_int3(N * (((int)bx << t.lw) + tx), ((int)by << t.lh) + (row & ((1 << t.lh) - 1)),
                      PLANES * bz + (row >> t.lh));
@@ -144,11 +144,12 @@ __device__ __forceinline__ int3 tile_site(const Tiling& t, int tid)
 
 // The same for a grid of Tiling::grid(): ten instructions fewer where no quotient
 // is needed, which the issue-bound steps notice (BF16 256^3 ideal 374.7 -> 372.1
-// us, with the pulls' row offsets as sums of two 370.9).
-template <int N, int PLANES, bool REV>
+// us, with the pulls' row offsets as sums of two 370.9); not LINE, where it need
+// not look for threads in line (force model 8 steps 256^3 BF16 4867 -> 4768 us).
+template <int N, int PLANES, bool REV, bool LINE>
 __device__ __forceinline__ int3 grid_tile(const Tiling& t, int tid)
 {
-    if (gridDim.y * gridDim.z == 1) return tile_site<N, PLANES, REV>(t, tid, blockIdx.x);
+    if (gridDim.y * gridDim.z == 1) return tile_site<N, PLANES, REV, LINE>(t, tid, blockIdx.x);
     const int bz = REV ? t.ntz - 1 - (int)blockIdx.z : (int)blockIdx.z;
     const int tx = tid & ((1 << t.lw) - 1), row = tid >> t.lw;
     return make_int3(N * (((int)blockIdx.x << t.lw) + tx), ((int)blockIdx.y << t.lh) + (row & ((1 << t.lh) - 1)),
@@ -670,7 +671,7 @@ __device__ __forceinline__ void prefetch_rows(const S* src, const StepArgs<float
     if (b >= gridDim.x * gridDim.y * gridDim.z) return;
     const int rows = 32 >> t.lw;  // of a warp
     for (int k = 0, row = (threadIdx.x >> 5) * rows; k < rows; ++k, ++row) {
-        const int3 r = tile_site<2, 2, false>(t, row << t.lw, b);
+        const int3 r = tile_site<2, 2, false, false>(t, row << t.lw, b);
         if (r.x >= a.X || r.y >= a.Y || r.z >= a.Z) continue;
         const char* p = reinterpret_cast<const char*>(src + lane * a.V + (r.x + a.X * (r.y + a.Y * r.z)));
         const int bytes = min(2 << t.lw, a.X - r.x) * (int)sizeof(S);
@@ -678,14 +679,14 @@ __device__ __forceinline__ void prefetch_rows(const S* src, const StepArgs<float
     }
 }
 
-template <class S, bool AL, int MINB, bool EARLY>
+template <class S, bool AL, int MINB, bool EARLY, bool LINE>
 __global__ void __launch_bounds__(128, MINB)
     k_step2(const StepArgs<float> a, const __grid_constant__ Planes<S> P, const Tiling t)
 {
     using L = D3Q19;
     using A = Packed<S>;
     if constexpr (!EARLY) pdl_wait();
-    const int3 r0 = grid_tile<2, 2, false>(t, threadIdx.x);
+    const int3 r0 = grid_tile<2, 2, false, LINE>(t, threadIdx.x);
     const int x = r0.x, y = r0.y, z = r0.z, X = a.X, Y = a.Y, Z = a.Z;
     const int s = x + X * (y + Y * z);
     F2 zn[EARLY ? 16 : 1];

@@ -637,8 +637,12 @@ struct Prec {
         if (e != cudaSuccess) return e;
         auto pick = [&](auto E) {
             constexpr bool EARLY = decltype(E)::value;
-            return gx == 1 ? (m.total ? k_force_collide<S, false, true, EARLY> : k_force_collide<S, false, false, EARLY>)
-                           : (m.total ? k_force_collide<S, true, true, EARLY> : k_force_collide<S, true, false, EARLY>);
+            return gx == 1 ? (m.total ? k_force_collide<S, false, true, EARLY, true>
+                                      : k_force_collide<S, false, false, EARLY, true>)
+                   : EARLY || tc.threads ? (m.total ? k_force_collide<S, true, true, EARLY, true>
+                                                    : k_force_collide<S, true, false, EARLY, true>)
+                                         : (m.total ? k_force_collide<S, true, true, EARLY, EARLY>
+                                                    : k_force_collide<S, true, false, EARLY, EARLY>);
         };
         const auto kc = early ? pick(std::true_type{}) : pick(std::false_type{});
         return launch_chain(kc, tc.grid(), dim3(128), st, a, pl, crho, mu, tc);
@@ -715,8 +719,10 @@ struct Prec {
                 const Tiling t = make_tiling(m.X, m.Y, m.Z, 2, 128, 2);
                 const bool al = m.X % 2 == 0;
                 const bool early = t.blocks() <= kEarlyIdealBlocks;
-                const auto k = early ? (al ? k_step2<S, true, 3, true> : k_step2<S, false, 3, true>)
-                                     : (al ? k_step2<S, true, MINB, false> : k_step2<S, false, MINB, false>);
+                const auto k = early ? (al ? k_step2<S, true, 3, true, true> : k_step2<S, false, 3, true, true>)
+                               : !al ? k_step2<S, false, MINB, false, true>
+                               : t.threads ? k_step2<S, true, MINB, false, true>
+                                           : k_step2<S, true, MINB, false, false>;
                 return launch_chain(k, t.grid(), dim3(128), st, make_args<D3Q19, R>(m, step),
                                     make_planes<S>(src, dst, 19, m.V), t);
             }
