@@ -226,7 +226,7 @@ __device__ __forceinline__ void block_rows(R v[NV], double* __restrict__ row)
 
 // densities of the states g^n (pre-collision deviations) blockIdx.y = 0, 1, ..
 template <class R>
-__global__ void __launch_bounds__(128) k_adj_density(const R* __restrict__ gn, R* __restrict__ drho, long V)
+__global__ void __launch_bounds__(128) k_adj_density(const R* gn, R* __restrict__ drho, long V)
 {
     pdl_wait();
     gn += (long)blockIdx.y * 19 * V;
@@ -278,8 +278,8 @@ __device__ __forceinline__ void put(R* p, T v, bool two)
 // W: rho Fbar (TOTAL: Fbar), three fields; rb1: -Fbar . grad mu.
 template <class T, class R, bool AL, bool FORCE, bool TOTAL>
 __global__ void __launch_bounds__(128, kSites<T> == 2 ? 3 : 2)
-    k_adj_collide(const AdjArgs<R> a, const R* __restrict__ gn, const R* __restrict__ drho, const R* __restrict__ mu,
-                  const R* __restrict__ lam_next, const R* __restrict__ rb_next, R* __restrict__ lam,
+    k_adj_collide(const AdjArgs<R> a, const R* gn, const R* drho, const R* mu,
+                  const R* lam_next, const R* rb_next, R* __restrict__ lam,
                   R* __restrict__ W, R* __restrict__ rb1, double* __restrict__ rows, const Tiling t)
 {
     pdl_wait();
@@ -352,7 +352,7 @@ __global__ void __launch_bounds__(128, kSites<T> == 2 ? 3 : 2)
 // cs^2 grad rho): rb1 += sum_i w_i c_i . Fbar(y - c_i) as well.
 template <class R, bool TOTAL>
 __global__ void __launch_bounds__(128)
-    k_adj_mu(const AdjArgs<R> a, const R* __restrict__ drho, const R* __restrict__ W, R* __restrict__ mubar,
+    k_adj_mu(const AdjArgs<R> a, const R* drho, const R* W, R* __restrict__ mubar,
              R* __restrict__ rb1, const Tiling t)
 {
     pdl_wait();
@@ -393,8 +393,8 @@ __global__ void __launch_bounds__(128)
 // -sum rho lap(mubar): the lattice Laplacian is symmetric.
 template <class R>
 __global__ void __launch_bounds__(128)
-    k_adj_rho(const AdjArgs<R> a, const R* __restrict__ drho, const R* __restrict__ mubar,
-              const R* __restrict__ rb1, R* __restrict__ lam, R* __restrict__ rb_out, double* __restrict__ rows,
+    k_adj_rho(const AdjArgs<R> a, const R* drho, const R* mubar,
+              const R* rb1, R* __restrict__ lam, R* __restrict__ rb_out, double* __restrict__ rows,
               const Tiling t)
 {
     pdl_wait();
@@ -432,7 +432,7 @@ __global__ void __launch_bounds__(128)
 
 // lam += rb on every population: the deferred density part of the last step
 template <class R>
-__global__ void k_add_rb(R* __restrict__ lam, const R* __restrict__ rb, long V)
+__global__ void k_add_rb(R* __restrict__ lam, const R* rb, long V)
 {
     pdl_wait();
     for (long s = blockIdx.x * (long)blockDim.x + threadIdx.x; s < V; s += (long)gridDim.x * blockDim.x) {
@@ -445,7 +445,7 @@ __global__ void k_add_rb(R* __restrict__ lam, const R* __restrict__ rb, long V)
 // Column blockIdx.x of the block rows of step blockIdx.y (nc rows of the
 // collision's three columns, then nr of k_adj_rho's) summed into
 // part[step * 6 + column].
-__global__ void __launch_bounds__(256) k_sum_grads(const double* __restrict__ rows, int nc, int nr,
+__global__ void __launch_bounds__(256) k_sum_grads(const double* rows, int nc, int nr,
                                                    double* __restrict__ part)
 {
     __shared__ double sh[256];
@@ -466,7 +466,7 @@ __global__ void __launch_bounds__(256) k_sum_grads(const double* __restrict__ ro
 // The steps' sums added to their parameters, the last step first: columns
 // (bulk, shear, ghost, kappa, A, B) go to grad (omega_shear, omega_bulk,
 // omega_ghost, kappa, A, B), the free-energy columns only for the non-ideal fluid.
-__global__ void k_add_grads(const double* __restrict__ part, int n, double* __restrict__ grad, int nonideal)
+__global__ void k_add_grads(const double* part, int n, double* __restrict__ grad, int nonideal)
 {
     pdl_wait();
     const int c = threadIdx.x;

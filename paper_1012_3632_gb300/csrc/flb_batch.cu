@@ -67,8 +67,8 @@ struct Tile {
 // are read anew for each; the thread's eight Philox calls in lock-step 1355).
 template <bool OFF32>
 __global__ void __launch_bounds__(128, 5)
-    k_step_batch(const __grid_constant__ BatchArgs A, const int4* __restrict__ tiles, int ntiles,
-                 const unsigned long long* __restrict__ d_step, unsigned long long* __restrict__ d_next)
+    k_step_batch(const __grid_constant__ BatchArgs A, const int4* tiles, int ntiles,
+                 const unsigned long long* d_step, unsigned long long* __restrict__ d_next)
 {
     using Off = typename std::conditional<OFF32, int, long>::type;
     using L = D3Q19;

@@ -18,7 +18,7 @@ namespace flb {
 // ---------------------------------------------------------------------------
 // Column sums (one block per column, fixed order: deterministic)
 // ---------------------------------------------------------------------------
-__global__ void k_sum_columns(const double* __restrict__ partials, int nrows, int ncol, double* __restrict__ out,
+__global__ void k_sum_columns(const double* partials, int nrows, int ncol, double* __restrict__ out,
                               double add0)
 {
     __shared__ double sh[256];
@@ -63,7 +63,7 @@ cudaError_t sum_lattices(const ModeSums& a, int ncol, double* out, cudaStream_t 
 
 // Step blockIdx.y: its rows are split over gridDim.x blocks; the block that
 // comes last adds their partial sums in block order (deterministic).
-__global__ void __launch_bounds__(256) k_sum_steps(const float4* __restrict__ rows, int nrows, int per,
+__global__ void __launch_bounds__(256) k_sum_steps(const float4* rows, int nrows, int per,
                                                    double* __restrict__ part, unsigned* __restrict__ ticks,
                                                    double* __restrict__ out, double add0)
 {
@@ -592,7 +592,7 @@ constexpr int kRegOccupancy = 512;
 
 template <int L, bool STRIDED, int IN, bool POWER>
 __global__ void __launch_bounds__(kRegThreads<L>, kRegOccupancy / kRegThreads<L>)
-    k_fft_reg(float2* __restrict__ data, const float* __restrict__ real, int es, int s_out, int n_in, int n_lines,
+    k_fft_reg(float2* data, const float* real, int es, int s_out, int n_in, int n_lines,
               const PowerOut pw, const __grid_constant__ WhiteIn white)
 {
     constexpr int B = kRegLines<L>, T = kRegThreads<L>, P = STRIDED ? B : B + 1;
@@ -757,7 +757,7 @@ __global__ void __launch_bounds__(256) k_dft_lines(T* __restrict__ data, const L
 
 // Longer lines: out of place, a root per term.
 template <class T>
-__global__ void k_dft_lines_naive(const T* __restrict__ in, T* __restrict__ out, const LineGeom g, int n_out)
+__global__ void k_dft_lines_naive(const T* in, T* __restrict__ out, const LineGeom g, int n_out)
 {
     using E = decltype(T::x);
     pdl_wait();
@@ -884,7 +884,7 @@ cudaError_t fft3d(float2* data, int X, int Y, int Z, float2* scratch, cudaStream
 // three passes instead of six: 82 -> 35 us with the register transforms.
 template <int L>
 __global__ void __launch_bounds__(kRegThreads<L>, kRegOccupancy / kRegThreads<L>)
-    k_swift_columns(const float2* __restrict__ in, float2* __restrict__ out, const float* __restrict__ chol, int X)
+    k_swift_columns(const float2* in, float2* __restrict__ out, const float* chol, int X)
 {
     constexpr int B = kRegLines<L>, H = B / 2;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -942,7 +942,7 @@ cudaError_t swift_noise_fp32(const PhiloxKeys& key, uint32_t step, uint32_t repl
     return fft_axis(out, work, X, 1, X, Y, (long)X * Y, 1, (long)X * Y, s);
 }
 
-__global__ void k_complex(const float* __restrict__ in, long V, float2* __restrict__ out)
+__global__ void k_complex(const float* in, long V, float2* __restrict__ out)
 {
     pdl_wait();
     for (long s = blockIdx.x * (long)blockDim.x + threadIdx.x; s < V; s += (long)gridDim.x * blockDim.x)
@@ -952,7 +952,7 @@ __global__ void k_complex(const float* __restrict__ in, long V, float2* __restri
 // p = |F|^2 / V (p = 0 at k = 0): acc += p and out = scale acc, or out = p.  The
 // square in the transform's type, the accumulation over snapshots in FP64.
 template <class T>
-__global__ void k_power(const T* __restrict__ d, long V, double* __restrict__ acc, double* __restrict__ out,
+__global__ void k_power(const T* d, long V, double* __restrict__ acc, double* __restrict__ out,
                         double scale)
 {
     using E = decltype(T::x);

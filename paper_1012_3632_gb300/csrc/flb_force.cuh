@@ -95,7 +95,10 @@ __global__ void __launch_bounds__(128, 7) k_force_density(const __grid_constant_
                     lo[i] = F2(v.y, v.z);
                     hi[i] = F2(v.w, A::keep1(r + xe));
                 }
-                if constexpr (STATE)
+            }
+            if constexpr (STATE) {  // after the loads: a store would hold back the loads behind it
+#pragma unroll
+                for (int i = 0; i < L::Q; ++i)
                     *reinterpret_cast<float4*>(P.dst[i] + (XY * z + X * y + x)) =
                         make_float4(lo[i].v.x, lo[i].v.y, hi[i].v.x, hi[i].v.y);
             }
@@ -121,7 +124,10 @@ __global__ void __launch_bounds__(128, 7) k_force_density(const __grid_constant_
                     g[i] = F2(A::plain1(r + xm), A::plain1(r + x));
                 else
                     g[i] = F2(A::plain1(r + x1), A::plain1(r + xe));
-                if constexpr (STATE) {
+            }
+            if constexpr (STATE) {
+#pragma unroll
+                for (int i = 0; i < L::Q; ++i) {
                     S* o = P.dst[i] + (XY * z + X * y + x);
                     if constexpr (GX == 2) {
                         *reinterpret_cast<float2*>(o) = g[i].v;
@@ -163,7 +169,7 @@ __global__ void __launch_bounds__(128, 7) k_force_density(const __grid_constant_
 // thread with its 9 rows).
 template <int GX>
 __global__ void __launch_bounds__(128)
-    k_force_mu(const StepArgs<float> a, const float* __restrict__ rho, float* __restrict__ mu, const Tiling t,
+    k_force_mu(const StepArgs<float> a, const float* rho, float* __restrict__ mu, const Tiling t,
                bool trigger)
 {
     using L = D3Q19;
@@ -231,8 +237,8 @@ __global__ void __launch_bounds__(128)
 // spilled) measured 474 -> 480 us at 256^3.
 template <class S, bool AL, bool TOTAL, bool EARLY, bool LINE>
 __global__ void __launch_bounds__(128, EARLY ? 3 : 4)
-    k_force_collide(const StepArgs<float> a, const __grid_constant__ Planes<S> P, const float* __restrict__ rho,
-                    const float* __restrict__ mu, const Tiling t)
+    k_force_collide(const StepArgs<float> a, const __grid_constant__ Planes<S> P, const float* rho,
+                    const float* mu, const Tiling t)
 {
     using L = D3Q19;
     using A = Packed<S>;
@@ -444,8 +450,8 @@ __global__ void __launch_bounds__(TX* TY / 2)
 // thread, by fewer instructions and no barrier.
 template <class S, bool AL>
 __global__ void __launch_bounds__(128)
-    k_step_swift2(const StepArgs<float> a, const __grid_constant__ Planes<S> P, const float* __restrict__ drho,
-                  const float2* __restrict__ xi, const Tiling t)
+    k_step_swift2(const StepArgs<float> a, const __grid_constant__ Planes<S> P, const float* drho,
+                  const float2* xi, const Tiling t)
 {
     using L = D2Q9;
     using A = Packed<S>;

@@ -24,7 +24,11 @@ namespace flb {
 // Programmatic dependent launch.  A kernel launched with launch_chain may start
 // while the last blocks of the kernel before it on the stream are ending:
 // pdl_wait waits until everything before this kernel is complete and visible
-// and comes before any access to memory.  A kernel triggers its dependent
+// and comes before any access to memory.  The source has to fix that order: loads
+// in inline PTX are asm volatile, which keep their place behind the wait, and a
+// pointer that a kernel reads through is not __restrict__ (data that nothing
+// writes while the kernel runs may be loaded at any point of it, and the kernel
+// before may still run).  A kernel triggers its dependent
 // before its blocks' end only where that one has work that needs no memory, the
 // noise, and both fit the chip (EARLY), and only after its own wait, so that no
 // more than two kernels are under way.  Elsewhere blocks that start while this
@@ -194,7 +198,7 @@ struct Vel<D3Q19> {
 
 // Pull g_i(r - c_i) for all i.
 template <class L, class R, class S>
-__device__ __forceinline__ void pull(const S* __restrict__ src, long V, const Nbhd& nb, R g[L::Q])
+__device__ __forceinline__ void pull(const S* src, long V, const Nbhd& nb, R g[L::Q])
 {
 #pragma unroll
     for (int i = 0; i < L::Q; ++i)
@@ -242,19 +246,19 @@ __device__ __forceinline__ void pull_planes(const Planes<S>& P, const Nbhd& nb, 
 __device__ __forceinline__ float2 ld_stream2(const float* p)
 {
     float2 v;
-    asm("ld.global.L1::no_allocate.L2::256B.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    asm volatile("ld.global.L1::no_allocate.L2::256B.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
     return v;
 }
 __device__ __forceinline__ float ld_stream1(const float* p)
 {
     float v;
-    asm("ld.global.L1::no_allocate.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    asm volatile("ld.global.L1::no_allocate.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
     return v;
 }
 __device__ __forceinline__ float4 ld_keep4(const float* p)
 {
     float4 v;
-    asm("ld.global.L1::evict_last.L2::256B.v4.f32 {%0, %1, %2, %3}, [%4];"
+    asm volatile("ld.global.L1::evict_last.L2::256B.v4.f32 {%0, %1, %2, %3}, [%4];"
         : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
         : "l"(p));
     return v;
@@ -262,7 +266,7 @@ __device__ __forceinline__ float4 ld_keep4(const float* p)
 __device__ __forceinline__ float ld_keep1(const float* p)
 {
     float v;
-    asm("ld.global.L1::evict_last.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    asm volatile("ld.global.L1::evict_last.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
     return v;
 }
 
@@ -291,25 +295,25 @@ struct Packed<__nv_bfloat16> {
     static __device__ __forceinline__ float2 stream2(const B* p)
     {
         uint32_t u;
-        asm("ld.global.L1::no_allocate.L2::256B.b32 %0, [%1];" : "=r"(u) : "l"(p));
+        asm volatile("ld.global.L1::no_allocate.L2::256B.b32 %0, [%1];" : "=r"(u) : "l"(p));
         return make_float2(lo(u), hi(u));
     }
     static __device__ __forceinline__ float stream1(const B* p)
     {
         unsigned short u;
-        asm("ld.global.L1::no_allocate.L2::256B.b16 %0, [%1];" : "=h"(u) : "l"(p));
+        asm volatile("ld.global.L1::no_allocate.L2::256B.b16 %0, [%1];" : "=h"(u) : "l"(p));
         return lo(u);
     }
     static __device__ __forceinline__ float4 keep4(const B* p)
     {
         uint32_t a, b;
-        asm("ld.global.L1::evict_last.L2::256B.v2.b32 {%0, %1}, [%2];" : "=r"(a), "=r"(b) : "l"(p));
+        asm volatile("ld.global.L1::evict_last.L2::256B.v2.b32 {%0, %1}, [%2];" : "=r"(a), "=r"(b) : "l"(p));
         return make_float4(lo(a), hi(a), lo(b), hi(b));
     }
     static __device__ __forceinline__ float keep1(const B* p)
     {
         unsigned short u;
-        asm("ld.global.L1::evict_last.L2::256B.b16 %0, [%1];" : "=h"(u) : "l"(p));
+        asm volatile("ld.global.L1::evict_last.L2::256B.b16 %0, [%1];" : "=h"(u) : "l"(p));
         return lo(u);
     }
     static __device__ __forceinline__ float2 plain2(const B* p)
@@ -351,7 +355,7 @@ constexpr int kSitesThreads = 128;
 
 template <class L, class R, class S>
 __global__ void __launch_bounds__(kSitesThreads)
-    k_density(const S* __restrict__ src, R* __restrict__ drho, int X, int Y, int Z, const Tiling t)
+    k_density(const S* src, R* __restrict__ drho, int X, int Y, int Z, const Tiling t)
 {
     pdl_wait();
     const int3 r = tile_site<1, L::D == 3 ? 2 : 1, false>(t, threadIdx.x);
@@ -378,8 +382,8 @@ __global__ void __launch_bounds__(kSitesThreads)
 // ---------------------------------------------------------------------------
 template <class L, class R, class S, bool FORCE, bool TOTAL, bool SPLIT>
 __global__ void __launch_bounds__(kSitesThreads)
-    k_sites(const StepArgs<R> a, const __grid_constant__ Planes<S> P, const R* __restrict__ drho,
-            const R* __restrict__ mu, const Tiling t)
+    k_sites(const StepArgs<R> a, const __grid_constant__ Planes<S> P, const R* drho,
+            const R* mu, const Tiling t)
 {
     constexpr int PLANES = L::D == 3 && !SPLIT ? 2 : 1, NPAIR = (L::NNC + 1) / 2;
     __shared__ R zs[SPLIT ? 2 * NPAIR : 1][32];
@@ -470,7 +474,7 @@ __global__ void __launch_bounds__(kSitesThreads)
 // (edge sum) - 4 rho (fewer operations on the slow pipe).
 template <class R>
 __global__ void __launch_bounds__(kSitesThreads)
-    k_mu_field(const StepArgs<R> a, const R* __restrict__ drho, R* __restrict__ mu, const Tiling t)
+    k_mu_field(const StepArgs<R> a, const R* drho, R* __restrict__ mu, const Tiling t)
 {
     using L = D3Q19;
     pdl_wait();
@@ -586,8 +590,8 @@ using NoiseField = typename std::conditional<std::is_same<R, double>::value, dou
 
 template <class R, class S, int TX, int TY>
 __global__ void __launch_bounds__(TX* TY)
-    k_step_swift(const StepArgs<R> a, const __grid_constant__ Planes<S> P, const R* __restrict__ drho,
-                 const NoiseField<R>* __restrict__ xi)
+    k_step_swift(const StepArgs<R> a, const __grid_constant__ Planes<S> P, const R* drho,
+                 const NoiseField<R>* xi)
 {
     using L = D2Q9;
     constexpr int RX = TX + 2, RY = TY + 2;

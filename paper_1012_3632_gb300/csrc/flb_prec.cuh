@@ -175,7 +175,7 @@ __global__ void k_set_pop(const double* __restrict__ in, S* __restrict__ dst, do
 // Pre-collision deviations in the storage type, [i][s] (pull of the stored
 // post-collision buffer) and the inverse scatter.
 template <class L, class S>
-__global__ void k_pull_state(const S* __restrict__ src, S* __restrict__ out, int X, int Y, int Z)
+__global__ void k_pull_state(const S* src, S* __restrict__ out, int X, int Y, int Z)
 {
     pdl_wait();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -190,7 +190,7 @@ __global__ void k_pull_state(const S* __restrict__ src, S* __restrict__ out, int
         out[(long)i * V + s] = src[(long)i * V + nb.src(Vel<L>::cx(i), Vel<L>::cy(i), Vel<L>::cz(i))];
 }
 template <class L, class S>
-__global__ void k_push_state(const S* __restrict__ in, S* __restrict__ dst, int X, int Y, int Z)
+__global__ void k_push_state(const S* in, S* __restrict__ dst, int X, int Y, int Z)
 {
     pdl_wait();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -458,7 +458,7 @@ __host__ __device__ constexpr int opposite(int i)
 
 template <class L, class R, class S>
 __global__ void __launch_bounds__(kConsThreads, sizeof(R) == 8 ? 2 : 3)
-    k_cons_partials(const S* __restrict__ src, double* __restrict__ partials, long V)
+    k_cons_partials(const S* src, double* __restrict__ partials, long V)
 {
     pdl_wait();
     constexpr int NP = (L::Q - 1) / 2;
@@ -492,7 +492,7 @@ __global__ void __launch_bounds__(kConsThreads, sizeof(R) == 8 ? 2 : 3)
 
 template <class L, class R, class S, class T>
 __global__ void __launch_bounds__(kSitesThreads)
-    k_mode_field(const S* __restrict__ src, int mode, T* __restrict__ out, int X, int Y, int Z, const Tiling t)
+    k_mode_field(const S* src, int mode, T* __restrict__ out, int X, int Y, int Z, const Tiling t)
 {
     pdl_wait();
     const int3 r = tile_site<1, L::D == 3 ? 2 : 1, false>(t, threadIdx.x);

@@ -47,7 +47,7 @@ __global__ void k_swift_white(PhiloxKeys key, uint32_t step, uint32_t replica, l
 
 // out(k) = conj(Ze'(k) + i Zp'(k)) with (Ze', Zp') = chol(k) (E, P).
 template <class T, class E = decltype(T::x)>
-__global__ void k_swift_colour(const T* __restrict__ Z, const E* __restrict__ chol, int X, int Y, T* __restrict__ out)
+__global__ void k_swift_colour(const T* Z, const E* chol, int X, int Y, T* __restrict__ out)
 {
     pdl_wait();
     const long V = (long)X * Y;
