@@ -61,10 +61,18 @@ cudaError_t sum_lattices(const ModeSums& a, int ncol, double* out, cudaStream_t 
     return launch_chain(k_sum_lattices, dim3(ncol, a.n), dim3(128), s, a, ncol, out);
 }
 
+// A load of what other blocks of this launch wrote (not from L1).
+__device__ __forceinline__ double ld_relaxed(const double* p)
+{
+    double v;
+    asm volatile("ld.relaxed.gpu.global.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+    return v;
+}
+
 // Step blockIdx.y: its rows are split over gridDim.x blocks; the block that
 // comes last adds their partial sums in block order (deterministic).
 __global__ void __launch_bounds__(256) k_sum_steps(const float4* rows, int nrows, int per,
-                                                   double* __restrict__ part, unsigned* __restrict__ ticks,
+                                                   double* part, unsigned* ticks,
                                                    double* __restrict__ out, double add0)
 {
     __shared__ double red[8][4];
@@ -99,9 +107,10 @@ __global__ void __launch_bounds__(256) k_sum_steps(const float4* rows, int nrows
         if (lane == 0)
             asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(old) : "l"(ticks + step) : "memory");
         if (__shfl_sync(0xffffffffu, old, 0) != (unsigned)nb - 1) return;
+        __syncwarp();  // orders what lane 0 acquired before the loads of the others, a shuffle does not
         if (lane == 0) ticks[step] = 0u;
         acc = 0.0;
-        for (int k = lane >> 2; k < nb; k += 8) acc += __ldcg(p + 4 * k + (lane & 3));
+        for (int k = lane >> 2; k < nb; k += 8) acc += ld_relaxed(p + 4 * k + (lane & 3));
         for (int o = 16; o > 2; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
     }
     if (lane < 4) out[4 * step + lane] = lane == 0 ? acc + add0 : acc;

@@ -60,3 +60,12 @@ def test_inline_ptx_that_touches_memory_is_volatile(path):
     for m in re.finditer(r"\basm\s*(volatile)?\s*\(\s*\"([a-z_]+)\.", _source(path)):
         if m.group(2) in ("ld", "st", "atom", "red", "prefetch", "griddepcontrol", "fence", "membar"):
             assert m.group(1), _source(path)[m.start():m.start() + 90]
+
+
+def test_sums_of_other_blocks_are_read_after_the_warp_is_in_order():
+    """Lane 0 acquires the other blocks' sums; only a __syncwarp orders that
+    before the loads of the other lanes, which have to be loads that see them."""
+    body = {name: body for name, _, body in _kernels()}["k_sum_steps"]
+    after = body[body.index("atom.acq_rel"):]
+    assert "__ldcg" not in after
+    assert after.index("__shfl_sync") < after.index("__syncwarp()") < after.index("ld_relaxed(")
