@@ -224,11 +224,17 @@ int build_tiles(flb_batch* b)
             for (int j = 0; j < ny; ++j)
                 for (int i = 0; i < nx; ++i) t.push_back(make_int4(r, i, j, k));
     }
+    // the list in use stays, with the parameters that go with it, unless the new one is there
+    int4* d_t = nullptr;
+    BCUDA(cudaMalloc(&d_t, t.size() * sizeof(int4)));
+    const cudaError_t e = cudaMemcpy(d_t, t.data(), t.size() * sizeof(int4), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) {
+        cudaFree(d_t);
+        return bfail(FLB_ECUDA, std::string("work list: ") + cudaGetErrorString(e));
+    }
     if (b->tiles) cudaFree(b->tiles);
-    b->tiles = nullptr;
+    b->tiles = d_t;
     b->ntiles = (int)t.size();
-    BCUDA(cudaMalloc(&b->tiles, t.size() * sizeof(int4)));
-    BCUDA(cudaMemcpy(b->tiles, t.data(), t.size() * sizeof(int4), cudaMemcpyHostToDevice));
     for (int p = 0; p < 2; ++p) {
         BatchArgs& A = b->args[p];
         std::memset(&A, 0, sizeof(A));
@@ -286,6 +292,19 @@ int make_graph(flb_batch* b, int p)
     cudaGraphDestroy(g);
     if (e != cudaSuccess) return bfail(FLB_ECUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
     return FLB_OK;
+}
+
+// n elements, once: each buffer for itself, so that one that could not be had is
+// asked for again by the next call.
+template <class T>
+int alloc_once(T** p, size_t n)
+{
+    if (*p) return FLB_OK;
+    const cudaError_t e = cudaMalloc(p, n * sizeof(T));
+    if (e == cudaSuccess) return FLB_OK;
+    *p = nullptr;
+    return bfail(e == cudaErrorMemoryAllocation ? FLB_ENOMEM : FLB_ECUDA,
+                 std::string("cudaMalloc(") + std::to_string(n * sizeof(T)) + "): " + cudaGetErrorString(e));
 }
 
 const float* rep_src(const flb_batch* b, int r) { return b->buf[b->cur] + b->off[r]; }
@@ -503,10 +522,8 @@ int flb_batch_mode_variance(flb_batch* b, double* out)
     a.n = 0;
     a.lat[0].first = 0;
     for (int r = 0; r < b->n; ++r) flb::mode_blocks(a, rep_src(b, r), b->m[r].X, b->m[r].Y, b->m[r].Z, 8);
-    if (!b->partials) {
-        BCUDA(cudaMalloc(&b->partials, (size_t)a.lat[a.n].first * 38 * sizeof(double)));
-        BCUDA(cudaMalloc(&b->red, (size_t)b->n * 38 * sizeof(double)));
-    }
+    if (int rc = alloc_once(&b->partials, (size_t)a.lat[a.n].first * 38)) return rc;
+    if (int rc = alloc_once(&b->red, (size_t)b->n * 38)) return rc;
     a.rows = b->partials;
     b->mv_count += 1;
     BCUDA(ops.mode_sums(a, 19, 8, b->stream));
@@ -533,17 +550,15 @@ int flb_batch_structure_factor(flb_batch* b, int replica, double* S, int mode, i
     Dev guard(b->device);
     const flb::PrecOps& ops = flb::ops_fp32();
     const HostModel& m = b->m[replica];
-    if (!b->fft) {
-        long vmax = 0;
-        for (auto& mm : b->m) vmax = std::max(vmax, mm.V);
-        BCUDA(cudaMalloc(&b->fft, (vmax + 1) * sizeof(double2)));
-        BCUDA(cudaMalloc(&b->fft_scratch, vmax * sizeof(double2)));
-        BCUDA(cudaMalloc(&b->sk_tmp, vmax * sizeof(double)));
-    }
+    long vmax = 0;
+    for (auto& mm : b->m) vmax = std::max(vmax, mm.V);
+    if (int rc = alloc_once(&b->fft, vmax + 1)) return rc;
+    if (int rc = alloc_once(&b->fft_scratch, vmax)) return rc;
+    if (int rc = alloc_once(&b->sk_tmp, vmax)) return rc;
     double* target = nullptr;
     if (accumulate) {
         auto& slot = b->sk_acc[{replica, mode}];
-        if (!slot.first) BCUDA(cudaMalloc(&slot.first, m.V * sizeof(double)));
+        if (int rc = alloc_once(&slot.first, m.V)) return rc;
         if (slot.second == 0) BCUDA(cudaMemsetAsync(slot.first, 0, m.V * sizeof(double), b->stream));
         target = slot.first;
         slot.second += 1;
