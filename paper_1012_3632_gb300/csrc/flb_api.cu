@@ -483,6 +483,51 @@ int flb_init(flb_ctx* c, const double* rho, const double* u, int thermal_init)
     return flb_reset_accumulators(c);
 }
 
+// Sums of states that the coming steps start from, formed step by step and added
+// up by one launch per batch of kmax: the partial rows wait in the context's
+// partial-sum buffer until flush().  Whatever else writes to that buffer (a check
+// of the totals) has to flush first.
+struct StepSums {
+    flb_ctx* c;
+    double* out;  // 4 doubles per step, of the first state that waits
+    int nrow;     // warp rows of the step's own density pass, or 0: the reduction before the step
+    int kmax;
+    int n = 0;    // states that wait
+
+    StepSums(flb_ctx* ctx, double* dev_sums)
+        : c(ctx), out(dev_sums), nrow(dev_sums ? ctx->ops->step_row_count(ctx->m) : 0),
+          kmax(nrow > 0 ? step_rows_capacity(ctx, nrow)
+                        : (int)std::min<size_t>(16, partial_bytes(ctx) / (32 * (size_t)flb::cons_rows(ctx->m.V))))
+    {
+    }
+    // where the density pass puts the next state's rows
+    float4* rows() const { return (float4*)(c->partials + 4 * (size_t)flb::kSumBlocksMax * kmax) + (size_t)n * nrow; }
+    // the reduction of a state
+    cudaError_t reduce(const void* src)
+    {
+        return c->ops->cons_partials(c->m, src, c->partials + 4 * (size_t)flb::cons_rows(c->m.V) * n, c->stream);
+    }
+    // one state more waits; `last`: no other joins it
+    cudaError_t push(bool last)
+    {
+        ++n;
+        return n == kmax || last ? flush() : cudaSuccess;
+    }
+    cudaError_t flush()
+    {
+        if (n == 0) return cudaSuccess;
+        const double m0 = c->m.rho0 * (double)c->m.V;
+        const int k = n;
+        double* to = out;
+        out += 4 * (size_t)n;
+        n = 0;
+        if (nrow > 0)
+            return flb::sum_steps((const float4*)(c->partials + 4 * (size_t)flb::kSumBlocksMax * kmax), nrow, k,
+                                  c->partials, ticks(c), to, m0, c->stream);
+        return flb::sum_columns(c->partials, flb::cons_rows(c->m.V), 4, to, c->stream, m0, k);
+    }
+};
+
 // The time steps of flb_step; with dev_sums (device, 4 doubles per step) also
 // the sums of the state each step starts from: the step kernel's own partial
 // sums where it provides them, else the conservation reduction before the step
@@ -490,14 +535,11 @@ int flb_init(flb_ctx* c, const double* rho, const double* u, int thermal_init)
 // with states (device, pop_bytes per step) each state a step starts from.
 static int step_impl(flb_ctx* c, int nsteps, double* dev_sums, char* states = nullptr)
 {
-    const double m0 = c->m.rho0 * (double)c->m.V;
-    const int nrow = dev_sums ? c->ops->step_row_count(c->m) : 0;
-    const int kmax = nrow > 0   ? step_rows_capacity(c, nrow)
-                     : dev_sums ? (int)std::min<size_t>(16, partial_bytes(c) / (32 * (size_t)flb::cons_rows(c->m.V)))
-                                : 1;
+    StepSums sums(c, dev_sums);
     for (int t = 0; t < nsteps; ++t) {
         const void* src = c->buf[c->cur];
         void* dst = c->buf[c->cur ^ 1];
+        const bool check = c->check_every > 0 && (c->step + 1) % (uint64_t)c->check_every == 0;
         size_t slot = 0;
         int rc;
         if (c->ops->step_needs_density(c->m)) {
@@ -509,33 +551,23 @@ static int step_impl(flb_ctx* c, int nsteps, double* dev_sums, char* states = nu
             if ((rc = timer_end(c, slot))) return rc;
         }
         if ((rc = timer_begin(c, 1, &slot))) return rc;
-        cudaError_t se;
-        if (dev_sums && nrow > 0) {
-            // the steps' warp rows side by side in the partial-sum buffer, summed
-            // together once it is full
-            float4* rows = (float4*)(c->partials + 4 * (size_t)flb::kSumBlocksMax * kmax);
-            se = c->ops->step_rows(c->m, c->step, src, dst, c->drho, rows + (size_t)(t % kmax) * nrow, c->stream);
-            if (se == cudaSuccess && (t % kmax == kmax - 1 || t == nsteps - 1))
-                se = flb::sum_steps(rows, nrow, t % kmax + 1, c->partials, ticks(c),
-                                    dev_sums + 4 * (size_t)(t - t % kmax), m0, c->stream);
+        if (dev_sums && sums.nrow > 0) {
+            FLB_CUDA(c->ops->step_rows(c->m, c->step, src, dst, c->drho, sums.rows(), c->stream));
+            FLB_CUDA(sums.push(check || t == nsteps - 1));
         } else if (dev_sums) {
-            // this step kernel has no partial sums: reduce the state first, the
-            // rows of kmax states (4 of the buffer's 2 Q columns each) together
-            const int rows = flb::cons_rows(c->m.V), k = t % kmax;
-            FLB_CUDA(c->ops->cons_partials(c->m, src, c->partials + 4 * (size_t)rows * k, c->stream));
-            if (k == kmax - 1 || t == nsteps - 1)
-                FLB_CUDA(flb::sum_columns(c->partials, rows, 4, dev_sums + 4 * (size_t)(t - k), c->stream, m0, k + 1));
-            se = c->ops->step(c->m, c->step, src, dst, c->drho, c->stream);
+            FLB_CUDA(sums.reduce(src));
+            FLB_CUDA(sums.push(check || t == nsteps - 1));
+            FLB_CUDA(c->ops->step(c->m, c->step, src, dst, c->drho, c->stream));
         } else if (states) {
-            se = c->ops->step_state(c->m, c->step, src, dst, c->drho, states + (size_t)t * c->pop_bytes(), c->stream);
+            FLB_CUDA(c->ops->step_state(c->m, c->step, src, dst, c->drho, states + (size_t)t * c->pop_bytes(),
+                                        c->stream));
         } else {
-            se = c->ops->step(c->m, c->step, src, dst, c->drho, c->stream);
+            FLB_CUDA(c->ops->step(c->m, c->step, src, dst, c->drho, c->stream));
         }
-        FLB_CUDA(se);
         if ((rc = timer_end(c, slot))) return rc;
         c->cur ^= 1;
         c->step += 1;
-        if (c->check_every > 0 && c->step % (uint64_t)c->check_every == 0) {
+        if (check) {
             double s[4];
             if ((rc = timer_begin(c, 2, &slot))) return rc;
             rc = conservation(c, s);
