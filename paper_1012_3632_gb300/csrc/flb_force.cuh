@@ -58,9 +58,11 @@ __device__ __forceinline__ void load_row(const float* p, int x, int x1, int xm, 
 // least 7 blocks per SM: the sums would take 88 registers and with them the
 // warps that hide the loads (a step with sums 716 us, at 6 blocks 727, 8: 740).
 // STATE: the pulled deviations go to P.dst as well, the states that the adjoint
-// keeps (FP32; 64^3 14.7 us, without them 8.3 and a pull of their own 9.5).
+// keeps (FP32; 64^3 14.7 us, without them 8.3 and a pull of their own 9.5), at 5
+// blocks per SM: they are held until the last load (20 steps of 64^3, forward and
+// back, 1000 -> 943 us).
 template <class S, int GX, bool SUMS, bool STATE = false>
-__global__ void __launch_bounds__(128, 7) k_force_density(const __grid_constant__ Planes<S> P, float* __restrict__ rho,
+__global__ void __launch_bounds__(128, STATE ? 5 : 7) k_force_density(const __grid_constant__ Planes<S> P, float* __restrict__ rho,
                                                        float* __restrict__ rows, int X, int Y, int Z, const Tiling t)
 {
     using L = D3Q19;
