@@ -1,6 +1,6 @@
 // flb_internal.h -- host-side interface between the C ABI (flb_api.cu) and the
 // precision-specific kernel instantiations (flb_fp64.cu, flb_fp32.cu,
-// flb_bf16.cu) and the precision-independent kernels (flb_fft.cu).
+// flb_bf16.cu) and the precision-independent kernels (flb_fft.cu, flb_sums.cu).
 #pragma once
 
 #include <cstdint>
@@ -74,7 +74,7 @@ inline int mode_blocks(ModeSums& a, const void* src, int X, int Y, int Z, int wa
     a.lat[++a.n].first = q.first + (int)nb;
     return (int)nb;
 }
-// Column sums of each lattice's rows: out[r * ncol + c] (flb_fft.cu).
+// Column sums of each lattice's rows: out[r * ncol + c] (flb_sums.cu).
 cudaError_t sum_lattices(const ModeSums& a, int ncol, double* out, cudaStream_t s);
 
 // Kernels whose code depends on the compute/storage type.  Pointers are device
@@ -150,7 +150,7 @@ cudaError_t launch_chain(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream
 
 // Deterministic column sums of k arrays of nrows rows, one after another:
 // out[i*ncol + c] = sum_r partials[(i*nrows + r)*ncol + c], plus add0 on the
-// columns 0 (flb_fft.cu).
+// columns 0 (flb_sums.cu).
 cudaError_t sum_columns(const double* partials, int nrows, int ncol, double* out, cudaStream_t s,
                         double add0 = 0.0, int k = 1);
 
@@ -163,7 +163,7 @@ inline int cons_rows(long V)
     return (int)(b < kConsBlocksMax ? b : kConsBlocksMax);
 }
 
-// Sums of k steps' warp rows (flb_fft.cu): rows holds k times nrows float4 rows
+// Sums of k steps' warp rows (flb_sums.cu): rows holds k times nrows float4 rows
 // (mass deviation and momentum); out[4 i ..] receives the sums of step i's, the
 // mass with add0.  part: kSumBlocksMax k doubles x 4, ticks: k counters that are
 // zero between launches.

@@ -1,0 +1,45 @@
+"""The first call of a kind in a process: it loads the code that goes with it, and
+nothing that takes longer than the call is worth.  Each kind in a process of its
+own, the faster of two (a loaded host), as milliseconds of wall time."""
+import os
+import subprocess
+import sys
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+PROGRAM = """
+import time
+import numpy as np
+from paper_1012_3632_gb300 import MODE_VAR, Batch, Context
+fe = dict(A=-0.01, B=0.1, rho_c=1.0, kappa=0.02)
+%s
+c.%s
+c.synchronize()
+t = time.perf_counter()
+c.%s
+c.synchronize()
+print(1e3 * (time.perf_counter() - t))
+"""
+FORCE = "c = Context(19, (48, 48, 48), 1.0, kT=1e-6, free_energy=fe)"
+IDEAL = "c = Context(19, (48, 48, 48), 1.0, kT=1e-6)"
+BATCH = "c = Batch([(32, 32, 32), (16, 18, 20)], [1.0, 1.0], [1e-5, 1e-5], [1, 2])"
+
+# what has to be loaded is well under a megabyte: about 0.3 ms, a few with a slow host
+LIMIT_MS = 5.0
+
+
+@pytest.mark.parametrize("make,before,call", [
+    (IDEAL, "step(1)", "conservation()"), (FORCE, "step(1)", "conservation()"), (FORCE, "step(1)", "step_sums(2)"),
+    (IDEAL, "step(1)", "moments(MODE_VAR)"), (BATCH, "step(1)", "mode_variance()"),
+], ids=["conservation", "conservation_force", "step_sums", "mode_var", "batch_var"])
+def test_first_call_is_not_held_up(make, before, call):
+    best = float("inf")
+    for _ in range(2):
+        r = subprocess.run([sys.executable, "-c", PROGRAM % (make, before, call)], capture_output=True, text=True,
+                           timeout=300, cwd=ROOT)
+        assert r.returncode == 0, r.stderr
+        best = min(best, float(r.stdout.split()[-1]))
+    assert best < LIMIT_MS, best
