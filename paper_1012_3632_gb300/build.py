@@ -18,7 +18,10 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libflb.so")
 SOURCES = ["flb_api.cu", "flb_fp64.cu", "flb_fp32.cu", "flb_bf16.cu", "flb_fft.cu", "flb_sums.cu", "flb_noalloc.cu", "flb_batch.cu", "flb_adjoint.cu", "flb_capillary.cu", "flb_swift.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2"]
+# --no-compress: nvcc compresses a translation unit's device code once it is large, and
+# the driver unpacks it when the first of its kernels is used (the transforms: 14 ms
+# against 2)
+FLAGS = ["-O3", "-std=c++17", "-lineinfo", "--no-compress", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2"]
 
 
 def nvcc() -> str:

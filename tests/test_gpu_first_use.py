@@ -25,16 +25,21 @@ print(1e3 * (time.perf_counter() - t))
 """
 FORCE = "c = Context(19, (48, 48, 48), 1.0, kT=1e-6, free_energy=fe)"
 IDEAL = "c = Context(19, (48, 48, 48), 1.0, kT=1e-6)"
+SWIFT = ("c = Context(9, (100, 64), 1.0, kT=1e-7, "
+         "free_energy=dict(A=-0.025, B=0.4, rho_c=0.75, kappa=0.08, total=True, model=1))")
 BATCH = "c = Batch([(32, 32, 32), (16, 18, 20)], [1.0, 1.0], [1e-5, 1e-5], [1, 2])"
 
-# what has to be loaded is well under a megabyte: about 0.3 ms, a few with a slow host
+# what has to be loaded is a few megabytes at most: 0.2 to 1.2 ms, more with a slow host
 LIMIT_MS = 5.0
 
 
 @pytest.mark.parametrize("make,before,call", [
     (IDEAL, "step(1)", "conservation()"), (FORCE, "step(1)", "conservation()"), (FORCE, "step(1)", "step_sums(2)"),
     (IDEAL, "step(1)", "moments(MODE_VAR)"), (BATCH, "step(1)", "mode_variance()"),
-], ids=["conservation", "conservation_force", "step_sums", "mode_var", "batch_var"])
+    (IDEAL, "step(1)", "structure_factor(0)"), (BATCH, "step(1)", "structure_factor(0, 0)"),
+    (SWIFT, "init()", "step(1)"),
+], ids=["conservation", "conservation_force", "step_sums", "mode_var", "batch_var", "spectrum", "batch_spectrum",
+        "coloured_noise"])
 def test_first_call_is_not_held_up(make, before, call):
     best = float("inf")
     for _ in range(2):
