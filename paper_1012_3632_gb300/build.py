@@ -17,6 +17,8 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libflb.so")
 SOURCES = ["flb_api.cu", "flb_fp64.cu", "flb_fp32.cu", "flb_bf16.cu", "flb_fft.cu", "flb_sums.cu", "flb_noalloc.cu", "flb_batch.cu", "flb_adjoint.cu", "flb_capillary.cu", "flb_swift.cu"]
+# compiled once per part (FLB_REG_PART), a share of the transform lengths each
+REG_SOURCE, REG_PARTS = "flb_fft_reg.cu", 12
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # --no-compress: nvcc compresses a translation unit's device code once it is large, and
 # the driver unpacks it when the first of its kernels is used (the transforms: 14 ms
@@ -50,16 +52,20 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) 
     extra = ["-Xptxas", "-v"] if ptxas_info else []
     extra += os.environ.get("FLB_NVCC_FLAGS", "").split()
 
-    def compile_one(src):
-        obj = os.path.join(BUILD, os.path.splitext(src)[0] + ".o")
-        cmd = [cc, *ARCH, *FLAGS, *extra, "-c", os.path.join(CSRC, src), "-o", obj]
+    units = [(f"{os.path.splitext(REG_SOURCE)[0]}{k}.o", REG_SOURCE, [f"-DFLB_REG_PART={k}"]) for k in range(REG_PARTS)]
+    units += [(os.path.splitext(src)[0] + ".o", src, []) for src in SOURCES]
+
+    def compile_one(unit):
+        name, src, defs = unit
+        obj = os.path.join(BUILD, name)
+        cmd = [cc, *ARCH, *FLAGS, *extra, *defs, "-c", os.path.join(CSRC, src), "-o", obj]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"nvcc failed for {src}:\n{r.stderr}")
         return obj, r.stderr
 
-    with cf.ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
-        results = list(ex.map(compile_one, SOURCES))
+    with cf.ThreadPoolExecutor(max_workers=max(len(SOURCES), os.cpu_count() or 1)) as ex:
+        results = list(ex.map(compile_one, units))
     if verbose or ptxas_info:
         for _, err in results:
             if err:

@@ -11,6 +11,7 @@
 
 #include "flb_internal.h"
 #include "flb_kernels.cuh"
+#include "flb_fft_reg.cuh"
 #include "flb_swift.cuh"
 
 namespace flb {
@@ -48,27 +49,6 @@ static bool make_plan(int L, FftPlan& p)
     }
     return n == 1 && p.nrad <= 32;
 }
-
-// Complex arithmetic on double2 (FP64 transforms) and float2 (FP32 transforms).
-template <class T>
-__device__ __forceinline__ T cmul(T a, T b)
-{
-    return T{a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x};
-}
-template <class T>
-__device__ __forceinline__ T cadd(T a, T b)
-{
-    return T{a.x + b.x, a.y + b.y};
-}
-template <class T>
-__device__ __forceinline__ T csub(T a, T b)
-{
-    return T{a.x - b.x, a.y - b.y};
-}
-
-// |a|^2 with the rounding fixed: the fused and the separate power spectrum agree
-// to the bit.
-__device__ __forceinline__ float norm2(float2 a) { return fmaf(a.y, a.y, __fmul_rn(a.x, a.x)); }
 
 // Line geometry: line (i0, i1) starts at i0*s_in + i1*s_out, elements es apart.
 struct LineGeom {
@@ -170,20 +150,11 @@ __device__ __forceinline__ void butterfly_p2(const T* __restrict__ in, T* __rest
     for (int r = 0; r < R; ++r) out[pad16(base + (r << lgNs))] = y[r];
 }
 
-// Twiddle table tw[m] = exp(-2 pi i m / L), m < L, built by every block of
-// k_fft_lines in shared memory.  FP32 transforms: one FP32 sincospi per entry.
-// FP64 transforms: m = a S + b with S = ceil(sqrt(L)), tw[m] = coarse[a] *
-// fine[b] with coarse[a] = exp(-2 pi i a S / L), fine[b] = exp(-2 pi i b / L):
-// about 2 sqrt(L) FP64 sincospi per block instead of L (FP64 is slow on this
-// part), each entry within a few ulp.  scratch: >= S + ceil(L / S) entries.
-__device__ __forceinline__ void fill_twiddles(float2* tw, int L, float2*)
-{
-    for (int m = threadIdx.x; m < L; m += blockDim.x) {
-        float s, c;
-        sincospif(-2.0f * ((float)m / (float)L), &s, &c);
-        tw[m] = make_float2(c, s);
-    }
-}
+// Twiddle table of FP64 transforms (those of FP32: flb_fft_reg.cuh): m = a S + b
+// with S = ceil(sqrt(L)), tw[m] = coarse[a] * fine[b] with
+// coarse[a] = exp(-2 pi i a S / L), fine[b] = exp(-2 pi i b / L): about 2 sqrt(L)
+// FP64 sincospi per block instead of L (FP64 is slow on this part), each entry
+// within a few ulp.  scratch: >= S + ceil(L / S) entries.
 __device__ __forceinline__ void fill_twiddles(double2* tw, int L, double2* scratch)
 {
     int S = 1;
@@ -304,298 +275,45 @@ __global__ void __launch_bounds__(kFftThreads) k_fft_lines(T* __restrict__ data,
     }
 }
 
-// ---------------------------------------------------------------------------
-// FP32 lines of the common lengths: two radix passes at a time in registers
-// ---------------------------------------------------------------------------
-// Bound by latency and shared-memory passes: the radix-by-radix kernel above
-// crosses shared memory once per radix and fetches a 2048-element block per
-// 256 threads.  Here a thread takes Ra Rb elements q + (r0 Rb + r') L / (Ra Rb)
-// of a line, which the radix-Ra butterflies j = q + r' L / (Ra Rb) and the
-// radix-Rb butterflies of the next pass exchange among themselves alone, so that
-// a length of up to 256 crosses shared memory once; strided lines load and
-// store straight from registers, blocks keep their twiddle table for several
-// groups of lines.  The arithmetic of every butterfly is that of the passes
-// above.  Structure factor of a 128^3 state 113 -> 59 us, 96^3 82 -> 22, 256^3
-// 703 -> 410 (density field and power spectrum included).
-template <int L>
-struct RegPlan {
-    static constexpr bool ok = false;
-};
-#define FLB_REG_PLAN(LEN, A0, B0, A1, B1, A2, B2)                                                \
-    template <>                                                                                  \
-    struct RegPlan<LEN> {                                                                        \
-        static constexpr bool ok = true;                                                         \
-        static constexpr int ra[3] = {A0, A1, A2}, rb[3] = {B0, B1, B2}, n = A2 > 1 ? 3 : 2;      \
-    }
-FLB_REG_PLAN(32, 4, 4, 2, 1, 1, 1);
-FLB_REG_PLAN(48, 4, 4, 3, 1, 1, 1);
-FLB_REG_PLAN(64, 4, 4, 4, 1, 1, 1);
-FLB_REG_PLAN(96, 4, 4, 2, 3, 1, 1);
-FLB_REG_PLAN(128, 4, 4, 4, 2, 1, 1);
-FLB_REG_PLAN(135, 3, 3, 3, 5, 1, 1);
-FLB_REG_PLAN(192, 4, 4, 4, 3, 1, 1);
-FLB_REG_PLAN(200, 4, 2, 5, 5, 1, 1);
-FLB_REG_PLAN(225, 3, 3, 5, 5, 1, 1);
-FLB_REG_PLAN(243, 3, 3, 3, 3, 3, 1);
-FLB_REG_PLAN(256, 4, 4, 4, 4, 1, 1);
-FLB_REG_PLAN(360, 4, 2, 3, 3, 5, 1);
-FLB_REG_PLAN(384, 4, 4, 4, 2, 3, 1);
-FLB_REG_PLAN(400, 4, 4, 5, 5, 1, 1);
-FLB_REG_PLAN(512, 4, 4, 4, 4, 2, 1);
-FLB_REG_PLAN(1024, 4, 4, 4, 4, 4, 1);
-#undef FLB_REG_PLAN
-
-// The R-point DFT of butterfly(), on registers.
-template <int R, class T>
-__device__ __forceinline__ void dft(const T (&v)[R], T (&y)[R], const T* __restrict__ tw, int L)
+// The kernels of a length with a plan in registers (flb_fft_reg.cuh), or NULL.
+static const RegKernels* reg_kernels(int L)
 {
-    using E = decltype(T::x);
-    if constexpr (R == 1) {
-        y[0] = v[0];
-    } else if constexpr (R == 2) {
-        y[0] = cadd(v[0], v[1]);
-        y[1] = csub(v[0], v[1]);
-    } else if constexpr (R == 4) {
-        const T a = cadd(v[0], v[2]), b = csub(v[0], v[2]);
-        const T c = cadd(v[1], v[3]), d = csub(v[1], v[3]);
-        y[0] = cadd(a, c);
-        y[2] = csub(a, c);
-        y[1] = T{b.x + d.y, b.y - d.x};  // b - i d
-        y[3] = T{b.x - d.y, b.y + d.x};  // b + i d
-    } else if constexpr (R == 3) {
-        const E h = E(0.86602540378443864676);  // sqrt(3)/2
-        const T t = cadd(v[1], v[2]), u = csub(v[1], v[2]);
-        y[0] = cadd(v[0], t);
-        const T m = T{v[0].x - E(0.5) * t.x, v[0].y - E(0.5) * t.y};
-        y[1] = T{m.x + h * u.y, m.y - h * u.x};  // m - i h u
-        y[2] = T{m.x - h * u.y, m.y + h * u.x};  // m + i h u
-    } else {  // R == 5
-        const int f = L / 5;
-#pragma unroll
-        for (int q = 0; q < 5; ++q) {
-            T acc = v[0];
-#pragma unroll
-            for (int r = 1; r < 5; ++r) acc = cadd(acc, cmul(v[r], tw[((q * r) % 5) * f]));
-            y[q] = acc;
-        }
-    }
-}
-
-// Passes Ra and Rb (N0: product of the radices before) of the items w, w + TL,
-// .. of a line: ld(i) its element i, st(i, v, n) the result, the thread's n-th.
-// pre(i, n) announces a result before the butterflies (what st adds to it is
-// loaded meanwhile).  sync stands between the last load and the first store.
-template <int L, int N0, int Ra, int Rb, class T, class LD, class PR, class ST, class SY>
-__device__ __forceinline__ void two_passes(const T* __restrict__ tw, int w, LD&& ld, PR&& pre, ST&& st, SY&& sync)
-{
-    constexpr int E = Ra * Rb, S = L / E, TL = (L + 15) / 16, IT = (S + TL - 1) / TL;
-    T v[IT][E];
-#pragma unroll
-    for (int it = 0; it < IT; ++it) {
-        const int q = w + it * TL;
-        if (S % TL == 0 || q < S)
-#pragma unroll
-            for (int e = 0; e < E; ++e) v[it][e] = ld(q + e * S);
-    }
-#pragma unroll
-    for (int it = 0; it < IT; ++it) {
-        const int q = w + it * TL, base = (q / N0) * (N0 * E) + q % N0;
-        if (S % TL == 0 || q < S)
-#pragma unroll
-            for (int e = 0; e < E; ++e) pre(base + N0 * e, it * E + e);
-    }
-    sync();
-#pragma unroll
-    for (int it = 0; it < IT; ++it) {
-        const int q = w + it * TL;
-        if (S % TL != 0 && q >= S) continue;
-        const int k = q % N0, A = q / N0;
-        T y[Rb][Ra];
-#pragma unroll
-        for (int rb = 0; rb < Rb; ++rb) {
-            T x[Ra];
-            x[0] = v[it][rb];
-#pragma unroll
-            for (int r = 1; r < Ra; ++r) {
-                x[r] = v[it][r * Rb + rb];
-                if (N0 > 1) x[r] = cmul(x[r], tw[r * k * (L / (N0 * Ra))]);
-            }
-            dft<Ra>(x, y[rb], tw, L);
-        }
-        const int base = A * (N0 * E) + k;
-#pragma unroll
-        for (int r = 0; r < Ra; ++r) {
-            T x[Rb], z[Rb];
-            x[0] = y[0][r];
-#pragma unroll
-            for (int rb = 1; rb < Rb; ++rb) x[rb] = cmul(y[rb][r], tw[rb * (k + r * N0) * (L / (N0 * E))]);
-            dft<Rb>(x, z, tw, L);
-#pragma unroll
-            for (int rb = 0; rb < Rb; ++rb) st(base + N0 * (r + rb * Ra), z[rb], it * E + r + rb * Ra);
-        }
-    }
-}
-
-// Results of a thread: the most over the passes.
-template <int L>
-constexpr int kRegSlots = 32;
-
-// Lines through shared memory: L elements of B lines at pitch P (element-major).
-template <int L, class T, class LD, class PR, class ST>
-__device__ __forceinline__ void reg_fft(const T* tw, T* sm, int P, int w, int l, LD&& ld, PR&& pre, ST&& st)
-{
-    using Pl = RegPlan<L>;
-    auto rd = [&](int i) { return sm[i * P + l]; };
-    auto wr = [&](int i, T v, int) { sm[i * P + l] = v; };
-    auto none = [](int, int) {};
-    auto sync = [] { __syncthreads(); };
-    constexpr int N1 = Pl::ra[0] * Pl::rb[0], N2 = N1 * Pl::ra[1] * Pl::rb[1];
-    two_passes<L, 1, Pl::ra[0], Pl::rb[0]>(tw, w, ld, none, wr, sync);  // sync: ld may read sm
-    __syncthreads();
-    if constexpr (Pl::n == 2) {
-        two_passes<L, N1, Pl::ra[1], Pl::rb[1]>(tw, w, rd, pre, st, sync);  // sync: st may write sm
-    } else {
-        two_passes<L, N1, Pl::ra[1], Pl::rb[1]>(tw, w, rd, none, wr, sync);
-        __syncthreads();
-        two_passes<L, N2, Pl::ra[2], Pl::rb[2]>(tw, w, rd, pre, st, sync);
-    }
-}
-
-// Lines per block: 128 threads or a little more, rows of 32 bytes or wider.
-template <int L>
-constexpr int kRegLines = L <= 32 ? 64 : L <= 64 ? 32 : L <= 192 ? 16 : L <= 512 ? 8 : 4;
-template <int L>
-constexpr int kRegThreads = kRegLines<L> * ((L + 15) / 16);
-
-// What the last pass of a strided axis leaves: the transform in place, or its
-// power spectrum.
-struct PowerOut {
-    double* acc;   // += p (or NULL)
-    double* out;   // = p, or with acc = scale * (acc + p) (or NULL)
-    double scale;
-    float inv;     // 1 / V
-};
-
-// Input of the rows: complex numbers in place, real numbers, or the white e/eps
-// normals of the modified equilibrium's noise.
-enum { kInComplex, kInReal, kInWhite };
-struct WhiteIn {
-    PhiloxKeys key;
-    uint32_t step, replica;
-};
-
-// STRIDED: line (i0, i1) starts at i0 + i1 s_out, elements es apart, i0 < n_in;
-// else lines are consecutive rows, n_lines of them.
-// threads per SM that the register kernels leave room for (128 registers): the
-// fastest of 256 to 1024 at 96^3 to 256^3
-constexpr int kRegOccupancy = 512;
-
-template <int L, bool STRIDED, int IN, bool POWER>
-__global__ void __launch_bounds__(kRegThreads<L>, kRegOccupancy / kRegThreads<L>)
-    k_fft_reg(float2* data, const float* real, int es, int s_out, int n_in, int n_lines,
-              const PowerOut pw, const __grid_constant__ WhiteIn white)
-{
-    constexpr int B = kRegLines<L>, T = kRegThreads<L>, P = STRIDED ? B : B + 1;
-    extern __shared__ __align__(16) unsigned char smraw[];
-    float2* tw = reinterpret_cast<float2*>(smraw);
-    float2* sm = tw + L;
-    const int tid = threadIdx.x, l = tid % B, w = tid / B;
-    fill_twiddles(tw, L, (float2*)nullptr);
-    pdl_wait();
-    __syncthreads();
-    // element offsets fit 32 bits: the field has V < 2^31 sites
-    const int groups = STRIDED ? (n_in + B - 1) / B : 1;
-    const int tasks = STRIDED ? (n_lines / n_in) * groups : (n_lines + B - 1) / B;
-    for (int task = blockIdx.x; task < tasks; task += gridDim.x) {
-        if constexpr (STRIDED) {
-            const int i1 = task / groups, i0 = (task - i1 * groups) * B + l;
-            const bool in = i0 < n_in;
-            const int s0 = (in ? i0 : 0) + i1 * s_out;
-            auto ld = [&](int i) { return data[s0 + i * es]; };
-            if constexpr (POWER) {
-                // the accumulator's values are loaded ahead: one load after another store
-                // to it would wait for memory each (128^3: 28 us)
-                double acc[kRegSlots<L>];
-                reg_fft<L>(tw, sm, P, w, l, ld, [&](int i, int n) { acc[n] = pw.acc ? pw.acc[s0 + i * es] : 0.0; },
-                           [&](int i, float2 v, int n) {
-                               if (!in) return;
-                               const int s = s0 + i * es;
-                               double p = s == 0 ? 0.0 : (double)(norm2(v) * pw.inv);
-                               if (pw.acc) {
-                                   p += acc[n];
-                                   pw.acc[s] = p;
-                                   p *= pw.scale;
-                               }
-                               if (pw.out) pw.out[s] = p;
-                           });
-            } else {
-                reg_fft<L>(tw, sm, P, w, l, ld, [](int, int) {}, [&](int i, float2 v, int) {
-                    if (in) data[s0 + i * es] = v;
-                });
-            }
-        } else {
-            const int r0 = task * B, nl = min(B, n_lines - r0), tot = nl * L;
-            float2* p = data + (long)r0 * L;
-#pragma unroll 4
-            for (int e = tid; e < tot; e += T) {
-                const int row = e / L, j = e - row * L;
-                if constexpr (IN == kInReal)
-                    sm[j * P + row] = make_float2(real[(long)r0 * L + e], 0.f);
-                else if constexpr (IN == kInWhite)
-                    sm[j * P + row] = swift_white<float2>(white.key, (uint32_t)(r0 * L + e), white.step, white.replica);
-                else
-                    sm[j * P + row] = p[e];
-            }
-            __syncthreads();
-            reg_fft<L>(tw, sm, P, w, l, [&](int i) { return sm[i * P + l]; }, [](int, int) {},
-                       [&](int i, float2 v, int) { sm[i * P + l] = v; });
-            __syncthreads();
-#pragma unroll 4
-            for (int e = tid; e < tot; e += T) {
-                const int row = e / L, j = e - row * L;
-                p[e] = sm[j * P + row];
+    struct Table {
+        const RegKernels* of[kRegMax + 1] = {};
+        Table()
+        {
+#define FLB_REG_ENTRY(K) reg_part_##K(),
+            const RegKernels* const part[kRegParts] = {FLB_REG_PARTS(FLB_REG_ENTRY)};
+#undef FLB_REG_ENTRY
+            for (int n = 0; n < kRegLengths; ++n) {
+                const RegKernels* k = part[n % kRegParts] + n / kRegParts;
+                of[k->L] = k;
             }
         }
-        __syncthreads();
-    }
+    };
+    static const Table t;
+    return L >= 0 && L <= kRegMax ? t.of[L] : nullptr;
 }
 
-template <int L, bool STRIDED, int IN, bool POWER>
-static cudaError_t launch_reg(float2* data, const float* real, long es, long s_out, int n_in, long n_lines,
-                                 const PowerOut& pw, const WhiteIn& white, cudaStream_t s)
+// blocks that stay resident keep their twiddles for several groups of lines
+static unsigned reg_grid(const RegKernels& k, long tasks)
 {
-    constexpr int B = kRegLines<L>;
-    const long tasks = STRIDED ? (n_lines / n_in) * ((n_in + B - 1) / B) : (n_lines + B - 1) / B;
-    // blocks that stay resident keep their twiddles for several groups of lines
-    const unsigned grid = (unsigned)std::min<long>(tasks, 152L * (2048 / kRegThreads<L> / 2));
-    return launch_chain_smem(k_fft_reg<L, STRIDED, IN, POWER>, dim3(grid), dim3(kRegThreads<L>),
-                             (L + (size_t)L * (STRIDED ? B : B + 1)) * sizeof(float2), s, data, real, (int)es,
-                             (int)s_out, n_in, (int)n_lines, pw, white);
+    return (unsigned)std::min<long>(tasks, 152L * (2048 / k.threads / 2));
 }
-
-// f(integral_constant<L>) for a length with a register plan; false otherwise.
-template <class F>
-static bool with_reg_length(int L, F&& f)
+static cudaError_t launch_rows(const RegKernels& k, float2* data, const float* real, long n_lines, RowInput in,
+                               const WhiteIn& white, cudaStream_t s)
 {
-    switch (L) {
-    case 32: f(std::integral_constant<int, 32>{}); return true;
-    case 48: f(std::integral_constant<int, 48>{}); return true;
-    case 64: f(std::integral_constant<int, 64>{}); return true;
-    case 96: f(std::integral_constant<int, 96>{}); return true;
-    case 128: f(std::integral_constant<int, 128>{}); return true;
-    case 135: f(std::integral_constant<int, 135>{}); return true;
-    case 192: f(std::integral_constant<int, 192>{}); return true;
-    case 200: f(std::integral_constant<int, 200>{}); return true;
-    case 225: f(std::integral_constant<int, 225>{}); return true;
-    case 243: f(std::integral_constant<int, 243>{}); return true;
-    case 256: f(std::integral_constant<int, 256>{}); return true;
-    case 360: f(std::integral_constant<int, 360>{}); return true;
-    case 384: f(std::integral_constant<int, 384>{}); return true;
-    case 400: f(std::integral_constant<int, 400>{}); return true;
-    case 512: f(std::integral_constant<int, 512>{}); return true;
-    case 1024: f(std::integral_constant<int, 1024>{}); return true;
-    default: return false;
-    }
+    return launch_chain_smem(k.rows, dim3(reg_grid(k, (n_lines + k.lines - 1) / k.lines)), dim3(k.threads),
+                             (k.L + (size_t)k.L * (k.lines + 1)) * sizeof(float2), s, data, real, (int)n_lines, in,
+                             white);
+}
+static cudaError_t launch_strided(const RegKernels& k, bool power, float2* data, long es, long s_out, int n_in,
+                                  int n_out, const PowerOut& pw, cudaStream_t s)
+{
+    return launch_chain_smem(power ? k.power : k.strided,
+                             dim3(reg_grid(k, (long)n_out * ((n_in + k.lines - 1) / k.lines))), dim3(k.threads),
+                             (k.L + (size_t)k.L * k.lines) * sizeof(float2), s, data, (int)es, (int)s_out, n_in,
+                             n_out, pw);
 }
 
 // Direct DFT for lengths with prime factors above 5, accumulated in double.
@@ -715,15 +433,9 @@ static cudaError_t fft_axis(T* data, T* scratch, int L, long es, long s_in, int 
 {
     if (L == 1) return cudaSuccess;
     if constexpr (std::is_same<T, float2>::value) {
-        cudaError_t e = cudaSuccess;
-        const auto go = [&](auto N) {
-            constexpr int LEN = decltype(N)::value;
-            e = es == 1 ? launch_reg<LEN, false, kInComplex, false>(data, nullptr, es, s_out, n_in, (long)n_in * n_out,
-                                                                    PowerOut{}, WhiteIn{}, s)
-                        : launch_reg<LEN, true, kInComplex, false>(data, nullptr, es, s_out, n_in, (long)n_in * n_out,
-                                                                   PowerOut{}, WhiteIn{}, s);
-        };
-        if (with_reg_length(L, go)) return e;
+        if (const RegKernels* k = reg_kernels(L))
+            return es == 1 ? launch_rows(*k, data, nullptr, (long)n_in * n_out, kInComplex, WhiteIn{}, s)
+                           : launch_strided(*k, false, data, es, s_out, n_in, n_out, PowerOut{}, s);
     }
     FftPlan plan;
     const LineGeom g{L, es, s_in, s_out, n_in};
@@ -777,69 +489,20 @@ cudaError_t fft3d(float2* data, int X, int Y, int Z, float2* scratch, cudaStream
 // ---------------------------------------------------------------------------
 // Coloured noise of the modified equilibrium, FP32 (flb_swift.cu has the method)
 // ---------------------------------------------------------------------------
-// The y transform of the columns nx and X - nx, the colouring of every
-// (ny, nx), (-ny, -nx) pair between them, and the y transform of the result, in
-// one pass over the field: H columns and their mirror images per block.  With
-// the white noise drawn into the x transform's rows a step of 1024 x 400 makes
-// three passes instead of six: 82 -> 35 us with the register transforms.
-template <int L>
-__global__ void __launch_bounds__(kRegThreads<L>, kRegOccupancy / kRegThreads<L>)
-    k_swift_columns(const float2* in, float2* __restrict__ out, const float* chol, int X)
-{
-    constexpr int B = kRegLines<L>, H = B / 2;
-    extern __shared__ __align__(16) unsigned char smraw[];
-    float2* tw = reinterpret_cast<float2*>(smraw);
-    float2* sm = tw + L;
-    const int l = threadIdx.x % B, w = threadIdx.x / B;
-    fill_twiddles(tw, L, (float2*)nullptr);
-    pdl_wait();
-    __syncthreads();
-    const int n0 = blockIdx.x * H + (l < H ? l : l - H);
-    const bool valid = n0 <= X / 2;
-    const int n = valid ? n0 : 0, nx = l < H ? n : (n == 0 ? 0 : X - n);  // this line's column
-    const int partner = l < H ? l + H : l - H;
-    reg_fft<L>(tw, sm, B, w, l, [&](int i) { return in[nx + X * i]; }, [](int, int) {},
-               [&](int i, float2 v, int) { sm[i * B + l] = v; });
-    __syncthreads();
-    reg_fft<L>(
-        tw, sm, B, w, l,
-        [&](int i) {
-            const float2 zk = sm[i * B + l], zm = sm[(i == 0 ? 0 : L - i) * B + partner];
-            // E = (Z(k) + conj Z(-k)) / 2, P = (Z(k) - conj Z(-k)) / (2i)
-            const float er = 0.5f * (zk.x + zm.x), ei = 0.5f * (zk.y - zm.y);
-            const float pr = 0.5f * (zk.y + zm.y), pi = -0.5f * (zk.x - zm.x);
-            const float* c = chol + 3 * (nx + X * i);
-            const float c11 = c[0], c21 = c[1], c22 = c[2];
-            // conjugate of E' + i P' = (Er - Pi) + i (Ei + Pr)
-            return make_float2(c11 * er - (c21 * ei + c22 * pi), -(c11 * ei + (c21 * er + c22 * pr)));
-        },
-        [](int, int) {},
-        [&](int i, float2 v, int) {
-            if (valid) out[nx + X * i] = v;
-        });
-}
-
-bool swift_noise_lengths(int X, int Y)
-{
-    return with_reg_length(X, [](auto) {}) && with_reg_length(Y, [](auto) {});
-}
+bool swift_noise_lengths(int X, int Y) { return reg_kernels(X) && reg_kernels(Y); }
 
 cudaError_t swift_noise_fp32(const PhiloxKeys& key, uint32_t step, uint32_t replica, int X, int Y, const float* chol,
                              float2* work, float2* out, cudaStream_t s)
 {
-    cudaError_t e = cudaSuccess;
-    with_reg_length(X, [&](auto N) {
-        e = launch_reg<decltype(N)::value, false, kInWhite, false>(work, nullptr, 1, 0, 0, Y, PowerOut{},
-                                                                   WhiteIn{key, step, replica}, s);
-    });
+    const RegKernels *kx = reg_kernels(X), *ky = reg_kernels(Y);
+    if (!kx || !ky) return cudaErrorInvalidValue;
+    cudaError_t e = launch_rows(*kx, work, nullptr, Y, kInWhite, WhiteIn{key, step, replica}, s);
     if (e != cudaSuccess) return e;
-    with_reg_length(Y, [&](auto N) {
-        constexpr int L = decltype(N)::value, H = kRegLines<L> / 2;
-        e = launch_chain_smem(k_swift_columns<L>, dim3((X / 2 + H) / H), dim3(kRegThreads<L>),
-                              (L + (size_t)L * kRegLines<L>) * sizeof(float2), s, (const float2*)work, out, chol, X);
-    });
+    const int H = ky->lines / 2;
+    e = launch_chain_smem(ky->columns, dim3((X / 2 + H) / H), dim3(ky->threads),
+                          (Y + (size_t)Y * ky->lines) * sizeof(float2), s, (const float2*)work, out, chol, X);
     if (e != cudaSuccess) return e;
-    return fft_axis(out, work, X, 1, X, Y, (long)X * Y, 1, (long)X * Y, s);
+    return launch_rows(*kx, out, nullptr, Y, kInComplex, WhiteIn{}, s);
 }
 
 __global__ void k_complex(const float* in, long V, float2* __restrict__ out)
@@ -895,10 +558,11 @@ cudaError_t spectrum(float2* data, const float* real, int X, int Y, int Z, float
     const PowerOut pw{acc, out, scale, 1.0f / (float)V};
     cudaError_t e = cudaSuccess;
     // x: from the real rows
-    const bool reg_x = with_reg_length(X, [&](auto N) {
-        e = launch_reg<decltype(N)::value, false, kInReal, false>(data, real, 1, 0, 0, (long)Y * Z, pw, WhiteIn{}, s);
-    });
-    if (e != cudaSuccess) return e;
+    const RegKernels* reg_x = reg_kernels(X);
+    if (reg_x) {
+        e = launch_rows(*reg_x, data, real, (long)Y * Z, kInReal, WhiteIn{}, s);
+        if (e != cudaSuccess) return e;
+    }
     if (!reg_x) {
         const long nb = std::min<long>((V + 255) / 256, 152 * 32);
         e = launch_chain(k_complex, dim3((unsigned)nb), dim3(256), s, real, V, data);
@@ -911,13 +575,8 @@ cudaError_t spectrum(float2* data, const float* real, int X, int Y, int Z, float
     for (int a = 0; a <= last; ++a) {
         const long es = a == 0 ? X : (long)X * Y, so = a == 0 ? (long)X * Y : X;
         const int no = a == 0 ? Z : Y;
-        if (a == last) {
-            const bool reg = with_reg_length(axes[a], [&](auto N) {
-                e = launch_reg<decltype(N)::value, true, kInComplex, true>(data, nullptr, es, so, X, (long)X * no, pw,
-                                                                       WhiteIn{}, s);
-            });
-            if (reg) return e;
-        }
+        if (a == last)
+            if (const RegKernels* k = reg_kernels(axes[a])) return launch_strided(*k, true, data, es, so, X, no, pw, s);
         if ((e = fft_axis(data, scratch, axes[a], es, 1, X, so, no, V, s)) != cudaSuccess) return e;
     }
     return power_t<float2>(data, V, acc, out, scale, s);
