@@ -389,8 +389,12 @@ __global__ void __launch_bounds__(128)
 
 // rhobar = rb1 + psi''(rho) mubar - kappa lap(mubar), added to every population
 // (or, with rb_out, stored for the next adjoint step of a segment to add);
-// kappa, A, B gradients.  The kappa gradient -sum mubar lap(rho) is formed as
-// -sum rho lap(mubar): the lattice Laplacian is symmetric.
+// kappa, A, B gradients.  The kappa gradient -sum mubar lap(rho) is formed from the
+// differences along each of the nine velocity pairs, 6 sum_k w_k (mubar(r + c_k) -
+// mubar(r)) (rho(r + c_k) - rho(r)): the lattice Laplacian is symmetric, and no part
+// of a field that is the same everywhere comes in.  (As -sum rho lap(mubar) the
+// rounding of the Laplacian was multiplied by rho - rho0: a fluid at rho0 - 0.5 lost
+// two to three digits.)
 template <class R>
 __global__ void __launch_bounds__(128)
     k_adj_rho(const AdjArgs<R> a, const R* drho, const R* mubar,
@@ -405,14 +409,21 @@ __global__ void __launch_bounds__(128)
         const int s = r.x + a.X * (r.y + a.Y * r.z);
         const Nbhd nb(r.x, r.y, r.z, a.X, a.Y, a.Z);
         const R mb = mubar[s], r0 = drho[s];
-        R ax = R(0), ed = R(0);
+        R ax = R(0), ed = R(0), kax = R(0), ked = R(0);
 #pragma unroll
         for (int i = 1; i < 19; ++i) {
-            const R v = mubar[nb.src(-Vel<L>::cx(i), -Vel<L>::cy(i), -Vel<L>::cz(i))] - mb;
+            const int q = nb.src(-Vel<L>::cx(i), -Vel<L>::cy(i), -Vel<L>::cz(i));
+            const R v = mubar[q] - mb;
             if (i < 7)
                 ax += v;
             else
                 ed += v;
+            if (i & 1) {  // c of the pair (c, -c)
+                if (i < 7)
+                    kax += v * (drho[q] - r0);
+                else
+                    ked += v * (drho[q] - r0);
+            }
         }
         const R lapm = R(1.0 / 3) * ax + R(1.0 / 6) * ed;  // 6 sum_i w_i (..)
         const R d = r0 + a.rho0_minus_rhoc;
@@ -423,9 +434,9 @@ __global__ void __launch_bounds__(128)
         else
 #pragma unroll
             for (int i = 0; i < 19; ++i) lam[(long)i * V + s] += rb;
-        gp[0] = -r0 * lapm;      // kappa
-        gp[1] = mb * d;          // A
-        gp[2] = mb * d * d * d;  // B
+        gp[0] = R(1.0 / 3) * kax + R(1.0 / 6) * ked;  // kappa
+        gp[1] = mb * d;                               // A
+        gp[2] = mb * d * d * d;                       // B
     }
     block_rows<3>(gp, rows + 3 * (long)blockIdx.x);
 }
