@@ -59,10 +59,6 @@ struct AdjArgs {
     R inv_om[3], dln_ns[3];
 };
 
-__device__ __forceinline__ double mad(double a, double b, double c) { return a * b + c; }
-__device__ __forceinline__ F2 mad(F2 a, F2 b, F2 c) { return mk2(__ffma2_rn(a.v, b.v, c.v)); }
-__device__ __forceinline__ F2 mad(float a, F2 b, F2 c) { return mk2(__ffma2_rn(make_float2(a, a), b.v, c.v)); }
-
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 

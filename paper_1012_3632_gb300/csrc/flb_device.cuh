@@ -226,6 +226,13 @@ __device__ __forceinline__ F2& operator*=(F2& a, F2 b)
     return a;
 }
 
+// a b + c in one rounding, as the compiler contracts it for single values: packed
+// products and sums are rounded apart unless this is asked for.
+__device__ __forceinline__ double mad(double a, double b, double c) { return a * b + c; }
+__device__ __forceinline__ float mad(float a, float b, float c) { return a * b + c; }
+__device__ __forceinline__ F2 mad(F2 a, F2 b, F2 c) { return mk2(__ffma2_rn(a.v, b.v, c.v)); }
+__device__ __forceinline__ F2 mad(float a, F2 b, F2 c) { return mk2(__ffma2_rn(make_float2(a, a), b.v, c.v)); }
+
 // reciprocal and square root: the FP32 paths use the SFU approximations (the
 // density is ~1 and the results feed terms far below FP32 storage rounding)
 __device__ __forceinline__ double rcp_(double x) { return 1.0 / x; }
@@ -312,19 +319,19 @@ struct D2Q9 {
     __device__ __forceinline__ static void add_back(const R Dm[9], R g[9])
     {
         const R De = Dm[3], Dw = Dm[4], Dxy = Dm[5], Dqx = Dm[6], Dqy = Dm[7], Dep = Dm[8];
-        g[0] += R(4.0 / 9.0) * (R(2) * (Dep - De));
+        g[0] = mad(R(4.0 / 9.0), (R(2) * (Dep - De)), g[0]);
         const R E1 = De + Dw - R(4) * Dep, O1 = Dm[1] - Dqx;
         const R E2 = De - Dw - R(4) * Dep, O2 = Dm[2] - Dqy;
         const R E3 = R(4) * De + Dxy + R(8) * Dep, O3 = Dm[1] + Dm[2] + R(2) * (Dqx + Dqy);
         const R E4 = R(4) * De - Dxy + R(8) * Dep, O4 = Dm[1] - Dm[2] + R(2) * (Dqx - Dqy);
-        g[1] += R(1.0 / 9.0) * (E1 + O1);
-        g[3] += R(1.0 / 9.0) * (E1 - O1);
-        g[2] += R(1.0 / 9.0) * (E2 + O2);
-        g[4] += R(1.0 / 9.0) * (E2 - O2);
-        g[5] += R(1.0 / 36.0) * (E3 + O3);
-        g[7] += R(1.0 / 36.0) * (E3 - O3);
-        g[8] += R(1.0 / 36.0) * (E4 + O4);
-        g[6] += R(1.0 / 36.0) * (E4 - O4);
+        g[1] = mad(R(1.0 / 9.0), (E1 + O1), g[1]);
+        g[3] = mad(R(1.0 / 9.0), (E1 - O1), g[3]);
+        g[2] = mad(R(1.0 / 9.0), (E2 + O2), g[2]);
+        g[4] = mad(R(1.0 / 9.0), (E2 - O2), g[4]);
+        g[5] = mad(R(1.0 / 36.0), (E3 + O3), g[5]);
+        g[7] = mad(R(1.0 / 36.0), (E3 - O3), g[7]);
+        g[8] = mad(R(1.0 / 36.0), (E4 + O4), g[8]);
+        g[6] = mad(R(1.0 / 36.0), (E4 - O4), g[6]);
     }
 
     // Populations w_i sum_a T_ai D_a of all modes (D_0 included), into g.
@@ -405,7 +412,7 @@ struct D2Q9 {
     // p_ww and p_xy; e and eps take the coloured noise (xe, xp) given per site,
     // the other non-conserved modes their white noise.
     template <class R, class PR>
-    __device__ __forceinline__ static void collide_swift(R g[9], R pex, R gx, R gy, R kappa, R xe, R xp,
+    __device__ __forceinline__ static void collide_swift(R g[9], R pex, R gx, R gy, PR kappa, R xe, R xp,
                                                          const Coll<PR>& P, uint32_t site, uint32_t step)
     {
         R m[9];
@@ -413,11 +420,10 @@ struct D2Q9 {
         const R rho = P.rho0 + m[0];
         const R ir = rcp_(rho);
         const R ux = m[1] * ir, uy = m[2] * ir;
-        const R uxx = ux * ux, uyy = uy * uy;
-        const R eq_e = R(3) * rho * (uxx + uyy) + R(6) * pex;
-        const R eq_w = rho * (uxx - uyy) + kappa * (gx * gx - gy * gy);
-        const R eq_xy = rho * ux * uy + kappa * gx * gy;
-        const R eq_eps = R(-6) * pex;
+        const R uyy = uy * uy, gyy = gy * gy;
+        const R eq_e = mad(R(6), pex, R(3) * rho * mad(ux, ux, uyy));
+        const R eq_w = mad(kappa, mad(gx, gx, R(-1) * gyy), rho * mad(ux, ux, R(-1) * uyy));
+        const R eq_xy = mad(kappa * gx, gy, (rho * ux) * uy);
         R Dm[9];
         Dm[0] = Dm[1] = Dm[2] = R(0);
         Dm[3] = P.rel[0] * (m[3] - eq_e);
@@ -425,17 +431,17 @@ struct D2Q9 {
         Dm[5] = P.rel[2] * (m[5] - eq_xy);
         Dm[6] = P.rel[3] * m[6];
         Dm[7] = P.rel[4] * m[7];
-        Dm[8] = P.rel[5] * (m[8] - eq_eps);
+        Dm[8] = P.rel[5] * mad(R(6), pex, m[8]);  // eq_eps = -6 pex
         if (P.noise) {
             const R sr = P.noise_local ? sqrt_(rho) : R(P.sqrt_rho0);
             R z[8];
             noise_normals<2>(P.key, site, step, P.replica, z);
 #pragma unroll
-            for (int k = 1; k < 5; ++k) Dm[3 + k] += P.ns[k] * (sr * z[k]);
+            for (int k = 1; k < 5; ++k) Dm[3 + k] = mad(P.ns[k], sr * z[k], Dm[3 + k]);
             // the coloured noise is built around rho0: sqrt(rho / rho0) for the local density
             const R sc = sr * rcp_(R(P.sqrt_rho0));
-            Dm[3] += (sc * xe) * R(1.0 / 4.0);   // / N_e
-            Dm[8] += (sc * xp) * R(1.0 / 16.0);  // / N_eps
+            Dm[3] = mad(sc, R(1.0 / 4.0) * xe, Dm[3]);   // / N_e
+            Dm[8] = mad(sc, R(1.0 / 16.0) * xp, Dm[8]);  // / N_eps
         }
         add_back(Dm, g);
     }

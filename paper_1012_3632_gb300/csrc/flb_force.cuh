@@ -492,14 +492,15 @@ __global__ void __launch_bounds__(128)
     F2 ax(0.f), ed(0.f);
 #pragma unroll
     for (int i = 1; i < L::Q; ++i) (i < 5 ? ax : ed) += at(Vel<L>::cx(i), Vel<L>::cy(i)) - rc;
-    const F2 lap = (6.0f / 9.0f) * ax + (6.0f / 36.0f) * ed;  // 6 sum_i w_i (rho_i - rho)
+    const F2 lap = mad(6.0f / 36.0f, ed, (6.0f / 9.0f) * ax);  // 6 sum_i w_i (rho_i - rho)
     const F2 d5 = at(1, 1) - at(-1, -1), d8 = at(1, -1) - at(-1, 1);
-    const F2 gx = (3.0f / 9.0f) * (at(1, 0) - at(-1, 0)) + (3.0f / 36.0f) * (d5 + d8);
-    const F2 gy = (3.0f / 9.0f) * (at(0, 1) - at(0, -1)) + (3.0f / 36.0f) * (d5 - d8);
+    const F2 gx = mad(3.0f / 36.0f, d5 + d8, (3.0f / 9.0f) * (at(1, 0) - at(-1, 0)));
+    const F2 gy = mad(3.0f / 36.0f, d5 - d8, (3.0f / 9.0f) * (at(0, 1) - at(0, -1)));
     const F2 rho = a.c.rho0 + rc, d = rc + a.rho0_minus_rhoc, dd = d * d;
-    const F2 psi = dd * (0.5f * a.A + 0.25f * a.B * dd), psip = d * (a.A + a.B * dd);
-    const F2 pex = rho * psip - psi - (a.pgrad * (1.0f / 3.0f)) * rho - a.kappa * (rho * lap);
-    L::collide_swift(g, pex, gx, gy, F2(a.kappa), ne, np, a.c, (uint32_t)site, a.c.step);
+    const F2 half = mad(0.25f * a.B, dd, F2(0.5f * a.A));  // psi = d^2 half
+    const F2 psip = d * mad(a.B, dd, F2(a.A));
+    const F2 pex = mad(rho, mad(-a.kappa, lap, F2(a.pgrad * (-1.0f / 3.0f))), mad(rho, psip, (-1.0f * dd) * half));
+    L::collide_swift(g, pex, gx, gy, a.kappa, ne, np, a.c, (uint32_t)site, a.c.step);
 #pragma unroll
     for (int i = 0; i < L::Q; ++i) {
         if constexpr (AL) {
