@@ -137,7 +137,8 @@ typedef struct {
     int device;          /* CUDA device ordinal; -1 (default): the current device */
     int check_every;     /* flb_step checks mass/momentum for NaN/Inf every this many
                             steps (0: never; default 0) */
-    int guard;           /* 1: the two population buffers and the density field get
+    int guard;           /* 1: the two population buffers, the density field and the
+                            chemical potential field of a step in passes get
                             64 KiB guard zones of a fixed byte pattern on both sides,
                             checked by flb_check_guards (a bounds check of the
                             kernels' writes for debugging; default 0) */

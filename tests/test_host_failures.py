@@ -77,3 +77,23 @@ num("fake_keep_arg").value = 1                    # the work list of the batch s
 b.step(1)
 assert ctypes.c_void_p.in_dll(fake, "fake_arg").value, "step over no work list"
 """)
+
+
+@pytest.mark.parametrize("field,offset,side", [(2, -1, "before its start"), (2, 256, "after its end"),
+                                               (3, -1, "before its start"), (3, 256, "after its end")])
+def test_fields_of_a_step_in_passes_have_guard_zones_of_their_own(fake, field, offset, side):
+    """Density and chemical potential (64 sites, 256 bytes each; allocations 2 and 3,
+    behind the population buffers): a write past one is not lost in the other."""
+    _run(fake, f"""
+c = Context(19, (4, 4, 4), 1.0, kT=1e-6, free_energy=dict(A=-0.01, B=0.1, rho_c=1.0, kappa=0.02), guard=True)
+c.check_guards()
+base = (ctypes.c_void_p * 256).in_dll(fake, "fake_ptr")[{field}]
+ctypes.memset(base + 65536 + {offset}, 0, 1)
+try:
+    c.check_guards()
+except FLBError as e:
+    assert e.code == -7 and {side!r} in str(e), e   # FLB_EBOUNDS
+    assert {"density field" if field == 2 else "chemical potential field"!r} in str(e), e
+else:
+    sys.exit("the write was not seen")
+""")
