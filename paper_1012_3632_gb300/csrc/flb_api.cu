@@ -670,8 +670,7 @@ int flb_moments(flb_ctx* c, double* out, int which)
         a.n = 0;
         a.rows = c->partials;
         a.lat[0].first = 0;
-        // one warp per block while that leaves SMs without a block
-        const int warps = ((long)((m.X + 31) / 32) * m.Y * m.Z) < 8 * 152 ? 1 : 8;
+        const int warps = flb::mode_warps(m.X, m.Y, m.Z);
         flb::mode_blocks(a, src, m.X, m.Y, m.Z, warps);
         FLB_CUDA(c->ops->mode_sums(a, m.Q, warps, c->stream));
         FLB_CUDA(flb::sum_lattices(a, 2 * m.Q, c->red, c->stream));

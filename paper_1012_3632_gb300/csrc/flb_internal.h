@@ -60,11 +60,17 @@ struct ModeSums {
 constexpr int kModeRowsMin = 512;  // rows that a partial-sum buffer holds at least
 // Append a lattice; returns its blocks.  Sixteen groups of 32 sites per warp and
 // at most six blocks per SM: long enough that the block's own sums do not count.
+// Lattices that give an SM fewer than eight groups go in small blocks, two per SM
+// (mode_warps): a warp per SM left an FP64 one waiting for its own chain of
+// operations, us of the whole call at 32^3 and 31 x 29 x 37, one warp 74 and 81, two
+// 47 and 44, eight 44 and 57 (FP32 42, 34, 33).
+inline int mode_warps(int X, int Y, int Z) { return (long)((X + 31) / 32) * Y * Z < 8 * 152 ? 2 : 8; }
 inline int mode_blocks(ModeSums& a, const void* src, int X, int Y, int Z, int warps)
 {
     const long groups = (long)((X + 31) / 32) * Y * Z, most = 6 * 152;
     long nb = (groups + 16 * warps - 1) / (16 * warps);
-    if (nb < 152) nb = (groups + warps - 1) / warps < 152 ? (groups + warps - 1) / warps : 152;
+    const long least = warps == 8 ? 152 : 2 * 152, one = (groups + warps - 1) / warps;  // <= kModeRowsMin rows
+    if (nb < least) nb = one < least ? one : least;
     if (nb > most) nb = most;
     ModeLattice& q = a.lat[a.n];
     q.src = src;
