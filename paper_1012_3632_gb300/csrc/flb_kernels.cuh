@@ -374,13 +374,18 @@ __global__ void __launch_bounds__(kSitesThreads)
 // SPLIT (FP64, small lattices): a block of four warps steps 32 sites; the first
 // pulls and collides, the others draw the normals meanwhile.
 //
+// LINE: t may have its threads in line (grid_tile).  Single precision is bound by
+// issue slots: with the tile number along one dimension, and idle lanes sent to the
+// first site before they return, BF16 2048 x 2048 took 62.3 us a step, now 54.2,
+// 255^3 478, now 461 to 465.
+//
 // FP64: the FP64 pipe (16 cycles per warp instruction of an SM) where the
 // lattice fills the chip, 64^3 force model 198 us a step (840 before: a column
 // march on 64 blocks that formed densities and mu several times over, normals
 // on the same pipe); below, the latency of one warp's chain of instructions,
 // 32 x 32 5.2 us (15.1 on 4 blocks of 256).
 // ---------------------------------------------------------------------------
-template <class L, class R, class S, bool FORCE, bool TOTAL, bool SPLIT>
+template <class L, class R, class S, bool FORCE, bool TOTAL, bool SPLIT, bool LINE>
 __global__ void __launch_bounds__(kSitesThreads)
     k_sites(const StepArgs<R> a, const __grid_constant__ Planes<S> P, const R* drho,
             const R* mu, const Tiling t)
@@ -389,9 +394,10 @@ __global__ void __launch_bounds__(kSitesThreads)
     __shared__ R zs[SPLIT ? 2 * NPAIR : 1][32];
     pdl_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, X = a.X, Y = a.Y, Z = a.Z;
-    const int3 r = tile_site<1, PLANES, false>(t, SPLIT ? lane : (int)threadIdx.x);
+    const int3 r = grid_tile<1, PLANES, false, LINE>(t, SPLIT ? lane : (int)threadIdx.x);
     const bool in = r.x < X && r.y < Y && r.z < Z;
-    const int x = in ? r.x : 0, y = in ? r.y : 0, z = in ? r.z : 0;  // idle lanes repeat the first site
+    if (!SPLIT && !in) return;
+    const int x = in ? r.x : 0, y = in ? r.y : 0, z = in ? r.z : 0;  // idle lanes of SPLIT repeat the first site
     const int s = x + X * (y + Y * z);
     if constexpr (SPLIT) {
         if (warp > 0) {
@@ -402,7 +408,6 @@ __global__ void __launch_bounds__(kSitesThreads)
             return;
         }
     }
-    if (!SPLIT && !in) return;
     const Nbhd nb(x, y, z, X, Y, Z);
     R g[L::Q];
     pull_planes<L, false>(P, nb, g);

@@ -582,13 +582,14 @@ struct Prec {
         if constexpr (std::is_same<R, double>::value) {
             if (split_sites(m)) {
                 const Tiling t = make_tiling(m.X, m.Y, m.Z, 1, 32, 1);
-                return launch_chain(k_sites<L, R, S, FORCE, TOTAL, true>, dim3(t.blocks()), dim3(kSitesThreads), st, a,
+                return launch_chain(k_sites<L, R, S, FORCE, TOTAL, true, true>, t.grid(), dim3(kSitesThreads), st, a,
                                     pl, drho, mu, t);
             }
         }
         const Tiling t = make_tiling(m.X, m.Y, m.Z, 1, kSitesThreads, L::D == 3 ? 2 : 1);
-        return launch_chain(k_sites<L, R, S, FORCE, TOTAL, false>, dim3(t.blocks()), dim3(kSitesThreads), st, a, pl,
-                            drho, mu, t);
+        const auto k = t.threads ? k_sites<L, R, S, FORCE, TOTAL, false, true>
+                                 : k_sites<L, R, S, FORCE, TOTAL, false, false>;
+        return launch_chain(k, t.grid(), dim3(kSitesThreads), st, a, pl, drho, mu, t);
     }
     // D3Q19 force model, one site per lane: density, mu and collision passes.
     static cudaError_t step_force_sites(const HostModel& m, uint64_t step, const void* src, void* dst, R* drho,
