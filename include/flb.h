@@ -249,11 +249,14 @@ int flb_check_guards(flb_ctx* ctx);
  * sums[4*t + 1..3] = sum_r sum_i f_i c_i (as flb_conservation), t < nsteps.
  * sums: host, 4*nsteps doubles, written when the call returns (it waits for
  * the context's stream once, at the end; device-addressable page-locked
- * memory is written in place by the reduction, other memory through a copy).  The D3Q19 force-model step with
- * FP32 or BF16 storage, even X and the excess free energy forms these sums inside its density pass (per-warp
- * partial sums of the mass deviation and momentum of the pulled populations,
- * those of several steps added up by one launch); every other step runs the
- * reduction of flb_conservation before the step.  Errors as flb_step. */
+ * memory is written in place by the reduction, other memory through a copy).
+ * The D3Q19 force-model step with FP32 or BF16 storage, even X and the excess
+ * free energy forms these sums inside its density pass (per-warp partial sums
+ * of the mass deviation and momentum of the pulled populations); every other
+ * step runs the reduction of flb_conservation before the step.  The sums of up
+ * to 16 steps are added up by one launch, in any case before a check
+ * (check_every): when that stops the run, page-locked memory holds the sums of
+ * the steps before it.  Errors as flb_step. */
 int flb_step_sums(flb_ctx* ctx, int nsteps, double* sums);
 
 /* flb_step_sums without the wait: enqueues the nsteps steps and the delivery
@@ -348,7 +351,7 @@ int flb_kernel_times(flb_ctx* ctx, double* ms, int* launches);
 /* ---- Batched replicas -------------------------------------------------------
  * Up to FLB_BATCH_MAX independent periodic D3Q19 ideal-gas lattices of uneven
  * sizes, advanced together for ensemble averages (the equilibration-ratio
- * statistics of Sec. VI).  Each time step is one persistent kernel launch over
+ * statistics of Sec. VI).  Each time step is one kernel launch over
  * the flattened (replica, tile) work list; steps are replayed from a captured
  * CUDA graph of two steps.  Populations are FP32 deviations.  Replica r uses
  * the Philox key seeds[r] and counter word replica = opt->replica + r, so its

@@ -1,6 +1,7 @@
 // flb_api.cu -- the C ABI declared in include/flb.h: context object, buffer
 // management, step sequencing, observables, checkpoints and error reporting.
-// All compute happens in the kernels of flb_prec.cuh / flb_fft.cu.
+// All compute happens in the kernels of flb_prec.cuh, flb_force.cuh, flb_fft.cu,
+// flb_sums.cu and the files of the models.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -302,6 +303,7 @@ int validate(int lattice, const int dims[3], double om_s, double om_b, double om
     if (o.check_every < 0) return fail(FLB_EINVAL, "check_every must be >= 0");
     if (o.guard != 0 && o.guard != 1) return fail(FLB_EINVAL, "guard must be 0 or 1");
     if (o.z_chunk < 0) return fail(FLB_EINVAL, "z_chunk must be >= 0");
+    // (no launch depends on z_chunk; the values that were refused still are)
     if (o.z_chunk > 0 && (dims[2] + o.z_chunk - 1) / o.z_chunk > 65535)
         return fail(FLB_EINVAL, "z_chunk too small for the launch grid (Z / z_chunk must be <= 65535)");
     if (fe && fe->enabled) {

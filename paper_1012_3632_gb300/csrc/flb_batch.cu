@@ -48,11 +48,6 @@ struct BatchArgs {
 };
 static_assert(sizeof(BatchArgs) < 32000, "batch parameters exceed the kernel parameter space");
 
-// Work item: replica and tile coordinates.
-struct Tile {
-    int r, bx, by, bz;
-};
-
 // 128 threads per tile of tx*ty*tz = 256 sites: one thread per site pair
 // (x, x+1) along x when the replica's X is even (packed FP32 arithmetic, as the
 // single-lattice kernel k_step2), otherwise one site per thread in two passes.

@@ -3,6 +3,10 @@
 // uses.
 #include <utility>
 
+#ifndef FLB_REG_PART
+#define FLB_REG_PART 0
+#endif
+
 #include "flb_fft_reg.cuh"
 
 namespace flb {

@@ -25,7 +25,7 @@ struct NvtxRange {
 };
 #define FLB_TRACE() ::flb::NvtxRange flb_trace_range_(__func__)
 
-// flb_z_chunk's answer for contexts that set no z_chunk of their own.
+// flb_z_chunk's answer for contexts that set no z_chunk of their own (no step has one).
 constexpr int kZChunkDefault = 16;
 
 // Model parameters in double; each instantiation converts to its compute type.

@@ -8,11 +8,12 @@
 // One step (Sec. V, Eq. (lbe-mom)) per site r, fused in one kernel:
 //   pull g_i(r - c_i) -> moments -> relax, force, noise -> back-transform
 //   -> write g*_i(r) into the other buffer.
-// The non-ideal fluid (App. A) first needs rho on a neighbourhood: the density
-// gather kernel writes drho(r) = sum_i g*_i(r - c_i) for every site, and the
-// step kernel stages drho of its tile plus a 2-site halo in shared memory,
-// evaluates mu = psi'(rho) - kappa lap rho on the tile plus a 1-site halo and
-// F = -rho grad mu at each site.
+// The non-ideal fluid (App. A) first needs rho on a neighbourhood, drho(r) =
+// sum_i g*_i(r - c_i), and mu = psi'(rho) - kappa lap rho on a smaller one.  D3Q19:
+// passes over the whole lattice write both fields before the collision reads them
+// (k_density, k_mu_field here; flb_force.cuh for packed storage).  D2Q9 force model:
+// density and mu of a tile with its halo in shared memory, one launch.  D2Q9
+// modified equilibrium: the density field is written first, no mu.
 #pragma once
 
 #include <type_traits>
@@ -225,24 +226,21 @@ Planes<S> make_planes(const void* src, void* dst, int Q, long V)
     return p;
 }
 
-// Pull g_i(r - c_i) through the plane pointers (LAST: last read of these
-// populations in this step).
-template <class L, bool LAST, class R, class S>
+// Pull g_i(r - c_i) through the plane pointers.
+template <class L, class R, class S>
 __device__ __forceinline__ void pull_planes(const Planes<S>& P, const Nbhd& nb, R g[L::Q])
 {
 #pragma unroll
-    for (int i = 0; i < L::Q; ++i) {
-        const S* p = P.src[i] + nb.src(Vel<L>::cx(i), Vel<L>::cy(i), Vel<L>::cz(i));
-        g[i] = LAST ? load_last<R>(p) : load_s<R>(p);
-    }
+    for (int i = 0; i < L::Q; ++i)
+        g[i] = load_s<R>(P.src[i] + nb.src(Vel<L>::cx(i), Vel<L>::cy(i), Vel<L>::cz(i)));
 }
 
 // Cache-hinted FP32 loads (PTX ld.global with an L1 eviction priority and an
-// L2 prefetch size).  stream2/stream1: populations read once per step by the
-// ideal step -- not allocated in L1, the L2 fetches 256-byte sectors.
-// keep4/keep1: the fused non-ideal step's density gather, whose lines the
-// collision of the same tile pulls again two planes later -- kept in L1 with
-// the evict_last priority, 256-byte L2 fetches.
+// L2 prefetch size).  stream2/stream1: populations read once per kernel by the
+// ideal step and the force collision -- not allocated in L1, the L2 fetches
+// 256-byte sectors.  keep4/keep1: the quads of the force model's density pass,
+// whose lines the loads of neighbouring sites (c_x = +-1) touch again -- kept in L1
+// with the evict_last priority, 256-byte L2 fetches.
 __device__ __forceinline__ float2 ld_stream2(const float* p)
 {
     float2 v;
@@ -273,7 +271,7 @@ __device__ __forceinline__ float ld_keep1(const float* p)
 // Storage access of the two-sites-per-thread kernels, FP32 in registers:
 // S = float, or __nv_bfloat16 (a bf16 widens to FP32 exactly by a 16-bit
 // shift; stores round to nearest even, as store_s does).  stream: the ideal
-// step's hints above; keep: the density gather's; plain: the collision's pull.
+// step's hints above; keep: the density pass's; plain: no hint.
 template <class S>
 struct Packed;
 template <>
@@ -410,7 +408,7 @@ __global__ void __launch_bounds__(kSitesThreads)
     }
     const Nbhd nb(x, y, z, X, Y, Z);
     R g[L::Q];
-    pull_planes<L, false>(P, nb, g);
+    pull_planes<L>(P, nb, g);
     R F[3] = {R(0), R(0), R(0)};
     if constexpr (FORCE) {
         if constexpr (std::is_same<R, float>::value) {
@@ -531,7 +529,7 @@ __global__ void __launch_bounds__(TX* TY)
     for (int e = tid; e < RY * RX; e += NT) {
         const Nbhd nh(wrap_any(x0 + e % RX, X), wrap_any(y0 + e / RX, Y), 0, X, Y, 1);
         R g[L::Q], m[L::Q];
-        pull_planes<L, false>(P, nh, g);
+        pull_planes<L>(P, nh, g);
         L::moments(g, m);
         srho[e] = m[0];
     }
@@ -575,7 +573,7 @@ __global__ void __launch_bounds__(TX* TY)
     }
     const Nbhd nb(x, y, 0, X, Y, 1);
     R g[L::Q];
-    pull_planes<L, false>(P, nb, g);
+    pull_planes<L>(P, nb, g);
     const int s = x + X * y;
     L::collide(g, fx, fy, a.c, (uint32_t)s, a.c.step);
 #pragma unroll
@@ -583,12 +581,13 @@ __global__ void __launch_bounds__(TX* TY)
 }
 
 // ---------------------------------------------------------------------------
-// Modified-equilibrium model (Sec. IV.C), D2Q9: the pressure
-// p = p0(rho) - kappa rho lap rho and the square-gradient stress enter the
-// equilibrium (D2Q9::collide_swift); no force.  The density deviation comes
-// from the gather kernel (tile + 1 halo in shared memory), the coloured e/eps
-// noise from swift_noise: xi_e = Re(xi[s]) / V, xi_eps = -Im(xi[s]) / V.
-// p0 = rho psi' - psi (+ rho cs^2 when psi is the excess free energy, pgrad = 0).
+// Modified-equilibrium model (Sec. IV.C), D2Q9 with FP64 storage (the others:
+// k_step_swift2): the pressure p = p0(rho) - kappa rho lap rho and the
+// square-gradient stress enter the equilibrium (D2Q9::collide_swift); no force.
+// The density deviation is read from its field (tile + 1 halo in shared memory), the
+// coloured e/eps noise comes from swift_noise: xi_e = Re(xi[s]) / V, xi_eps =
+// -Im(xi[s]) / V.  p0 = rho psi' - psi (+ rho cs^2 when psi is the excess free
+// energy, pgrad = 0).
 // ---------------------------------------------------------------------------
 template <class R>
 using NoiseField = typename std::conditional<std::is_same<R, double>::value, double2, float2>::type;
@@ -632,18 +631,12 @@ __global__ void __launch_bounds__(TX* TY)
     R xe = R(0), xp = R(0);
     if (a.c.noise) {
         const NoiseField<R> v = xi[s];
-        if constexpr (std::is_same<R, float>::value) {
-            // v / V with 1 / V in two floats: rounded once, and off the FP64 pipe
-            xe = fmaf(v.x, a.inv_v, v.x * a.inv_v_lo);
-            xp = -fmaf(v.y, a.inv_v, v.y * a.inv_v_lo);
-        } else {
-            xe = v.x * a.inv_v;
-            xp = -v.y * a.inv_v;
-        }
+        xe = v.x * a.inv_v;
+        xp = -v.y * a.inv_v;
     }
     const Nbhd nb(x, y, 0, X, Y, 1);
     R g[L::Q];
-    pull_planes<L, false>(P, nb, g);
+    pull_planes<L>(P, nb, g);
     L::collide_swift(g, pex, gx, gy, a.kappa, xe, xp, a.c, (uint32_t)s, a.c.step);
 #pragma unroll
     for (int i = 0; i < L::Q; ++i) store_stream(P.dst[i] + s, g[i]);

@@ -658,12 +658,14 @@ struct Prec {
         if (e != cudaSuccess) return e;
         auto pick = [&](auto E) {
             constexpr bool EARLY = decltype(E)::value;
-            return gx == 1 ? (m.total ? k_force_collide<S, false, true, EARLY, true>
-                                      : k_force_collide<S, false, false, EARLY, true>)
-                   : EARLY || tc.threads ? (m.total ? k_force_collide<S, true, true, EARLY, true>
-                                                    : k_force_collide<S, true, false, EARLY, true>)
-                                         : (m.total ? k_force_collide<S, true, true, EARLY, EARLY>
-                                                    : k_force_collide<S, true, false, EARLY, EARLY>);
+            if (gx == 1)
+                return m.total ? k_force_collide<S, false, true, EARLY, true>
+                               : k_force_collide<S, false, false, EARLY, true>;
+            if constexpr (!EARLY)
+                if (!tc.threads)
+                    return m.total ? k_force_collide<S, true, true, false, false>
+                                   : k_force_collide<S, true, false, false, false>;
+            return m.total ? k_force_collide<S, true, true, EARLY, true> : k_force_collide<S, true, false, EARLY, true>;
         };
         const auto kc = early ? pick(std::true_type{}) : pick(std::false_type{});
         return launch_chain(kc, tc.grid(), dim3(128), st, a, pl, crho, mu, tc);
@@ -818,10 +820,8 @@ struct Prec {
     {
         return m.Q == 19 ? mu_force_l<D3Q19>(m, drho, mu, F, st) : mu_force_l<D2Q9>(m, drho, mu, F, st);
     }
-    // The D2Q9 non-ideal step reads a density field gathered beforehand; the
-    // D3Q19 one gathers the density itself.
-    // a density field written before the step: only the modified-equilibrium
-    // step reads one (the force-model steps gather their density themselves)
+    // a density field written before the step: only the modified-equilibrium step
+    // reads one (the force-model steps form their density themselves)
     static int needs_density(const HostModel& m) { return m.nonideal && m.Q == 9 && m.model == 1 ? 1 : 0; }
     static int site_blocks(const HostModel& m)
     {
