@@ -82,9 +82,8 @@ struct flb_ctx {
 
     void* buf[2] = {nullptr, nullptr};  // post-collision populations of the last step
     int cur = 0;
-    void* drho = nullptr;               // density deviation field (compute type); without guard
-                                        // zones a step in passes has its chemical potential behind it
-    void* mu = nullptr;                 // chemical potential (else)
+    void* drho = nullptr;               // density deviation field (compute type)
+    void* mu = nullptr;                 // chemical potential (steps in passes, observables)
     void* F = nullptr;                  // force field, 3 components (observables)
     double* partials = nullptr;         // per-block reduction rows
     double* red = nullptr;              // reduced columns (device)
@@ -246,9 +245,6 @@ int ensure_partials(flb_ctx* c)
 // Counters of sum_steps (zero between launches), behind the reduced columns.
 unsigned* ticks(flb_ctx* c) { return (unsigned*)(c->red + 64); }
 
-// Byte offset of the chemical potential behind the density field.
-size_t mu_offset(const flb_ctx* c) { return (c->field_bytes() + 255) / 256 * 256; }
-
 // Steps whose warp rows (nrow float4 each) and block sums fit the partial-sum
 // buffer together: at least 4 (nrow <= 4 rows_max), at most kSumStepsMax.
 int step_rows_capacity(const flb_ctx* c, int nrow)
@@ -399,13 +395,10 @@ int flb_create(flb_ctx** out, int lattice, const int dims[3], double omega_shear
     c->sk_count.assign(m.Q, 0);
     c->mv_sum.assign(m.Q, 0.0);
 
-    // one allocation for both fields of a step in passes (flb_create 255 -> 230 us at
-    // 64^3); with guard zones each between its own
-    const bool mu_behind = c->ops->step_in_passes(m) && !c->guard;
     if ((rc = alloc_guarded(c, &c->buf[0], c->pop_bytes(), "population buffer 0")) ||
         (rc = alloc_guarded(c, &c->buf[1], c->pop_bytes(), "population buffer 1")) ||
-        (rc = alloc_guarded(c, &c->drho, (mu_behind ? mu_offset(c) : 0) + c->field_bytes(), "density field")) ||
-        (c->ops->step_in_passes(m) && !mu_behind &&
+        (rc = alloc_guarded(c, &c->drho, c->field_bytes(), "density field")) ||
+        (c->ops->step_in_passes(m) &&
          (rc = alloc_guarded(c, &c->mu, c->field_bytes(), "chemical potential field"))) ||
         (rc = ensure_partials(c))) {
         free_all(c);
@@ -413,7 +406,7 @@ int flb_create(flb_ctx** out, int lattice, const int dims[3], double omega_shear
         return rc;
     }
     if (c->ops->step_in_passes(m)) {
-        m.mu = mu_behind ? (char*)c->drho + mu_offset(c) : c->mu;
+        m.mu = c->mu;
         const cudaError_t ce = cudaMemsetAsync(ticks(c), 0, flb::kSumStepsMax * sizeof(unsigned), c->stream);
         if (ce != cudaSuccess) {
             free_all(c);
@@ -695,12 +688,12 @@ int flb_moments(flb_ctx* c, double* out, int which)
     cudaError_t e = cudaSuccess;
     const void* F = nullptr;
     if (which == FLB_U && m.nonideal && m.model == 0) {
-        if ((!m.mu && (rc = alloc(&c->mu, c->field_bytes()))) || (rc = alloc(&c->F, 3 * c->field_bytes()))) {
+        if ((rc = alloc(&c->mu, c->field_bytes())) || (rc = alloc(&c->F, 3 * c->field_bytes()))) {
             cudaFree(d_out);
             return rc;
         }
         e = c->ops->density(m, src, c->drho, c->stream);
-        if (e == cudaSuccess) e = c->ops->mu_force(m, c->drho, m.mu ? m.mu : c->mu, c->F, c->stream);
+        if (e == cudaSuccess) e = c->ops->mu_force(m, c->drho, c->mu, c->F, c->stream);
         F = c->F;
     }
     if (e == cudaSuccess) e = c->ops->moments(m, src, d_out, which, F, c->stream);
