@@ -27,7 +27,7 @@
 // At 64^3 a launch takes little more than its latency, so that fields which the
 // states of several steps give at once are not a launch per step, neighbours are
 // read once (30 values for mubar, not 90) and the launches are chained: a segment
-// of 20 steps, recomputed and swept back, takes 1.07 ms; with density, mu, force
+// of 20 steps, recomputed and swept back, takes 0.94 ms; with density, mu, force
 // and gradient launches per step and its states pulled apart it took 1.8 ms.
 #include <cuda_runtime.h>
 
