@@ -69,9 +69,9 @@ __device__ __forceinline__ double value_sum(double v, bool) { return v; }
 __device__ __forceinline__ float value_sum(F2 v, bool two) { return two ? v.v.x + v.v.y : v.v.x; }
 
 // d_a = sum_i T_ai w_i l_i: L::moments of w l, the weights (axis pairs 1/18, edge
-// pairs 1/36) taken out of the sums.  (w l first rounds every value once more: error
-// of a step back 7.3e-8, with single values, whose products the compiler
-// contracts, 7.0e-8, so 6.4e-8.)
+// pairs 1/36) taken out of the sums.  (w l first rounds every value once more, for a
+// sum and a difference: error of a step back 7.3e-8, one site per thread 7.0e-8, so
+// 6.4e-8.)
 template <class T>
 __device__ __forceinline__ void weighted_moments(const T l[19], T d[19])
 {

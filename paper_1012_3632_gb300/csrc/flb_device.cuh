@@ -217,10 +217,10 @@ __device__ __forceinline__ F2& operator*=(F2& a, F2 b)
     return a;
 }
 
-// a b + c in one rounding, as the compiler contracts it for single values: packed
-// products and sums are rounded apart unless this is asked for.
+// a b + c in one rounding.  The compiler contracts a packed product with the sum it
+// goes into, but not with a difference, which is itself a fused operation with -1, nor
+// where the product is used twice.
 __device__ __forceinline__ double mad(double a, double b, double c) { return a * b + c; }
-__device__ __forceinline__ float mad(float a, float b, float c) { return a * b + c; }
 __device__ __forceinline__ F2 mad(F2 a, F2 b, F2 c) { return mk2(__ffma2_rn(a.v, b.v, c.v)); }
 __device__ __forceinline__ F2 mad(float a, F2 b, F2 c) { return mk2(__ffma2_rn(make_float2(a, a), b.v, c.v)); }
 
@@ -310,19 +310,19 @@ struct D2Q9 {
     __device__ __forceinline__ static void add_back(const R Dm[9], R g[9])
     {
         const R De = Dm[3], Dw = Dm[4], Dxy = Dm[5], Dqx = Dm[6], Dqy = Dm[7], Dep = Dm[8];
-        g[0] = mad(R(4.0 / 9.0), (R(2) * (Dep - De)), g[0]);
+        g[0] += R(4.0 / 9.0) * (R(2) * (Dep - De));
         const R E1 = De + Dw - R(4) * Dep, O1 = Dm[1] - Dqx;
         const R E2 = De - Dw - R(4) * Dep, O2 = Dm[2] - Dqy;
         const R E3 = R(4) * De + Dxy + R(8) * Dep, O3 = Dm[1] + Dm[2] + R(2) * (Dqx + Dqy);
         const R E4 = R(4) * De - Dxy + R(8) * Dep, O4 = Dm[1] - Dm[2] + R(2) * (Dqx - Dqy);
-        g[1] = mad(R(1.0 / 9.0), (E1 + O1), g[1]);
-        g[3] = mad(R(1.0 / 9.0), (E1 - O1), g[3]);
-        g[2] = mad(R(1.0 / 9.0), (E2 + O2), g[2]);
-        g[4] = mad(R(1.0 / 9.0), (E2 - O2), g[4]);
-        g[5] = mad(R(1.0 / 36.0), (E3 + O3), g[5]);
-        g[7] = mad(R(1.0 / 36.0), (E3 - O3), g[7]);
-        g[8] = mad(R(1.0 / 36.0), (E4 + O4), g[8]);
-        g[6] = mad(R(1.0 / 36.0), (E4 - O4), g[6]);
+        g[1] += R(1.0 / 9.0) * (E1 + O1);
+        g[3] += R(1.0 / 9.0) * (E1 - O1);
+        g[2] += R(1.0 / 9.0) * (E2 + O2);
+        g[4] += R(1.0 / 9.0) * (E2 - O2);
+        g[5] += R(1.0 / 36.0) * (E3 + O3);
+        g[7] += R(1.0 / 36.0) * (E3 - O3);
+        g[8] += R(1.0 / 36.0) * (E4 + O4);
+        g[6] += R(1.0 / 36.0) * (E4 - O4);
     }
 
     // Populations w_i sum_a T_ai D_a of all modes (D_0 included), into g.

@@ -449,9 +449,10 @@ __global__ void __launch_bounds__(TX* TY / 2)
 // Modified-equilibrium step of D2Q9 (k_step_swift), a site pair per thread with
 // the density rows read from the field: no shared tile to wait for.
 // 1024 x 400 FP32: a step with its noise passes 35.3 -> 31.5 us against one site per
-// thread, by fewer instructions and no barrier; 31.0 with products and sums fused
-// (mad), which also keeps the rounding of single values: error against 64 bits
-// 1.06e-7 after 20 steps of 256 x 96, 1.21e-7 without.
+// thread, by fewer instructions and no barrier; 31.0 with the differences of the
+// pressure and the stresses as fused operations (mad), which also keeps the rounding
+// of single values: error against 64 bits 1.06e-7 after 20 steps of 256 x 96, 1.21e-7
+// with the products rounded before they were subtracted.
 template <class S, bool AL>
 __global__ void __launch_bounds__(128)
     k_step_swift2(const StepArgs<float> a, const __grid_constant__ Planes<S> P, const float* drho,

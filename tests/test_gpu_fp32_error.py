@@ -1,6 +1,6 @@
 """FP32 rounding of the kernels that work on two sites at once: no larger than that
-of one site per thread, whose products and sums the compiler contracts.  The bounds
-are the errors against 64 bits that the one-site kernels had on these states."""
+of one site per thread.  The bounds are the errors against 64 bits that the one-site
+kernels had on these states."""
 import math
 
 import numpy as np
